@@ -8,10 +8,13 @@
 //   h^{Y_m}_s = sum_{l=l_m}^{L_m} sum_r K^{Y_m,Omega_l}_{s r} v^{Omega_l}_r (coupling)
 //   f~_j = sum_s L_s^{Y_m}(s_j) h^{Y_m}_s + g_{L_m+1}  (s_j in Y_m),  g_1 (s_j in Y_M)
 //
-// Kernels: k_lap_minmax (interval ends y_1 = max s, xi_1 = max t, validity),
-// k_lap_band (band of every t_k and s_j), k_lap_moments (moments and band sums,
-// deterministic: per-warp tables, warp-ordered group sums, block partials
-// reduced in block order by k_lap_reduce), k_lap_couple (h and g), k_lap_eval.
+// Kernels of a planned transform: k_lap_minmax (interval ends y_1 = max s,
+// xi_1 = max t, validity), k_lap_band (band of every t_k and s_j), and per
+// execute k_lap_moments_cheb, k_lap_reduce_items, k_lap_couple_cheb and
+// k_lap_eval_cheb, which carry the moments and the band functions as Chebyshev
+// sums (the same interpolants, see the note at k_lap_kcheb).  The
+// allocation-free call keeps the barycentric form (k_lap_moments, k_lap_reduce,
+// k_lap_couple, k_lap_eval): it has no plan to hold the tables.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -73,9 +76,8 @@ __global__ void k_lap_band(int64_t n, const double* __restrict__ v, double v1, i
 // for every 32 consecutive t_k it takes, lanes are grouped by band
 // (match_any) and each group's sum is formed in lane order and added by the
 // group's lowest lane, so the result does not depend on scheduling.
-template <typename T, bool BANDS_FROM_VALUES = false>
-__global__ void k_lap_moments(int64_t N, const double* __restrict__ t,
-                              const uint8_t* __restrict__ tband, const T* __restrict__ c,
+template <typename T>
+__global__ void k_lap_moments(int64_t N, const double* __restrict__ t, const T* __restrict__ c,
                               int levels, int q, double xi1, const double* __restrict__ cheb,
                               T* __restrict__ partial) {
     extern __shared__ unsigned char smem_raw[];
@@ -91,7 +93,7 @@ __global__ void k_lap_moments(int64_t N, const double* __restrict__ t,
     for (int64_t ch = (int64_t)blockIdx.x * nw + w; ch < nchunk; ch += (int64_t)gridDim.x * nw) {
         const int64_t k = ch * 32 + lane;
         const bool valid = k < N;
-        const int l = !valid ? 255 : (BANDS_FROM_VALUES ? lap_band(t[k], xi1, levels) : tband[k]);
+        const int l = valid ? lap_band(t[k], xi1, levels) : 255;
         const double cv = valid ? (double)c[k] : 0.0;
         // barycentric denominator on Omega_l (only for interpolated bands)
         double tau = 0.0, inv_den = 1.0;
@@ -135,10 +137,6 @@ __global__ void k_lap_moments(int64_t N, const double* __restrict__ t,
     }
 }
 
-// Largest rank any Laplace plan uses (Algorithm 1: kMaxQ; the generalised
-// algorithm: kGenMaxQ below): the size of the per-element weight arrays.
-constexpr int kLapMaxRank = 64;
-
 // Barycentric weights w_r = lambda_r / (tau - t_r), r < q, with one division:
 // Montgomery's batch inversion (prefix products of d_r = tau - t_r, one
 // reciprocal, a backward sweep), about 3q ulps instead of 1/2 ulp per weight.
@@ -163,77 +161,6 @@ __device__ __forceinline__ bool bary_batch(double tau, int q, const double* __re
         w[r] = cheb[q + r] * ir;
     }
     return true;
-}
-
-// The moments of k_lap_moments for t_k in band order (plan time, a stable
-// sort by band): t, tband sorted, c read through tperm.  A warp's 32 elements
-// then form runs of equal band, so each moment is summed per run by a
-// segmented shuffle scan (5 steps instead of 32) whose last lane adds it to
-// the warp's table; the runs of one chunk have distinct bands, so no two lanes
-// add to one entry and the order stays fixed.  Each weight lambda_r / (tau - t_r)
-// is formed once.
-template <typename T>
-__global__ void k_lap_moments_sorted(int64_t N, const double* __restrict__ t,
-                                     const uint8_t* __restrict__ tband,
-                                     const int32_t* __restrict__ tperm, const T* __restrict__ c,
-                                     int levels, int q, double xi1, const double* __restrict__ cheb,
-                                     T* __restrict__ partial) {
-    extern __shared__ unsigned char smem_raw[];
-    T* tab = reinterpret_cast<T*>(smem_raw);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nw = blockDim.x >> 5;
-    const int row = q + 1;
-    const int entries = (levels + 1) * row;
-    for (int i = threadIdx.x; i < nw * entries; i += blockDim.x) tab[i] = (T)0;
-    __syncthreads();
-    T* mytab = tab + w * entries;
-    const int64_t nchunk = (N + 31) / 32;
-    for (int64_t ch = (int64_t)blockIdx.x * nw + w; ch < nchunk; ch += (int64_t)gridDim.x * nw) {
-        const int64_t k = ch * 32 + lane;
-        const bool valid = k < N;
-        const int l = valid ? tband[k] : 255;       // invalid lanes: a run of their own at the end
-        const double cv = valid ? (double)c[tperm[k]] : 0.0;
-        double tau = 0.0, inv_den = 1.0;
-        double wr[kLapMaxRank];
-        int hit = -1;
-        const bool interp = valid && l < levels;
-        if (interp) {
-            const double a = ldexp(xi1, -l);
-            tau = (t[k] - 1.5 * a) / (0.5 * a);
-            if (bary_batch(tau, q, cheb, wr, &hit)) {
-                double den = 0.0;
-                for (int r = 0; r < q; ++r) den += wr[r];
-                inv_den = 1.0 / den;
-            }
-        }
-        // runs of equal band: s0 = first lane of my run, tail = last lane of it
-        const int lprev = __shfl_up_sync(0xffffffffu, l, 1);
-        const bool head = lane == 0 || lprev != l;
-        const unsigned heads = __ballot_sync(0xffffffffu, head);
-        const int s0 = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-        const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
-        for (int r = 0; r <= q; ++r) {
-            T val = (T)0;
-            if (r == q) {
-                val = (T)cv;
-            } else if (interp) {
-                const double Lr = (hit >= 0) ? (r == hit ? 1.0 : 0.0) : wr[r] * inv_den;
-                val = (T)(Lr * cv);
-            }
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const T x = __shfl_up_sync(0xffffffffu, val, off);
-                if (lane - off >= s0) val += x;
-            }
-            if (valid && tail) mytab[l * row + r] += val;
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < entries; i += blockDim.x) {
-        T s = (T)0;
-        for (int ww = 0; ww < nw; ++ww) s += tab[ww * entries + i];
-        partial[(int64_t)blockIdx.x * entries + i] = s;
-    }
 }
 
 // vS[i] = sum over blocks of partial[b][i]: one warp per entry, lane l summing
@@ -298,46 +225,295 @@ __global__ void k_lap_ktable(int levels, int q, double y1, double xi1, const int
     }
 }
 
-// k_lap_couple with the coupling blocks read from the plan's table (same
-// summation order, so the same h).
-__global__ void k_lap_couple_tab(int levels, int q, const int* __restrict__ ell,
-                                 const int64_t* __restrict__ koff, const double* __restrict__ Kt,
-                                 const double* __restrict__ vS, double* __restrict__ h,
-                                 double* __restrict__ g) {
-    const int m = blockIdx.x + 1;
-    const int row = q + 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        g[levels + 1] = 0.0;
-        for (int l = levels; l >= 1; --l) g[l] = g[l + 1] + vS[l * row + q];
+// Chebyshev form of a planned transform.  On Omega_l the Lagrange weights of
+// the q Chebyshev points are L_r(t) = sum_j C_j(r) T_j(tau), C_j(r) =
+// (2 - [j = 0]) / q T_j(t_r) (discrete orthogonality of the T_j, j < q), and
+// likewise on Y_m, so with
+//   u^{Omega_l}_j = sum_{t_k in Omega_l} T_j(tau_k) c_k   (u_0: the band sum S_l)
+//   K''_{ij} = sum_s sum_r C_i(s) K^{Y_m,Omega_l}_{s r} C_j(r)   (plan time, in place)
+//   a^{Y_m}_i = sum_l sum_j K''_{ij} u^{Omega_l}_j
+// the same interpolant is f~_j = sum_i T_i(sigma_j) a_i + g_{L_m+1}.  An element
+// costs three operations per degree instead of the weights' products, their
+// inversion and a scan over the warp: no division, no exact-hit case.
+__global__ void k_lap_kcheb(int q, double* __restrict__ Kt) {
+    extern __shared__ double ksm[];                 // C (q x q), K (q x q), K C^T (q x q)
+    double *C = ksm, *K = ksm + q * q, *X = ksm + 2 * q * q;
+    double* out = Kt + (int64_t)blockIdx.x * q * q;
+    for (int i = threadIdx.x; i < q * q; i += blockDim.x) {
+        const int j = i / q, r = i % q;
+        C[i] = cospi((double)(j * (2 * r + 1) % (4 * q)) / (2.0 * q)) * ((j ? 2.0 : 1.0) / q);
+        K[i] = out[i];
     }
-    if (m >= levels) return;
-    // one warp per s: lanes stride over the (l, r) terms, a fixed shuffle tree
-    // combines them
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int l0 = ell[m];
-    const int tot = max(levels - m - l0 + 1, 0) * q;
-    const double* K = Kt + koff[m];
-    for (int s = warp; s < q; s += nw) {
-        double acc = 0.0;
-        for (int i = lane; i < tot; i += 32) {
-            const int li = i / q, r = i - li * q;
-            acc += K[((int64_t)li * q + s) * q + r] * vS[(l0 + li) * row + r];
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) h[m * q + s] = acc;
+    __syncthreads();
+    for (int i = threadIdx.x; i < q * q; i += blockDim.x) {
+        const int s = i / q, j = i % q;
+        double a = 0.0;
+        for (int r = 0; r < q; ++r) a += K[s * q + r] * C[j * q + r];
+        X[i] = a;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < q * q; i += blockDim.x) {
+        const int ii = i / q, j = i % q;
+        double a = 0.0;
+        for (int s = 0; s < q; ++s) a += C[ii * q + s] * X[s * q + j];
+        out[i] = a;
     }
 }
 
+// tau_k = (t_k - 3/2 a) / (a/2), a = v1 / 2^band, of every value (0 in the last
+// band): double, or a float pair for the FP32 form, so that an execute needs no
+// FP64 arithmetic per element there.
+template <typename T> struct lap_tau { using type = double; };
+template <> struct lap_tau<float> { using type = ff; };
+template <typename T> using LapTau = typename lap_tau<T>::type;
+
+template <typename T>
+__global__ void k_lap_tau(int64_t n, const double* __restrict__ v, const uint8_t* __restrict__ band,
+                          double v1, int levels, LapTau<T>* __restrict__ tau) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int l = band[i];
+    double x = 0.0;
+    if (l < levels) {
+        const double a = ldexp(v1, -l);
+        x = (v[i] - 1.5 * a) / (0.5 * a);
+    }
+    tau[i] = LapTau<T>(x);
+}
+
+// first[l] = first position of band l among the n bands in ascending order,
+// l = 0 .. levels + 1.
+__global__ void k_lap_starts(int64_t n, const uint8_t* __restrict__ band, int levels, int64_t* __restrict__ first) {
+    const int l = threadIdx.x;
+    if (l > levels + 1) return;
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (band[mid] < l) lo = mid + 1;
+        else hi = mid;
+    }
+    first[l] = lo;
+}
+
+// T_j(tau), j = 0 .. q - 1, handed to f(j, T_j(|tau|)) together with the sign of
+// the odd degrees (T_j(-x) = (-1)^j T_j(x)).  Doubles step the differences
+// d_{j+1} = T_{j+1} - T_j = d_j + 2 (|tau| - 1) T_j, whose rounding grows with j
+// where the three-term recurrence's grows with j^2 near the ends of the
+// interval; in float pairs j^2 2^-48 is far below the FP32 form's rounding, and
+// the plain recurrence on tau itself is cheaper.
+__device__ __forceinline__ float ff_round(ff a) { return a.hi + a.lo; }
+
+// acc[j] += c T_j(tau), j < q <= P.
+template <int P>
+__device__ __forceinline__ void cheb_moments(double tau, double c, int q, double* acc) {
+    const double e = fabs(tau) - 1.0, e2 = 2.0 * e, co = tau < 0.0 ? -c : c;
+    double t = 1.0, d = e;
+    acc[0] += c;
+#pragma unroll
+    for (int j = 1; j < P; ++j) {
+        if (j < q) {
+            if (j > 1) d = fma(e2, t, d);
+            t += d;
+            acc[j] = fma(j & 1 ? co : c, t, acc[j]);
+        }
+    }
+}
+template <int P>
+__device__ __forceinline__ void cheb_moments(ff tau, float c, int q, float* acc) {
+    const ff x2 = ff(2.f * tau.hi, 2.f * tau.lo);
+    ff t0 = ff(1.f), t1 = tau;
+    acc[0] += c;
+#pragma unroll
+    for (int j = 1; j < P; ++j) {
+        if (j < q) {
+            if (j > 1) {
+                const ff t2 = x2 * t1 - t0;
+                t0 = t1;
+                t1 = t2;
+            }
+            acc[j] = fmaf(c, ff_round(t1), acc[j]);
+        }
+    }
+}
+
+// sum_i T_i(tau) a_i, i < q.
+__device__ __forceinline__ double cheb_sum(double tau, const double* __restrict__ a, int q) {
+    const double e = fabs(tau) - 1.0, e2 = 2.0 * e;
+    double t = 1.0, d = e, even = a[0], odd = 0.0;
+    for (int i = 1; i < q; i += 2) {
+        if (i > 1) d = fma(e2, t, d);
+        t += d;
+        odd = fma(a[i], t, odd);
+        if (i + 1 < q) {
+            d = fma(e2, t, d);
+            t += d;
+            even = fma(a[i + 1], t, even);
+        }
+    }
+    return tau < 0.0 ? even - odd : even + odd;
+}
+__device__ __forceinline__ ff cheb_sum(ff tau, const ff* __restrict__ a, int q) {
+    const ff x2 = ff(2.f * tau.hi, 2.f * tau.lo);
+    ff t0 = ff(1.f), t1 = tau, s = a[0];
+    for (int i = 1; i < q; ++i) {
+        s += a[i] * t1;
+        const ff t2 = x2 * t1 - t0;
+        t0 = t1;
+        t1 = t2;
+    }
+    return s;
+}
+
+// Work items of the moments: runs of consecutive elements of one band.
+constexpr int kLapThreads = 256;
+constexpr int kLapMaxPer = 16;     // elements per thread of an item, at most
+struct LapItem {
+    int64_t k0;
+    int count;
+    int band;
+};
+
+__device__ __forceinline__ float lap_shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double lap_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+// Sums v[0 .. 2 H) over the lanes of a warp by halving: in step OFF a lane keeps
+// one half of its values and takes the partner's sums for it, so all P values
+// cost about P exchanges instead of 5 P; at the end lane l holds in v[0 .. P/32)
+// (P >= 32) or v[0] the sums of the entries it kept.
+template <int H, int OFF, typename T> __device__ __forceinline__ void halve_sum(T* v, int lane) {
+    if constexpr (OFF > 0) {
+        if constexpr (H > 0) {
+            const bool up = lane & OFF;
+#pragma unroll
+            for (int i = 0; i < H; ++i) {
+                const T give = up ? v[i] : v[i + H];
+                const T keep = up ? v[i + H] : v[i];
+                v[i] = keep + lap_shfl(give, OFF);
+            }
+        } else {
+            v[0] += lap_shfl(v[0], OFF);
+        }
+        halve_sum<H / 2, OFF / 2>(v, lane);
+    }
+}
+
+// Moments u_j of one item, j < q <= P: each thread sums its elements over the
+// degrees in registers, a halving exchange sums the warp, shared memory the
+// warps, all in a fixed order.  Bound by the FP64 pipe (3 q operations per
+// element, 0.53e12 per second) in the FP64 form; N = 2^16, q = 11: 38.7 us for
+// the barycentric weights and the scan per degree, see k_lap_eval_cheb for what
+// it takes now.  In the FP32 form the recurrence runs in float pairs (N = 10^6:
+// 354 us before).
+template <typename T, int P>
+__global__ void __launch_bounds__(kLapThreads)
+    k_lap_moments_cheb(const LapItem* __restrict__ items, const LapTau<T>* __restrict__ tau,
+                       const int32_t* __restrict__ tperm, const T* __restrict__ c, int levels, int q,
+                       T* __restrict__ partial) {
+    __shared__ T red[kLapThreads / 32][P];
+    const LapItem it = items[blockIdx.x];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int qb = it.band < levels ? q : 1;         // the last band: its sum only
+    T acc[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j) acc[j] = (T)0;
+    for (int e = threadIdx.x; e < it.count; e += kLapThreads) {
+        const int64_t k = it.k0 + e;
+        cheb_moments<P>(tau[k], c[tperm[k]], qb, acc);
+    }
+    halve_sum<P / 2, 16>(acc, lane);
+    // the entry lane l holds in v[i]: bit 16 chose the upper P/2, bit 8 the upper P/4, ...
+    constexpr int R = P >= 32 ? P / 32 : 1;
+    int e0 = 0;
+#pragma unroll
+    for (int h = P / 2, off = 16; off > 0 && h > 0; h >>= 1, off >>= 1)
+        if (lane & off) e0 += h;
+    const bool own = P >= 32 || (lane & (32 / P - 1)) == 0;
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+        if (own) red[w][e0 + i] = acc[i];
+    __syncthreads();
+    if (threadIdx.x < P && threadIdx.x < q) {
+        T s = (T)0;
+        for (int ww = 0; ww < kLapThreads / 32; ++ww) s += red[ww][threadIdx.x];
+        partial[(int64_t)blockIdx.x * q + threadIdx.x] = s;
+    }
+}
+
+// u[l q + j] = sum over the items of band l of partial[item][j]: one warp per
+// entry, the lanes striding over the items, a fixed shuffle tree.
+template <typename T>
+__global__ void k_lap_reduce_items(int levels, int q, const int* __restrict__ first,
+                                   const T* __restrict__ partial, double* __restrict__ u) {
+    const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (i >= (levels + 1) * q) return;               // uniform across the warp
+    const int l = i / q, j = i - l * q;
+    double s = 0.0;
+    for (int b = first[l] + lane; b < first[l + 1]; b += 32) s += (double)partial[(int64_t)b * q + j];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) u[i] = s;
+}
+
+// a^{Y_m}_i = sum_{l = lo(m)}^{hi(m)} sum_j K''(m, l)_{ij} u^{Omega_l}_j, m = blockIdx.x
+// + 1, one warp per i (blockIdx.y: groups of 8), lanes striding over (l, j), a
+// fixed shuffle tree; written as LapTau<T> values.  Algorithm 1 (ell != nullptr):
+// l = l_m .. M - m; the generalised algorithm: l = 1 .. M - 1.  Block (0, 0)
+// also forms g_l = sum_{l' >= l} S_{l'} (S = u_0), g_{levels+1} = 0.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_lap_couple_cheb(int levels, int q, const int* __restrict__ ell, const int64_t* __restrict__ koff,
+                      const double* __restrict__ Kt, const double* __restrict__ u,
+                      LapTau<T>* __restrict__ ha, LapTau<T>* __restrict__ g) {
+    const int m = blockIdx.x + 1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        double s = 0.0;
+        g[levels + 1] = LapTau<T>(0.0);
+        for (int l = levels; l >= 1; --l) {
+            s += u[l * q];
+            g[l] = LapTau<T>(s);
+        }
+    }
+    const int i = blockIdx.y * 8 + warp;
+    if (m >= levels || i >= q) return;
+    const int l0 = ell ? ell[m] : 1, l1 = ell ? levels - m : levels - 1;
+    const int tot = max(l1 - l0 + 1, 0) * q;
+    const double* K = Kt + (ell ? koff[m] : (int64_t)(m - 1) * (levels - 1) * q * q) + i * q;
+    double acc = 0.0;
+    for (int x = lane; x < tot; x += 32) {
+        const int li = x / q, j = x - li * q;
+        acc += K[(int64_t)li * q * q + j] * u[(l0 + li) * q + j];
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if (lane == 0) ha[m * q + i] = LapTau<T>(acc);
+}
+
+// f~_j = sum_i T_i(sigma_j) a_i + g_{L_m+1} (s_j in Y_m), g_1 (s_j in Y_M); the
+// FP32 form in float pairs throughout.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_lap_eval_cheb(int64_t M, const LapTau<T>* __restrict__ sigma, const uint8_t* __restrict__ sband,
+                    int levels, int q, const LapTau<T>* __restrict__ ha, const LapTau<T>* __restrict__ g,
+                    T* __restrict__ f) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= M) return;
+    const int m = sband[j];
+    LapTau<T> v = g[m >= levels ? 1 : levels - m + 1];
+    if (m < levels) v = cheb_sum(sigma[j], ha + m * q, q) + v;
+    if constexpr (sizeof(T) == 4) f[j] = ff_round(v);
+    else f[j] = v;
+}
+
 // f~_j: barycentric weights of s_j on Y_m (double), then sum_s L_s h_s + g_{L_m + 1}.
-template <typename T, bool BANDS_FROM_VALUES = false>
-__global__ void k_lap_eval(int64_t M, const double* __restrict__ sv,
-                           const uint8_t* __restrict__ sband, int levels, int q, double y1,
+template <typename T>
+__global__ void k_lap_eval(int64_t M, const double* __restrict__ sv, int levels, int q, double y1,
                            const double* __restrict__ cheb, const double* __restrict__ h,
                            const double* __restrict__ g, T* __restrict__ f) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= M) return;
-    const int m = BANDS_FROM_VALUES ? lap_band(sv[j], y1, levels) : sband[j];
+    const int m = lap_band(sv[j], y1, levels);
     if (m >= levels) {
         f[j] = (T)g[1];
         return;
@@ -380,7 +556,7 @@ __global__ void k_lap_cheb(int q, double* cheb) {
 // (the example there, y, xi > 0).
 
 constexpr int kGenMaxQ = 64;
-static_assert(kGenMaxQ <= kLapMaxRank && kMaxQ <= kLapMaxRank, "weight arrays of the moments kernel");
+static_assert(kGenMaxQ <= 64 && kMaxQ <= 64, "degrees of k_lap_moments_cheb");
 
 __device__ __forceinline__ double gen_kappa(int kind, double y, double xi) {
     const double x = y * xi;
@@ -402,35 +578,14 @@ __global__ void k_gen_ktable(int kind, int levels, int q, double y1, double xi1,
     }
 }
 
-// h^{Y_m}_s = sum_{l = 1}^{M - 1} sum_r Kt(m, l)_{s r} v^{Omega_l}_r, m = blockIdx.x + 1.
-// One warp per s: lanes stride over the (l, r) terms, a fixed shuffle tree
-// combines them.
-__global__ void k_gen_couple(int levels, int q, const double* __restrict__ Kt,
-                             const double* __restrict__ vS, double* __restrict__ h) {
-    const int m = blockIdx.x + 1, row = q + 1, nb = levels - 1;
-    if (m >= levels) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int tot = nb * q;
-    for (int s = warp; s < q; s += nw) {
-        double acc = 0.0;
-        for (int i = lane; i < tot; i += 32) {
-            const int li = i / q, r = i - li * q;      // l = li + 1
-            acc += Kt[(((int64_t)(m - 1) * nb + li) * q + s) * q + r] * vS[(li + 1) * row + r];
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) h[m * q + s] = acc;
-    }
-}
-
-// f~_j: s_j in Y_m (m < M): sum_s L_s^{Y_m}(s_j) h^{Y_m}_s plus the Omega_M near
+// f~_j: s_j in Y_m (m < M): the Chebyshev sum of the band plus the Omega_M near
 // field sum_{t_k in Omega_M} c_k kappa(s_j, t_k); s_j in Y_M: the direct sum.
 template <typename T, int KIND>
-__global__ void k_gen_eval(int64_t M, const double* __restrict__ sv,
-                           const uint8_t* __restrict__ sband, int levels, int q, double y1,
-                           const double* __restrict__ cheb, const double* __restrict__ h, int64_t N,
-                           const double* __restrict__ t, const T* __restrict__ c,
-                           const int32_t* __restrict__ nearT, int64_t nnear, T* __restrict__ f) {
+__global__ void k_gen_eval(int64_t M, const double* __restrict__ sv, const LapTau<T>* __restrict__ stau,
+                           const uint8_t* __restrict__ sband, int levels, int q,
+                           const LapTau<T>* __restrict__ ha, int64_t N, const double* __restrict__ t,
+                           const T* __restrict__ c, const int32_t* __restrict__ nearT, int64_t nnear,
+                           T* __restrict__ f) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= M) return;
     const int m = sband[j];
@@ -439,18 +594,7 @@ __global__ void k_gen_eval(int64_t M, const double* __restrict__ sv,
     if (m >= levels) {
         for (int64_t k = 0; k < N; ++k) acc += (double)c[k] * gen_kappa(KIND, sj, t[k]);
     } else {
-        const double a = ldexp(y1, -m);
-        const double tau = (sj - 1.5 * a) / (0.5 * a);
-        double den = 0.0, num = 0.0;
-        int hit = -1;
-        for (int s = 0; s < q; ++s) {
-            const double d = tau - cheb[s];
-            if (d == 0.0) hit = s;
-            const double wgt = cheb[q + s] / d;
-            den += wgt;
-            num += wgt * h[m * q + s];
-        }
-        acc = (hit >= 0) ? h[m * q + hit] : num / den;
+        acc = (double)cheb_sum(stau[j], ha + m * q, q);
         for (int64_t i = 0; i < nnear; ++i) {
             const int32_t k = nearT[i];
             acc += (double)c[k] * gen_kappa(KIND, sj, t[k]);
@@ -522,17 +666,14 @@ static bool lap_params(double eps, int q_in, double y1, double xi1, LapParams* P
     return true;
 }
 
-// Launches moments -> reduce -> couple -> eval on `scratch` (layout above),
-// with nblocks moment blocks; the layout reserves partial sums for
-// layout_blocks >= nblocks blocks (0: nblocks).
-template <typename T, bool BANDS_FROM_VALUES = false>
-static cudaError_t lap_run(int64_t N, int64_t M, const double* t, const double* s,
-                           const uint8_t* tband, const uint8_t* sband, const LapParams& P,
-                           const double* cheb, const T* c, T* f, unsigned char* scratch,
-                           int nblocks, cudaStream_t st, Plan* timed,
-                           const double* Kt = nullptr, const int64_t* koff = nullptr,
-                           const int32_t* tperm = nullptr, int layout_blocks = 0) {
-    const LapLayout L = lap_layout(P.levels, P.q, std::max(nblocks, layout_blocks), sizeof(T));
+// The allocation-free call: launches moments -> reduce -> couple -> eval on
+// `scratch` (layout above), with nblocks moment blocks; the layout reserves
+// partial sums for layout_blocks >= nblocks blocks.
+template <typename T>
+static cudaError_t noalloc_run(int64_t N, int64_t M, const double* t, const double* s, const LapParams& P,
+                               const double* cheb, const T* c, T* f, unsigned char* scratch, int nblocks,
+                               int layout_blocks, cudaStream_t st) {
+    const LapLayout L = lap_layout(P.levels, P.q, layout_blocks, sizeof(T));
     const int entries = (P.levels + 1) * (P.q + 1);
     T* partial = (T*)(scratch + L.partial);
     double* vS = (double*)(scratch + L.vS);
@@ -540,40 +681,20 @@ static cudaError_t lap_run(int64_t N, int64_t M, const double* t, const double* 
     double* g = (double*)(scratch + L.g);
     const int* ell = (const int*)(scratch + L.ell);
     const size_t smem = (size_t)kLapWarps * entries * sizeof(T);
-    int slot = -1;
     if (N > 0) {
-        auto kern = k_lap_moments<T, BANDS_FROM_VALUES>;
-        cudaError_t e = tperm ? cudaFuncSetAttribute(k_lap_moments_sorted<T>,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                              : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_lap_moments<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
         if (e != cudaSuccess) return e;
-        if (timed) timer_begin(*timed, "lap_moments", (double)N * (8 + 1 + 4 + sizeof(T)), st, &slot);
-        if (tperm)   // t in band order (plans of fl_plan_laplace)
-            k_lap_moments_sorted<T><<<nblocks, kLapWarps * 32, smem, st>>>(
-                N, t, tband, tperm, c, P.levels, P.q, P.xi1, cheb, partial);
-        else
-            kern<<<nblocks, kLapWarps * 32, smem, st>>>(N, t, tband, c, P.levels, P.q, P.xi1, cheb,
-                                                        partial);
-        if (timed) timer_end(*timed, slot, st);
+        k_lap_moments<T><<<nblocks, kLapWarps * 32, smem, st>>>(N, t, c, P.levels, P.q, P.xi1, cheb, partial);
         k_lap_reduce<T><<<(entries * 32 + 255) / 256, 256, 0, st>>>(nblocks, entries, partial, vS);
     } else {
         cudaError_t e = cudaMemsetAsync(vS, 0, entries * sizeof(double), st);
         if (e != cudaSuccess) return e;
     }
-    if (Kt)
-        k_lap_couple_tab<<<std::max(1, P.levels - 1), 32 * std::min(P.q, 32), 0, st>>>(
-            P.levels, P.q, ell, koff, Kt, vS, h, g);
-    else
-        k_lap_couple<<<std::max(1, P.levels - 1), std::max(32, ((P.q + 31) / 32) * 32), 0, st>>>(
-            P.levels, P.q, P.y1, P.xi1, ell, cheb, vS, h, g);
-    if (M > 0) {
-        if (timed) timer_begin(*timed, "lap_eval", (double)M * (8 + 1 + sizeof(T)), st, &slot);
-        k_lap_eval<T, BANDS_FROM_VALUES><<<(unsigned)((M + 255) / 256), 256, 0, st>>>(
-            M, s, sband, P.levels, P.q, P.y1, cheb, h, g, f);
-        if (timed) timer_end(*timed, slot, st);
-    }
-    if (timed) timed->launches += (N > 0 ? 2 : 0) + 1 + (M > 0 ? 1 : 0);
+    k_lap_couple<<<std::max(1, P.levels - 1), std::max(32, ((P.q + 31) / 32) * 32), 0, st>>>(
+        P.levels, P.q, P.y1, P.xi1, ell, cheb, vS, h, g);
+    if (M > 0)
+        k_lap_eval<T><<<(unsigned)((M + 255) / 256), 256, 0, st>>>(M, s, P.levels, P.q, P.y1, cheb, h, g, f);
     return cudaGetLastError();
 }
 
@@ -585,46 +706,72 @@ static fl_status lap_fail(fl_status s, const std::string& m) { return set_error(
 
 namespace fl {
 
-// Moment tables per block for the generalised algorithm: up to kLapWarps, as
-// many as fit 200 KB of shared memory (0: the tables do not fit).
-static int gen_moment_warps(int entries, size_t tsize) {
-    const size_t per = (size_t)entries * tsize;
-    return (int)std::min<size_t>(kLapWarps, (size_t)(200 * 1024) / per);
+// Scratch of a planned transform: item partials, moments u, band functions a, g.
+struct LapPlanLayout {
+    size_t partial, u, ha, g, ell, first, total;
+};
+
+static LapPlanLayout lap_plan_layout(int levels, int q, int64_t items, size_t tsize) {
+    LapPlanLayout L;
+    size_t off = 0;
+    L.partial = off; off = align256(off + (size_t)items * q * tsize);
+    L.u = off;       off = align256(off + (size_t)(levels + 1) * q * sizeof(double));
+    L.ha = off;      off = align256(off + (size_t)(levels + 1) * q * sizeof(double));
+    L.g = off;       off = align256(off + (size_t)(levels + 2) * sizeof(double));
+    L.ell = off;     off = align256(off + (size_t)(levels + 1) * sizeof(int));
+    L.first = off;   off = align256(off + (size_t)(levels + 2) * sizeof(int));
+    L.total = off;
+    return L;
 }
 
+template <typename T, int P>
+static void lap_moments_launch(Plan& p, const T* c, T* partial, cudaStream_t st) {
+    k_lap_moments_cheb<T, P><<<(unsigned)p.n_lap_items, kLapThreads, 0, st>>>(
+        (const LapItem*)p.d_lapitems, (const LapTau<T>*)p.d_ttau, p.d_tperm, c, p.levels, p.q, partial);
+}
+
+// moments -> reduce -> couple -> eval, both forms of the algorithm.
 template <typename T>
-static cudaError_t gen_run(Plan& p, const T* c, T* f, cudaStream_t st) {
-    const LapLayout L = lap_layout(p.levels, p.q, p.lap_blocks, sizeof(T));
-    const int entries = (p.levels + 1) * (p.q + 1);
+static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
+    const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items, sizeof(T));
     unsigned char* scratch = (unsigned char*)p.d_lap;
     T* partial = (T*)(scratch + L.partial);
-    double* vS = (double*)(scratch + L.vS);
-    double* h = (double*)(scratch + L.h);
-    const int nw = gen_moment_warps(entries, sizeof(T));
-    const size_t smem = (size_t)nw * entries * sizeof(T);
+    double* u = (double*)(scratch + L.u);
+    LapTau<T>* ha = (LapTau<T>*)(scratch + L.ha);
+    LapTau<T>* g = (LapTau<T>*)(scratch + L.g);
+    const int* first = (const int*)(scratch + L.first);
+    const bool gen = p.lap_kernel != 0;
     int slot = -1;
-    if (p.N > 0 && p.levels > 1) {
-        cudaError_t e = cudaFuncSetAttribute(k_lap_moments_sorted<T>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        timer_begin(p, "lap_moments", (double)p.N * (8 + 1 + 4 + sizeof(T)), st, &slot);
-        k_lap_moments_sorted<T><<<p.lap_blocks, nw * 32, smem, st>>>(
-            p.N, p.d_ts, p.d_tbs, p.d_tperm, c, p.levels, p.q, p.xi1, p.d_cheb, partial);
+    if (p.n_lap_items > 0) {
+        timer_begin(p, "lap_moments", (double)p.N * (8 + 4 + sizeof(T)), st, &slot);
+        if (p.q <= 8) lap_moments_launch<T, 8>(p, c, partial, st);
+        else if (p.q <= 16) lap_moments_launch<T, 16>(p, c, partial, st);
+        else if (p.q <= 32) lap_moments_launch<T, 32>(p, c, partial, st);
+        else lap_moments_launch<T, 64>(p, c, partial, st);
         timer_end(p, slot, st);
-        k_lap_reduce<T><<<(entries * 32 + 255) / 256, 256, 0, st>>>(p.lap_blocks, entries, partial, vS);
-        k_gen_couple<<<p.levels - 1, 32 * std::min(p.q, 32), 0, st>>>(p.levels, p.q, p.d_lapK, vS, h);
-        p.launches += 3;
+        ++p.launches;
+    }
+    // (bands without items sum to zero: no elements, no moments)
+    if (!gen || (p.N > 0 && p.levels > 1)) {
+        const int entries = (p.levels + 1) * p.q;
+        k_lap_reduce_items<T><<<(entries * 32 + 255) / 256, 256, 0, st>>>(p.levels, p.q, first, partial, u);
+        const dim3 grid((unsigned)std::max(1, p.levels - 1), (unsigned)((p.q + 7) / 8));
+        k_lap_couple_cheb<T><<<grid, 256, 0, st>>>(p.levels, p.q, gen ? nullptr : (const int*)(scratch + L.ell),
+                                                   p.d_lapKoff, p.d_lapK, u, ha, g);
+        p.launches += 2;
     }
     if (p.M > 0) {
         timer_begin(p, "lap_eval", (double)p.M * (8 + 1 + sizeof(T)), st, &slot);
+        const unsigned grid = (unsigned)((p.M + 255) / 256);
+        const LapTau<T>* sg = (const LapTau<T>*)p.d_stau;
         if (p.lap_kernel == 2)
-            k_gen_eval<T, 2><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
-                p.M, p.d_s, p.d_sband, p.levels, p.q, p.y1, p.d_cheb, h, p.N, p.d_t, c, p.d_nearT,
-                p.n_nearT, f);
+            k_gen_eval<T, 2><<<grid, 256, 0, st>>>(p.M, p.d_s, sg, p.d_sband, p.levels, p.q, ha, p.N, p.d_t, c,
+                                                   p.d_nearT, p.n_nearT, f);
+        else if (p.lap_kernel == 1)
+            k_gen_eval<T, 1><<<grid, 256, 0, st>>>(p.M, p.d_s, sg, p.d_sband, p.levels, p.q, ha, p.N, p.d_t, c,
+                                                   p.d_nearT, p.n_nearT, f);
         else
-            k_gen_eval<T, 1><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
-                p.M, p.d_s, p.d_sband, p.levels, p.q, p.y1, p.d_cheb, h, p.N, p.d_t, c, p.d_nearT,
-                p.n_nearT, f);
+            k_lap_eval_cheb<T><<<grid, 256, 0, st>>>(p.M, sg, p.d_sband, p.levels, p.q, ha, g, f);
         timer_end(p, slot, st);
         p.launches += 1;
     }
@@ -632,23 +779,8 @@ static cudaError_t gen_run(Plan& p, const T* c, T* f, cudaStream_t st) {
 }
 
 cudaError_t run_laplace(Plan& p, const void* c, void* f, cudaStream_t st) {
-    if (p.lap_kernel != 0)
-        return p.prec == FL_FP64 ? gen_run<double>(p, (const double*)c, (double*)f, st)
-                                 : gen_run<float>(p, (const float*)c, (float*)f, st);
-    LapParams P;
-    memset(&P, 0, sizeof(P));
-    P.q = p.q;
-    P.levels = p.levels;
-    P.y1 = p.y1;
-    P.xi1 = p.xi1;
-    for (int m = 1; m < p.levels && m < (int)p.bands.size(); ++m) P.ell[m] = p.bands[m].ell;
-    if (p.prec == FL_FP64)
-        return lap_run<double>(p.N, p.M, p.d_ts, p.d_s, p.d_tbs, p.d_sband, P, p.d_cheb,
-                               (const double*)c, (double*)f, (unsigned char*)p.d_lap, p.lap_blocks,
-                               st, &p, p.d_lapK, p.d_lapKoff, p.d_tperm);
-    return lap_run<float>(p.N, p.M, p.d_ts, p.d_s, p.d_tbs, p.d_sband, P, p.d_cheb, (const float*)c,
-                          (float*)f, (unsigned char*)p.d_lap, p.lap_blocks, st, &p, p.d_lapK,
-                          p.d_lapKoff, p.d_tperm);
+    return p.prec == FL_FP64 ? lap_plan_run<double>(p, (const double*)c, (double*)f, st)
+                             : lap_plan_run<float>(p, (const float*)c, (float*)f, st);
 }
 
 }  // namespace fl
@@ -713,6 +845,84 @@ static cudaError_t sort_t_by_band(Plan& p, cudaStream_t st) {
     return e;   // on failure the plan's destructor frees what was allocated
 }
 
+// Plan time, after sort_t_by_band: tau of the t_k in band order and of the s_j,
+// and the moment items -- runs of up to 256 E elements of one band, E so that
+// the launch has about four items per SM up to E = kLapMaxPer (N = 2^16: 256
+// items of 256 elements, which the FP64 pipes of all SMs share; longer runs
+// only pay once that many items are there).  last: whether the last band is
+// summed too.  The sorted copies of the t_k are released.
+template <typename T>
+static cudaError_t lap_tables(Plan& p, bool last, std::vector<LapItem>* items, std::vector<int>* first,
+                              cudaStream_t st) {
+    items->clear();
+    first->assign(p.levels + 2, 0);
+    cudaError_t e = cudaSuccess;
+    if (p.M > 0) {
+        e = cudaMalloc(&p.d_stau, p.M * sizeof(LapTau<T>));
+        if (e != cudaSuccess) return e;
+        k_lap_tau<T><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(p.M, p.d_s, p.d_sband, p.y1, p.levels,
+                                                                    (LapTau<T>*)p.d_stau);
+    }
+    if (p.N == 0) return cudaGetLastError();
+    e = cudaMalloc(&p.d_ttau, p.N * sizeof(LapTau<T>));
+    int64_t* d_first = nullptr;
+    std::vector<int64_t> start(p.levels + 2);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_first, start.size() * sizeof(int64_t));
+    if (e == cudaSuccess) {
+        k_lap_tau<T><<<(unsigned)((p.N + 255) / 256), 256, 0, st>>>(p.N, p.d_ts, p.d_tbs, p.xi1, p.levels,
+                                                                    (LapTau<T>*)p.d_ttau);
+        k_lap_starts<<<1, FL_MAX_LEVELS + 32, 0, st>>>(p.N, p.d_tbs, p.levels, d_first);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(start.data(), d_first, start.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFree(d_first);
+    if (e != cudaSuccess) return e;
+    cudaFree(p.d_ts);
+    cudaFree(p.d_tbs);
+    p.d_ts = nullptr;
+    p.d_tbs = nullptr;
+    const int64_t per = std::min<int64_t>(kLapMaxPer, std::max<int64_t>(1, p.N / (kLapThreads * 4 * 152)));
+    for (int l = 1; l <= p.levels; ++l) {
+        (*first)[l] = (int)items->size();
+        if (l == p.levels && !last) break;
+        for (int64_t k = start[l]; k < start[l + 1]; k += per * kLapThreads)
+            items->push_back({k, (int)std::min<int64_t>(per * kLapThreads, start[l + 1] - k), l});
+    }
+    (*first)[p.levels + 1] = (int)items->size();
+    return cudaSuccess;
+}
+
+// The plan's scratch with the item starts, the items, and (nk blocks of the
+// coupling table) the table's Chebyshev form.
+static cudaError_t lap_upload(Plan& p, const std::vector<LapItem>& items, const std::vector<int>& first,
+                              const std::vector<int>& ell, int64_t nk, size_t* scratch, cudaStream_t st) {
+    p.n_lap_items = (int64_t)items.size();
+    const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items, p.prec == FL_FP64 ? 8 : 4);
+    *scratch = L.total + items.size() * sizeof(LapItem);
+    cudaError_t e = cudaMalloc(&p.d_lap, L.total);
+    unsigned char* base = (unsigned char*)p.d_lap;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(base + L.first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !ell.empty())
+        e = cudaMemcpyAsync(base + L.ell, ell.data(), ell.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && !items.empty()) {
+        e = cudaMalloc(&p.d_lapitems, items.size() * sizeof(LapItem));
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(p.d_lapitems, items.data(), items.size() * sizeof(LapItem),
+                                cudaMemcpyHostToDevice, st);
+    }
+    if (e == cudaSuccess && nk > 0) {
+        const size_t smem = 3 * (size_t)p.q * p.q * sizeof(double);   // <= 96 KiB (q <= 64)
+        e = cudaFuncSetAttribute(k_lap_kcheb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_lap_kcheb<<<(unsigned)nk, 256, smem, st>>>(p.q, p.d_lapK);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
 static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, int q,
                                    cudaStream_t st) {
     // interval ends and validity
@@ -768,18 +978,16 @@ static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, in
     }
     LAP_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * kMaxQ * sizeof(double)), "cudaMalloc cheb");
     k_lap_cheb<<<1, 64, 0, st>>>(P.q, p.d_cheb);
-    p.lap_blocks = lap_blocks(p.N);
     const size_t tsz = p.prec == FL_FP64 ? 8 : 4;
     if ((size_t)kLapWarps * (P.levels + 1) * (P.q + 1) * tsz > 200 * 1024)
         return lap_fail(FL_EUNSUPPORTED, "fl_plan_laplace: moment tables exceed shared memory "
                                          "(too many levels for this q)");
-    const LapLayout L = lap_layout(P.levels, P.q, p.lap_blocks, p.prec == FL_FP64 ? 8 : 4);
-    LAP_CUDA(cudaMalloc(&p.d_lap, L.total), "cudaMalloc scratch");
-    std::vector<int> ell(P.levels + 1, 0);
+    std::vector<int> ell(P.levels + 1, 0), first;
     for (int m = 1; m < P.levels; ++m) ell[m] = P.ell[m];
-    LAP_CUDA(cudaMemcpyAsync((unsigned char*)p.d_lap + L.ell, ell.data(), ell.size() * sizeof(int),
-                             cudaMemcpyHostToDevice, st),
-             "copy l_m");
+    std::vector<LapItem> items;
+    LAP_CUDA(p.prec == FL_FP64 ? lap_tables<double>(p, true, &items, &first, st)
+                               : lap_tables<float>(p, true, &items, &first, st),
+             "fl_plan_laplace: moment items");
     // coupling blocks K^{Y_m, Omega_l}, l = l_m .. L_m, as a table
     std::vector<int64_t> koff(P.levels + 1, 0);
     int64_t ktot = 0;
@@ -787,20 +995,27 @@ static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, in
         koff[m] = ktot;
         ktot += (int64_t)std::max(0, P.levels - m - P.ell[m] + 1) * P.q * P.q;
     }
+    int* d_ell = nullptr;   // l_m for the table kernel
+    LAP_CUDA(cudaMalloc((void**)&p.d_lapKoff, koff.size() * sizeof(int64_t)), "cudaMalloc coupling offsets");
+    LAP_CUDA(cudaMemcpyAsync(p.d_lapKoff, koff.data(), koff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st),
+             "copy coupling offsets");
     if (ktot > 0) {
         LAP_CUDA(cudaMalloc((void**)&p.d_lapK, ktot * sizeof(double)), "cudaMalloc coupling table");
-        LAP_CUDA(cudaMalloc((void**)&p.d_lapKoff, koff.size() * sizeof(int64_t)), "cudaMalloc coupling offsets");
-        LAP_CUDA(cudaMemcpyAsync(p.d_lapKoff, koff.data(), koff.size() * sizeof(int64_t),
-                                 cudaMemcpyHostToDevice, st),
-                 "copy coupling offsets");
-        k_lap_ktable<<<P.levels - 1, 256, 0, st>>>(P.levels, P.q, y1, xi1,
-                                                   (const int*)((unsigned char*)p.d_lap + L.ell),
-                                                   p.d_lapKoff, p.d_cheb, p.d_lapK);
+        LAP_CUDA(cudaMalloc((void**)&d_ell, ell.size() * sizeof(int)), "cudaMalloc l_m");
+        e = cudaMemcpyAsync(d_ell, ell.data(), ell.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) {
+            k_lap_ktable<<<P.levels - 1, 256, 0, st>>>(P.levels, P.q, y1, xi1, d_ell, p.d_lapKoff, p.d_cheb,
+                                                       p.d_lapK);
+            e = cudaGetLastError();
+        }
     }
-    LAP_CUDA(cudaGetLastError(), "fl_plan_laplace: launch");
-    LAP_CUDA(cudaStreamSynchronize(st), "fl_plan_laplace: synchronise");
+    size_t scratch = 0;
+    if (e == cudaSuccess) e = lap_upload(p, items, first, ell, ktot / (P.q * P.q), &scratch, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the host arrays are released on return
+    cudaFree(d_ell);
+    LAP_CUDA(e, "fl_plan_laplace: tables");
     const size_t ts = p.prec == FL_FP64 ? 8 : 4;
-    p.scratch_bytes = (double)L.total + N * 9.0 + M * 9.0;
+    p.scratch_bytes = (double)scratch + (N + M) * (9.0 + 8.0);
     p.model_bytes = (double)N * (8 + 1 + ts) + (double)M * (8 + 1 + ts);
     return FL_OK;
 }
@@ -875,12 +1090,15 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
     }
     LAP_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * kGenMaxQ * sizeof(double)), "cudaMalloc cheb");
     k_lap_cheb<<<1, kGenMaxQ, 0, st>>>(qq, p.d_cheb);
-    p.lap_blocks = lap_blocks(p.N);
     const size_t tsz = p.prec == FL_FP64 ? 8 : 4;
-    if (gen_moment_warps((levels + 1) * (qq + 1), tsz) < 1)
+    if ((size_t)(levels + 1) * (qq + 1) * tsz > 200 * 1024)
         return lap_fail(FL_EUNSUPPORTED, "fl_plan_kernel: moment tables exceed shared memory");
-    const LapLayout L = lap_layout(levels, qq, p.lap_blocks, tsz);
-    LAP_CUDA(cudaMalloc(&p.d_lap, L.total), "cudaMalloc scratch");
+    std::vector<LapItem> items;
+    std::vector<int> first;
+    LAP_CUDA(p.prec == FL_FP64 ? lap_tables<double>(p, false, &items, &first, st)
+                               : lap_tables<float>(p, false, &items, &first, st),
+             "fl_plan_kernel: moment items");
+    int64_t nk = 0;   // blocks of the coupling table
     // the Omega_M near field: indices of the t_k in the last frequency band
     if (N && levels > 1) {
         std::vector<uint8_t> tb(N);
@@ -896,14 +1114,15 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
                                      cudaMemcpyHostToDevice, st),
                      "copy near field");
         }
-        const int64_t ktot = (int64_t)(levels - 1) * (levels - 1) * qq * qq;
-        LAP_CUDA(cudaMalloc((void**)&p.d_lapK, ktot * sizeof(double)), "cudaMalloc coupling table");
+        nk = (int64_t)(levels - 1) * (levels - 1);
+        LAP_CUDA(cudaMalloc((void**)&p.d_lapK, nk * qq * qq * sizeof(double)), "cudaMalloc coupling table");
         k_gen_ktable<<<levels - 1, 256, 0, st>>>(kind, levels, qq, y1, xi1, p.d_cheb, p.d_lapK);
     }
     LAP_CUDA(cudaGetLastError(), "fl_plan_kernel: launch");
+    size_t scratch = 0;
+    LAP_CUDA(lap_upload(p, items, first, std::vector<int>(), nk, &scratch, st), "fl_plan_kernel: tables");
     LAP_CUDA(cudaStreamSynchronize(st), "fl_plan_kernel: synchronise");
-    p.scratch_bytes = (double)L.total + N * 9.0 + M * 9.0 +
-                      (levels > 1 ? (double)(levels - 1) * (levels - 1) * qq * qq * 8.0 : 0.0);
+    p.scratch_bytes = (double)scratch + (N + M) * (9.0 + 8.0) + (double)nk * qq * qq * 8.0;
     p.model_bytes = (double)N * (8 + 1 + tsz) + (double)M * (8 + 1 + tsz);
     return FL_OK;
 }
@@ -1107,15 +1326,11 @@ fl_status fl_laplace_real_noalloc(int64_t N, int64_t M, const double* t_dev, con
     for (int m = 0; m < FL_MAX_LEVELS; ++m) ea.v[m] = (m < P.levels) ? P.ell[m] : 0;
     k_store_ell<<<1, FL_MAX_LEVELS, 0, st>>>(ea, P.levels + 1, (int*)(lap + L.ell));
     LAP_CUDA(cudaGetLastError(), "fl_laplace_real_noalloc: launch");
-    cudaError_t e;
-    if (prec == FL_FP64)
-        e = lap_run<double, true>(N, M, t_dev, s_dev, nullptr, nullptr, P, cheb, (const double*)c_dev,
-                                  (double*)f_dev, lap, nblocks, st, nullptr, nullptr, nullptr, nullptr,
-                                  kLapMaxBlocks);
-    else
-        e = lap_run<float, true>(N, M, t_dev, s_dev, nullptr, nullptr, P, cheb, (const float*)c_dev,
-                                 (float*)f_dev, lap, nblocks, st, nullptr, nullptr, nullptr, nullptr,
-                                 kLapMaxBlocks);
+    const cudaError_t e =
+        prec == FL_FP64 ? noalloc_run<double>(N, M, t_dev, s_dev, P, cheb, (const double*)c_dev, (double*)f_dev, lap,
+                                              nblocks, kLapMaxBlocks, st)
+                        : noalloc_run<float>(N, M, t_dev, s_dev, P, cheb, (const float*)c_dev, (float*)f_dev, lap,
+                                             nblocks, kLapMaxBlocks, st);
     LAP_CUDA(e, "fl_laplace_real_noalloc");
     return FL_OK;
 }

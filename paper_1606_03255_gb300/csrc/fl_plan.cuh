@@ -269,14 +269,17 @@ struct Plan {
     double* d_t = nullptr;
     double* d_s = nullptr;
     uint8_t* d_tband = nullptr;    // band of every t_k
-    double* d_ts = nullptr;        // the t_k in band order (stable), for the moments
-    uint8_t* d_tbs = nullptr;      // their bands
+    double* d_ts = nullptr;        // planning only: the t_k in band order (stable)
+    uint8_t* d_tbs = nullptr;      // planning only: their bands
+    void* d_ttau = nullptr;        // tau of the t_k in band order (double, or ff in the FP32 form)
+    void* d_stau = nullptr;        // tau of the s_j
+    void* d_lapitems = nullptr;    // moment work items
+    int64_t n_lap_items = 0;
     int32_t* d_tperm = nullptr;    // original index of the k-th t in band order
     uint8_t* d_sband = nullptr;    // band of every s_j
     void* d_lap = nullptr;         // moments and partial sums
-    double* d_lapK = nullptr;      // coupling blocks K^{Y_m, Omega_l} (plan-time table)
+    double* d_lapK = nullptr;      // coupling blocks K^{Y_m, Omega_l} between Chebyshev degrees
     int64_t* d_lapKoff = nullptr;  // offset of band m's blocks in d_lapK
-    int lap_blocks = 0;
     int lap_kernel = 0;            // 0 Algorithm 1 (exp), 1 generalised exp, 2 generalised K_1/2
     int32_t* d_nearT = nullptr;    // generalised Algorithm 1: the t_k in Omega_M
     int64_t n_nearT = 0;

@@ -72,6 +72,26 @@ def test_matches_structured_algorithm1(fl, eps):
     assert oracle.error_E(ref, f, c) <= eps
 
 
+@pytest.mark.parametrize("q", [1, 2, 7, 8, 9, 16, 17, 32, 33, 40])
+@pytest.mark.parametrize("N", [255, 256, 257, 5000])
+def test_ranks_at_the_edges_of_the_moment_kernels(fl, q, N):
+    # the compiled degrees (8, 16, 32, 64) and the 256-element items, against
+    # the same K~ c in numpy: rounding only (a moment of degree j sums values
+    # |T_j c| <= |c| with a few j units of rounding: 64 units cover q = 40
+    # twice over, times the Lebesgue constants (2 + (2/pi) ln q)^2 < 20 of the
+    # two interpolations)
+    c, t, s = W.laplace_inputs(N, 300, seed=40 + q)
+    eps = 1e-6
+    f, info = _run(fl, c, t, s, eps, "fp64", q=q)
+    assert info["q"] == q
+    fs, P = S.laplace_alg1(c, t, s, eps, q=q)
+    assert np.max(np.abs(f - fs)) <= 64 * 20 * 2.0 ** -53 * np.sum(np.abs(c))
+    f32, _ = _run(fl, c.astype(np.float32), t, s, eps, "fp32", q=q)
+    c32 = c.astype(np.float32).astype(np.float64)
+    fs32, _ = S.laplace_alg1(c32, t, s, eps, q=q)
+    assert np.max(np.abs(f32 - fs32)) <= 32 * 20 * U32 * np.sum(np.abs(c32))
+
+
 @pytest.mark.parametrize("N,M", [(1, 1), (31, 5), (32, 33), (33, 1), (1000, 100), (4097, 77),
                                  (0, 10), (10, 0)])
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
