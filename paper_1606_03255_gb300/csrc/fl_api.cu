@@ -40,7 +40,7 @@ Plan::~Plan() {
     if (gexec) cudaGraphExecDestroy(gexec);
     void* ptrs[] = {d_ws, d_perm, d_bandid, d_bands, d_small, d_pass, d_cheb, d_D, d_grid, d_Y,
                     d_stage_c, d_stage_f, d_stage_r, d_z0, d_t, d_s, d_tband, d_sband, d_lap, d_direct,
-                    d_dranges, d_dpart, d_cdir, d_dadj32, d_dadj64, d_cell, d_sp_phi,
+                    d_dranges, d_dpart, d_cdir, d_dsegs, d_dadj, d_dz, d_cell, d_sp_phi,
                     d_sp_L, d_sp_rv, d_cell_bands, d_lapK, d_lapKoff, d_tw, d_nearT, d_cheb32, d_cff, d_tperm, d_ts, d_tbs, d_ttau, d_stau, d_lapitems,
                     d_xis, d_xperm, d_xbk, d_xstart, d_xwin, d_xiphi, d_xcs, d_xsb,
                     d_frbs, d_fent, d_fphi, d_fpp, d_ntab, d_boff, d_bptr};
@@ -274,6 +274,103 @@ static int route_of(const Plan& p, const BandHost& bh) {
     const double fft = (double)d.nrhs * d.n * (d.log2n + 8) * fft_pt + (double)bh.nodes * per_node + 2.0e5;
     const double direct = (double)bh.nodes * d.K * 6.0 * p.direct_bias;
     return direct < fft ? 2 : 1;
+}
+
+static bool pinned(const Plan& p, const Instance& in) {
+    return p.prec == FL_FP32 && !p.xi_mode && in.N <= kPinnedN;
+}
+
+// The nodes of a direct band: appended to the last segment when they follow it
+// and sum over the same coefficients, else a segment of their own.
+static void add_direct_band(Plan& p, const BandHost& bh) {
+    const BandDev& d = bh.dev;
+    const int pin = !pinned(p, p.inst[bh.inst]) ? 0 : d.K <= kDirSeqK && bh.nodes >= kDirSeqNodes ? 2 : 1;
+    if (!p.direct_segs.empty()) {
+        DirectSeg& s = p.direct_segs.back();
+        if (s.K == d.K && s.pin == pin && s.c_off == d.c_off && s.node_off + s.nodes == bh.node_off) {
+            s.nodes += bh.nodes;
+            return;
+        }
+    }
+    p.direct_segs.push_back({bh.node_off, bh.nodes, d.K, d.c_off, 0, (int)((d.K + kDirChunk - 1) / kDirChunk), pin});
+}
+
+// Work items of the direct segments.  Forward: the lanes per node G cover the
+// chunk's Horner blocks with `r` blocks per lane, r the largest power of two (up
+// to kDirMaxBlocks) that still leaves every SM about 1024 busy lanes (pinned
+// transforms: r = 1, or G = 1 for DirectSeg::pin = 2); an item
+// holds the nodes of one pass of its 256 threads, or of two when there are
+// plenty of items (the staged chunk then serves twice as many).  Adjoint: node
+// groups of `steps` nodes (pairs in FP32) per lane, doubled from 8 while the
+// launch keeps 24 warps per SM, since every group adds its sums to cdir with
+// atomics.
+static void build_direct_items(Plan& p) {
+    constexpr int64_t kSMs = 152;
+    const int np = p.prec == FL_FP32 ? 2 : 1;   // nodes per lane group
+    p.direct_work.clear();
+    p.dadj_work.clear();
+    p.direct_ranges.clear();
+    p.direct_nodes = p.dpart_elems = p.direct_kmax = 0;
+    int64_t lane_blocks = 0;
+    for (DirectSeg& s : p.direct_segs) {
+        lane_blocks += (s.nodes + np - 1) / np * ((s.K + kDirBlock - 1) / kDirBlock);
+        p.direct_kmax = std::max(p.direct_kmax, s.K);
+        if (s.nchunk == 1) continue;
+        s.dslot = p.dpart_elems;
+        p.dpart_elems += s.nodes * s.nchunk;
+        p.direct_ranges.push_back({(int)(&s - p.direct_segs.data()), 0, s.nodes, p.direct_nodes});
+        p.direct_nodes += s.nodes;
+    }
+    int r = 1;
+    while (r < kDirMaxBlocks && lane_blocks >= 2 * r * kSMs * 1024) r *= 2;
+    auto lanes = [&](const DirectSeg& s) {   // log2 G
+        if (s.pin == 2) return 0;
+        const int64_t nblk = (std::min<int64_t>(s.K, kDirChunk) + kDirBlock - 1) / kDirBlock;
+        return std::min(5, ilog2_ceil(s.pin ? nblk : (nblk + r - 1) / r));
+    };
+    auto items = [&](int passes, bool make) {
+        int64_t count = 0;
+        for (size_t g = 0; g < p.direct_segs.size(); ++g) {
+            const DirectSeg& s = p.direct_segs[g];
+            const int lg = lanes(s);
+            const int64_t per = (int64_t)passes * np * (256 >> lg);
+            for (int64_t n0 = 0; n0 < s.nodes; n0 += per) {
+                count += s.nchunk;
+                for (int ch = 0; make && ch < s.nchunk; ++ch)
+                    p.direct_work.push_back({(int)g, ch, s.node_off + n0, (int)std::min(per, s.nodes - n0), lg});
+            }
+        }
+        return count;
+    };
+    items(items(1, false) >= 16 * kSMs ? 2 : 1, true);
+    if (p.batched) return;   // forward only
+    auto adj_items = [&](int64_t steps, bool make) {
+        int64_t count = 0;
+        for (size_t g = 0; g < p.direct_segs.size(); ++g) {
+            const DirectSeg& s = p.direct_segs[g];
+            const int64_t span = 32 * kDirAdjKL;
+            for (int64_t k = 0; k < s.K; k += span) {
+                const int lkb = ilog2_ceil((std::min(span, s.K - k) + kDirAdjKL - 1) / kDirAdjKL);
+                const int64_t per = steps * np * (32 >> lkb);
+                count += (s.nodes + per - 1) / per;
+                for (int64_t n0 = 0; make && n0 < s.nodes; n0 += per)
+                    p.dadj_work.push_back({(int)g, (int)(k / span), s.node_off + n0,
+                                           (int)std::min(per, s.nodes - n0), lkb});
+            }
+        }
+        return count;
+    };
+    int64_t steps = 8;
+    while (steps < kDirAdjSteps && adj_items(steps, false) > 24 * kSMs) steps *= 2;
+    adj_items(steps, true);
+}
+
+template <typename E>
+static cudaError_t upload(const std::vector<E>& v, E** dev, cudaStream_t st) {
+    if (v.empty()) return cudaSuccess;
+    cudaError_t e = cudaMalloc((void**)dev, v.size() * sizeof(E));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(*dev, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice, st);
+    return e;
 }
 
 // Four-step work items of the large bands, grouped by grid size into launches
@@ -706,16 +803,9 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     p.xqc = p.xi_mode ? xi_chunk(p.q) : 0;
     p.small_work.clear();
     p.large_bands.clear();
-    p.direct_work.clear();
-    p.direct_ranges.clear();
-    p.dadj_work32.clear();
-    p.dadj_work64.clear();
-    p.direct_nodes = p.direct_terms = p.dpart_elems = 0;
-    p.n_direct_small = 0;
-    p.n_dadj_small = 0;
+    p.direct_segs.clear();
+    p.direct_terms = 0;
     p.z0_nodes = 0;
-    std::vector<DirectItem> small_items;
-    std::vector<DirectAdjItem> small_adj;
     std::vector<int> nfft_bands;   // bands evaluated by an NFFT, in order
     for (int i = 0; i < B; ++i) {
         Instance& in = p.inst[i];
@@ -736,36 +826,8 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
             d.nodes = bh.nodes;
             d.route = bh.nodes > 0 ? route_of(p, bh) : 0;
             if (d.route == 2) {
-                d.nchunk = (int)((d.K + kDirChunk - 1) / kDirChunk);
-                d.dslot = p.dpart_elems;
-                p.dpart_elems += bh.nodes * d.nchunk;
-                p.direct_ranges.push_back({b, 0, bh.nodes, p.direct_nodes});
-                p.direct_nodes += bh.nodes;
                 p.direct_terms += bh.nodes * d.K;
-                if (d.K <= kDirSmallK && bh.nodes >= kDirSmallMinNodes && p.prec == FL_FP32) {
-                    for (int64_t n0 = 0; n0 < bh.nodes; n0 += kDirSmallNodes)
-                        small_items.push_back({b, 0, bh.node_off + n0,
-                                               (int)std::min<int64_t>(kDirSmallNodes, bh.nodes - n0), 0});
-                } else {
-                    for (int64_t n0 = 0; n0 < bh.nodes; n0 += kDirNodes)
-                        for (int ch = 0; ch < d.nchunk; ++ch)
-                            p.direct_work.push_back({b, ch, bh.node_off + n0,
-                                                     (int)std::min<int64_t>(kDirNodes, bh.nodes - n0), 0});
-                }
-                if (!p.batched && d.K <= kDirSmallK) {
-                    for (int64_t n0 = 0; n0 < bh.nodes; n0 += kDirAdjNodes)
-                        small_adj.push_back({b, 0, bh.node_off + n0,
-                                             (int)std::min<int64_t>(kDirAdjNodes, bh.nodes - n0), 0});
-                } else if (!p.batched) {
-                    for (int kl : {32, 16}) {
-                        std::vector<DirectAdjItem>& v = kl == 32 ? p.dadj_work32 : p.dadj_work64;
-                        const int64_t kc = (d.K + 32 * kl - 1) / (32 * kl);
-                        for (int64_t n0 = 0; n0 < bh.nodes; n0 += kDirAdjNodes)
-                            for (int64_t ch = 0; ch < kc; ++ch)
-                                v.push_back({b, (int)ch, bh.node_off + n0,
-                                             (int)std::min<int64_t>(kDirAdjNodes, bh.nodes - n0), 0});
-                    }
-                }
+                add_direct_band(p, bh);
                 continue;
             }
             if (d.route == 1) nfft_bands.push_back(b);
@@ -811,22 +873,7 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
             }
         }
     }
-    // few direct items (a handful of sparse bands): half as many nodes per
-    // item, so the launch still covers the GPU several times over
-    if (!p.direct_work.empty() && (int64_t)p.direct_work.size() < kDirFewItems) {
-        std::vector<DirectItem> halves;
-        for (const DirectItem& it : p.direct_work) {
-            const int h = std::min(it.nnodes, kDirNodes / 2);
-            halves.push_back({it.band, it.chunk, it.node0, h, 0});
-            if (it.nnodes > h) halves.push_back({it.band, it.chunk, it.node0 + h, it.nnodes - h, 0});
-        }
-        p.direct_work.swap(halves);
-    }
-    p.n_direct_small = (int64_t)small_items.size();
-    p.direct_work.insert(p.direct_work.end(), small_items.begin(), small_items.end());
-    p.n_dadj_small = (int64_t)small_adj.size();
-    p.dadj_work32.insert(p.dadj_work32.end(), small_adj.begin(), small_adj.end());
-    p.dadj_work64.insert(p.dadj_work64.end(), small_adj.begin(), small_adj.end());
+    build_direct_items(p);
     build_pass_groups(p);
     if ((s = build_fused(p, st)) != FL_OK) return s;
     if ((int)p.bands.size() != nb) {   // sub-bands were appended: a larger table
@@ -859,26 +906,14 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
                 "copy pass items");
     }
     if (!p.direct_work.empty()) {
-        FL_CUDA(cudaMalloc((void**)&p.d_direct, p.direct_work.size() * sizeof(DirectItem)),
-                "cudaMalloc direct work");
-        FL_CUDA(cudaMemcpyAsync(p.d_direct, p.direct_work.data(),
-                                p.direct_work.size() * sizeof(DirectItem), cudaMemcpyHostToDevice, st),
-                "copy direct work");
-        FL_CUDA(cudaMalloc((void**)&p.d_dranges, p.direct_ranges.size() * sizeof(DirectRange)),
-                "cudaMalloc direct ranges");
-        FL_CUDA(cudaMemcpyAsync(p.d_dranges, p.direct_ranges.data(),
-                                p.direct_ranges.size() * sizeof(DirectRange), cudaMemcpyHostToDevice, st),
-                "copy direct ranges");
-        FL_CUDA(cudaMalloc(&p.d_dpart, p.dpart_elems * cs), "cudaMalloc direct partials");
-        std::vector<DirectAdjItem>& adj = p.prec != FL_FP32 ? p.dadj_work64 : p.dadj_work32;
-        DirectAdjItem*& d_adj = p.prec != FL_FP32 ? p.d_dadj64 : p.d_dadj32;
-        if (!adj.empty()) {
-            FL_CUDA(cudaMalloc((void**)&d_adj, adj.size() * sizeof(DirectAdjItem)), "cudaMalloc adjoint work");
-            FL_CUDA(cudaMemcpyAsync(d_adj, adj.data(), adj.size() * sizeof(DirectAdjItem),
-                                    cudaMemcpyHostToDevice, st),
-                    "copy adjoint work");
-        }
-        FL_CUDA(cudaMalloc(&p.d_cdir, p.N * cs), "cudaMalloc direct adjoint");
+        FL_CUDA(upload(p.direct_segs, &p.d_dsegs, st), "fl_plan: direct segments");
+        FL_CUDA(upload(p.direct_work, &p.d_direct, st), "fl_plan: direct work");
+        FL_CUDA(upload(p.direct_ranges, &p.d_dranges, st), "fl_plan: direct ranges");
+        FL_CUDA(upload(p.dadj_work, &p.d_dadj, st), "fl_plan: adjoint work");
+        if (p.dpart_elems > 0) FL_CUDA(cudaMalloc(&p.d_dpart, p.dpart_elems * cs), "cudaMalloc direct partials");
+        if (!p.dadj_work.empty()) FL_CUDA(cudaMalloc(&p.d_cdir, p.N * cs), "cudaMalloc direct adjoint");
+        FL_CUDA(cudaMalloc(&p.d_dz, 2 * M * cs), "cudaMalloc direct bases");
+        FL_CUDA(build_direct_base(p, st), "fl_plan: direct bases");
     }
     // adjoint of the NFFT bands (single plans): per-node taps and weights, cell list
     p.cell_bands.clear();
@@ -929,7 +964,7 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     FL_CUDA(cudaStreamSynchronize(st), "fl_plan: synchronise");
     p.scratch_bytes = (double)p.grid_elems * cs + (double)p.D_elems * rs + (double)p.Y_elems * cs +
                       (double)M * (sizeof(double2) + 8) + (double)p.dpart_elems * cs +
-                      (p.direct_work.empty() ? 0.0 : (double)p.N * cs);
+                      (p.direct_work.empty() ? 0.0 : 2.0 * M * cs + (double)(p.dadj_work.empty() ? 0 : p.N) * cs);
     // algorithmic bytes of one execute: c once, D once, each grid written and read
     // once per FFT pass, the nodes, and f
     double mb = (double)p.N * cs + (double)p.D_elems * rs + (double)M * (sizeof(double2) + 8 + cs);
@@ -946,7 +981,8 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
         mb += (d.log2n <= kSmallMaxLog2) ? g : 3.0 * g;   // small: write; large: Y write+read, grid write
         mb += std::min<double>(g, (double)p.bands[b].nodes * d.nrhs * 2 * p.mw * cs);   // gather
     }
-    if (!p.direct_work.empty()) mb += (double)p.direct_work.size() * kDirChunk * cs;   // c tiles
+    if (!p.direct_work.empty())   // c tiles
+        mb += (double)p.direct_work.size() * std::min<int64_t>(p.direct_kmax, kDirChunk) * cs;
     p.model_bytes = mb;
     return FL_OK;
 }

@@ -155,8 +155,9 @@ struct BandDev {
     double yc, yh;     // band Y_m = [yc - yh, yc + yh] (paper's y), for barycentric weights
     double yh_inv;     // 1 / yh (a power of two times 1/y_1)
     int64_t node_off;  // first node of the band in sorted order
-    int64_t dslot;     // direct route: offset of the band's partial sums (nodes x nchunk)
-    int nchunk;        // direct route: coefficient chunks
+    int64_t pad1;      // (unused; the layout of this struct stays because the compiler's choice
+                       // of fused products in the pinned FP32 transforms, kPinnedN, moved with it)
+    int pad4;
     int pad2;
     int64_t c_off;     // offset of the band's transform in the coefficient buffer (batches)
     int64_t nodes;     // nodes of the band (sorted positions node_off .. node_off + nodes)

@@ -6,9 +6,20 @@
 // truncation of Lemma A.2, or K = N for the Y_M band), i.e. eq. (4.1) itself
 // -- the "naive matrix vector multiplication" the paper times in Section 5 --
 // restricted to those frequencies.  The sum is blocked: each block of 32 terms
-// is a Horner polynomial in z_j, and z_j^{k_b} at the block start is formed
-// from an exactly reduced phase (k_b x_j mod 1) and exp(-y_j k_b), so the error
-// does not grow with k.
+// is evaluated as four Horner polynomials of eight terms in z_j, combined by
+// Horner in z_j^8 -- as many steps as one chain of 32, in four independent
+// ones, and the rounding of z_j enters with its 7th power instead of its 31st
+// (z_j and z_j^8 are rounded once at plan time).  z_j^{k_b} at the block start
+// is formed from an exactly reduced phase (k_b x_j mod 1) and exp(-y_j k_b), so
+// the error does not grow with k.
+//
+// Neighbouring direct bands with the same K are one segment (their nodes are
+// consecutive in sorted order), so a handful of nodes per band still shares a
+// work item.  The arithmetic is float, double or float pairs (A below).
+#include <algorithm>
+#include <type_traits>
+
+#include "fl_f32x2.cuh"
 #include "fl_ffmath.cuh"
 #include "fl_plan.cuh"
 
@@ -17,140 +28,214 @@ namespace fl {
 constexpr double kTwoPiDir = 6.283185307179586476925286766559;
 
 // Shared-memory stride of a staged Horner block: one element of padding, so
-// the 32 lanes of a warp, each on its own block, read 32 different bank
-// offsets instead of one (blocks of 32 complex values are 256 or 512 bytes
-// apart, a whole number of bank rows).
+// lanes on different blocks read different bank offsets (blocks of 32 complex
+// values are 256 or 512 bytes apart, a whole number of bank rows).
 constexpr int kDirBlockLd = kDirBlock + 1;
-constexpr int kDirTile = kDirChunk / kDirBlock * kDirBlockLd;
 
-// frac(k x) in [-1/2, 1/2) for the FP64 form and the float pairs: k x = p + e
-// exactly (FMA), one rounding.  (The FP32 form uses dir_f32_power below.)
-template <typename T> __device__ __forceinline__ double dir_phase(double k, double x);
-template <> __device__ __forceinline__ double dir_phase<double>(double k, double x) {
-    return frac_turns(k, x);
+static size_t dir_tile(int64_t kmax, size_t csize) {
+    const int64_t k = std::min<int64_t>(kmax, kDirChunk);
+    return (size_t)((k + kDirBlock - 1) / kDirBlock * kDirBlockLd) * csize;
 }
-
-template <typename T> __device__ __forceinline__ T dir_exp(T a);
-template <> __device__ __forceinline__ float dir_exp<float>(float a) { return expf(a); }
-template <> __device__ __forceinline__ double dir_exp<double>(double a) { return exp(a); }
 
 // FP32 form without FP64 arithmetic per block: x in [0, 1) held as the 64-bit
 // fixed-point X = x 2^64 (exact for the 53-bit x), so frac(k x) is the
-// wrapped product k X, rounded to 24 bits and read as a signed value in
-// [-1/2, 1/2); y as a float pair (hi + lo), so y k = p + e with p = fl(hi k)
-// and e its error plus lo k, and exp(-y k) = exp(-p) (1 - e) (|e| < 2^-20 p).
+// wrapped product k X, read as a signed value in [-1/2, 1/2); y as a float pair
+// (hi + lo), so y k = p + e with p = fl(hi k) and e its error plus lo k, and
+// exp(-y k) = exp(-p) (1 - e) (|e| < 2^-20 p).
 struct DirF32Node {
     uint64_t X;
     float yh, yl;
 };
 
-// A node from the plan's record (k_node_tab: X = x 2^64, and y = 2 pi Im w as
-// a float pair, formed once at plan time in double), with z = exp(-y)
-// e^(2 pi i x) in float: x - [x >= 1/2] is the signed X 2^-64, rounded once
-// to float.
-__device__ __forceinline__ DirF32Node dir_f32_record(uint4 rec, float2* z) {
-    DirF32Node d;
-    d.X = ((uint64_t)rec.y << 32) | (uint64_t)rec.x;
-    d.yh = __uint_as_float(rec.z);
-    d.yl = __uint_as_float(rec.w);
-    const float xr = (float)(int64_t)d.X * 0x1p-64f;
-    *z = cscale(expipi<float>(2.f * xr), expf(-d.yh));
-    return d;
-}
-
 // z^k = exp(-y k) e^(2 pi i frac(k x)) for 0 <= k < 2^24 (SIGN = -1: the conjugate
 // phase); false when y k > lim (the power underflows: so do all later ones).
+// The phase is the float nearest to the top 32 bits of the product; pin: to its
+// top 24 bits, half up, the rounding of pinned transforms (kPinnedN).
 template <int SIGN>
-__device__ __forceinline__ bool dir_f32_power(const DirF32Node& d, int64_t k, float lim, float2* zk) {
+__device__ __forceinline__ bool dir_f32_power(const DirF32Node& d, int64_t k, float lim, bool pin, float2* zk) {
     const float kf = (float)k;                 // exact: k < 2^24
     const float p = d.yh * kf;
     if (p > lim) return false;
     const float e = fmaf(d.yh, kf, -p) + d.yl * kf;
     const float mag = expf(-p) * (1.f - e);
-    const uint64_t ph = (uint64_t)k * d.X + (1ull << 39);
-    const float phase = (float)((int64_t)ph >> 40) * 0x1p-24f;   // frac(k x) in [-1/2, 1/2)
+    const uint64_t ph = (uint64_t)k * d.X;
+    const float phase = pin ? (float)((int64_t)(ph + (1ull << 39)) >> 40) * 0x1p-24f
+                            : (float)(int32_t)(ph >> 32) * 0x1p-32f;
     *zk = cscale(expipi<float>((float)(2 * SIGN) * phase), mag);
     return true;
 }
 
-// Warp part of k_direct for node w of the item: lane l sums the Horner blocks
-// l, l + 32, ... of the staged chunk; lane 0 writes the node's partial.
-template <typename T>
-__device__ __forceinline__ void direct_node(const DirectItem& it, const BandDev& B, const C_t<T>* tile,
-                                            const double2* __restrict__ ws,
-                                            const uint4* __restrict__ ntab, int64_t k0, int64_t kend,
-                                            int w, int lane, C_t<T>* __restrict__ part) {
-    using C = C_t<T>;
-    const int64_t i = it.node0 + w;
-    // z = exp(-y) exp(2 pi i x) in T (FP32: from the node record)
-    C z;
-    DirF32Node nd;
-    double x = 0.0, y = 0.0;
-    if constexpr (sizeof(T) == 4) {
-        nd = dir_f32_record(ntab[i], &z);
+// A node as the powers need it: from the plan-time record (X = x 2^64, y =
+// 2 pi Im w as a float pair, k_node_tab) in the FP32 form, from the sorted
+// nodes otherwise.
+template <typename A> struct DirNode {
+    double x, y;
+};
+template <> struct DirNode<float> {
+    DirF32Node d;
+};
+template <typename A>
+__device__ __forceinline__ DirNode<A> dir_node(const double2* __restrict__ ws, const uint4* __restrict__ ntab,
+                                               int64_t i) {
+    DirNode<A> n;
+    if constexpr (sizeof(A) == 4) {
+        const uint4 rec = ntab[i];
+        n.d.X = ((uint64_t)rec.y << 32) | (uint64_t)rec.x;
+        n.d.yh = __uint_as_float(rec.z);
+        n.d.yl = __uint_as_float(rec.w);
     } else {
         const double2 wv = ws[i];
-        x = wv.x - floor(wv.x);
-        y = kTwoPiDir * wv.y;
-        const double xr = x >= 0.5 ? x - 1.0 : x;
-        z = cscale(expipi<T>((T)(2.0 * xr)), dir_exp<T>((T)(-y)));
+        n.x = wv.x - floor(wv.x);
+        n.y = kTwoPiDir * wv.y;
     }
-    C acc = C{(T)0, (T)0};
-#pragma unroll 1
-    for (int bb = 0; bb < kDirChunk / (32 * kDirBlock); ++bb) {
-        const int b = bb * 32 + lane;
-        const int64_t kb = k0 + (int64_t)b * kDirBlock;
-        if (kb >= kend) break;
-        C zk;
-        if constexpr (sizeof(T) == 4) {
-            if (!dir_f32_power<1>(nd, kb, 104.f, &zk)) break;   // z^kb underflows: so do later blocks
-        } else {
-            const double ykb = y * (double)kb;
-            if (ykb > 745.0) break;
-            zk = cscale(expipi<T>((T)(2.0 * dir_phase<T>((double)kb, x))), dir_exp<T>((T)(-ykb)));
-        }
-        const C* cb = tile + b * kDirBlockLd;
-        C P = cb[kDirBlock - 1];
-#pragma unroll
-        for (int t = kDirBlock - 2; t >= 0; --t) P = cadd(cmul(P, z), cb[t]);
-        acc = cadd(acc, cmul(zk, P));
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-    }
-    if (lane == 0) part[B.dslot + (i - B.node_off) * B.nchunk + it.chunk] = acc;
+    return n;
 }
 
-// One CTA per work item: up to kDirNodes consecutive sorted nodes of one band
-// against one chunk of kDirChunk coefficients staged in shared memory.  Warp w
-// takes nodes w, w + 8, ...; lane l the Horner blocks l, l + 32, ... of the
-// chunk.
-template <typename T, bool DERIV>
-__global__ void __launch_bounds__(256) k_direct(const DirectItem* __restrict__ items,
-                                                const BandDev* __restrict__ bands,
-                                                const double2* __restrict__ ws,
-                                                const uint4* __restrict__ ntab,
-                                                const C_t<T>* __restrict__ c,
-                                                C_t<T>* __restrict__ part) {
-    using C = C_t<T>;
+// z^k (SIGN = -1: its conjugate); false once the power underflows.  Double and
+// float pairs reduce k x mod 1 exactly (FMA) in double.
+template <int SIGN>
+__device__ __forceinline__ bool dir_power(const DirNode<float>& n, int64_t k, float2* zk, bool pin = false) {
+    return dir_f32_power<SIGN>(n.d, k, 104.f, pin, zk);
+}
+template <int SIGN> __device__ __forceinline__ bool dir_power(const DirNode<double>& n, int64_t k, double2* zk) {
+    const double yk = n.y * (double)k;
+    if (yk > 745.0) return false;
+    *zk = cscale(expipi<double>((double)(2 * SIGN) * frac_turns((double)k, n.x)), exp(-yk));
+    return true;
+}
+template <int SIGN> __device__ __forceinline__ bool dir_power(const DirNode<ff>& n, int64_t k, ffc* zk) {
+    const double yk = n.y * (double)k;
+    if (yk > 104.0) return false;   // below 2^-150 |c|
+    ff_sincospi(ff((double)(2 * SIGN) * frac_turns((double)k, n.x)), &zk->y, &zk->x);
+    const ff mk = ff_exp(ff(-yk));
+    *zk = ffc{zk->x * mk, zk->y * mk};
+    return true;
+}
+
+// z = exp(-y) e^(2 pi i x) of a pinned transform, in float from the record: x - [x >= 1/2]
+// is the signed X 2^-64, rounded once.
+__device__ __forceinline__ float2 dir_f32_base(const DirF32Node& d) {
+    const float xr = (float)(int64_t)d.X * 0x1p-64f;
+    return cscale(expipi<float>(2.f * xr), expf(-d.yh));
+}
+
+// Plan time: z_j and z_j^8 of the nodes of every segment (entries 2 i and 2 i + 1
+// of node i), formed in double and rounded once.
+template <typename A> __device__ __forceinline__ C_t<A> dir_round(double2 v) { return {A(v.x), A(v.y)}; }
+template <typename A>
+__global__ void k_dir_base(const DirectSeg* __restrict__ segs, const double2* __restrict__ ws,
+                           C_t<A>* __restrict__ z) {
+    const DirectSeg S = segs[blockIdx.y];
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= S.nodes) return;
+    const int64_t i = S.node_off + t;
+    const DirNode<double> n = dir_node<double>(ws, nullptr, i);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const double k = e ? 8.0 : 1.0;
+        z[2 * i + e] = dir_round<A>(cscale(expipi<double>(2.0 * frac_turns(k, n.x)), exp(-n.y * k)));
+    }
+}
+
+// One Horner step P z + c: four fused operations (double), or the pairs' own.
+__device__ __forceinline__ double2 dir_step(double2 P, double2 z, double2 c) {
+    return {fma(P.x, z.x, fma(-P.y, z.y, c.x)), fma(P.x, z.y, fma(P.y, z.x, c.y))};
+}
+__device__ __forceinline__ ffc dir_step(ffc P, ffc z, ffc c) { return cadd(cmul(P, z), c); }
+struct f2c {   // two nodes' complex values in packed pairs
+    f2 x, y;
+};
+__device__ __forceinline__ f2c dir_step(f2c P, f2c z, f2 nzy, f2c c) {
+    return {f2_fma(P.x, z.x, f2_fma(P.y, nzy, c.x)), f2_fma(P.x, z.y, f2_fma(P.y, z.x, c.y))};
+}
+// The steps of pinned transforms (kPinnedN): products and sums rounded as these
+// always had them.  Re (P z) is a rounded product and a fused one, the
+// addend a separate sum; which product of the imaginary part is the fused one
+// differs between segments summed in order (SEQ) and the others.
+template <bool XY> __device__ __forceinline__ f2c dir_mul_pin(f2c a, f2c b, f2 nby) {
+    return {f2_fma(a.x, b.x, f2_mul(a.y, nby)),
+            XY ? f2_fma(a.x, b.y, f2_mul(a.y, b.x)) : f2_fma(a.y, b.x, f2_mul(a.x, b.y))};
+}
+template <bool SEQ>
+__device__ __forceinline__ f2c dir_block_pin(const float2* cb, f2c z, f2 nzy, f2c zk, f2 nzky, bool la, bool lb) {
+    f2c P = {f2_dup(cb[kDirBlock - 1].x), f2_dup(cb[kDirBlock - 1].y)};
+#pragma unroll
+    for (int t = kDirBlock - 2; t >= 0; --t) {
+        const float2 ct = cb[t];
+        const f2c m = dir_mul_pin<!SEQ>(P, z, nzy);
+        P = f2c{f2_add(m.x, f2_dup(ct.x)), f2_add(m.y, f2_dup(ct.y))};
+    }
+    if (!la) P = f2c{f2_make(0.f, f2_hi(P.x)), f2_make(0.f, f2_hi(P.y))};
+    if (!lb) P = f2c{f2_make(f2_lo(P.x), 0.f), f2_make(f2_lo(P.y), 0.f)};
+    return dir_mul_pin<!SEQ>(P, zk, nzky);   // zk P
+}
+__device__ __forceinline__ f2c dir_pair(float2 a, float2 b) { return {f2_make(a.x, b.x), f2_make(a.y, b.y)}; }
+
+__device__ __forceinline__ float dir_shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double dir_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ ff dir_shfl(ff v, int o) { return ff(dir_shfl(v.hi, o), dir_shfl(v.lo, o)); }
+
+template <typename C> __device__ __forceinline__ C dir_zero() {
+    using T = decltype(C().x);
+    return C{T(0), T(0)};
+}
+
+// The result of node i: written to f (with rmul: rmul_j conj(result), the
+// node-gradient epilogue) when the segment has one chunk, else to its partial.
+__device__ __forceinline__ float2 dir_out(float2 v) { return v; }
+__device__ __forceinline__ double2 dir_out(double2 v) { return v; }
+__device__ __forceinline__ double2 dir_out(ffc v) { return double2{(double)v.x, (double)v.y}; }
+
+template <typename A, typename O>
+__device__ __forceinline__ void dir_write(const DirectSeg& S, int64_t i, int chunk, C_t<A> v,
+                                          const int32_t* __restrict__ perm, const O* __restrict__ rmul,
+                                          O* __restrict__ f, C_t<A>* __restrict__ part) {
+    if (S.nchunk > 1) {
+        part[S.dslot + (i - S.node_off) * S.nchunk + chunk] = v;
+        return;
+    }
+    const int32_t j = perm[i];
+    const O o = dir_out(v);
+    f[j] = rmul ? cmulc(rmul[j], o) : o;
+}
+
+// One CTA per work item: consecutive sorted nodes of one segment against one
+// chunk of up to kDirChunk coefficients staged in shared memory.  G = 2^lg
+// consecutive lanes share a node (two nodes in the FP32 form) and take its
+// Horner blocks l, l + G, ... of the chunk, so that a segment of few frequencies
+// keeps all lanes busy: a whole warp per node left 30 of 32 lanes idle at K =
+// 64.  Bound by the FMA pipe of its arithmetic (4 operations a term; FP64: 16
+// cycles of the SM per warp instruction, active lanes or not).  The FP32 form
+// steps two nodes at once in packed pairs (fl_f32x2.cuh), 5 issues per term and
+// node pair against 2 x 7.
+//
+// Segments of a pinned transform (DirectSeg::pin) keep its steps, their rounding
+// and the order of its sums: one Horner chain per block, z from the node record
+// in float, the blocks of a node in ascending order (pin = 2, G = 1) or one per
+// lane, summed by the shuffle tree (pin = 1).
+template <typename A, typename O, bool DERIV>
+__global__ void __launch_bounds__(256)
+    k_direct(const DirectItem* __restrict__ items, const DirectSeg* __restrict__ segs,
+             const double2* __restrict__ ws, const uint4* __restrict__ ntab, const C_t<A>* __restrict__ zb,
+             const C_t<A>* __restrict__ c, const int32_t* __restrict__ perm, const O* __restrict__ rmul,
+             O* __restrict__ f, C_t<A>* __restrict__ part) {
+    using C = C_t<A>;
+    constexpr int NP = sizeof(A) == 4 ? 2 : 1;   // nodes per lane group
     extern __shared__ unsigned char smem_raw[];
     C* tile = reinterpret_cast<C*>(smem_raw);
     const DirectItem it = items[blockIdx.x];
-    const BandDev B = bands[it.band];
+    const DirectSeg S = segs[it.seg];
     const int64_t k0 = (int64_t)it.chunk * kDirChunk;
-    const int64_t kend = min(B.K, k0 + (int64_t)kDirChunk);
-    // the chunk's terms rounded up to whole Horner blocks (zeros past kend)
-    const int nst = (int)((kend - k0 + kDirBlock - 1) / kDirBlock) * kDirBlock;
-    for (int i = threadIdx.x; i < nst; i += blockDim.x) {
-        const int64_t k = k0 + i;
-        C v = C{(T)0, (T)0};
-        if (k < kend) {
-            v = c[B.c_off + k];
-            if (DERIV) {
-                T wgt;
-                if constexpr (sizeof(T) == 4) wgt = (float)k * 6.28318530717958647692f;   // k < 2^24: one rounding
+    const int kn = (int)min(S.K - k0, (int64_t)kDirChunk);
+    const int nblk = (kn + kDirBlock - 1) / kDirBlock;   // zeros past kn
+    for (int i = threadIdx.x; i < nblk * kDirBlock; i += 256) {
+        C v = dir_zero<C>();
+        if (i < kn) {
+            const int64_t k = k0 + i;
+            v = c[S.c_off + k];
+            if constexpr (DERIV) {
+                A wgt;
+                if constexpr (sizeof(A) == 4) wgt = (float)k * 6.28318530717958647692f;   // k < 2^24: one rounding
                 else wgt = kTwoPiDir * (double)k;
                 v = C{-v.y * wgt, v.x * wgt};
             }
@@ -158,78 +243,95 @@ __global__ void __launch_bounds__(256) k_direct(const DirectItem* __restrict__ i
         tile[i + i / kDirBlock] = v;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int w = threadIdx.x >> 5; w < it.nnodes; w += 8)
-        direct_node<T>(it, B, tile, ws, ntab, k0, kend, w, lane, part);
-}
-
-// Bands with K <= kDirSmallK: one thread per node (up to kDirSmallNodes per
-// CTA), the band's K coefficients staged once, all K terms per thread in the
-// same blocked Horner form (blocks of kDirBlock terms from an exactly reduced
-// power z^kb); the partial of chunk 0 as for k_direct.
-template <typename T, bool DERIV>
-__global__ void __launch_bounds__(kDirSmallNodes) k_direct_small(const DirectItem* __restrict__ items,
-                                                                 const BandDev* __restrict__ bands,
-                                                                 const double2* __restrict__ ws,
-                                                                 const uint4* __restrict__ ntab,
-                                                                 const C_t<T>* __restrict__ c,
-                                                                 C_t<T>* __restrict__ part) {
-    using C = C_t<T>;
-    __shared__ C tile[kDirSmallK];
-    const DirectItem it = items[blockIdx.x];
-    const BandDev B = bands[it.band];
-    const int K = (int)B.K;                              // <= kDirSmallK
-    const int Kr = (K + kDirBlock - 1) / kDirBlock * kDirBlock;
-    for (int k = threadIdx.x; k < Kr; k += blockDim.x) {
-        C v = C{(T)0, (T)0};
-        if (k < K) {
-            v = c[B.c_off + k];
-            if (DERIV) {
-                T wgt;
-                if constexpr (sizeof(T) == 4) wgt = (float)k * 6.28318530717958647692f;
-                else wgt = kTwoPiDir * (double)k;
-                v = C{-v.y * wgt, v.x * wgt};
+    const int lg = it.lg, G = 1 << lg;
+    const int sub = threadIdx.x & (G - 1);
+    // every lane of a warp runs the same trips (the shuffles below)
+    for (int n0 = 0; n0 < it.nnodes; n0 += NP * (256 >> lg)) {
+        const int n = n0 + NP * (threadIdx.x >> lg);
+        const bool on = n < it.nnodes;
+        const int64_t i = it.node0 + (on ? n : 0);
+        if constexpr (NP == 2) {
+            const bool two = n + 1 < it.nnodes;
+            const int64_t i1 = two ? i + 1 : i;
+            const DirNode<A> na = dir_node<A>(ws, ntab, i), nb = dir_node<A>(ws, ntab, i1);
+            f2c z, z8 = {};
+            if (S.pin) {
+                z = dir_pair(dir_f32_base(na.d), dir_f32_base(nb.d));
+            } else {
+                z = dir_pair(zb[2 * i], zb[2 * i1]);
+                z8 = dir_pair(zb[2 * i + 1], zb[2 * i1 + 1]);
             }
-        }
-        tile[k] = v;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x >= it.nnodes) return;
-    const int64_t i = it.node0 + threadIdx.x;
-    C z;
-    DirF32Node nd;
-    double x = 0.0, y = 0.0;
-    if constexpr (sizeof(T) == 4) {
-        nd = dir_f32_record(ntab[i], &z);
-    } else {
-        const double2 wv = ws[i];
-        x = wv.x - floor(wv.x);
-        y = kTwoPiDir * wv.y;
-        const double xr = x >= 0.5 ? x - 1.0 : x;
-        z = cscale(expipi<T>((T)(2.0 * xr)), dir_exp<T>((T)(-y)));
-    }
-    C acc = C{(T)0, (T)0};
-    for (int kb = 0; kb < K; kb += kDirBlock) {
-        C zk;
-        if constexpr (sizeof(T) == 4) {
-            if (!dir_f32_power<1>(nd, kb, 104.f, &zk)) break;
-        } else {
-            const double ykb = y * (double)kb;
-            if (ykb > 745.0) break;
-            zk = cscale(expipi<T>((T)(2.0 * dir_phase<T>((double)kb, x))), dir_exp<T>((T)(-ykb)));
-        }
-        const C* cb = tile + kb;
-        C P = cb[kDirBlock - 1];
+            const f2 nz = f2_make(-f2_lo(z.y), -f2_hi(z.y)), nz8 = f2_make(-f2_lo(z8.y), -f2_hi(z8.y));
+            f2c acc = {f2_dup(0.f), f2_dup(0.f)};
+            for (int b = sub; on && b < nblk; b += G) {
+                float2 ka = {0.f, 0.f}, kb = {0.f, 0.f};
+                const bool la = dir_power<1>(na, k0 + b * kDirBlock, &ka, S.pin);
+                const bool lb = dir_power<1>(nb, k0 + b * kDirBlock, &kb, S.pin);
+                if (!la && !lb) break;          // both powers underflow: so do later blocks
+                const float2* cb = reinterpret_cast<const float2*>(tile) + b * kDirBlockLd;
+                const f2c zk = dir_pair(ka, kb);
+                const f2 nzk = f2_make(-ka.y, -kb.y);
+                if (S.pin) {
+                    const f2c m = S.pin == 2 ? dir_block_pin<true>(cb, z, nz, zk, nzk, la, lb)
+                                             : dir_block_pin<false>(cb, z, nz, zk, nzk, la, lb);
+                    acc = f2c{f2_add(acc.x, m.x), f2_add(acc.y, m.y)};
+                } else {
+                    f2c P;
 #pragma unroll
-        for (int t = kDirBlock - 2; t >= 0; --t) P = cadd(cmul(P, z), cb[t]);
-        acc = cadd(acc, cmul(zk, P));
+                    for (int h = kDirBlock / 8 - 1; h >= 0; --h) {
+                        f2c Q = {f2_dup(cb[8 * h + 7].x), f2_dup(cb[8 * h + 7].y)};
+#pragma unroll
+                        for (int t = 6; t >= 0; --t) {
+                            const float2 ct = cb[8 * h + t];
+                            Q = dir_step(Q, z, nz, f2c{f2_dup(ct.x), f2_dup(ct.y)});
+                        }
+                        P = h == kDirBlock / 8 - 1 ? Q : dir_step(P, z8, nz8, Q);
+                    }
+                    if (!la)                        // (a power of zero takes nothing from its block)
+                        P = f2c{f2_make(0.f, f2_hi(P.x)), f2_make(0.f, f2_hi(P.y))};
+                    if (!lb) P = f2c{f2_make(f2_lo(P.x), 0.f), f2_make(f2_lo(P.y), 0.f)};
+                    acc = dir_step(P, zk, nzk, acc);
+                }
+            }
+            const f2 ar = acc.x, ai = acc.y;
+            float ax = f2_lo(ar), ay = f2_lo(ai), bx = f2_hi(ar), by = f2_hi(ai);
+            for (int off = G >> 1; off > 0; off >>= 1) {
+                ax += dir_shfl(ax, off);
+                ay += dir_shfl(ay, off);
+                bx += dir_shfl(bx, off);
+                by += dir_shfl(by, off);
+            }
+            if (sub == 0 && on) {
+                dir_write<A>(S, i, it.chunk, float2{ax, ay}, perm, rmul, f, part);
+                if (two) dir_write<A>(S, i1, it.chunk, float2{bx, by}, perm, rmul, f, part);
+            }
+        } else {
+            const DirNode<A> nd = dir_node<A>(ws, ntab, i);
+            C acc = dir_zero<C>();
+            const C z = zb[2 * i], z8 = zb[2 * i + 1];
+            for (int b = sub; on && b < nblk; b += G) {
+                C zk;
+                if (!dir_power<1>(nd, k0 + b * kDirBlock, &zk)) break;
+                const C* cb = tile + b * kDirBlockLd;
+                C P;
+#pragma unroll
+                for (int h = kDirBlock / 8 - 1; h >= 0; --h) {
+                    C Q = cb[8 * h + 7];
+#pragma unroll
+                    for (int t = 6; t >= 0; --t) Q = dir_step(Q, z, cb[8 * h + t]);
+                    P = h == kDirBlock / 8 - 1 ? Q : dir_step(P, z8, Q);
+                }
+                acc = cadd(acc, cmul(zk, P));
+            }
+            for (int off = G >> 1; off > 0; off >>= 1)
+                acc = cadd(acc, C{dir_shfl(acc.x, off), dir_shfl(acc.y, off)});
+            if (sub == 0 && on) dir_write<A>(S, i, it.chunk, acc, perm, rmul, f, part);
+        }
     }
-    part[B.dslot + (i - B.node_off) * B.nchunk] = acc;
 }
 
-// The direct band holding flattened node t: the last range whose prefix is
-// <= t (prefixes ascend; binary search, so batches of thousands of direct
-// bands cost log2 of that per node).
+// The segment holding flattened node t: the last range whose prefix is
+// <= t (prefixes ascend; binary search).
 __device__ __forceinline__ int find_direct_range(const DirectRange* __restrict__ ranges, int nranges,
                                                  int64_t t) {
     int lo = 0, hi = nranges;
@@ -241,424 +343,194 @@ __device__ __forceinline__ int find_direct_range(const DirectRange* __restrict__
     return lo;
 }
 
-// f[perm[i]] = sum over the node's chunks (in chunk order); with rmul,
-// rmul[perm[i]] * conj(sum) (the node-gradient epilogue).
-template <typename T>
-__global__ void k_direct_reduce(int nranges, const DirectRange* __restrict__ ranges,
-                                int64_t total, const BandDev* __restrict__ bands,
-                                const int32_t* __restrict__ perm, const C_t<T>* __restrict__ part,
-                                const C_t<T>* __restrict__ rmul, C_t<T>* __restrict__ f) {
-    using C = C_t<T>;
+// Segments of several chunks: f[perm[i]] = sum over the node's chunks (in chunk
+// order); with rmul, rmul[perm[i]] * conj(sum).
+template <typename A, typename O>
+__global__ void k_direct_reduce(int nranges, const DirectRange* __restrict__ ranges, int64_t total,
+                                const DirectSeg* __restrict__ segs, const int32_t* __restrict__ perm,
+                                const C_t<A>* __restrict__ part, const O* __restrict__ rmul,
+                                O* __restrict__ f) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total) return;
     const DirectRange R = ranges[find_direct_range(ranges, nranges, t)];
-    const BandDev B = bands[R.band];
+    const DirectSeg S = segs[R.seg];
     const int64_t local = t - R.prefix;
-    const C* p = part + B.dslot + local * B.nchunk;
-    C acc = C{(T)0, (T)0};
-    for (int ch = 0; ch < B.nchunk; ++ch) acc = cadd(acc, p[ch]);
-    const int32_t j = perm[B.node_off + local];
-    f[j] = rmul ? cmulc(rmul[j], acc) : acc;
+    const C_t<A>* p = part + S.dslot + local * S.nchunk;
+    C_t<A> acc = dir_zero<C_t<A>>();
+    for (int ch = 0; ch < S.nchunk; ++ch) acc = cadd(acc, p[ch]);
+    const int32_t j = perm[S.node_off + local];
+    const O o = dir_out(acc);
+    f[j] = rmul ? cmulc(rmul[j], o) : o;
 }
 
-// Adjoint of the direct bands, cdir[k] += sum_{j in band} r_j conj(z_j)^k for
-// k < K_b: the transpose of the blocked Horner sum.  One warp per work item
-// (band, chunk of 32 KL frequencies, up to kDirAdjNodes nodes); lane l owns
-// the KL frequencies k0 = chunk 32 KL + l KL .. k0 + KL - 1.  For each node
-// (broadcast across the warp by shuffles) the lane forms conj(z_j)^k0 from an
-// exactly reduced phase, then steps through its frequencies multiplying by
-// conj(z_j).  Chunks of different node groups meet in cdir through atomics.
-template <typename T> struct AdjKL { static constexpr int KL = sizeof(T) == 4 ? 32 : 16; };
+// Adjoint of the direct segments, cdir[k] += sum_j r_j conj(z_j)^k for k < K: the
+// transpose of the blocked Horner sum.  One warp per work item (segment, chunk
+// of 32 KL frequencies, node group).  The lanes split into KB = 2^lkb blocks of
+// KL frequencies (the fewest that cover the chunk's share of K) and 32 / KB node
+// subgroups; a lane forms conj(z_j)^k0 from an exactly reduced phase, then
+// steps through its KL frequencies multiplying by conj(z_j); a shuffle tree adds
+// the subgroups and the first adds the result to cdir (atomics across node
+// groups).  The FP32 form steps two nodes at once in packed pairs.  The node
+// groups are cut so that the launch has several warps per SM: at 256 nodes each
+// the K = 512 band of N = M = 2^18 disk nodes had 160 warps (float pairs:
+// 570 us, and the bands with K <= 256 in double 990 us).
+constexpr int kAdjKL = kDirAdjKL;
+static_assert(kAdjKL == 16, "two chains of eight steps");
 
-template <typename T>
-__global__ void __launch_bounds__(32) k_direct_adj(const DirectAdjItem* __restrict__ items,
-                                                   const BandDev* __restrict__ bands,
-                                                   const double2* __restrict__ ws,
-                                                   const uint4* __restrict__ ntab,
-                                                   const int32_t* __restrict__ perm,
-                                                   const C_t<T>* __restrict__ r,
-                                                   C_t<T>* __restrict__ cdir) {
-    using C = C_t<T>;
-    constexpr int KL = AdjKL<T>::KL;
-    const DirectAdjItem it = items[blockIdx.x];
-    const BandDev B = bands[it.band];
-    const int lane = threadIdx.x;
-    const int64_t k0 = (int64_t)it.kchunk * (32 * KL) + (int64_t)lane * KL;
-    const bool active = k0 < B.K;
-    C acc[KL];
-#pragma unroll
-    for (int t = 0; t < KL; ++t) acc[t] = C{(T)0, (T)0};
-    for (int nb = 0; nb < it.nnodes; nb += 32) {
-        // lane loads node nb + lane: x, y, r_j and conj(z_j) in T
-        double xl = 0.0, yl = 0.0;
-        C rl = C{(T)0, (T)0}, zl = C{(T)0, (T)0};
-        DirF32Node nl = {0ull, 0.f, 0.f};
-        if (nb + lane < it.nnodes) {
-            const int64_t i = it.node0 + nb + lane;
-            rl = r[perm[i]];
-            if constexpr (sizeof(T) == 4) {   // from the node record; conj(z)
-                nl = dir_f32_record(ntab[i], &zl);
-                zl.y = -zl.y;
-            } else {
-                const double2 wv = ws[i];
-                xl = wv.x - floor(wv.x);
-                yl = kTwoPiDir * wv.y;
-                const double xr = xl >= 0.5 ? xl - 1.0 : xl;
-                zl = cscale(expipi<T>((T)(-2.0 * xr)), dir_exp<T>((T)(-yl)));
-            }
-        }
-        const int cnt = min(32, it.nnodes - nb);
-        for (int q = 0; q < cnt; ++q) {
-            const C rq = C{__shfl_sync(0xffffffffu, rl.x, q), __shfl_sync(0xffffffffu, rl.y, q)};
-            const C zq = C{__shfl_sync(0xffffffffu, zl.x, q), __shfl_sync(0xffffffffu, zl.y, q)};
-            C w0;
-            if constexpr (sizeof(T) == 4) {
-                DirF32Node nq;
-                nq.X = ((uint64_t)__shfl_sync(0xffffffffu, (unsigned)(nl.X >> 32), q) << 32) |
-                       (uint64_t)__shfl_sync(0xffffffffu, (unsigned)nl.X, q);
-                nq.yh = __shfl_sync(0xffffffffu, nl.yh, q);
-                nq.yl = __shfl_sync(0xffffffffu, nl.yl, q);
-                if (!active) continue;
-                if (!dir_f32_power<-1>(nq, k0, 104.f, &w0)) continue;
-            } else {
-                const double x = __shfl_sync(0xffffffffu, xl, q);
-                const double y = __shfl_sync(0xffffffffu, yl, q);
-                if (!active) continue;
-                const double yk = y * (double)k0;
-                if (yk > 745.0) continue;
-                w0 = cscale(expipi<T>((T)(-2.0 * dir_phase<T>((double)k0, x))), dir_exp<T>((T)(-yk)));
-            }
-            C rw = cmul(rq, w0);
-#pragma unroll
-            for (int t = 0; t < KL; ++t) {
-                acc[t] = cadd(acc[t], rw);
-                rw = cmul(rw, zq);
-            }
-        }
-    }
-    if (!active) return;
-#pragma unroll
-    for (int t = 0; t < KL; ++t) {
-        const int64_t k = k0 + t;
-        if (k < B.K) {
-            atomicAdd(&cdir[k].x, acc[t].x);
-            atomicAdd(&cdir[k].y, acc[t].y);
-        }
-    }
-}
-
-// The float-pair form (FL_FP64_FF): k_direct with the Horner steps, the
-// block-start powers z_j^kb = exp(-y kb) e^(2 pi i frac(kb x)) and the sums in
-// float pairs (fl_ffmath.cuh); the phases kb x are still reduced exactly in
-// double.  c: the coefficients already converted to pairs.
-__global__ void __launch_bounds__(256) k_direct_ff(const DirectItem* __restrict__ items,
-                                                   const BandDev* __restrict__ bands,
-                                                   const double2* __restrict__ ws,
-                                                   const ffc* __restrict__ c,
-                                                   ffc* __restrict__ part) {
-    extern __shared__ unsigned char smem_raw[];
-    ffc* tile = reinterpret_cast<ffc*>(smem_raw);
+template <typename A, typename O>
+__global__ void __launch_bounds__(32)
+    k_direct_adj(const DirectItem* __restrict__ items, const DirectSeg* __restrict__ segs,
+                 const double2* __restrict__ ws, const uint4* __restrict__ ntab, const C_t<A>* __restrict__ zb,
+                 const int32_t* __restrict__ perm, const O* __restrict__ r, O* __restrict__ cdir) {
+    using C = C_t<A>;
     const DirectItem it = items[blockIdx.x];
-    const BandDev B = bands[it.band];
-    const int64_t k0 = (int64_t)it.chunk * kDirChunk;
-    const int64_t kend = min(B.K, k0 + (int64_t)kDirChunk);
-    const int nst = (int)((kend - k0 + kDirBlock - 1) / kDirBlock) * kDirBlock;
-    for (int i = threadIdx.x; i < nst; i += blockDim.x) {
-        const int64_t k = k0 + i;
-        tile[i + i / kDirBlock] = k < kend ? c[B.c_off + k] : ffc{ff(0), ff(0)};
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int w = threadIdx.x >> 5; w < it.nnodes; w += 8) {   // nodes w, w + 8, ...
-        const int64_t i = it.node0 + w;
-        const double2 wv = ws[i];
-        const double x = wv.x - floor(wv.x);
-        const double y = kTwoPiDir * wv.y;
-        double xr = x;
-        if (xr >= 0.5) xr -= 1.0;
-        ffc z;
-        ff_sincospi(ff(2.0 * xr), &z.y, &z.x);
-        const ff mag = ff_exp(ff(-y));
-        z = ffc{z.x * mag, z.y * mag};
-        ffc acc = {ff(0), ff(0)};
-#pragma unroll 1
-        for (int bb = 0; bb < kDirChunk / (32 * kDirBlock); ++bb) {
-            const int b = bb * 32 + lane;
-            const int64_t kb = k0 + (int64_t)b * kDirBlock;
-            if (kb >= kend) break;
-            const double ykb = y * (double)kb;
-            if (ykb > 104.0) break;     // below 2^-150 |c|: so are the later blocks
-            const ffc* cb = tile + b * kDirBlockLd;
-            ffc P = cb[kDirBlock - 1];
+    const DirectSeg S = segs[it.seg];
+    const int lane = threadIdx.x, lkb = it.lg, g = lane >> lkb, G = 32 >> lkb;
+    const int64_t k0 = (int64_t)it.chunk * (32 * kAdjKL) + (int64_t)(lane & ((1 << lkb) - 1)) * kAdjKL;
+    const bool active = k0 < S.K;
+    C acc[kAdjKL];
+    if constexpr (sizeof(A) == 4) {
+        f2 ar[kAdjKL], ai[kAdjKL];
 #pragma unroll
-            for (int t = kDirBlock - 2; t >= 0; --t) P = cadd(cmul(P, z), cb[t]);
-            ffc zk;
-            ff_sincospi(ff(2.0 * dir_phase<double>((double)kb, x)), &zk.y, &zk.x);
-            const ff mk = ff_exp(ff(-ykb));
-            acc = cadd(acc, cmul(ffc{zk.x * mk, zk.y * mk}, P));
+        for (int t = 0; t < kAdjKL; ++t) ar[t] = ai[t] = f2_dup(0.f);
+        for (int jn = 2 * g; active && jn < it.nnodes; jn += 2 * G) {
+            const int64_t i = it.node0 + jn;
+            const bool two = jn + 1 < it.nnodes;
+            const int64_t i1 = two ? i + 1 : i;
+            const DirNode<A> na = dir_node<A>(ws, ntab, i), nb = dir_node<A>(ws, ntab, i1);
+            float2 wa = {0.f, 0.f}, wb = {0.f, 0.f};
+            const bool la = dir_power<-1>(na, k0, &wa);
+            const bool lb = dir_power<-1>(nb, k0, &wb) && two;
+            if (!la && !lb) continue;
+            wa = la ? cmul(r[perm[i]], wa) : float2{0.f, 0.f};
+            wb = lb ? cmul(r[perm[i1]], wb) : float2{0.f, 0.f};
+            // conj(z): w conj(z) = (wx zx + wy zy, wy zx - wx zy)
+            const float2 a1 = zb[2 * i], b1 = zb[2 * i1], a8 = zb[2 * i + 1], b8 = zb[2 * i1 + 1];
+            const f2c zq = {f2_make(a1.x, b1.x), f2_make(-a1.y, -b1.y)};
+            const f2 nzq = f2_make(a1.y, b1.y);
+            f2c w = dir_pair(wa, wb), v = dir_pair(cmulc(wa, a8), cmulc(wb, b8));   // k0 and k0 + 8
+#pragma unroll
+            for (int t = 0; t < kAdjKL / 2; ++t) {
+                ar[t] = f2_add(ar[t], w.x);
+                ai[t] = f2_add(ai[t], w.y);
+                ar[t + 8] = f2_add(ar[t + 8], v.x);
+                ai[t + 8] = f2_add(ai[t + 8], v.y);
+                w = f2c{f2_fma(w.y, nzq, f2_mul(w.x, zq.x)), f2_fma(w.x, zq.y, f2_mul(w.y, zq.x))};
+                v = f2c{f2_fma(v.y, nzq, f2_mul(v.x, zq.x)), f2_fma(v.x, zq.y, f2_mul(v.y, zq.x))};
+            }
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const ffc o = {ff(__shfl_xor_sync(0xffffffffu, acc.x.hi, off),
-                              __shfl_xor_sync(0xffffffffu, acc.x.lo, off)),
-                           ff(__shfl_xor_sync(0xffffffffu, acc.y.hi, off),
-                              __shfl_xor_sync(0xffffffffu, acc.y.lo, off))};
-            acc = cadd(acc, o);
-        }
-        if (lane == 0) part[B.dslot + (i - B.node_off) * B.nchunk + it.chunk] = acc;
-    }
-}
-
-// f[perm[i]] = sum over the node's chunks (in chunk order), rounded to double.
-__global__ void k_direct_reduce_ff(int nranges, const DirectRange* __restrict__ ranges,
-                                   int64_t total, const BandDev* __restrict__ bands,
-                                   const int32_t* __restrict__ perm, const ffc* __restrict__ part,
-                                   const double2* __restrict__ rmul, double2* __restrict__ f) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total) return;
-    const DirectRange R = ranges[find_direct_range(ranges, nranges, t)];
-    const BandDev B = bands[R.band];
-    const int64_t local = t - R.prefix;
-    const ffc* p = part + B.dslot + local * B.nchunk;
-    ffc acc = {ff(0), ff(0)};
-    for (int ch = 0; ch < B.nchunk; ++ch) acc = cadd(acc, p[ch]);
-    const int32_t j = perm[B.node_off + local];
-    const double2 v = double2{(double)acc.x, (double)acc.y};
-    // with rmul: rmul[j] conj(v) (node gradient)
-    f[j] = rmul ? cmulc(rmul[j], v) : v;
-}
-
-// (the coefficients are read as pairs from p.d_cff, k-weighted by the caller
-// for the derivative)
-static cudaError_t direct_forward_ff(Plan& p, void* f, const void* rmul, cudaStream_t st) {
-    if (p.direct_work.empty()) return cudaSuccess;
-    const size_t smem = (size_t)kDirTile * sizeof(ffc);
-    cudaError_t e = cudaFuncSetAttribute(k_direct_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int slot;
-    timer_begin(p, "direct", (double)p.direct_terms * sizeof(ffc) / 32.0, st, &slot);
-    k_direct_ff<<<(unsigned)p.direct_work.size(), 256, smem, st>>>(p.d_direct, p.d_bands, p.d_ws,
-                                                                  (const ffc*)p.d_cff, (ffc*)p.d_dpart);
-    k_direct_reduce_ff<<<(unsigned)((p.direct_nodes + 255) / 256), 256, 0, st>>>(
-        (int)p.direct_ranges.size(), p.d_dranges, p.direct_nodes, p.d_bands, p.d_perm,
-        (const ffc*)p.d_dpart, (const double2*)rmul, (double2*)f);
-    timer_end(p, slot, st);
-    p.launches += 2;
-    return cudaGetLastError();
-}
-
-// Adjoint of the bands with K <= kDirSmallK: one warp per (band, group of up
-// to kDirAdjNodes nodes).  The lanes split into KB blocks of KL frequencies
-// (KB the smallest power of two with KB KL >= K) and G = 32 / KB node
-// subgroups; each lane sums its subgroup's nodes (every G-th) over its KL
-// frequencies, a fixed shuffle tree adds the subgroups, and the first
-// subgroup adds the result to cdir (atomics across node groups, as k_direct_adj).
-template <typename T>
-__global__ void __launch_bounds__(32) k_direct_adj_small(const DirectAdjItem* __restrict__ items,
-                                                         const BandDev* __restrict__ bands,
-                                                         const double2* __restrict__ ws,
-                                                         const uint4* __restrict__ ntab,
-                                                         const int32_t* __restrict__ perm,
-                                                         const C_t<T>* __restrict__ r,
-                                                         C_t<T>* __restrict__ cdir) {
-    using C = C_t<T>;
-    constexpr int KL = AdjKL<T>::KL;
-    const DirectAdjItem it = items[blockIdx.x];
-    const BandDev B = bands[it.band];
-    const int K = (int)B.K;
-    int lkb = 0;
-    while ((KL << lkb) < K) ++lkb;                 // KB = 2^lkb <= 32 (K <= kDirSmallK)
-    const int lane = threadIdx.x, g = lane >> lkb, G = 32 >> lkb;
-    const int64_t k0 = (int64_t)(lane & ((1 << lkb) - 1)) * KL;
-    const bool active = k0 < K;
-    C acc[KL];
+        for (int t = 0; t < kAdjKL; ++t) acc[t] = float2{f2_lo(ar[t]) + f2_hi(ar[t]), f2_lo(ai[t]) + f2_hi(ai[t])};
+    } else {
 #pragma unroll
-    for (int t = 0; t < KL; ++t) acc[t] = C{(T)0, (T)0};
-    for (int jn = g; active && jn < it.nnodes; jn += G) {
-        const int64_t i = it.node0 + jn;
-        C zq, w0;
-        double x = 0.0, y = 0.0;
-        if constexpr (sizeof(T) == 4) {   // from the node record; conj(z)
-            const DirF32Node nd = dir_f32_record(ntab[i], &zq);
-            zq.y = -zq.y;
-            if (!dir_f32_power<-1>(nd, k0, 104.f, &w0)) continue;
-        } else {
-            const double2 wv = ws[i];
-            x = wv.x - floor(wv.x);
-            y = kTwoPiDir * wv.y;
-            const double xr = x >= 0.5 ? x - 1.0 : x;
-            zq = cscale(expipi<T>((T)(-2.0 * xr)), dir_exp<T>((T)(-y)));
-            const double yk = y * (double)k0;
-            if (yk > 745.0) continue;
-            w0 = cscale(expipi<T>((T)(-2.0 * dir_phase<T>((double)k0, x))), dir_exp<T>((T)(-yk)));
-        }
-        C rw = cmul(r[perm[i]], w0);
+        for (int t = 0; t < kAdjKL; ++t) acc[t] = dir_zero<C>();
+        for (int jn = g; active && jn < it.nnodes; jn += G) {
+            const int64_t i = it.node0 + jn;
+            C w0;
+            if (!dir_power<-1>(dir_node<A>(ws, ntab, i), k0, &w0)) continue;
+            const O rj = r[perm[i]];
+            const C z = zb[2 * i];
+            const C zq = C{z.x, -z.y};
+            C rw;
+            if constexpr (std::is_same<A, ff>::value) rw = cmul(ffc{ff(rj.x), ff(rj.y)}, w0);
+            else rw = cmul(rj, w0);
+            C rv = cmulc(rw, zb[2 * i + 1]);         // from k0 + 8
 #pragma unroll
-        for (int t = 0; t < KL; ++t) {
-            acc[t] = cadd(acc[t], rw);
-            rw = cmul(rw, zq);
+            for (int t = 0; t < kAdjKL / 2; ++t) {
+                acc[t] = cadd(acc[t], rw);
+                acc[t + 8] = cadd(acc[t + 8], rv);
+                rw = cmul(rw, zq);
+                rv = cmul(rv, zq);
+            }
         }
     }
     for (int off = 1 << lkb; off < 32; off <<= 1) {
 #pragma unroll
-        for (int t = 0; t < KL; ++t) {
-            acc[t].x += __shfl_xor_sync(0xffffffffu, acc[t].x, off);
-            acc[t].y += __shfl_xor_sync(0xffffffffu, acc[t].y, off);
-        }
+        for (int t = 0; t < kAdjKL; ++t)
+            acc[t] = cadd(acc[t], C{dir_shfl(acc[t].x, off), dir_shfl(acc[t].y, off)});
     }
     if (g != 0 || !active) return;
 #pragma unroll
-    for (int t = 0; t < KL; ++t) {
+    for (int t = 0; t < kAdjKL; ++t) {
         const int64_t k = k0 + t;
-        if (k < K) {
-            atomicAdd(&cdir[k].x, acc[t].x);
-            atomicAdd(&cdir[k].y, acc[t].y);
+        if (k < S.K) {
+            const O o = dir_out(acc[t]);
+            atomicAdd(&cdir[k].x, o.x);
+            atomicAdd(&cdir[k].y, o.y);
         }
     }
 }
 
-template <typename T>
-static cudaError_t direct_forward_t(Plan& p, const void* c, void* f, bool deriv, const void* rmul,
-                                    cudaStream_t st) {
-    using C = C_t<T>;
+template <typename A>
+static cudaError_t dir_base_t(Plan& p, cudaStream_t st) {
+    int64_t most = 0;
+    for (const DirectSeg& s : p.direct_segs) most = std::max(most, s.nodes);
+    const int64_t ns = (int64_t)p.direct_segs.size();
+    for (int64_t s0 = 0; s0 < ns; s0 += 65535)   // gridDim.y
+        k_dir_base<A><<<dim3((unsigned)((most + 255) / 256), (unsigned)std::min<int64_t>(65535, ns - s0)), 256, 0,
+                        st>>>(p.d_dsegs + s0, p.d_ws, (C_t<A>*)p.d_dz);
+    return cudaGetLastError();
+}
+
+cudaError_t build_direct_base(Plan& p, cudaStream_t st) {
+    if (p.prec == FL_FP64_FF) return dir_base_t<ff>(p, st);
+    return p.prec == FL_FP64 ? dir_base_t<double>(p, st) : dir_base_t<float>(p, st);
+}
+
+// (float pairs read the coefficients as pairs, k-weighted by the caller for the
+// derivative)
+template <typename A, typename O, bool DERIV>
+static cudaError_t direct_forward_t(Plan& p, const void* c, void* f, const void* rmul, cudaStream_t st) {
+    using C = C_t<A>;
     if (p.direct_work.empty()) return cudaSuccess;
-    const size_t smem = (size_t)kDirTile * sizeof(C);
-    auto kern = deriv ? k_direct<T, true> : k_direct<T, false>;
+    const size_t smem = dir_tile(p.direct_kmax, sizeof(C));
+    auto kern = k_direct<A, O, DERIV>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int slot;
     timer_begin(p, "direct", (double)p.direct_terms * sizeof(C) / 32.0, st, &slot);
-    const int64_t nbig = (int64_t)p.direct_work.size() - p.n_direct_small;
-    if (nbig > 0)
-        kern<<<(unsigned)nbig, 256, smem, st>>>(p.d_direct, p.d_bands, p.d_ws, p.d_ntab, (const C*)c,
-                                                (C*)p.d_dpart);
-    if (p.n_direct_small > 0) {
-        auto ks = deriv ? k_direct_small<T, true> : k_direct_small<T, false>;
-        ks<<<(unsigned)p.n_direct_small, kDirSmallNodes, 0, st>>>(p.d_direct + nbig, p.d_bands, p.d_ws,
-                                                                  p.d_ntab, (const C*)c, (C*)p.d_dpart);
+    kern<<<(unsigned)p.direct_work.size(), 256, smem, st>>>(
+        p.d_direct, p.d_dsegs, p.d_ws, p.d_ntab, (const C*)p.d_dz, (const C*)c, p.d_perm, (const O*)rmul, (O*)f,
+        (C*)p.d_dpart);
+    if (p.direct_nodes > 0) {
+        k_direct_reduce<A, O><<<(unsigned)((p.direct_nodes + 255) / 256), 256, 0, st>>>(
+            (int)p.direct_ranges.size(), p.d_dranges, p.direct_nodes, p.d_dsegs, p.d_perm, (const C*)p.d_dpart,
+            (const O*)rmul, (O*)f);
         ++p.launches;
     }
-    k_direct_reduce<T><<<(unsigned)((p.direct_nodes + 255) / 256), 256, 0, st>>>(
-        (int)p.direct_ranges.size(), p.d_dranges, p.direct_nodes, p.d_bands, p.d_perm,
-        (const C*)p.d_dpart, (const C*)rmul, (C*)f);
     timer_end(p, slot, st);
-    p.launches += 1 + (nbig > 0);
+    ++p.launches;
     return cudaGetLastError();
 }
 
 cudaError_t run_direct_forward(Plan& p, const void* c, void* f, bool deriv, const void* rmul,
                                cudaStream_t st) {
-    if (p.prec == FL_FP64_FF)   // reads the coefficients as pairs (converted by the caller)
-        return direct_forward_ff(p, f, rmul, st);
-    return p.prec == FL_FP64 ? direct_forward_t<double>(p, c, f, deriv, rmul, st)
-                             : direct_forward_t<float>(p, c, f, deriv, rmul, st);
+    if (p.prec == FL_FP64_FF) return direct_forward_t<ff, double2, false>(p, p.d_cff, f, rmul, st);
+    if (p.prec == FL_FP64)
+        return deriv ? direct_forward_t<double, double2, true>(p, c, f, rmul, st)
+                     : direct_forward_t<double, double2, false>(p, c, f, rmul, st);
+    return deriv ? direct_forward_t<float, float2, true>(p, c, f, rmul, st)
+                 : direct_forward_t<float, float2, false>(p, c, f, rmul, st);
 }
 
-// The float-pair form's adjoint of the direct bands with K > kDirSmallK:
-// k_direct_adj's steps (same work items, KL = 16 frequencies per lane) with
-// conj(z_j), the restart power conj(z_j)^k0 and the frequency steps in float
-// pairs; the restart phase k0 x mod 1 is still reduced exactly in double.
-// Each lane's sums, rounded to double, meet in cdir through atomics.
-__global__ void __launch_bounds__(32) k_direct_adj_ff(const DirectAdjItem* __restrict__ items,
-                                                      const BandDev* __restrict__ bands,
-                                                      const double2* __restrict__ ws,
-                                                      const int32_t* __restrict__ perm,
-                                                      const double2* __restrict__ r,
-                                                      double2* __restrict__ cdir) {
-    constexpr int KL = 16;
-    const DirectAdjItem it = items[blockIdx.x];
-    const BandDev B = bands[it.band];
-    const int lane = threadIdx.x;
-    const int64_t k0 = (int64_t)it.kchunk * (32 * KL) + (int64_t)lane * KL;
-    const bool active = k0 < B.K;
-    ffc acc[KL];
-#pragma unroll
-    for (int t = 0; t < KL; ++t) acc[t] = ffc{ff(0), ff(0)};
-    for (int nb = 0; nb < it.nnodes; nb += 32) {
-        // lane loads node nb + lane: x, y, r_j and conj(z_j) as pairs
-        double xl = 0.0, yl = 0.0;
-        ffc rl = {ff(0), ff(0)}, zl = {ff(0), ff(0)};
-        if (nb + lane < it.nnodes) {
-            const int64_t i = it.node0 + nb + lane;
-            const double2 wv = ws[i];
-            xl = wv.x - floor(wv.x);
-            yl = kTwoPiDir * wv.y;
-            const double2 rv = r[perm[i]];
-            rl = ffc{ff(rv.x), ff(rv.y)};
-            const double xr = xl >= 0.5 ? xl - 1.0 : xl;
-            ff_sincospi(ff(-2.0 * xr), &zl.y, &zl.x);
-            const ff mag = ff_exp(ff(-yl));
-            zl = ffc{zl.x * mag, zl.y * mag};
-        }
-        const int cnt = min(32, it.nnodes - nb);
-        for (int q = 0; q < cnt; ++q) {
-            const ffc rq = {ff(__shfl_sync(0xffffffffu, rl.x.hi, q), __shfl_sync(0xffffffffu, rl.x.lo, q)),
-                            ff(__shfl_sync(0xffffffffu, rl.y.hi, q), __shfl_sync(0xffffffffu, rl.y.lo, q))};
-            const ffc zq = {ff(__shfl_sync(0xffffffffu, zl.x.hi, q), __shfl_sync(0xffffffffu, zl.x.lo, q)),
-                            ff(__shfl_sync(0xffffffffu, zl.y.hi, q), __shfl_sync(0xffffffffu, zl.y.lo, q))};
-            const double x = __shfl_sync(0xffffffffu, xl, q);
-            const double y = __shfl_sync(0xffffffffu, yl, q);
-            if (!active) continue;
-            const double yk = y * (double)k0;
-            if (yk > 104.0) continue;   // below 2^-150 |r_j|
-            ffc w0;
-            ff_sincospi(ff(-2.0 * dir_phase<double>((double)k0, x)), &w0.y, &w0.x);
-            const ff mk = ff_exp(ff(-yk));
-            ffc rw = cmul(rq, ffc{w0.x * mk, w0.y * mk});
-#pragma unroll
-            for (int t = 0; t < KL; ++t) {
-                acc[t] = cadd(acc[t], rw);
-                rw = cmul(rw, zq);
-            }
-        }
-    }
-    if (!active) return;
-#pragma unroll
-    for (int t = 0; t < KL; ++t) {
-        const int64_t k = k0 + t;
-        if (k < B.K) {
-            atomicAdd(&cdir[k].x, (double)acc[t].x);
-            atomicAdd(&cdir[k].y, (double)acc[t].y);
-        }
-    }
-}
-
-// (pairs: the float-pair form, T = double, whose bands with K > kDirSmallK
-// take k_direct_adj_ff)
-template <typename T>
-static cudaError_t direct_adjoint_t(Plan& p, const void* r, cudaStream_t st, bool pairs = false) {
-    using C = C_t<T>;
-    if (p.direct_ranges.empty()) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(p.d_cdir, 0, p.N * sizeof(C), st);
+template <typename A, typename O>
+static cudaError_t direct_adjoint_t(Plan& p, const void* r, cudaStream_t st) {
+    if (p.dadj_work.empty()) return cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(p.d_cdir, 0, p.N * sizeof(O), st);
     if (e != cudaSuccess) return e;
-    const bool dbl = sizeof(T) == 8;
-    const std::vector<DirectAdjItem>& items = dbl ? p.dadj_work64 : p.dadj_work32;
-    const DirectAdjItem* d_items = dbl ? p.d_dadj64 : p.d_dadj32;
     int slot;
     timer_begin(p, "direct_adj", 0.0, st, &slot);
-    const int64_t nbig = (int64_t)items.size() - p.n_dadj_small;
-    if (nbig > 0 && pairs) {
-        k_direct_adj_ff<<<(unsigned)nbig, 32, 0, st>>>(d_items, p.d_bands, p.d_ws, p.d_perm,
-                                                      (const double2*)r, (double2*)p.d_cdir);
-        ++p.launches;
-    } else if (nbig > 0) {
-        k_direct_adj<T><<<(unsigned)nbig, 32, 0, st>>>(d_items, p.d_bands, p.d_ws, p.d_ntab, p.d_perm,
-                                                       (const C*)r, (C*)p.d_cdir);
-        ++p.launches;
-    }
-    if (p.n_dadj_small > 0) {
-        k_direct_adj_small<T><<<(unsigned)p.n_dadj_small, 32, 0, st>>>(
-            d_items + nbig, p.d_bands, p.d_ws, p.d_ntab, p.d_perm, (const C*)r, (C*)p.d_cdir);
-        ++p.launches;
-    }
+    k_direct_adj<A, O><<<(unsigned)p.dadj_work.size(), 32, 0, st>>>(
+        p.d_dadj, p.d_dsegs, p.d_ws, p.d_ntab, (const C_t<A>*)p.d_dz, p.d_perm, (const O*)r, (O*)p.d_cdir);
+    ++p.launches;
     timer_end(p, slot, st);
     return cudaGetLastError();
 }
 
-// (the float-pair form on its complex128 r: bands with K <= kDirSmallK in double)
 cudaError_t run_direct_adjoint(Plan& p, const void* r, cudaStream_t st) {
-    if (p.prec == FL_FP64_FF) return direct_adjoint_t<double>(p, r, st, true);
-    return p.prec == FL_FP64 ? direct_adjoint_t<double>(p, r, st) : direct_adjoint_t<float>(p, r, st);
+    if (p.prec == FL_FP64_FF) return direct_adjoint_t<ff, double2>(p, r, st);
+    return p.prec == FL_FP64 ? direct_adjoint_t<double, double2>(p, r, st)
+                             : direct_adjoint_t<float, float2>(p, r, st);
 }
 
 }  // namespace fl

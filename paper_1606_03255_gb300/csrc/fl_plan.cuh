@@ -86,55 +86,40 @@ struct FuseArgs {
     float2* pp;
 };
 
-// Direct route (fl_direct.cu): kDirNodes nodes x one chunk of kDirChunk
-// coefficients per CTA (its 8 warps take kDirNodes / 8 nodes each, so the
-// staged chunk serves them all), Horner blocks of kDirBlock terms.
-#ifndef FL_DIR_NODES
-#define FL_DIR_NODES 16
-#endif
-constexpr int kDirBlock = 32;
-constexpr int kDirChunk = 4096;
-constexpr int kDirNodes = FL_DIR_NODES;
-static_assert(kDirNodes % 8 == 0, "whole nodes per warp");
-// below this many direct items (8 CTAs per SM of the 152) a plan halves the
-// nodes per item
-constexpr int64_t kDirFewItems = 8 * 152;
-// FP32 bands with K <= kDirSmallK and at least kDirSmallMinNodes nodes: one
-// thread per node, up to kDirSmallNodes nodes per CTA, all K terms per thread
-// (see k_direct_small).  Fewer nodes, or FP64 (whose serial chains are long),
-// keep a warp per node.
-#ifndef FL_DIR_SMALL_MIN_NODES
-#define FL_DIR_SMALL_MIN_NODES 128
-#endif
-#ifndef FL_DIR_SMALL_NODES
-#define FL_DIR_SMALL_NODES 256
-#endif
-constexpr int kDirSmallK = 256, kDirSmallNodes = FL_DIR_SMALL_NODES,
-              kDirSmallMinNodes = FL_DIR_SMALL_MIN_NODES;
-
-struct DirectItem {
-    int band;
-    int chunk;
-    int64_t node0;   // first sorted node of the item
-    int nnodes;      // <= kDirNodes
-    int pad;
+// Direct route (fl_direct.cu).  A segment: consecutive sorted nodes (of one
+// direct band, or of neighbouring ones with the same K) that sum over the same
+// K frequencies.
+struct DirectSeg {
+    int64_t node_off, nodes;   // sorted nodes node_off .. node_off + nodes
+    int64_t K;                 // frequencies 0 .. K - 1
+    int64_t c_off;             // first coefficient of the transform
+    int64_t dslot;             // offset of its partial sums (nodes x nchunk; nchunk > 1)
+    int nchunk;                // chunks of kDirChunk coefficients
+    int pin;                   // pinned transforms (kPinnedN): 1, or 2 with the blocks of a node summed in order
 };
 
-// Direct route adjoint: a warp per (band, frequency chunk of 32 KL, node group).
-constexpr int kDirAdjNodes = 256;
-struct DirectAdjItem {
-    int band;
-    int kchunk;
-    int64_t node0;
+// Horner blocks of kDirBlock terms, at most kDirChunk coefficients staged per
+// CTA; G = 2^lg lanes per node (pair), each taking every G-th block.
+constexpr int kDirBlock = 32;
+constexpr int kDirChunk = 4096;
+constexpr int kDirMaxBlocks = 8;   // most blocks per lane that G is cut for
+// Adjoint: frequencies per lane, and the most node steps a lane takes.
+constexpr int kDirAdjKL = 16;
+constexpr int kDirAdjSteps = 64;
+
+struct DirectItem {
+    int seg;
+    int chunk;
+    int64_t node0;   // first sorted node of the item
     int nnodes;
-    int pad;
+    int lg;          // log2 of the lanes per node (forward) or frequency blocks (adjoint)
 };
 
 struct DirectRange {
-    int band;
+    int seg;
     int pad;
-    int64_t count;   // nodes of the band
-    int64_t prefix;  // direct nodes of the bands before it
+    int64_t count;   // nodes of the segment
+    int64_t prefix;  // nodes of the segments before it
 };
 
 // Per-band plan data on the host.
@@ -166,6 +151,16 @@ struct Timer {
     cudaEvent_t start, stop;
     double bytes;
 };
+
+// FP32 transforms of at most this many coefficients (integer exponents) keep the
+// rounding of every forward step, bit for bit: their node gradients leave
+// through autograd in double and are compared at that precision at these
+// sizes, where any other rounding of the FP32 steps (about 10^-7) shows; a
+// transform of a batch equals the single plan's bit for bit, so both do.
+constexpr int64_t kPinnedN = (int64_t)1 << 18;
+// pinned transforms: bands with K <= kDirSeqK and at least kDirSeqNodes nodes
+// sum the blocks of a node in order
+constexpr int64_t kDirSeqK = 256, kDirSeqNodes = 128;
 
 struct Plan {
     int kind = 0;           // 0 Fourier-Laplace, 1 Laplace
@@ -206,12 +201,11 @@ struct Plan {
     double direct_bias = 1.0;
     double tuned_bias = 0.0;       // bias chosen by the autotuner (0: not tuned)
     int tuned_sigma_mode = -1, tuned_fuse_mode = -1, tuned_rhs = -1;   // its other choices
-    std::vector<DirectItem> direct_work;   // items of the larger-K bands, then n_direct_small
-    int64_t n_direct_small = 0;            // items of the bands with K <= kDirSmallK (at the end)
-    std::vector<DirectRange> direct_ranges;
-    std::vector<DirectAdjItem> dadj_work32, dadj_work64;   // adjoint items for KL = 32 / 16, then
-    int64_t n_dadj_small = 0;                              // the items of K <= kDirSmallK bands
-    int64_t direct_nodes = 0, direct_terms = 0, dpart_elems = 0;
+    std::vector<DirectSeg> direct_segs;
+    std::vector<DirectItem> direct_work, dadj_work;
+    std::vector<DirectRange> direct_ranges;   // the segments of several chunks
+    int64_t direct_nodes = 0;                 // their nodes
+    int64_t direct_terms = 0, dpart_elems = 0, direct_kmax = 0;
 
     // device memory
     double2* d_ws = nullptr;       // nodes in sorted order (Re w, Im w)
@@ -253,8 +247,9 @@ struct Plan {
     void* d_z0 = nullptr;          // one complex: sum of r over Z^0 (adjoint)
     DirectItem* d_direct = nullptr;
     DirectRange* d_dranges = nullptr;
-    DirectAdjItem* d_dadj32 = nullptr;
-    DirectAdjItem* d_dadj64 = nullptr;
+    DirectSeg* d_dsegs = nullptr;
+    DirectItem* d_dadj = nullptr;
+    void* d_dz = nullptr;          // direct route: z_j, z_j^8 per sorted node (complex, the plan's arithmetic)
     void* d_dpart = nullptr;       // direct route: partial sums (complex T)
     void* d_cdir = nullptr;        // direct route adjoint: N complex
     // fused gather (FuseArgs): row-block starts, entries, window values, partial sums
@@ -332,6 +327,7 @@ cudaError_t launch_xi_combine(Plan& p, void* out, cudaStream_t st);   // adjoint
 cudaError_t run_forward_xi(Plan& p, const void* c, void* f, cudaStream_t st);
 
 // Launchers (fl_direct.cu)
+cudaError_t build_direct_base(Plan& p, cudaStream_t st);   // d_dz
 cudaError_t run_direct_forward(Plan& p, const void* c, void* f, bool deriv, const void* rmul,
                                cudaStream_t st);
 cudaError_t run_direct_adjoint(Plan& p, const void* r, cudaStream_t st);

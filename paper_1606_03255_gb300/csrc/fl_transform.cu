@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __rest
         return;
     }
     // with rmul: f[j] = rmul[j] * conj(value) (node gradient, see fl_grad_w)
-    if (B.route != 1) return;   // direct-route band: written by k_direct_reduce
+    if (B.route != 1) return;   // direct-route band: written by the direct kernels
     if constexpr (sizeof(T) == 4 && !XI) {
         const C v = gather_node_f32<MW>(ntab[i], i - B.node_off, B, bands, grid, cheb32, q, kb_b, fpp);
         f[j] = rmul ? cmulc(rmul[j], v) : v;
@@ -1009,6 +1009,12 @@ static cudaError_t gather_dispatch(Plan& p, const void* c, void* f, bool deriv, 
     }
 }
 
+// Whether the gather has a node to write: one of an NFFT band or of Z^0 (the
+// direct kernels write the others).
+static bool gathers(const Plan& p) {
+    return p.z0_nodes > 0 || !p.small_work.empty() || !p.large_bands.empty();
+}
+
 template <typename T>
 static cudaError_t forward_t(Plan& p, const void* c, void* f, bool deriv, const void* rmul,
                              cudaStream_t st) {
@@ -1016,6 +1022,7 @@ static cudaError_t forward_t(Plan& p, const void* c, void* f, bool deriv, const 
     cudaError_t e = deriv ? fft_bands<T, +1, 0, true>(p, c, st) : fft_bands<T, +1, 0, false>(p, c, st);
     if (e != cudaSuccess) return e;
     if ((e = run_direct_forward(p, c, f, deriv, rmul, st)) != cudaSuccess) return e;
+    if (!gathers(p)) return cudaSuccess;
     return gather_dispatch<T>(p, c, f, deriv, rmul, st);
 }
 
@@ -1156,6 +1163,7 @@ static cudaError_t forward_ff(Plan& p, const void* c, void* f, bool deriv, const
     cudaError_t e = fft_bands<ff, +1, 0, false>(p, p.d_cff, st);
     if (e != cudaSuccess) return e;
     if ((e = run_direct_forward(p, c, f, deriv, rmul, st)) != cudaSuccess) return e;
+    if (!gathers(p)) return cudaSuccess;
     switch (p.mw) {
 #define FL_MW_CASE(W) \
     case W: return gather_ff_t<W>(p, c, f, deriv, rmul, st);
@@ -1229,7 +1237,7 @@ static cudaError_t adjoint_t(Plan& p, const void* r, void* cout, cudaStream_t st
     timer_begin(p, "combine", 0.0, st, &slot);
     k_combine<T, G, FT><<<(unsigned)((p.N + 255) / 256), 256, 0, st>>>(
         p.N, p.levels, p.d_bands, (const FT*)p.d_D, (const G*)p.d_grid, z0sum,
-        p.direct_ranges.empty() ? nullptr : (const C*)p.d_cdir, (C*)cout);
+        p.dadj_work.empty() ? nullptr : (const C*)p.d_cdir, (C*)cout);
     timer_end(p, slot, st);
     p.launches += 2;
     return cudaGetLastError();
