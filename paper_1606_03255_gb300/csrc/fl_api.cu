@@ -108,6 +108,7 @@ static int onesided_rank(double eps_K) {
 static fl_status select_common(Plan& p, int q_in) {
     p.eps_K = p.eps / 3.0;
     p.eps_A = p.eps / 3.0;
+    p.q_given = q_in > 0;
     if (q_in > 0)
         p.q = q_in;
     else if (p.variant == 1)
@@ -270,7 +271,7 @@ static int route_of(const Plan& p, const BandHost& bh) {
     const BandDev& d = bh.dev;
     const bool dbl = p.prec != FL_FP32;   // float pairs: gather and direct bands in double
     const double fft_pt = dbl ? 2.0 : 1.0, win = dbl ? 150.0 : 20.0, div = dbl ? 40.0 : 4.0;
-    const double per_node = (double)d.nrhs * 2 * p.mw * 2 + 2.0 * p.mw * win + (d.nrhs > 1 ? p.q * div : 0.0);
+    const double per_node = (double)d.nrhs * 2 * p.mw * 2 + 2.0 * p.mw * win + (d.nrhs > 1 ? d.nrhs * div : 0.0);
     const double fft = (double)d.nrhs * d.n * (d.log2n + 8) * fft_pt + (double)bh.nodes * per_node + 2.0e5;
     const double direct = (double)bh.nodes * d.K * 6.0 * p.direct_bias;
     return direct < fft ? 2 : 1;
@@ -407,6 +408,30 @@ static void build_pass_groups(Plan& p) {
     }
 }
 
+// Estimated cost of a gather from the grids, all right-hand sides.
+static double unfused_cost(int64_t nodes, int nrhs, int mw) {
+    return (double)nodes * ((double)nrhs * 2 * mw * 2 + 2.0 * mw * 20.0);
+}
+
+// FP32 transforms that may merge bands (not pinned): the same with the traffic
+// of the grids and partial sums, in the same units (0.26 ps: an FFT point costs
+// log2 n + 8 of them, 7 ps measured at N = M = 2^20; a byte of HBM about 0.56).
+// A gather from the grid pays for writing it and reads it once, or 128 bytes
+// per node, whichever is less (it measured 0.16 ms for 1.5*10^5 nodes and 35
+// grids of 2^21 points); a fused one writes and reads a partial sum per node
+// and tile.  *fuse: the cheaper of the two.
+static double free_gather_cost(int64_t nodes, int nrhs, int64_t n, int log2n, int mw, bool fusable, bool* fuse) {
+    const double bytes = std::min<double>(8.0 * n, 128.0 * nodes);
+    const double grid = unfused_cost(nodes, nrhs, mw) + nrhs * (0.56 * 8.0 * n + 0.8 * bytes);
+    *fuse = false;
+    if (!fusable || log2n <= kSmallMaxLog2) return grid;
+    const int TR = pass_tiles(8, (log2n + 1) / 2, FL_P2_THREADS_F32);
+    const int parts = (2 * mw - 1 + TR - 1) / TR + 1;
+    const double fused = nrhs * ((double)nodes * (TR + 2 * mw - 1) / TR * 24.0 + (double)nodes * parts * 15.0);
+    *fuse = fused < grid;
+    return std::min(fused, grid);
+}
+
 // Window gather fused into pass 2 (FP32 forward, four-step grids).  A band
 // qualifies when its nodes are few for its grid: per right-hand side the
 // unfused path writes the grid (8 n bytes) and gathers about three 32-byte
@@ -444,8 +469,9 @@ static fl_status build_fused(Plan& p, cudaStream_t st) {
         const double parts = (double)(TR + taps - 1) / TR;
         const double unfused = 8.0 * d.n + std::min<double>(8.0 * d.n, 96.0 * bh.nodes);
         const double fused = bh.nodes * parts * (8.0 + 16.0 * NQ + 8.0) + 8.0 * P * bh.nodes;
-        // sub-bands (parent >= 0) have no other gather: always fused
-        if (p.fuse_mode == 2 || d.parent >= 0 || fused <= 0.5 * unfused) cands.push_back({b, l1, l2, TR, P});
+        bool fuse = d.parent >= 0 || fused <= 0.5 * unfused;   // pinned transforms: sub-bands always
+        if (!pinned(p, p.inst[bh.inst])) free_gather_cost(bh.nodes, d.nrhs, d.n, d.log2n, p.mw, true, &fuse);
+        if (p.fuse_mode == 2 || fuse) cands.push_back({b, l1, l2, TR, P});
     }
     if (cands.empty()) return FL_OK;
     std::vector<double2> hw(p.M);
@@ -581,10 +607,6 @@ static double fused_cost(int64_t nodes, int log2n, int mw) {   // per right-hand
     return entries * 24.0 + (double)nodes * parts * 6.0;
 }
 
-static double unfused_cost(int64_t nodes, int nrhs, int mw) {
-    return (double)nodes * ((double)nrhs * 2 * mw * 2 + 2.0 * mw * 20.0);
-}
-
 struct SplitChoice {
     int P = 1, log2n = 0;
     int64_t Kp = 0, Nc = 0;
@@ -597,10 +619,14 @@ static SplitChoice best_split(const Plan& p, const BandHost& bh, double smin, in
     const BandDev& d = bh.dev;
     SplitChoice best;
     const bool four_step = d.log2n > kSmallMaxLog2;
-    // FP32: sub-bands gather inside pass 2 (fused); FP64: from their grids
+    // FP32: sub-bands gather inside pass 2 (fused; from their grids where that is
+    // cheaper, not in pinned transforms); FP64: from their grids
     const bool fusable = p.prec == FL_FP32 && p.fuse_mode != 1;
+    const bool free32 = p.prec == FL_FP32 && !p.xi_mode && !pinned(p, p.inst[bh.inst]);
+    bool fz = false;
     double c1 = fft_cost(d.nrhs, d.n, d.log2n) +
-                (four_step && fusable
+                (free32 ? free_gather_cost(bh.nodes, d.nrhs, d.n, d.log2n, mw, fusable, &fz)
+                 : four_step && fusable
                      ? std::min(d.nrhs * fused_cost(bh.nodes, d.log2n, mw), unfused_cost(bh.nodes, d.nrhs, mw))
                      : unfused_cost(bh.nodes, d.nrhs, mw));
     double bc = force ? (double)d.n : c1;
@@ -619,7 +645,9 @@ static SplitChoice best_split(const Plan& p, const BandHost& bh, double smin, in
             // the half-width this sigma needs, and the FP32 limit at it
             const int mc = std::max(mw, window_width(p.eps_A, (double)n / (double)Nc));
             if (deconv_gain((double)n / (double)Nc, mc) > gain_max) continue;
-            const double gather = fusable ? d.nrhs * fused_cost(bh.nodes, lg, mc) : unfused_cost(bh.nodes, d.nrhs, mc);
+            const double gather = free32    ? free_gather_cost(bh.nodes, d.nrhs, n, lg, mc, fusable, &fz)
+                                  : fusable ? d.nrhs * fused_cost(bh.nodes, lg, mc)
+                                            : unfused_cost(bh.nodes, d.nrhs, mc);
             const double c = force ? (double)P * n : P * (fft_cost(d.nrhs, n, lg) + gather);
             if (c < bc) {
                 bc = c;
@@ -701,6 +729,155 @@ static fl_status plan_splits(Plan& p, const std::vector<int>& nfft, cudaStream_t
     return FL_OK;
 }
 
+// ---------------------------------------------------------------------------
+// Merged bands.  The dyadic bands with l_m = 1 all keep the same K frequencies,
+// each with q right-hand sides, although on the ones near the circle y xi is
+// small and exp(-y xi) all but linear there.  Neighbouring ones are therefore
+// interpolated together, in y alone (the weights exp(-y_s k) are exact at the
+// Chebyshev points y_s of the union), at the rank that leaves no larger an
+// error than rank q leaves on a single dyadic band: at N = M = 2^20, eps = 1e-6 the
+// six bands of the clustered nodes take 35 right-hand sides instead of 72, at
+// 2^18 and 1e-12 nine bands 82 instead of 198.
+
+// Bounds of the interpolation error of exp(-y x) on y in [a, b], relative to the
+// kernel's bound 1, at 0 .. kMaxQ points: the Chebyshev coefficients of
+// exp(-(c + h t) x) are 2 (-1)^j I_j(h x) e^{-c x}, and interpolation at q Chebyshev
+// points errs by at most twice the sum of the coefficients from q on; the
+// largest over x in (0, xmax] (sampled on a logarithmic grid; the bounds are
+// smooth and unimodal in x).
+static void interp_error(double a, double b, double xmax, double* err) {
+    constexpr int kTerms = 128, kSamples = 24;
+    const double h = 0.5 * (b - a);
+    for (int q = 0; q <= kMaxQ; ++q) err[q] = 0.0;
+    for (int i = 0; i < kSamples; ++i) {
+        const double x = xmax * pow(2.0, -0.25 * i), z = h * x;
+        // e^-z I_j(z) by backward recurrence, normalised by I_0 + 2 sum I_j = e^z
+        double v[kTerms + 2];
+        v[kTerms + 1] = 0.0;
+        v[kTerms] = 1e-280;
+        double sum = 2.0 * v[kTerms];
+        for (int j = kTerms; j > 0; --j) {
+            v[j - 1] = v[j + 1] + 2.0 * j / z * v[j];
+            if (v[j - 1] > 1e250) {   // rescale
+                for (int t = j - 1; t <= kTerms; ++t) v[t] *= 1e-250;
+                sum *= 1e-250;
+            }
+            sum += (j > 1 ? 2.0 : 1.0) * v[j - 1];
+        }
+        const double scale = 4.0 * exp(-a * x) / sum;
+        double tail = 0.0;
+        for (int j = kTerms; j >= 0; --j) {
+            tail += v[j] * scale;
+            if (j <= kMaxQ) err[j] = std::max(err[j], tail);
+        }
+    }
+}
+
+// The smallest rank whose bound on [a, 2^octaves a], x <= xmax, is at most tol
+// (kMaxQ + 1: none).  It depends on a xmax alone, rounded up to a sixteenth of an
+// octave and kept per plan (a batch asks for the same few again and again).
+static int merged_rank(Plan& p, double a, int octaves, double xmax, double tol) {
+    const int key = (int)ceil(16.0 * log2(a * xmax));
+    const auto hit = p.rank_memo.find({octaves, key});
+    if (hit != p.rank_memo.end()) return hit->second;
+    double err[kMaxQ + 1];
+    interp_error(1.0, ldexp(1.0, octaves), pow(2.0, key / 16.0), err);
+    int r = 2;
+    while (r <= kMaxQ && err[r] > tol) ++r;
+    p.rank_memo[{octaves, key}] = r;
+    return r;
+}
+
+// Estimated cost of an NFFT band (the units of route_of), at its best split.
+static double nfft_cost(const Plan& p, const BandHost& bh) {
+    double best = 0.0;
+    const bool split = p.sigma_mode != 1 && !p.xi_mode && p.prec != FL_FP64_FF;
+    for (double smin : {2.0, 1.75, 1.5, 1.25}) {
+        double c = 0.0;
+        best_split(p, bh, smin, p.mw, false, &c);
+        if (smin == 2.0 || c < best) best = c;
+        if (!split) break;
+    }
+    return best + 2.0e5;
+}
+
+// Merges neighbouring non-empty bands of a transform with l_m = 1 (where bands
+// are routed by cost and the rank comes from eps: a caller's q is that of every
+// band; and not in pinned transforms): the partition of least
+// estimated cost by dynamic programming; a band left alone keeps its route and
+// Algorithm 2's weights.  The nodes of a merged band are put in cell order (they
+// are consecutive and share a grid size) under its first band.
+static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
+    if ((p.route_mode != 0 && !p.xi_mode) || p.q_given || pinned(p, in)) return FL_OK;
+    std::vector<int> list;   // candidates, ascending band
+    for (int lb = 1; lb < in.levels; ++lb)
+        if (p.bands[in.band_base + lb].nodes > 0 && p.bands[in.band_base + lb].ell == 1) list.push_back(lb);
+    const int n = (int)list.size();
+    if (n == 0) return FL_OK;
+    double tol;
+    {
+        double err[kMaxQ + 1];   // the dyadic band at rank q, over every x
+        interp_error(1.0, 2.0, 64.0, err);
+        tol = err[p.q];
+    }
+    struct Part {
+        double cost;
+        int from, rank;
+    };
+    std::vector<Part> best(n + 1, Part{0.0, 0, 0});
+    auto merged = [&](int i, int j, int rank) {   // candidates list[i .. j] as one band
+        BandHost g = p.bands[in.band_base + list[i]];
+        g.nodes = 0;
+        for (int t = i; t <= j; ++t) g.nodes += p.bands[in.band_base + list[t]].nodes;
+        const double a = ldexp(p.y1, -list[j]), b = ldexp(p.y1, 1 - list[i]);
+        g.dev.nodes = g.nodes;
+        g.dev.yc = 0.5 * (a + b);
+        g.dev.yh = 0.5 * (b - a);
+        g.dev.yh_inv = 1.0 / g.dev.yh;
+        g.dev.nrhs = rank;
+        return g;
+    };
+    for (int j = 0; j < n; ++j) {
+        const BandHost& alone = p.bands[in.band_base + list[j]];
+        const double single = alone.dev.route == 2 ? (double)alone.nodes * alone.dev.K * 6.0 * p.direct_bias
+                                                   : nfft_cost(p, alone);
+        best[j + 1] = Part{best[j].cost + single, j, 0};
+        for (int i = j; i >= 0; --i) {
+            const int r = merged_rank(p, ldexp(p.y1, -list[j]), list[j] - list[i] + 1, in.xi1, tol);
+            if (r > kMaxQ) break;
+            if (i == j && r >= p.q) continue;
+            const double c = best[i].cost + nfft_cost(p, merged(i, j, r));
+            if (c < best[j + 1].cost) best[j + 1] = Part{c, i, r};
+        }
+    }
+    for (int j = n; j > 0; j = best[j].from) {
+        const int i = best[j].from, r = best[j].rank;
+        if (r == 0) continue;
+        const int lead = in.band_base + list[i];
+        const BandHost g = merged(i, j - 1, r);
+        for (int t = i; t < j; ++t) {
+            BandHost& bh = p.bands[in.band_base + list[t]];
+            bh.leader = lead;
+            bh.nodes = bh.dev.nodes = 0;
+            bh.dev.route = 0;
+        }
+        const int64_t own = p.bands[lead].own;
+        p.bands[lead] = g;
+        p.bands[lead].own = own;
+        p.bands[lead].leader = lead;
+        p.bands[lead].dev.route = 1;
+        int off = 0, k = 0;
+        while (k < (int)p.ranks.size() && p.ranks[k] != r) off += p.ranks[k++];
+        if (k == (int)p.ranks.size()) p.ranks.push_back(r);
+        p.bands[lead].dev.choff = off;
+        p.qmax = std::max(p.qmax, r);
+        if (i == j - 1) continue;   // one band at a lower rank: its nodes are in order
+        const cudaError_t e = launch_cell_sort(p, g.node_off, g.nodes, lead, st);
+        if (e != cudaSuccess) return cuda_fail(e, "fl_plan: merged bands");
+    }
+    return FL_OK;
+}
+
 // Plans the transforms Ns[i] x Ms[i], i < B, whose nodes are consecutive in
 // `nodes` (a single plan is B = 1).  Every band of every transform gets an
 // entry of one global band table, and each kernel launch of fl_execute covers
@@ -738,8 +915,6 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     for (int b = 0; b < nb; ++b) hb[b] = p.bands[b].dev;
     FL_CUDA(cudaMemcpyAsync(p.d_bands, hb.data(), nb * sizeof(BandDev), cudaMemcpyHostToDevice, st),
             "copy bands");
-    FL_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * kMaxQ * sizeof(double)), "cudaMalloc cheb");
-    FL_CUDA(cudaMalloc((void**)&p.d_cheb32, 4 * kMaxQ * sizeof(float)), "cudaMalloc cheb32");
     FL_CUDA(cudaMalloc(&p.d_z0, 2 * sizeof(double)), "cudaMalloc z0");
 
     // classify and sort the nodes of every transform into its slice
@@ -806,6 +981,10 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     p.direct_segs.clear();
     p.direct_terms = 0;
     p.z0_nodes = 0;
+    p.ranks.assign(1, p.q);
+    p.qmax = p.q;
+    p.own_gather = false;
+    for (const Instance& in : p.inst) p.own_gather = p.own_gather || !pinned(p, in);
     std::vector<int> nfft_bands;   // bands evaluated by an NFFT, in order
     for (int i = 0; i < B; ++i) {
         Instance& in = p.inst[i];
@@ -818,13 +997,19 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
         for (int lb = 1; lb <= in.levels; ++lb) {
             const int b = in.band_base + lb;
             BandHost& bh = p.bands[b];
-            bh.nodes = counts[b];
+            bh.nodes = bh.own = counts[b];
             bh.node_off = off;
             off += counts[b];
             BandDev& d = bh.dev;
             d.node_off = bh.node_off;
             d.nodes = bh.nodes;
             d.route = bh.nodes > 0 ? route_of(p, bh) : 0;
+        }
+        if ((s = merge_bands(p, in, st)) != FL_OK) return s;
+        for (int lb = 1; lb <= in.levels; ++lb) {
+            const int b = in.band_base + lb;
+            BandHost& bh = p.bands[b];
+            BandDev& d = bh.dev;
             if (d.route == 2) {
                 p.direct_terms += bh.nodes * d.K;
                 add_direct_band(p, bh);
@@ -942,7 +1127,7 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
                                     p.cell_bands.size() * sizeof(Plan::CellBand), cudaMemcpyHostToDevice, st),
                     "copy cell bands");
             FL_CUDA(cudaMalloc(&p.d_sp_phi, (size_t)M * 2 * p.mw * rs), "cudaMalloc adjoint taps");
-            FL_CUDA(cudaMalloc(&p.d_sp_L, (size_t)M * p.q * rs), "cudaMalloc adjoint weights");
+            FL_CUDA(cudaMalloc(&p.d_sp_L, (size_t)M * p.qmax * rs), "cudaMalloc adjoint weights");
             FL_CUDA(cudaMalloc(&p.d_sp_rv, (size_t)M * cs), "cudaMalloc adjoint residuals");
         }
     }
@@ -958,6 +1143,10 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     }
     if (p.prec == FL_FP64_FF)
         FL_CUDA(cudaMalloc(&p.d_cff, (size_t)p.N * sizeof(ffc)), "cudaMalloc float-pair coefficients");
+    int cheb_len = 0;
+    for (int r : p.ranks) cheb_len += r;
+    FL_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * cheb_len * sizeof(double)), "cudaMalloc cheb");
+    FL_CUDA(cudaMalloc((void**)&p.d_cheb32, 4 * cheb_len * sizeof(float)), "cudaMalloc cheb32");
     FL_CUDA(build_cheb(p, st), "fl_plan: tables");
     for (int i = 0; i < B; ++i)
         if (!shares_D[i]) FL_CUDA(build_tables(p, p.inst[i], st), "fl_plan: tables");
@@ -1632,19 +1821,20 @@ fl_status fl_get_info(fl_plan_t h, fl_info* info) {
     if (p.kind == 0) {   // bands of all transforms: routes counted over the batch
         for (const BandHost& bh : p.bands) {
             if (bh.local == 0 || bh.dev.parent >= 0) continue;   // sub-bands count with their band
-            if (bh.dev.route == 1) ++info->n_bands_fft;
+            if (bh.dev.route == 1 || bh.leader >= 0) ++info->n_bands_fft;
             if (bh.dev.route == 2) ++info->n_bands_direct;
         }
     }
     const int nb_first = p.kind == 0 && !p.inst.empty() ? p.inst[0].levels + 1 : (int)p.bands.size();
     for (int b = 1; b < nb_first && b < (int)p.bands.size() && b < FL_MAX_LEVELS; ++b) {
         const BandHost& bh = p.bands[b];
+        const BandDev& ev = p.kind == 0 && bh.leader >= 0 ? p.bands[bh.leader].dev : bh.dev;   // what evaluates it
         info->band_ell[b] = bh.ell;
-        info->band_route[b] = bh.dev.route;
-        info->band_nodes[b] = bh.nodes;
+        info->band_route[b] = ev.route;
+        info->band_nodes[b] = bh.own;
         info->band_K[b] = bh.dev.K;
-        info->band_n[b] = bh.dev.n;
-        info->band_parts[b] = bh.dev.nsub > 0 ? bh.dev.nsub : 1;
+        info->band_n[b] = ev.n;
+        info->band_parts[b] = ev.nsub > 0 ? ev.nsub : 1;
     }
     info->model_bytes = p.model_bytes;
     info->direct_bias = p.tuned_bias > 0 ? p.tuned_bias : p.direct_bias;

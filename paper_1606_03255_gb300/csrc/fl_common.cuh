@@ -147,7 +147,7 @@ struct BandDev {
     int64_t K;         // frequencies 0..K-1 carry nonzero weight
     int64_t grid_off;  // element offset of the band's grids (nrhs x n) in the grid buffer
     int64_t D_off;     // element offset of the band's weight table (nrhs x K)
-    int nrhs;          // right-hand sides: q for interpolated bands, 1 for Y_M
+    int nrhs;          // right-hand sides: the rank (q; less or more for a merged band), 1 for Y_M
     int log2n;
     int route;         // 0 empty, 1 NFFT, 2 direct sum
     int dld;           // 0: weights D[s K + k]; > 0 (real exponents): one row of
@@ -157,7 +157,8 @@ struct BandDev {
     int64_t node_off;  // first node of the band in sorted order
     int64_t pad1;      // (unused; the layout of this struct stays because the compiler's choice
                        // of fused products in the pinned FP32 transforms, kPinnedN, moved with it)
-    int pad4;
+    int choff;         // its interpolation points: entry choff of the tables d_cheb, d_cheb32 (ranks
+                       // packed one after the other)
     int pad2;
     int64_t c_off;     // offset of the band's transform in the coefficient buffer (batches)
     int64_t nodes;     // nodes of the band (sorted positions node_off .. node_off + nodes)

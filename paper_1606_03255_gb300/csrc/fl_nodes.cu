@@ -245,4 +245,53 @@ cudaError_t launch_cell_shift(int32_t* cell, int64_t off, int64_t n, int shift, 
     return cudaGetLastError();
 }
 
+__global__ void k_cell_keys(int64_t n, const int32_t* __restrict__ cell, uint32_t* __restrict__ keys,
+                            int32_t* __restrict__ vals) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    keys[i] = (uint32_t)cell[i];
+    vals[i] = (int32_t)i;
+}
+
+__global__ void k_cell_permute(int64_t n, const uint32_t* __restrict__ keys, const int32_t* __restrict__ vals,
+                               const double2* __restrict__ ws_src, const int32_t* __restrict__ perm_src, int band,
+                               double2* __restrict__ ws, int32_t* __restrict__ perm,
+                               int32_t* __restrict__ bandid, int32_t* __restrict__ cell) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int32_t j = vals[i];
+    ws[i] = ws_src[j];
+    perm[i] = perm_src[j];
+    bandid[i] = band;
+    cell[i] = (int32_t)keys[i];
+}
+
+cudaError_t launch_cell_sort(Plan& p, int64_t off, int64_t n, int band, cudaStream_t st) {
+    if (n == 0) return cudaSuccess;
+    const int64_t blocks = (n + 2047) / 2048;          // radix-sort tiles
+    const size_t kb = (n * 4 + 255) / 256 * 256;
+    unsigned char* tmp = nullptr;                       // keys, vals (twice), perm, nodes, histogram
+    cudaError_t e = cudaMallocAsync((void**)&tmp, 5 * kb + n * sizeof(double2) + 256 * blocks * 4, st);
+    if (e != cudaSuccess) return e;
+    uint32_t *keys = (uint32_t*)tmp, *keys2 = (uint32_t*)(tmp + kb);
+    int32_t *vals = (int32_t*)(tmp + 2 * kb), *vals2 = (int32_t*)(tmp + 3 * kb), *perm = (int32_t*)(tmp + 4 * kb);
+    double2* ws = (double2*)(tmp + 5 * kb);
+    uint32_t* hist = (uint32_t*)(tmp + 5 * kb + n * sizeof(double2));
+    const unsigned grid = (unsigned)((n + 255) / 256);
+    e = cudaMemcpyAsync(perm, p.d_perm + off, n * 4, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(ws, p.d_ws + off, n * sizeof(double2), cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) {
+        k_cell_keys<<<grid, 256, 0, st>>>(n, p.d_cell + off, keys, vals);
+        e = radix_sort_pairs(keys, vals, keys2, vals2, hist, n, 32, st);
+    }
+    if (e == cudaSuccess) {
+        k_cell_permute<<<grid, 256, 0, st>>>(n, keys, vals, ws, perm, band, p.d_ws + off, p.d_perm + off,
+                                             p.d_bandid + off, p.d_cell + off);
+        e = cudaGetLastError();
+    }
+    const cudaError_t e2 = cudaFreeAsync(tmp, st);
+    return e != cudaSuccess ? e : e2;
+}
+
 }  // namespace fl

@@ -5,7 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "fl.h"
@@ -130,6 +132,8 @@ struct BandHost {
     int64_t nodes = 0;      // nodes of the band
     int64_t node_off = 0;   // first node of the band in sorted order
     int64_t fentries = 0;   // entries of the fused gather (0: not fused)
+    int64_t own = 0;        // nodes before bands were merged (what fl_get_info reports)
+    int leader = -1;        // merged band: the band that evaluates its nodes (the leader: itself)
     BandDev dev{};
 };
 
@@ -181,6 +185,11 @@ struct Plan {
     int fuse_mode = 0;             // window gather in pass 2: 0 by cost, 1 never, 2 wherever possible
     int sigma_mode = 0;            // oversampling: 0 by cost, 1 sigma = 2, 2 sub-bands wherever allowed
     double sigma_min = 2.0;        // smallest oversampling of the plan's grids
+    int qmax = 0;                  // largest rank of a band (q unless bands were merged)
+    bool q_given = false;          // q is the caller's, not from eps
+    bool own_gather = false;       // bands may have ranks of their own (see merge_bands)
+    std::map<std::pair<int, int>, int> rank_memo;   // see merged_rank
+    std::vector<int> ranks;        // ranks of the tables d_cheb, d_cheb32, in order
     int route_mode = 0;            // 0 by cost, 1 all NFFT, 2 all direct
     int variant = 0;               // 0 Algorithm 2 weights, 1 one-sided interpolation
     // real exponents xi_k >= 1 (fl_plan_xi): the Fourier factor is an NNFFT
@@ -230,9 +239,9 @@ struct Plan {
     BandDev* d_bands = nullptr;    // levels + 1 descriptors
     SmallWork* d_small = nullptr;
     PassItem* d_pass = nullptr;
-    double* d_cheb = nullptr;      // t_s (q), lambda_s (q)
-    float* d_cheb32 = nullptr;     // t_s as (hi, lo) float pairs, lambda_s in float, and the
-                                   // low part of lambda_s (4 q)
+    double* d_cheb = nullptr;      // per rank r: t_s (r), lambda_s (r)
+    float* d_cheb32 = nullptr;     // per rank r: t_s as (hi, lo) float pairs, lambda_s in float, and
+                                   // the low part of lambda_s (4 r)
     void* d_D = nullptr;           // weight tables (T)
     void* d_grid = nullptr;        // band grids (complex T)
     void* d_Y = nullptr;           // four-step intermediate (complex T)
@@ -308,6 +317,9 @@ cudaError_t launch_permute(Plan& p, const Instance& in, const double* nodes, con
                            const int32_t* vals, cudaStream_t st);
 cudaError_t launch_copy_sorted(Plan& p, const Instance& in, const Instance& twin, cudaStream_t st);
 // cell[off .. off + n) >>= shift (node cells of a band moved to a grid 2^shift times smaller)
+// nodes [off, off + n), all of bands with one grid size, put in cell order (stable)
+// as the nodes of `band`
+cudaError_t launch_cell_sort(Plan& p, int64_t off, int64_t n, int band, cudaStream_t st);
 cudaError_t launch_cell_shift(int32_t* cell, int64_t off, int64_t n, int shift, cudaStream_t st);
 
 // Launchers (fl_transform.cu)

@@ -149,7 +149,7 @@ static cudaError_t build_tables_t(Plan& p, const Instance& in, cudaStream_t st) 
     int64_t kt_max = 0;
     for (int lb = 1; lb <= in.levels; ++lb) {
         const BandHost& bh = p.bands[in.band_base + lb];
-        if (bh.dev.route != 1 || bh.dev.nrhs == 1 || p.variant == 1) continue;
+        if (bh.dev.route != 1 || bh.dev.nrhs == 1 || p.variant == 1 || bh.leader >= 0) continue;
         kt_max = std::max<int64_t>(kt_max, (int64_t)(bh.Lm - bh.ell + 1) * p.q * p.q);
     }
     if (kt_max > 0) {
@@ -159,7 +159,7 @@ static cudaError_t build_tables_t(Plan& p, const Instance& in, cudaStream_t st) 
     for (int lb = 1; lb <= in.levels; ++lb) {
         const BandHost& bh = p.bands[in.band_base + lb];
         if (bh.dev.route != 1) continue;
-        if (bh.dev.nrhs > 1 && p.variant == 0) {
+        if (bh.dev.nrhs > 1 && p.variant == 0 && bh.leader < 0) {
             const int64_t nk = (int64_t)(bh.Lm - bh.ell + 1) * p.q * p.q;
             k_coupling<<<(unsigned)((nk + 255) / 256), 256, 0, st>>>(p.y1, in.xi1, lb, bh.ell, bh.Lm,
                                                                      p.q, p.d_cheb, Kt);
@@ -167,9 +167,10 @@ static cudaError_t build_tables_t(Plan& p, const Instance& in, cudaStream_t st) 
         // a split band: the weights of each sub-band's frequencies (same coupling blocks)
         for (int c = 0; c < std::max(1, bh.dev.nsub); ++c) {
             const BandDev& d = bh.dev.nsub > 0 ? p.bands[bh.dev.sub0 + c].dev : bh.dev;
+            const bool merged = bh.leader >= 0;   // interpolation in y alone, at the merged band's points
             k_weights<T><<<(unsigned)((d.K + 255) / 256), 256, 0, st>>>(
-                d, bh.ell, bh.Lm, p.q, in.xi1, in.levels, p.d_cheb, Kt, p.mw, p.kb_b, p.variant,
-                p.xi_mode ? p.d_xis : nullptr, (T*)p.d_D);
+                d, bh.ell, bh.Lm, merged ? d.nrhs : p.q, in.xi1, in.levels, p.d_cheb + 2 * d.choff, Kt, p.mw,
+                p.kb_b, merged ? 1 : p.variant, p.xi_mode ? p.d_xis : nullptr, (T*)p.d_D);
         }
     }
     e = cudaGetLastError();
@@ -267,7 +268,11 @@ cudaError_t build_node_table(Plan& p, cudaStream_t st) {
 }
 
 cudaError_t build_cheb(Plan& p, cudaStream_t st) {
-    k_cheb<<<1, 64, 0, st>>>(p.q, p.d_cheb, p.d_cheb32);
+    int off = 0;
+    for (int r : p.ranks) {
+        k_cheb<<<1, 64, 0, st>>>(r, p.d_cheb + 2 * off, p.d_cheb32 + 4 * off);
+        off += r;
+    }
     return cudaGetLastError();
 }
 
@@ -426,7 +431,9 @@ __device__ __forceinline__ float2 split_rhs_f32(const float2* __restrict__ pp,
 // phase reduction -- the grid cell and its fraction floor/frac(n x), the
 // centring shift (N_m/2) x mod 1, a sub-band's kc x mod 1 -- is an exact
 // shift or wrapped product of X, so no FP64 arithmetic runs per node.
-template <int MW>
+// SUB: the sub-bands of a split band may be gathered from their grids (one set of
+// window values at the sub-band grid, a centre phase each).
+template <int MW, bool SUB>
 __device__ __forceinline__ float2 gather_node_f32(const uint4 nd, int64_t jl, const BandDev& B,
                                                   const BandDev* __restrict__ bands,
                                                   const float2* __restrict__ grid,
@@ -434,6 +441,26 @@ __device__ __forceinline__ float2 gather_node_f32(const uint4 nd, int64_t jl, co
                                                   const float2* __restrict__ fpp) {
     const uint64_t X = ((uint64_t)nd.y << 32) | nd.x;
     const float th = __uint_as_float(nd.z), tl = __uint_as_float(nd.w);
+    if constexpr (SUB) {
+        if (B.nsub > 0 && !bands[B.sub0].fused) {
+            const int64_t u = (int64_t)(X >> (64 - B.log2n));
+            const float fr = (float)((X << B.log2n) >> 40) * 0x1p-24f;
+            float phi[2 * MW];
+#pragma unroll
+            for (int t = 0; t < 2 * MW; ++t)
+                phi[t] = kb_window<float>(fr + (float)(MW - 1 - t), (float)MW, (float)B.kb);
+            float2 acc = {0.f, 0.f};
+            for (int c = 0; c < B.nsub; ++c) {
+                const BandDev& S = bands[B.sub0 + c];
+                const float2* g = grid + S.grid_off;
+                const float2 a = B.nrhs > 1 ? gather_rhs_f32<MW>(g, B, u - (MW - 1), B.n - 1, phi, th, tl, q, cheb32)
+                                            : tap_sum<MW>(g, u - (MW - 1), B.n - 1, phi);
+                const float ph = fixed_turns(X, (uint64_t)(S.k0 + (S.Nm >> 1)));
+                acc = cadd(acc, cmul(a, expipi<float>(2.f * ph)));
+            }
+            return acc;
+        }
+    }
     if (B.nsub > 0) return split_rhs_f32(fpp, bands, B, jl, th, tl, X, q, cheb32);
     float2 acc;
     if (B.fused) {
@@ -459,7 +486,9 @@ __device__ __forceinline__ float2 gather_node_f32(const uint4 nd, int64_t jl, co
 // XI (real exponents): the outer NFFT of the band's NNFFT runs at x/2, Z^0
 // nodes receive 0, and the epilogue is exp(2 pi i xc x) / Phi(x/2) instead of
 // the centring shift.
-template <typename T, int MW, bool XI = false>
+// OWN: every band interpolates at its own rank and points (B.nrhs, B.choff);
+// FP32 plans without a transform that may merge bands keep the kernel of one rank.
+template <typename T, int MW, bool XI = false, bool OWN = true>
 __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __restrict__ ws,
                                                 const int32_t* __restrict__ perm,
                                                 const int32_t* __restrict__ bandid,
@@ -484,8 +513,13 @@ __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __rest
     }
     // with rmul: f[j] = rmul[j] * conj(value) (node gradient, see fl_grad_w)
     if (B.route != 1) return;   // direct-route band: written by the direct kernels
+    if constexpr (OWN) {
+        q = B.nrhs;
+        cheb += 2 * B.choff;
+        cheb32 += 4 * B.choff;
+    }
     if constexpr (sizeof(T) == 4 && !XI) {
-        const C v = gather_node_f32<MW>(ntab[i], i - B.node_off, B, bands, grid, cheb32, q, kb_b, fpp);
+        const C v = gather_node_f32<MW, OWN>(ntab[i], i - B.node_off, B, bands, grid, cheb32, q, kb_b, fpp);
         f[j] = rmul ? cmulc(rmul[j], v) : v;
         return;
     }
@@ -579,7 +613,7 @@ __global__ void __launch_bounds__(256) k_spread_prep_ff(int64_t M, const double2
                                                         const int32_t* __restrict__ bandid,
                                                         const BandDev* __restrict__ bands,
                                                         const double2* __restrict__ r,
-                                                        const float* __restrict__ cheb32, int q,
+                                                        const float* __restrict__ cheb32, int ldl,
                                                         ff* __restrict__ sp_phi, ff* __restrict__ sp_L,
                                                         ffc* __restrict__ sp_rv) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -601,6 +635,8 @@ __global__ void __launch_bounds__(256) k_spread_prep_ff(int64_t M, const double2
 #pragma unroll
     for (int t = 0; t < 2 * MW; ++t) sp_phi[i * (2 * MW) + t] = ff_kb_window(fr + ff(MW - 1 - t), (float)MW, kb);
     if (B.nrhs > 1) {
+        const int q = B.nrhs;
+        cheb32 += 4 * B.choff;
         const ff tf = ff((kTwoPiD * wv.y - B.yc) * B.yh_inv);
         ff L[kMaxQ];
         ff den = ff(0);
@@ -616,7 +652,7 @@ __global__ void __launch_bounds__(256) k_spread_prep_ff(int64_t M, const double2
             den += L[s];
         }
         for (int s = 0; s < q; ++s)
-            sp_L[i * q + s] = hit >= 0 ? (s == hit ? ff(1) : ff(0)) : ff_div(L[s], den);
+            sp_L[i * ldl + s] = hit >= 0 ? (s == hit ? ff(1) : ff(0)) : ff_div(L[s], den);
     }
 }
 
@@ -631,7 +667,7 @@ __global__ void __launch_bounds__(256) k_spread_prep(int64_t M, const double2* _
                                                      const int32_t* __restrict__ bandid,
                                                      const BandDev* __restrict__ bands,
                                                      const C_t<T>* __restrict__ r,
-                                                     const double* __restrict__ cheb, int q, T kb_b,
+                                                     const double* __restrict__ cheb, int ldl, T kb_b,
                                                      T* __restrict__ sp_phi, T* __restrict__ sp_L,
                                                      C_t<T>* __restrict__ sp_rv) {
     using C = C_t<T>;
@@ -668,8 +704,8 @@ __global__ void __launch_bounds__(256) k_spread_prep(int64_t M, const double2* _
         sp_phi[i * (2 * MW) + t] = kb_window<T>(fr + (T)(MW - 1 - t), (T)MW, kb);
     if (B.nrhs > 1) {
         T Ls[kMaxQ];
-        bary_weights<T>(kTwoPiD * wv.y, B, q, cheb, Ls);
-        for (int s = 0; s < q; ++s) sp_L[i * q + s] = Ls[s];
+        bary_weights<T>(kTwoPiD * wv.y, B, B.nrhs, cheb + 2 * B.choff, Ls);
+        for (int s = 0; s < B.nrhs; ++s) sp_L[i * ldl + s] = Ls[s];
     }
 }
 
@@ -695,7 +731,7 @@ __device__ __forceinline__ void spread_cell_sum(const BandDev& B, int64_t l,
                                                 const T* __restrict__ sp_phi,
                                                 const T* __restrict__ sp_L,
                                                 const C_t<T>* __restrict__ sp_rv,
-                                                const double2* __restrict__ ws, int q,
+                                                const double2* __restrict__ ws, int ldl,
                                                 int lane, int stride, C_t<T>* acc) {
     using C = C_t<T>;
     // a sub-band: node j's value carries exp(-2 pi i kc x_j), kc its centre
@@ -734,7 +770,7 @@ __device__ __forceinline__ void spread_cell_sum(const BandDev& B, int64_t l,
                 acc[0] = cadd(acc[0], w);
             } else {
                 for (int s = 0; s < nr; ++s) {
-                    const T L = sp_L[j * q + s];
+                    const T L = sp_L[j * ldl + s];
                     acc[s].x += L * w.x;
                     acc[s].y += L * w.y;
                 }
@@ -770,7 +806,7 @@ __global__ void __launch_bounds__(256) k_spread_cells(int ncb, const Plan::CellB
                                                       const T* __restrict__ sp_phi,
                                                       const T* __restrict__ sp_L,
                                                       const C_t<T>* __restrict__ sp_rv,
-                                                      const double2* __restrict__ ws, int q,
+                                                      const double2* __restrict__ ws, int ldl,
                                                       G* __restrict__ grid) {
     using C = C_t<T>;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -780,7 +816,7 @@ __global__ void __launch_bounds__(256) k_spread_cells(int ncb, const Plan::CellB
     const int64_t l = g - cbs[cb].prefix;
     C acc[kMaxQ];
     for (int s = 0; s < B.nrhs; ++s) acc[s] = C{(T)0, (T)0};
-    spread_cell_sum<T, MW>(B, l, cell, sp_phi, sp_L, sp_rv, ws, q, 0, 1, acc);
+    spread_cell_sum<T, MW>(B, l, cell, sp_phi, sp_L, sp_rv, ws, ldl, 0, 1, acc);
     G* gb = grid + B.grid_off + l;
     for (int s = 0; s < B.nrhs; ++s) gb[(int64_t)s * B.n] = grid_value<G>(acc[s]);
 }
@@ -804,7 +840,7 @@ __global__ void __launch_bounds__(kSpreadDense) k_spread_cells_warp(int ncb, con
                                                                     const T* __restrict__ sp_phi,
                                                                     const T* __restrict__ sp_L,
                                                                     const C_t<T>* __restrict__ sp_rv,
-                                                                    const double2* __restrict__ ws, int q,
+                                                                    const double2* __restrict__ ws, int ldl,
                                                                     G* __restrict__ grid) {
     using C = C_t<T>;
     __shared__ C red[kSpreadDense / 32][kMaxQ];
@@ -816,7 +852,7 @@ __global__ void __launch_bounds__(kSpreadDense) k_spread_cells_warp(int ncb, con
     const int64_t l = g - cbs[cb].prefix;
     C acc[kMaxQ];
     for (int s = 0; s < B.nrhs; ++s) acc[s] = C{(T)0, (T)0};
-    spread_cell_sum<T, MW>(B, l, cell, sp_phi, sp_L, sp_rv, ws, q, threadIdx.x, kSpreadDense, acc);
+    spread_cell_sum<T, MW>(B, l, cell, sp_phi, sp_L, sp_rv, ws, ldl, threadIdx.x, kSpreadDense, acc);
     for (int s = 0; s < B.nrhs; ++s) {
         T x = acc[s].x, y = acc[s].y;
 #pragma unroll
@@ -988,7 +1024,10 @@ static cudaError_t gather_t(Plan& p, const void* c, void* f, bool deriv, const v
     }
     int slot;
     timer_begin(p, "gather", bytes, st, &slot);
-    k_gather<T, MW><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
+    auto kern = k_gather<T, MW>;
+    if constexpr (sizeof(T) == 4)
+        if (!p.own_gather) kern = k_gather<T, MW, false, false>;
+    kern<<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
         p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const C*)p.d_grid, p.d_cheb, p.d_cheb32,
         p.q, (T)p.kb_b, (const C*)c, deriv ? 1 : 0, (const C*)rmul, p.d_fpp, p.d_ntab, (C*)f);
     timer_end(p, slot, st);
@@ -1070,7 +1109,7 @@ __global__ void __launch_bounds__(256) k_gather_ff(int64_t M, const double2* __r
                                                    const int32_t* __restrict__ bandid,
                                                    const BandDev* __restrict__ bands,
                                                    const ffc* __restrict__ grid,
-                                                   const float* __restrict__ cheb32, int q,
+                                                   const float* __restrict__ cheb32,
                                                    double kb_b, const double2* __restrict__ c,
                                                    int deriv, const double2* __restrict__ rmul,
                                                    double2* __restrict__ f) {
@@ -1084,6 +1123,8 @@ __global__ void __launch_bounds__(256) k_gather_ff(int64_t M, const double2* __r
         return;
     }
     if (B.route != 1) return;     // direct-route band: written by the direct kernels
+    const int q = B.nrhs;
+    cheb32 += 4 * B.choff;
     const double2 wv = ws[i];
     const double x = wv.x - floor(wv.x);
     const double t0 = (double)B.n * x;
@@ -1145,7 +1186,7 @@ static cudaError_t gather_ff_t(Plan& p, const void* c, void* f, bool deriv, cons
     int slot;
     timer_begin(p, "gather", bytes, st, &slot);
     k_gather_ff<MW><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
-        p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const ffc*)p.d_grid, p.d_cheb32, p.q,
+        p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const ffc*)p.d_grid, p.d_cheb32,
         p.kb_b, (const double2*)c, deriv ? 1 : 0, (const double2*)rmul, (double2*)f);
     timer_end(p, slot, st);
     ++p.launches;
@@ -1189,23 +1230,23 @@ static cudaError_t spread_t(Plan& p, const void* r, cudaStream_t st) {
     timer_begin(p, "spread", 0.0, st, &slot);
     if constexpr (std::is_same<T, ff>::value) {
         k_spread_prep_ff<MW><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
-            p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const double2*)r, p.d_cheb32, p.q,
+            p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const double2*)r, p.d_cheb32, p.qmax,
             (ff*)p.d_sp_phi, (ff*)p.d_sp_L, (ffc*)p.d_sp_rv);
     } else {
         auto prep = p.xi_mode ? k_spread_prep<T, MW, true> : k_spread_prep<T, MW, false>;
         prep<<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
-            p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const C*)r, p.d_cheb, p.q, (T)p.kb_b,
+            p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const C*)r, p.d_cheb, p.qmax, (T)p.kb_b,
             (T*)p.d_sp_phi, (T*)p.d_sp_L, (C*)p.d_sp_rv);
     }
     if (p.cells_total > 0)
         k_spread_cells<T, MW, G><<<(unsigned)((p.cells_total + 255) / 256), 256, 0, st>>>(
             (int)p.n_sparse_cb, p.d_cell_bands, p.cells_total, p.d_bands, p.d_cell,
-            (const T*)p.d_sp_phi, (const T*)p.d_sp_L, (const C*)p.d_sp_rv, p.d_ws, p.q, (G*)p.d_grid);
+            (const T*)p.d_sp_phi, (const T*)p.d_sp_L, (const C*)p.d_sp_rv, p.d_ws, p.qmax, (G*)p.d_grid);
     if (p.cells_dense > 0)
         k_spread_cells_warp<T, MW, G><<<(unsigned)p.cells_dense, kSpreadDense, 0, st>>>(
             (int)(p.cell_bands.size() - p.n_sparse_cb), p.d_cell_bands + p.n_sparse_cb,
             p.cells_dense, p.d_bands, p.d_cell, (const T*)p.d_sp_phi, (const T*)p.d_sp_L,
-            (const C*)p.d_sp_rv, p.d_ws, p.q, (G*)p.d_grid);
+            (const C*)p.d_sp_rv, p.d_ws, p.qmax, (G*)p.d_grid);
     timer_end(p, slot, st);
     p.launches += 1 + (p.cells_total > 0) + (p.cells_dense > 0);
     return cudaGetLastError();
