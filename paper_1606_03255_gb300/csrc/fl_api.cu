@@ -41,7 +41,7 @@ Plan::~Plan() {
     void* ptrs[] = {d_ws, d_perm, d_bandid, d_bands, d_small, d_pass, d_cheb, d_D, d_grid, d_Y,
                     d_stage_c, d_stage_f, d_stage_r, d_z0, d_t, d_s, d_tband, d_sband, d_lap, d_direct,
                     d_dranges, d_dpart, d_cdir, d_dsegs, d_dadj, d_dz, d_cell, d_sp_phi,
-                    d_sp_L, d_sp_rv, d_cell_bands, d_lapK, d_lapKoff, d_tw, d_nearT, d_cheb32, d_cff, d_tperm, d_ts, d_tbs, d_ttau, d_stau, d_lapitems,
+                    d_sp_L, d_sp_rv, d_sp_e, d_sp_blocks, d_dn_groups, d_sp_ranges, d_dn_start, d_comb, d_lapK, d_lapKoff, d_tw, d_nearT, d_cheb32, d_cff, d_tperm, d_ts, d_tbs, d_ttau, d_stau, d_lapitems,
                     d_xis, d_xperm, d_xbk, d_xstart, d_xwin, d_xiphi, d_xcs, d_xsb,
                     d_frbs, d_fent, d_fphi, d_fpp, d_ntab, d_boff, d_bptr};
     for (void* q : ptrs)
@@ -1100,34 +1100,13 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
         FL_CUDA(cudaMalloc(&p.d_dz, 2 * M * cs), "cudaMalloc direct bases");
         FL_CUDA(build_direct_base(p, st), "fl_plan: direct bases");
     }
-    // adjoint of the NFFT bands (single plans): per-node taps and weights, cell list
-    p.cell_bands.clear();
-    p.cells_total = p.cells_dense = 0;
-    p.n_sparse_cb = 0;
+    // adjoint of the NFFT bands (single plans): per-node taps and weights, cell lists
     if (!p.batched && M > 0) {
-        // dense: on average >= 32 window contributions per cell (warp per cell)
-        auto dense = [&](const BandHost& bh) { return bh.nodes * 2 * p.mw >= 32 * bh.dev.n; };
-        for (int b = 0; b < nb; ++b) {
-            const BandDev& d = p.bands[b].dev;
-            if (d.route != 1 || d.nsub > 0 || dense(p.bands[b])) continue;
-            p.cell_bands.push_back({b, 0, p.cells_total});
-            p.cells_total += d.n;
-        }
-        p.n_sparse_cb = (int)p.cell_bands.size();
-        for (int b = 0; b < nb; ++b) {
-            const BandDev& d = p.bands[b].dev;
-            if (d.route != 1 || d.nsub > 0 || !dense(p.bands[b])) continue;
-            p.cell_bands.push_back({b, 0, p.cells_dense});
-            p.cells_dense += d.n;
-        }
-        if (!p.cell_bands.empty()) {
-            FL_CUDA(cudaMalloc((void**)&p.d_cell_bands, p.cell_bands.size() * sizeof(Plan::CellBand)),
-                    "cudaMalloc cell bands");
-            FL_CUDA(cudaMemcpyAsync(p.d_cell_bands, p.cell_bands.data(),
-                                    p.cell_bands.size() * sizeof(Plan::CellBand), cudaMemcpyHostToDevice, st),
-                    "copy cell bands");
+        FL_CUDA(build_spread(p, st), "fl_plan: adjoint lists");
+        if (p.n_sp_blocks + p.n_dn_groups[0] + p.n_dn_groups[1] > 0) {
             FL_CUDA(cudaMalloc(&p.d_sp_phi, (size_t)M * 2 * p.mw * rs), "cudaMalloc adjoint taps");
             FL_CUDA(cudaMalloc(&p.d_sp_L, (size_t)M * p.qmax * rs), "cudaMalloc adjoint weights");
+            FL_CUDA(cudaMalloc(&p.d_sp_e, (size_t)M * cs), "cudaMalloc adjoint shifts");
             FL_CUDA(cudaMalloc(&p.d_sp_rv, (size_t)M * cs), "cudaMalloc adjoint residuals");
         }
     }
@@ -1148,6 +1127,7 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     FL_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * cheb_len * sizeof(double)), "cudaMalloc cheb");
     FL_CUDA(cudaMalloc((void**)&p.d_cheb32, 4 * cheb_len * sizeof(float)), "cudaMalloc cheb32");
     FL_CUDA(build_cheb(p, st), "fl_plan: tables");
+    if (p.d_sp_phi) FL_CUDA(build_node_weights(p, st), "fl_plan: node weights");
     for (int i = 0; i < B; ++i)
         if (!shares_D[i]) FL_CUDA(build_tables(p, p.inst[i], st), "fl_plan: tables");
     FL_CUDA(cudaStreamSynchronize(st), "fl_plan: synchronise");

@@ -124,6 +124,15 @@ struct DirectRange {
     int64_t prefix;  // nodes of the segments before it
 };
 
+// One grid of the adjoint's combination (an NFFT band or sub-band).
+struct CombineItem {
+    int64_t k0, K;             // its frequencies k0 .. k0 + K - 1
+    int64_t D_off, grid_off;
+    int64_t half, n;           // N_m / 2, grid points
+    int nrhs;
+    int pad;
+};
+
 // Per-band plan data on the host.
 struct BandHost {
     int ell = 0, Lm = 0;    // l_m, L_m (Definition 3.2); 0 for the Y_M band
@@ -223,19 +232,17 @@ struct Plan {
     int32_t* d_cell = nullptr;     // grid cell floor(n_m x) of each sorted node
     uint4* d_ntab = nullptr;       // FP32 plans: per sorted node x 2^64 (64-bit fixed point) and
                                    // the barycentric tau of its band as a float pair
-    void* d_sp_phi = nullptr;      // adjoint: window taps per node (M x 2 m_w, T)
-    void* d_sp_L = nullptr;        // adjoint: barycentric weights per node (M x q, T)
-    void* d_sp_rv = nullptr;       // adjoint: shifted residual per node (M, complex T)
-    struct CellBand {              // adjoint: the cells of one NFFT band
-        int band;
-        int pad;
-        int64_t prefix;            // cells of the NFFT bands before it
-    };
-    std::vector<CellBand> cell_bands;   // sparse bands first, then dense ones
-    CellBand* d_cell_bands = nullptr;
-    int n_sparse_cb = 0;
-    int64_t cells_total = 0;            // cells of the sparse bands
-    int64_t cells_dense = 0;            // cells of the dense bands
+    // single plans: per sorted node its window taps (M x 2 m_w), interpolation
+    // weights (M x qmax), shift (M complex), and the adjoint's shifted values
+    void *d_sp_phi = nullptr, *d_sp_L = nullptr, *d_sp_e = nullptr, *d_sp_rv = nullptr;
+    // adjoint spreading (fl_adjoint.cu): the sparse bands with their first blocks
+    // and the nodes of every block, the dense bands with their first cell groups
+    // and the cell starts; the grids of the combination
+    int4 *d_sp_blocks = nullptr, *d_dn_groups = nullptr, *d_sp_ranges = nullptr;
+    int32_t* d_dn_start = nullptr;
+    CombineItem* d_comb = nullptr;
+    int n_sp_bands = 0, n_dn_bands[2] = {0, 0}, n_comb = 0;
+    int64_t n_sp_blocks = 0, n_dn_groups[2] = {0, 0};   // dense: by warp, by CTA
     BandDev* d_bands = nullptr;    // levels + 1 descriptors
     SmallWork* d_small = nullptr;
     PassItem* d_pass = nullptr;
@@ -337,6 +344,12 @@ cudaError_t build_xi_tables(Plan& p, cudaStream_t st);
 cudaError_t launch_xi_spread(Plan& p, const void* c, cudaStream_t st);
 cudaError_t launch_xi_combine(Plan& p, void* out, cudaStream_t st);   // adjoint: grids -> c
 cudaError_t run_forward_xi(Plan& p, const void* c, void* f, cudaStream_t st);
+
+// Launchers (fl_adjoint.cu)
+cudaError_t build_spread(Plan& p, cudaStream_t st);         // cell lists
+cudaError_t build_node_weights(Plan& p, cudaStream_t st);   // d_sp_phi, d_sp_L, d_sp_e
+cudaError_t launch_spread(Plan& p, const void* r, cudaStream_t st);
+cudaError_t launch_combine(Plan& p, const void* r, void* c_out, cudaStream_t st);
 
 // Launchers (fl_direct.cu)
 cudaError_t build_direct_base(Plan& p, cudaStream_t st);   // d_dz

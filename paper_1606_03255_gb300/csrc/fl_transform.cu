@@ -167,6 +167,7 @@ static cudaError_t build_tables_t(Plan& p, const Instance& in, cudaStream_t st) 
         // a split band: the weights of each sub-band's frequencies (same coupling blocks)
         for (int c = 0; c < std::max(1, bh.dev.nsub); ++c) {
             const BandDev& d = bh.dev.nsub > 0 ? p.bands[bh.dev.sub0 + c].dev : bh.dev;
+            if (d.K == 0) continue;   // real exponents: none below the band's cut
             const bool merged = bh.leader >= 0;   // interpolation in y alone, at the merged band's points
             k_weights<T><<<(unsigned)((d.K + 255) / 256), 256, 0, st>>>(
                 d, bh.ell, bh.Lm, merged ? d.nrhs : p.q, in.xi1, in.levels, p.d_cheb + 2 * d.choff, Kt, p.mw,
@@ -488,6 +489,8 @@ __device__ __forceinline__ float2 gather_node_f32(const uint4 nd, int64_t jl, co
 // the centring shift.
 // OWN: every band interpolates at its own rank and points (B.nrhs, B.choff);
 // FP32 plans without a transform that may merge bands keep the kernel of one rank.
+// FP64 single plans read each node's taps and weights from the plan's tables
+// (phi_tab, L_tab; null for batches, which form them here).
 template <typename T, int MW, bool XI = false, bool OWN = true>
 __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __restrict__ ws,
                                                 const int32_t* __restrict__ perm,
@@ -500,7 +503,9 @@ __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __rest
                                                 const C_t<T>* __restrict__ rmul,
                                                 const float2* __restrict__ fpp,
                                                 const uint4* __restrict__ ntab,
-                                                C_t<T>* __restrict__ f) {
+                                                C_t<T>* __restrict__ f,
+                                                const T* __restrict__ phi_tab = nullptr,
+                                                const T* __restrict__ L_tab = nullptr, int ldl = 0) {
     using C = C_t<T>;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M) return;
@@ -533,15 +538,27 @@ __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __rest
     const int64_t lo = (int64_t)u - (MW - 1);
     T phi[2 * MW];
     const T kb = XI ? kb_b : (T)B.kb;   // the window shape of the band's grids
+    bool tab = false;
+    if constexpr (sizeof(T) == 8) {
+        if (phi_tab) {
+            tab = true;
 #pragma unroll
-    for (int t = 0; t < 2 * MW; ++t) phi[t] = kb_window<T>(fr + (T)(MW - 1 - t), (T)MW, kb);
+            for (int t = 0; t < 2 * MW; ++t) phi[t] = phi_tab[i * (2 * MW) + t];
+        }
+    }
+    if (!tab) {
+#pragma unroll
+        for (int t = 0; t < 2 * MW; ++t) phi[t] = kb_window<T>(fr + (T)(MW - 1 - t), (T)MW, kb);
+    }
     const int64_t nmask = B.n - 1;
     const C* g = grid + B.grid_off;
     if constexpr (sizeof(T) == 8 && !XI) {
         if (B.nsub > 0) {   // split band (FP64): its sub-bands' grids, each with its centre phase
-            T Ls[kMaxQ];
-            if (B.nrhs > 1) bary_weights<T>(kTwoPiD * wv.y, B, q, cheb, Ls);
-            else Ls[0] = (T)1;   // the Y_M band: one right-hand side
+            T Lw[kMaxQ];
+            const T* Ls = Lw;
+            if (B.nrhs == 1) Lw[0] = (T)1;   // the Y_M band: one right-hand side
+            else if (tab) Ls = L_tab + i * ldl;
+            else bary_weights<T>(kTwoPiD * wv.y, B, q, cheb, Lw);
             for (int sb = 0; sb < B.nsub; ++sb) {
                 const BandDev S = bands[B.sub0 + sb];
                 const C* gs = grid + S.grid_off;
@@ -569,8 +586,10 @@ __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __rest
     } else if (B.nrhs == 1) {
         acc = tap_sum<MW>(g, lo, nmask, phi);
     } else if constexpr (sizeof(T) == 8) {
-        T Ls[kMaxQ];
-        bary_weights<T>(kTwoPiD * wv.y, B, q, cheb, Ls);
+        T Lw[kMaxQ];
+        const T* Ls = Lw;
+        if (tab) Ls = L_tab + i * ldl;
+        else bary_weights<T>(kTwoPiD * wv.y, B, q, cheb, Lw);
         for (int s = 0; s < q; ++s) {
             const C a = tap_sum<MW>(g + (int64_t)s * B.n, lo, nmask, phi);
             acc.x += Ls[s] * a.x;
@@ -598,338 +617,6 @@ __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __rest
         val = cmul(acc, expipi<T>((T)(2.0 * ph)));
     }
     f[j] = rmul ? cmulc(rmul[j], val) : val;
-}
-
-// ---------------------------------------------------------------------------
-// Adjoint: spread (transpose of the gather), FFT with sign -, combine.
-
-// The float-pair form's spreading preparation: k_spread_prep's per-node
-// window taps, barycentric weights and shifted r_j in pairs (the window from
-// one pair exponential, the weights as in k_gather_ff); the phase (N_m/2) x
-// mod 1 is reduced exactly in double.
-template <int MW>
-__global__ void __launch_bounds__(256) k_spread_prep_ff(int64_t M, const double2* __restrict__ ws,
-                                                        const int32_t* __restrict__ perm,
-                                                        const int32_t* __restrict__ bandid,
-                                                        const BandDev* __restrict__ bands,
-                                                        const double2* __restrict__ r,
-                                                        const float* __restrict__ cheb32, int ldl,
-                                                        ff* __restrict__ sp_phi, ff* __restrict__ sp_L,
-                                                        ffc* __restrict__ sp_rv) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
-    const BandDev B = bands[bandid[i]];
-    if (B.route != 1) return;
-    const double2 wv = ws[i];
-    const double x = wv.x - floor(wv.x);
-    const double t0 = (double)B.n * x;
-    const ff fr = ff(t0 - floor(t0));
-    double ph = (double)(B.Nm >> 1) * x;   // N_m a power of two: exact
-    ph -= floor(ph);
-    if (ph >= 0.5) ph -= 1.0;
-    ffc e;
-    ff_sincospi(ff(2.0 * ph), &e.y, &e.x);
-    const double2 rj = r[perm[i]];
-    sp_rv[i] = cmulc(ffc{ff(rj.x), ff(rj.y)}, e);
-    const ff kb = ff(B.kb);
-#pragma unroll
-    for (int t = 0; t < 2 * MW; ++t) sp_phi[i * (2 * MW) + t] = ff_kb_window(fr + ff(MW - 1 - t), (float)MW, kb);
-    if (B.nrhs > 1) {
-        const int q = B.nrhs;
-        cheb32 += 4 * B.choff;
-        const ff tf = ff((kTwoPiD * wv.y - B.yc) * B.yh_inv);
-        ff L[kMaxQ];
-        ff den = ff(0);
-        int hit = -1;
-        for (int s = 0; s < q; ++s) {
-            const ff d = tf - ff(cheb32[s], cheb32[q + s]);
-            if (d.hi == 0.f && d.lo == 0.f) {
-                hit = s;
-                L[s] = ff(0);
-                continue;
-            }
-            L[s] = ff_div(ff(cheb32[2 * q + s], cheb32[3 * q + s]), d);
-            den += L[s];
-        }
-        for (int s = 0; s < q; ++s)
-            sp_L[i * ldl + s] = hit >= 0 ? (s == hit ? ff(1) : ff(0)) : ff_div(L[s], den);
-    }
-}
-
-// Adjoint spreading, the transpose of the gather, without atomics in two
-// steps.  k_spread_prep: for every sorted node of an NFFT band its 2 m_w window
-// taps, its barycentric weights L_s(y_j) and rv_j = r_j exp(-2 pi i (N_m/2) x_j).
-// XI (real exponents): taps at x_j/2 and rv_j = r_j exp(-2 pi i xc x_j) /
-// Phi(x_j/2), the conjugate of the forward epilogue.
-template <typename T, int MW, bool XI = false>
-__global__ void __launch_bounds__(256) k_spread_prep(int64_t M, const double2* __restrict__ ws,
-                                                     const int32_t* __restrict__ perm,
-                                                     const int32_t* __restrict__ bandid,
-                                                     const BandDev* __restrict__ bands,
-                                                     const C_t<T>* __restrict__ r,
-                                                     const double* __restrict__ cheb, int ldl, T kb_b,
-                                                     T* __restrict__ sp_phi, T* __restrict__ sp_L,
-                                                     C_t<T>* __restrict__ sp_rv) {
-    using C = C_t<T>;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M) return;
-    const BandDev B = bands[bandid[i]];
-    if (B.route != 1) return;
-    const double2 wv = ws[i];
-    const double xs = XI ? 0.5 * wv.x : wv.x;
-    const double x = xs - floor(xs);
-    const double t0 = (double)B.n * x;
-    const T fr = (T)(t0 - floor(t0));
-    if (B.nsub > 0) {   // split band: each sub-band applies its own centre phase
-        sp_rv[i] = r[perm[i]];
-    } else if constexpr (XI) {
-        const double ph = frac_turns(B.xc, wv.x);
-        const T v = (T)(kTwoPiD * 0.5 * wv.x);
-        const T arg = kb_b * kb_b - v * v;
-        const T rr = (T)MW * sqrt(arg > (T)0 ? arg : (T)0);
-        T i0;
-        if constexpr (sizeof(T) == 4) i0 = cyl_bessel_i0f(rr);
-        else i0 = cyl_bessel_i0(rr);
-        const C rv = cmulc(r[perm[i]], expipi<T>((T)(2.0 * ph)));
-        sp_rv[i] = cscale(rv, (T)1 / ((T)kPi * i0));
-    } else {
-        double ph = (double)(B.Nm >> 1) * x;   // N_m a power of two: exact
-        ph -= floor(ph);
-        if (ph >= 0.5) ph -= 1.0;
-        sp_rv[i] = cmulc(r[perm[i]], expipi<T>((T)(2.0 * ph)));
-    }
-    const T kb = XI ? kb_b : (T)B.kb;   // the window shape of the band's grid
-#pragma unroll
-    for (int t = 0; t < 2 * MW; ++t)
-        sp_phi[i * (2 * MW) + t] = kb_window<T>(fr + (T)(MW - 1 - t), (T)MW, kb);
-    if (B.nrhs > 1) {
-        T Ls[kMaxQ];
-        bary_weights<T>(kTwoPiD * wv.y, B, B.nrhs, cheb + 2 * B.choff, Ls);
-        for (int s = 0; s < B.nrhs; ++s) sp_L[i * ldl + s] = Ls[s];
-    }
-}
-
-// First sorted node of [lo, hi) whose cell is >= v (cells ascend within a band).
-__device__ __forceinline__ int64_t lower_cell(const int32_t* __restrict__ cell, int64_t lo,
-                                              int64_t hi, int64_t v) {
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (cell[mid] < v) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// Sum over the nodes that cover grid cell l of one NFFT band: the nodes whose
-// cell u lies in [l - m_w, l + m_w - 1] (mod n) form a contiguous range of the
-// band's cell-sorted nodes (two near the ends); node j adds window tap
-// t = l - u + m_w - 1 times rv_j, times L_s(y_j) for right-hand side s.  The
-// lanes lane, lane + stride, ... of the range are summed into acc.
-template <typename T, int MW>
-__device__ __forceinline__ void spread_cell_sum(const BandDev& B, int64_t l,
-                                                const int32_t* __restrict__ cell,
-                                                const T* __restrict__ sp_phi,
-                                                const T* __restrict__ sp_L,
-                                                const C_t<T>* __restrict__ sp_rv,
-                                                const double2* __restrict__ ws, int ldl,
-                                                int lane, int stride, C_t<T>* acc) {
-    using C = C_t<T>;
-    // a sub-band: node j's value carries exp(-2 pi i kc x_j), kc its centre
-    const double kc = (double)(B.k0 + (B.Nm >> 1));
-    const int64_t n = B.n, nb0 = B.node_off, nend = B.node_off + B.nodes;
-    int64_t ra[2][2];
-    int nrange = 0;
-    const int64_t c0 = l - MW, c1 = l + MW - 1;
-    if (c0 < 0) {
-        ra[0][0] = n + c0; ra[0][1] = n - 1;
-        ra[1][0] = 0; ra[1][1] = c1;
-        nrange = 2;
-    } else if (c1 >= n) {
-        ra[0][0] = c0; ra[0][1] = n - 1;
-        ra[1][0] = 0; ra[1][1] = c1 - n;
-        nrange = 2;
-    } else {
-        ra[0][0] = c0; ra[0][1] = c1;
-        nrange = 1;
-    }
-    const int nr = B.nrhs;
-    for (int rr = 0; rr < nrange; ++rr) {
-        const int64_t j0 = lower_cell(cell, nb0, nend, ra[rr][0]);
-        const int64_t j1 = lower_cell(cell, j0, nend, ra[rr][1] + 1);
-        for (int64_t j = j0 + lane; j < j1; j += stride) {
-            int64_t t = (l - cell[j] + MW - 1) % n;
-            if (t < 0) t += n;
-            C w = cscale(sp_rv[j], sp_phi[j * (2 * MW) + t]);
-            if constexpr (!std::is_same<T, ff>::value) {   // (no sub-bands in float pairs)
-                if (B.parent >= 0) {
-                    const double xj = ws[j].x - floor(ws[j].x);
-                    w = cmul(w, expipi<T>((T)(-2.0 * frac_turns(kc, xj))));
-                }
-            }
-            if (nr == 1) {
-                acc[0] = cadd(acc[0], w);
-            } else {
-                for (int s = 0; s < nr; ++s) {
-                    const T L = sp_L[j * ldl + s];
-                    acc[s].x += L * w.x;
-                    acc[s].y += L * w.y;
-                }
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ int find_cell_band(const Plan::CellBand* __restrict__ cbs, int ncb,
-                                              int64_t g) {
-    int lo = 0, hi = ncb;   // last entry with prefix <= g
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (cbs[mid].prefix <= g) lo = mid;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// A spread grid value as stored: C_t<T>, or rounded to a float pair (the grids
-// of the float-pair form, whose spreading runs in double).
-template <typename G, typename C> __device__ __forceinline__ G grid_value(const C& v) {
-    if constexpr (std::is_same<G, ffc>::value) return ffc{ff(v.x), ff(v.y)};
-    else return v;
-}
-
-// k_spread_cells: one thread per (sparse NFFT band, grid cell l); writes a_s[l]
-// for every right-hand side s.
-template <typename T, int MW, typename G = C_t<T>>
-__global__ void __launch_bounds__(256) k_spread_cells(int ncb, const Plan::CellBand* __restrict__ cbs,
-                                                      int64_t total, const BandDev* __restrict__ bands,
-                                                      const int32_t* __restrict__ cell,
-                                                      const T* __restrict__ sp_phi,
-                                                      const T* __restrict__ sp_L,
-                                                      const C_t<T>* __restrict__ sp_rv,
-                                                      const double2* __restrict__ ws, int ldl,
-                                                      G* __restrict__ grid) {
-    using C = C_t<T>;
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= total) return;
-    const int cb = find_cell_band(cbs, ncb, g);
-    const BandDev B = bands[cbs[cb].band];
-    const int64_t l = g - cbs[cb].prefix;
-    C acc[kMaxQ];
-    for (int s = 0; s < B.nrhs; ++s) acc[s] = C{(T)0, (T)0};
-    spread_cell_sum<T, MW>(B, l, cell, sp_phi, sp_L, sp_rv, ws, ldl, 0, 1, acc);
-    G* gb = grid + B.grid_off + l;
-    for (int s = 0; s < B.nrhs; ++s) gb[(int64_t)s * B.n] = grid_value<G>(acc[s]);
-}
-
-__device__ __forceinline__ float shfl_xor_t(float v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
-__device__ __forceinline__ double shfl_xor_t(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
-__device__ __forceinline__ ff shfl_xor_t(ff v, int off) {
-    return ff(__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off));
-}
-
-// Dense NFFT bands (many nodes per cell): one CTA of kSpreadDense threads per
-// cell, threads strided over the covering nodes; the thread sums are combined
-// in a fixed order (a shuffle tree per warp, then the warps in order).
-constexpr int kSpreadDense = 256;
-
-template <typename T, int MW, typename G = C_t<T>>
-__global__ void __launch_bounds__(kSpreadDense) k_spread_cells_warp(int ncb, const Plan::CellBand* __restrict__ cbs,
-                                                                    int64_t total,
-                                                                    const BandDev* __restrict__ bands,
-                                                                    const int32_t* __restrict__ cell,
-                                                                    const T* __restrict__ sp_phi,
-                                                                    const T* __restrict__ sp_L,
-                                                                    const C_t<T>* __restrict__ sp_rv,
-                                                                    const double2* __restrict__ ws, int ldl,
-                                                                    G* __restrict__ grid) {
-    using C = C_t<T>;
-    __shared__ C red[kSpreadDense / 32][kMaxQ];
-    const int64_t g = blockIdx.x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (g >= total) return;
-    const int cb = find_cell_band(cbs, ncb, g);
-    const BandDev B = bands[cbs[cb].band];
-    const int64_t l = g - cbs[cb].prefix;
-    C acc[kMaxQ];
-    for (int s = 0; s < B.nrhs; ++s) acc[s] = C{(T)0, (T)0};
-    spread_cell_sum<T, MW>(B, l, cell, sp_phi, sp_L, sp_rv, ws, ldl, threadIdx.x, kSpreadDense, acc);
-    for (int s = 0; s < B.nrhs; ++s) {
-        T x = acc[s].x, y = acc[s].y;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            x += shfl_xor_t(x, off);
-            y += shfl_xor_t(y, off);
-        }
-        if (lane == 0) red[w][s] = C{x, y};
-    }
-    __syncthreads();
-    const int s = threadIdx.x;
-    if (s < B.nrhs) {
-        C sum = red[0][s];
-        for (int ww = 1; ww < kSpreadDense / 32; ++ww) sum = cadd(sum, red[ww][s]);
-        grid[B.grid_off + l + (int64_t)s * B.n] = grid_value<G>(sum);
-    }
-}
-
-// Sum of r over the Z^0 nodes (the first z0 sorted nodes): c_out[0] gets it.
-template <typename T>
-__global__ void k_z0_sum(int64_t z0, const int32_t* __restrict__ perm,
-                         const C_t<T>* __restrict__ r, C_t<T>* __restrict__ out) {
-    __shared__ T sx[256], sy[256];
-    T ax = 0, ay = 0;
-    for (int64_t i = threadIdx.x; i < z0; i += 256) {
-        const C_t<T> v = r[perm[i]];
-        ax += v.x;
-        ay += v.y;
-    }
-    sx[threadIdx.x] = ax;
-    sy[threadIdx.x] = ay;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h) {
-            sx[threadIdx.x] += sx[threadIdx.x + h];
-            sy[threadIdx.x] += sy[threadIdx.x + h];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = C_t<T>{sx[0], sy[0]};
-}
-
-// c_out[k] = [k == 0] z0sum + sum_bands sum_s D[s][k] b_s[(k - N_m/2) mod n],
-// accumulated in T (double for the float-pair form, whose grids G and weights
-// DT are float pairs).
-template <typename T, typename G = C_t<T>, typename DT = T>
-__global__ void k_combine(int64_t N, int levels, const BandDev* __restrict__ bands,
-                          const DT* __restrict__ D, const G* __restrict__ grid,
-                          const C_t<T>* __restrict__ z0sum, const C_t<T>* __restrict__ cdir,
-                          C_t<T>* __restrict__ cout) {
-    using C = C_t<T>;
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= N) return;
-    C acc = (k == 0) ? *z0sum : C{(T)0, (T)0};
-    if (cdir) acc = cadd(acc, cdir[k]);
-    for (int b = 1; b <= levels; ++b) {
-        BandDev B = bands[b];
-        if (B.route != 1 || k >= B.K) continue;
-        for (int c = 0; c < B.nsub; ++c) {   // split band: the sub-band holding k
-            const BandDev S = bands[B.sub0 + c];
-            if (k >= S.k0 && k < S.k0 + S.K) {
-                B = S;
-                break;
-            }
-        }
-        const int64_t kl = k - B.k0;   // frequency within the (sub-)band
-        const int64_t i = (kl - (B.Nm >> 1)) & (B.n - 1);
-        const DT* Dk = D + B.D_off + kl;
-        const G* g = grid + B.grid_off + i;
-        for (int s = 0; s < B.nrhs; ++s) {
-            const T d = (T)Dk[(int64_t)s * B.K];
-            const G v = g[(int64_t)s * B.n];
-            acc.x += d * (T)v.x;
-            acc.y += d * (T)v.y;
-        }
-    }
-    cout[k] = acc;
 }
 
 // ---------------------------------------------------------------------------
@@ -1005,7 +692,8 @@ static cudaError_t gather_t(Plan& p, const void* c, void* f, bool deriv, const v
         timer_begin(p, "gather", 0.0, st, &slot);
         k_gather<T, MW, true><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
             p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const C_t<T>*)p.d_grid, p.d_cheb,
-            p.d_cheb32, p.q, (T)p.kb_b, (const C_t<T>*)c, 0, nullptr, nullptr, nullptr, (C_t<T>*)f);
+            p.d_cheb32, p.q, (T)p.kb_b, (const C_t<T>*)c, 0, nullptr, nullptr, nullptr, (C_t<T>*)f,
+            (const T*)p.d_sp_phi, (const T*)p.d_sp_L, p.qmax);
         timer_end(p, slot, st);
         ++p.launches;
         return cudaGetLastError();
@@ -1029,7 +717,8 @@ static cudaError_t gather_t(Plan& p, const void* c, void* f, bool deriv, const v
         if (!p.own_gather) kern = k_gather<T, MW, false, false>;
     kern<<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
         p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const C*)p.d_grid, p.d_cheb, p.d_cheb32,
-        p.q, (T)p.kb_b, (const C*)c, deriv ? 1 : 0, (const C*)rmul, p.d_fpp, p.d_ntab, (C*)f);
+        p.q, (T)p.kb_b, (const C*)c, deriv ? 1 : 0, (const C*)rmul, p.d_fpp, p.d_ntab, (C*)f,
+        sizeof(T) == 8 ? (const T*)p.d_sp_phi : nullptr, (const T*)p.d_sp_L, p.qmax);
     timer_end(p, slot, st);
     ++p.launches;
     return cudaGetLastError();
@@ -1099,7 +788,7 @@ __global__ void k_to_ff(int64_t n, const double2* __restrict__ in, int deriv, ff
 
 // The gather of the float-pair form: k_gather's steps with the window values,
 // tap sums, barycentric weights and recombination in float pairs (fl_ffmath.cuh)
-// instead of double; the phases n x mod 1 and (N_m/2) x mod 1 and tau are
+// instead of double (taps and weights of single plans from the plan's tables); the phases n x mod 1 and (N_m/2) x mod 1 and tau are
 // still reduced exactly in double (once per node).  The barycentric sum is
 // accumulated in one pass, sum_s L_s a_s / sum_s L_s with L_s = lambda_s /
 // (tau - t_s); an exact hit tau = t_s returns a_s.
@@ -1112,7 +801,8 @@ __global__ void __launch_bounds__(256) k_gather_ff(int64_t M, const double2* __r
                                                    const float* __restrict__ cheb32,
                                                    double kb_b, const double2* __restrict__ c,
                                                    int deriv, const double2* __restrict__ rmul,
-                                                   double2* __restrict__ f) {
+                                                   double2* __restrict__ f, const ff* __restrict__ phi_tab,
+                                                   const ff* __restrict__ L_tab, int ldl) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M) return;
     const int b = bandid[i];
@@ -1133,13 +823,26 @@ __global__ void __launch_bounds__(256) k_gather_ff(int64_t M, const double2* __r
     const int64_t lo = (int64_t)u - (MW - 1);
     const ff bb = ff(kb_b);
     ff phi[2 * MW];
+    if (phi_tab) {
 #pragma unroll
-    for (int t = 0; t < 2 * MW; ++t) phi[t] = ff_kb_window(fr + ff(MW - 1 - t), (float)MW, bb);
+        for (int t = 0; t < 2 * MW; ++t) phi[t] = phi_tab[i * (2 * MW) + t];
+    } else {
+#pragma unroll
+        for (int t = 0; t < 2 * MW; ++t) phi[t] = ff_kb_window(fr + ff(MW - 1 - t), (float)MW, bb);
+    }
     const int64_t nmask = B.n - 1;
     const ffc* g = grid + B.grid_off;
     ffc acc;
     if (B.nrhs == 1) {
         acc = tap_sum<MW>(g, lo, nmask, phi);
+    } else if (phi_tab) {
+        const ff* L = L_tab + i * ldl;
+        acc = ffc{ff(0), ff(0)};
+        for (int s = 0; s < q; ++s) {
+            const ffc a = tap_sum<MW>(g + (int64_t)s * B.n, lo, nmask, phi);
+            acc.x += L[s] * a.x;
+            acc.y += L[s] * a.y;
+        }
     } else {
         const ff tf = ff((kTwoPiD * wv.y - B.yc) * B.yh_inv);
         ff den = ff(0);
@@ -1187,7 +890,8 @@ static cudaError_t gather_ff_t(Plan& p, const void* c, void* f, bool deriv, cons
     timer_begin(p, "gather", bytes, st, &slot);
     k_gather_ff<MW><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
         p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const ffc*)p.d_grid, p.d_cheb32,
-        p.kb_b, (const double2*)c, deriv ? 1 : 0, (const double2*)rmul, (double2*)f);
+        p.kb_b, (const double2*)c, deriv ? 1 : 0, (const double2*)rmul, (double2*)f,
+        (const ff*)p.d_sp_phi, (const ff*)p.d_sp_L, p.qmax);
     timer_end(p, slot, st);
     ++p.launches;
     return cudaGetLastError();
@@ -1222,70 +926,20 @@ cudaError_t run_forward(Plan& p, const void* c, void* f, bool deriv, cudaStream_
                              : forward_t<float>(p, c, f, deriv, rmul, st);
 }
 
-template <typename T, int MW, typename G = C_t<T>>
-static cudaError_t spread_t(Plan& p, const void* r, cudaStream_t st) {
-    using C = C_t<T>;
-    if (p.cell_bands.empty()) return cudaSuccess;
-    int slot;
-    timer_begin(p, "spread", 0.0, st, &slot);
-    if constexpr (std::is_same<T, ff>::value) {
-        k_spread_prep_ff<MW><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
-            p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const double2*)r, p.d_cheb32, p.qmax,
-            (ff*)p.d_sp_phi, (ff*)p.d_sp_L, (ffc*)p.d_sp_rv);
-    } else {
-        auto prep = p.xi_mode ? k_spread_prep<T, MW, true> : k_spread_prep<T, MW, false>;
-        prep<<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
-            p.M, p.d_ws, p.d_perm, p.d_bandid, p.d_bands, (const C*)r, p.d_cheb, p.qmax, (T)p.kb_b,
-            (T*)p.d_sp_phi, (T*)p.d_sp_L, (C*)p.d_sp_rv);
-    }
-    if (p.cells_total > 0)
-        k_spread_cells<T, MW, G><<<(unsigned)((p.cells_total + 255) / 256), 256, 0, st>>>(
-            (int)p.n_sparse_cb, p.d_cell_bands, p.cells_total, p.d_bands, p.d_cell,
-            (const T*)p.d_sp_phi, (const T*)p.d_sp_L, (const C*)p.d_sp_rv, p.d_ws, p.qmax, (G*)p.d_grid);
-    if (p.cells_dense > 0)
-        k_spread_cells_warp<T, MW, G><<<(unsigned)p.cells_dense, kSpreadDense, 0, st>>>(
-            (int)(p.cell_bands.size() - p.n_sparse_cb), p.d_cell_bands + p.n_sparse_cb,
-            p.cells_dense, p.d_bands, p.d_cell, (const T*)p.d_sp_phi, (const T*)p.d_sp_L,
-            (const C*)p.d_sp_rv, p.d_ws, p.qmax, (G*)p.d_grid);
-    timer_end(p, slot, st);
-    p.launches += 1 + (p.cells_total > 0) + (p.cells_dense > 0);
-    return cudaGetLastError();
-}
-
-// T: the arithmetic of the direct bands and the combine; FT: that of the
-// spreading and the FFTs (T, or float pairs ff with T = double for the
-// float-pair form, whose combine reads pair grids and weights in double).
-template <typename T, typename FT = T>
+// Spread, FFTs of sign -, direct bands, combination (fl_adjoint.cu); FT: the
+// arithmetic of the spreading, the FFTs and the combination.
+template <typename FT>
 static cudaError_t adjoint_t(Plan& p, const void* r, void* cout, cudaStream_t st) {
-    using C = C_t<T>;
-    using G = C_t<FT>;
-    cudaError_t e;
-    switch (p.mw) {
-#define FL_MW_CASE(W) \
-    case W: e = spread_t<FT, W, G>(p, r, st); break;
-        FL_MW_CASE(2) FL_MW_CASE(3) FL_MW_CASE(4) FL_MW_CASE(5) FL_MW_CASE(6) FL_MW_CASE(7)
-        FL_MW_CASE(8) FL_MW_CASE(9) FL_MW_CASE(10) FL_MW_CASE(11) FL_MW_CASE(12)
-#undef FL_MW_CASE
-        default: e = cudaErrorInvalidValue;
-    }
+    cudaError_t e = launch_spread(p, r, st);
     if (e != cudaSuccess) return e;
     if ((e = fft_bands<FT, -1, 1, false>(p, nullptr, st)) != cudaSuccess) return e;
     if (p.xi_mode) return launch_xi_combine(p, cout, st);   // no direct bands, Z^0 adds 0
     if ((e = run_direct_adjoint(p, r, st)) != cudaSuccess) return e;
-    C* z0sum = (C*)p.d_z0;
-    k_z0_sum<T><<<1, 256, 0, st>>>(p.z0_nodes, p.d_perm, (const C*)r, z0sum);
-    int slot;
-    timer_begin(p, "combine", 0.0, st, &slot);
-    k_combine<T, G, FT><<<(unsigned)((p.N + 255) / 256), 256, 0, st>>>(
-        p.N, p.levels, p.d_bands, (const FT*)p.d_D, (const G*)p.d_grid, z0sum,
-        p.dadj_work.empty() ? nullptr : (const C*)p.d_cdir, (C*)cout);
-    timer_end(p, slot, st);
-    p.launches += 2;
-    return cudaGetLastError();
+    return launch_combine(p, r, cout, st);
 }
 
 cudaError_t run_adjoint(Plan& p, const void* r, void* cout, cudaStream_t st) {
-    if (p.prec == FL_FP64_FF) return adjoint_t<double, ff>(p, r, cout, st);
+    if (p.prec == FL_FP64_FF) return adjoint_t<ff>(p, r, cout, st);
     return p.prec == FL_FP64 ? adjoint_t<double>(p, r, cout, st) : adjoint_t<float>(p, r, cout, st);
 }
 
@@ -1310,7 +964,7 @@ static cudaError_t transposed_t(Plan& p, const void* g, void* out, cudaStream_t 
         k_conj<T><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(p.M, (const C*)g, (C*)p.d_stage_r);
         ++p.launches;
     }
-    cudaError_t e = adjoint_t<T, FT>(p, p.M > 0 ? p.d_stage_r : g, out, st);
+    cudaError_t e = adjoint_t<FT>(p, p.M > 0 ? p.d_stage_r : g, out, st);
     if (e != cudaSuccess) return e;
     k_conj<T><<<(unsigned)((p.N + 255) / 256), 256, 0, st>>>(p.N, (const C*)out, (C*)out);
     ++p.launches;

@@ -93,3 +93,22 @@ def test_merged_bands_real_exponents(fl, kind, prec, eps):
     assert oracle.error_E(ref, f[:300], c) <= _bound(prec, eps, ref, c)
     refg = oracle.xi_transposed(r, xi[:300], w)
     assert oracle.error_E(refg, g[:300], r) <= _bound(prec, eps, refg, r)
+
+
+@pytest.mark.parametrize("prec,eps", [("fp32", 1e-6), ("fp64", 1e-10)])
+def test_real_exponents_band_without_exponents(fl, prec, eps):
+    # every exponent above the low bands' cuts: those bands' sums are empty
+    N, M = 500, 400
+    dev = torch.device("cuda")
+    cdt = torch.complex64 if prec == "fp32" else torch.complex128
+    w = W.nodes_disk_uniform(M, seed=11)
+    w[:, 0] -= 0.5
+    xi = np.random.default_rng(12).uniform(900.0, 1000.0, N)
+    c, r = W.coefficients(N, seed=1), W.coefficients(M, seed=2)
+    plan = fl.XiPlan(torch.from_numpy(xi).to(dev), torch.from_numpy(w).to(dev), eps, precision=prec)
+    f = plan.execute(torch.from_numpy(c).to(cdt).to(dev)).cpu().numpy().astype(np.complex128)
+    g = plan.transposed(torch.from_numpy(r).to(cdt).to(dev)).cpu().numpy().astype(np.complex128)
+    plan.close()
+    ref, refg = oracle.xi_direct(c, xi, w), oracle.xi_transposed(r, xi, w)
+    assert oracle.error_E(ref, f, c) <= _bound(prec, eps, ref, c)
+    assert oracle.error_E(refg, g, r) <= _bound(prec, eps, refg, r)
