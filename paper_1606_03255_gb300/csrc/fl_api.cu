@@ -819,6 +819,9 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
         double err[kMaxQ + 1];   // the dyadic band at rank q, over every x
         interp_error(1.0, 2.0, 64.0, err);
         tol = err[p.q];
+        // in double an error below half a unit of rounding is none (rank 22 at
+        // eps = 1e-12 leaves 6e-18)
+        if (p.prec != FL_FP32) tol = std::max(tol, ldexp(1.0, -54));
     }
     struct Part {
         double cost;
@@ -1116,7 +1119,7 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
         FL_CUDA(cudaMemsetAsync(p.d_D, 0, p.D_elems * rs, st), "clear weights");
     if (p.Y_elems) FL_CUDA(cudaMalloc(&p.d_Y, p.Y_elems * cs), "cudaMalloc intermediate");
     if (p.Y_elems || !p.small_work.empty()) {   // stage twiddles of the passes and the small FFTs
-        FL_CUDA(cudaMalloc(&p.d_tw, (size_t)(kTwEntries + (p.prec == FL_FP64_FF ? 8192 : 0)) * cs),
+        FL_CUDA(cudaMalloc(&p.d_tw, (size_t)(kTwEntries + (p.prec != FL_FP32 ? 8192 : 0)) * cs),
                 "cudaMalloc twiddles");
         FL_CUDA(build_twiddles(p, st), "fl_plan: twiddles");
     }

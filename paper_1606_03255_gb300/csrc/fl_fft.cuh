@@ -100,14 +100,25 @@ template <typename T, int D> __device__ __forceinline__ int swz_step(int bs, int
     return (bs ^ (((r * D) >> 4) & (P - 1))) + r * D;
 }
 
-// 16-point DFT in registers (4 x 4 with internal twiddles), sign SIGN.
-template <int SIGN, typename T> __device__ __forceinline__ void dft16(C_t<T>* a) {
+// 16-point DFT in registers (4 x 4 with internal twiddles), sign SIGN.  OUTER: the
+// inputs 4 .. 11 are zero (not read), half the additions of the first layer.
+template <int SIGN, typename T, bool OUTER = false> __device__ __forceinline__ void dft16(C_t<T>* a) {
     using C = C_t<T>;
     const T c1 = (T)0.92387953251128675612818318939679;   // cos(pi/8)
     const T s1 = (T)0.38268343236508977172845998403040;   // sin(pi/8)
     const T h = (T)0.70710678118654752440084436210485;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) dft4<SIGN>(a[b], a[4 + b], a[8 + b], a[12 + b]);
+    for (int b = 0; b < 4; ++b) {
+        if constexpr (OUTER) {
+            const C x = a[b], y = a[12 + b], iy = mul_i<SIGN>(y);
+            a[b] = cadd(x, y);
+            a[4 + b] = csub(x, iy);
+            a[8 + b] = csub(x, y);
+            a[12 + b] = cadd(x, iy);
+        } else {
+            dft4<SIGN>(a[b], a[4 + b], a[8 + b], a[12 + b]);
+        }
+    }
     // a[b + 4 k1] *= W16^(b k1), W16 = exp(SIGN 2 pi i / 16)
     a[5] = cmul(a[5], C{c1, SIGN * s1});      // W^1
     a[6] = cmul(a[6], C{h, SIGN * h});        // W^2
@@ -193,6 +204,12 @@ template <int SIGN> __device__ __forceinline__ ffc ff_twiddle24(const ffc* __res
     return SIGN < 0 ? ffc{w.x, -w.y} : w;
 }
 
+// The same in double (FP64 form).
+template <int SIGN> __device__ __forceinline__ double2 ff_twiddle24(const double2* __restrict__ tab, int e) {
+    const double2 w = cmul(__ldg(tab + (e >> 12)), __ldg(tab + 4096 + (e & 4095)));
+    return SIGN < 0 ? double2{w.x, -w.y} : w;
+}
+
 // v[1 .. R-1] *= w^(r k) from the stage table tws (pairs, see fl_common.cuh).
 template <int R, int NS, int SIGN, typename C>
 __device__ __forceinline__ void apply_stage_twiddles(C* v, const C* __restrict__ tws, int k) {
@@ -266,6 +283,15 @@ template <int LOG2L, int SIGN, typename T>
 __device__ __forceinline__ void fft_first_from_regs(C_t<T>* v, C_t<T>* buf, int t) {
     dft16<SIGN, T>(v);
     // swz(16 t + r) = (16 t + mask) ^ r, mask = t & (P - 1) < 16
+    const int bs = swz<T>(t * 16);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) buf[bs ^ r] = v[r];
+    __syncthreads();
+}
+
+// Its store alone, for a first stage already done in registers.
+template <int LOG2L, typename T>
+__device__ __forceinline__ void fft_first_store(const C_t<T>* v, C_t<T>* buf, int t) {
     const int bs = swz<T>(t * 16);
 #pragma unroll
     for (int r = 0; r < 16; ++r) buf[bs ^ r] = v[r];
@@ -391,6 +417,7 @@ __global__ void __launch_bounds__(PassTile<T, LOG2L, PassBudget<T>::P1, FL_P1_SE
     const int i1 = blockIdx.x * TC + col;
     C* buf = sm + col * LD;
     C v[16];
+    [[maybe_unused]] bool outer = false;   // the first stage is done, on rows 0 .. 3 and 12 .. 15
     if constexpr (MODE == 0) {
         const T* Ds = D + B.D_off + (int64_t)s * B.K;
         const int K = (int)B.K, half = (int)(B.Nm >> 1), k0 = (int)B.k0;
@@ -400,7 +427,21 @@ __global__ void __launch_bounds__(PassTile<T, LOG2L, PassBudget<T>::P1, FL_P1_SE
         // sigma < 2 reaches into them)
         const C* cb = c + B.c_off;
         const int i0 = i1 + (t << log2n1), di = (L / 16) << log2n1;   // row r: i0 + r di
-        if (4 * half <= n && 4 * (K - half) <= n) {
+        if constexpr (sizeof(T) == 8) {
+            // FP64 and float pairs are bound by their arithmetic: the zero rows'
+            // additions are left out (2 of about 50 operations per point)
+            outer = 4 * half <= n && 4 * (K - half) <= n;
+            if (outer) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    v[r] = prep_value32<T, DERIV, false>(i0 + r * di, n, half, K, k0, cb, Ds);
+                    v[12 + r] = prep_value32<T, DERIV, true>(i0 + (12 + r) * di, n, half, K, k0, cb, Ds);
+                }
+                dft16<SIGN, T, true>(v);
+            }
+        }
+        if (outer) {
+        } else if (4 * half <= n && 4 * (K - half) <= n) {
 #pragma unroll
             for (int r = 0; r < 16; ++r)
                 v[r] = (r >= 4 && r < 12) ? C{(T)0, (T)0}
@@ -418,7 +459,12 @@ __global__ void __launch_bounds__(PassTile<T, LOG2L, PassBudget<T>::P1, FL_P1_SE
         for (int r = 0; r < 16; ++r) v[r] = in[i1 + ((t + r * (L / 16)) << log2n1)];
     }
     const C* twr = tw + tw_region(LOG2L, 4);
-    fft_first_from_regs<LOG2L, SIGN, T>(v, buf, t);
+    if constexpr (sizeof(T) == 8 && MODE == 0) {
+        if (!outer) dft16<SIGN, T>(v);
+        fft_first_store<LOG2L, T>(v, buf, t);
+    } else {
+        fft_first_from_regs<LOG2L, SIGN, T>(v, buf, t);
+    }
     fft_middle<LOG2L, 4, SIGN, T>(buf, t, twr);
     fft_last_to_regs<LOG2L, 4, SIGN, T>(buf, t, v, twr);
     // outputs l2 = jj + r NS, jj = t + jb L/16, twiddled by exp(SIGN 2 pi i i1 l2 / n)
@@ -426,15 +472,17 @@ __global__ void __launch_bounds__(PassTile<T, LOG2L, PassBudget<T>::P1, FL_P1_SE
     // step = exp(.. i1 NS): three sincospi values and short products
     constexpr int R = SP::LAST_R, NS = SP::LAST_NS, J = 16 / R;
     C* out = Y + item.y_off;
-    if constexpr (std::is_same<T, ff>::value) {
-        // float pairs: the same factorisation w0 rho^jb step^r as below, with
-        // the base factors from the two plan-time tables after the stage table
-        // (exponents i1 l2 < n <= 2^24, scaled to units of 2^-24 turns) and the
-        // powers of step formed by products at most three deep
+    if constexpr (sizeof(T) == 8) {
+        // FP64 and float pairs: the same factorisation w0 rho^jb step^r as below,
+        // with the base factors from the two plan-time tables after the stage
+        // table (exponents i1 l2 < n <= 2^24, scaled to units of 2^-24 turns; in
+        // double the sincospi of three factors per thread were a fifth of the
+        // pass's FP64 operations) and the powers of step formed by products at
+        // most three deep
         const C* tab = tw + kTwEntries;
         const int sh = 24 - (log2n1 + LOG2L);
         C step[R];
-        step[0] = C{ff(1), ff(0)};
+        step[0] = C{T(1), T(0)};
         if constexpr (R >= 2) step[1] = ff_twiddle24<SIGN>(tab, ((i1 * NS) & (n - 1)) << sh);
         if constexpr (R >= 4) {
             step[2] = cmul(step[1], step[1]);

@@ -253,7 +253,7 @@ struct Plan {
     void* d_grid = nullptr;        // band grids (complex T)
     void* d_Y = nullptr;           // four-step intermediate (complex T)
     void* d_tw = nullptr;          // four-step stage twiddles (complex T, kTwEntries;
-                                   // float pairs: + 8192 pass-1 output twiddles)
+                                   // FP64, float pairs: + 8192 pass-1 output twiddles)
     void* d_stage_c = nullptr;     // staging for fl_execute_host and fl_execute_batched_ptrs
     void* d_stage_f = nullptr;
     int64_t* d_boff = nullptr;     // batched: instance offsets of c (B + 1) then of f (B + 1)

@@ -212,25 +212,26 @@ __global__ void k_twiddles(C_t<T>* __restrict__ tw) {
     tw[i] = v;
 }
 
-// Float pairs: the pass-1 output twiddles as products of two tables,
+// Float pairs and FP64: the pass-1 output twiddles as products of two tables,
 // tab[a] = exp(2 pi i a / 2^12) and tab[4096 + b] = exp(2 pi i b / 2^24),
 // a, b < 4096, each computed in FP64 (exact arguments) and rounded once.
-__global__ void k_ff_tables(ffc* __restrict__ tab) {
+template <typename T> __global__ void k_ff_tables(C_t<T>* __restrict__ tab) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 8192) return;
     const double x = i < 4096 ? ldexp((double)i, -11) : ldexp((double)(i - 4096), -23);
     double sn, cs;
     sincospi(x, &sn, &cs);
-    tab[i] = ffc{ff(cs), ff(sn)};
+    tab[i] = C_t<T>{T(cs), T(sn)};
 }
 
 cudaError_t build_twiddles(Plan& p, cudaStream_t st) {
     const unsigned blocks = (unsigned)((kTwEntries + 255) / 256);
     if (p.prec == FL_FP64_FF) {
         k_twiddles<ff><<<blocks, 256, 0, st>>>((ffc*)p.d_tw);
-        k_ff_tables<<<8192 / 256, 256, 0, st>>>((ffc*)p.d_tw + kTwEntries);
+        k_ff_tables<ff><<<8192 / 256, 256, 0, st>>>((ffc*)p.d_tw + kTwEntries);
     } else if (p.prec == FL_FP64) {
         k_twiddles<double><<<blocks, 256, 0, st>>>((C_t<double>*)p.d_tw);
+        k_ff_tables<double><<<8192 / 256, 256, 0, st>>>((C_t<double>*)p.d_tw + kTwEntries);
     } else {
         k_twiddles<float><<<blocks, 256, 0, st>>>((C_t<float>*)p.d_tw);
     }
