@@ -230,19 +230,26 @@ __global__ void k_lap_ktable(int levels, int q, double y1, double xi1, const int
 // (2 - [j = 0]) / q T_j(t_r) (discrete orthogonality of the T_j, j < q), and
 // likewise on Y_m, so with
 //   u^{Omega_l}_j = sum_{t_k in Omega_l} T_j(tau_k) c_k   (u_0: the band sum S_l)
-//   K''_{ij} = sum_s sum_r C_i(s) K^{Y_m,Omega_l}_{s r} C_j(r)   (plan time, in place)
+//   K''_{ij} = sum_s sum_r C_i(s) K^{Y_m,Omega_l}_{s r} C_j(r)   (plan time; stored as rows
+//              over (l, j) per (m, i), so that a sum reads consecutive entries)
 //   a^{Y_m}_i = sum_l sum_j K''_{ij} u^{Omega_l}_j
 // the same interpolant is f~_j = sum_i T_i(sigma_j) a_i + g_{L_m+1}.  An element
 // costs three operations per degree instead of the weights' products, their
 // inversion and a scan over the warp: no division, no exact-hit case.
-__global__ void k_lap_kcheb(int q, double* __restrict__ Kt) {
+__global__ void k_lap_kcheb(int levels, int q, const int* __restrict__ ell, const int64_t* __restrict__ koff,
+                            const double* __restrict__ Kt, double* __restrict__ Kc) {
     extern __shared__ double ksm[];                 // C (q x q), K (q x q), K C^T (q x q)
     double *C = ksm, *K = ksm + q * q, *X = ksm + 2 * q * q;
-    double* out = Kt + (int64_t)blockIdx.x * q * q;
+    const int m = blockIdx.x + 1, li = blockIdx.y;
+    const int nl = ell ? levels - m - ell[m] + 1 : levels - 1;
+    if (li >= nl) return;
+    const int64_t base = ell ? koff[m] : (int64_t)(m - 1) * nl * q * q;
+    const double* src = Kt + base + (int64_t)li * q * q;
+    double* out = Kc + base + (int64_t)li * q;
     for (int i = threadIdx.x; i < q * q; i += blockDim.x) {
         const int j = i / q, r = i % q;
         C[i] = cospi((double)(j * (2 * r + 1) % (4 * q)) / (2.0 * q)) * ((j ? 2.0 : 1.0) / q);
-        K[i] = out[i];
+        K[i] = src[i];
     }
     __syncthreads();
     for (int i = threadIdx.x; i < q * q; i += blockDim.x) {
@@ -256,7 +263,7 @@ __global__ void k_lap_kcheb(int q, double* __restrict__ Kt) {
         const int ii = i / q, j = i % q;
         double a = 0.0;
         for (int s = 0; s < q; ++s) a += C[ii * q + s] * X[s * q + j];
-        out[i] = a;
+        out[(int64_t)ii * nl * q + j] = a;
     }
 }
 
@@ -295,17 +302,36 @@ __global__ void k_lap_starts(int64_t n, const uint8_t* __restrict__ band, int le
     first[l] = lo;
 }
 
-// T_j(tau), j = 0 .. q - 1, handed to f(j, T_j(|tau|)) together with the sign of
-// the odd degrees (T_j(-x) = (-1)^j T_j(x)).  Doubles step the differences
-// d_{j+1} = T_{j+1} - T_j = d_j + 2 (|tau| - 1) T_j, whose rounding grows with j
-// where the three-term recurrence's grows with j^2 near the ends of the
-// interval; in float pairs j^2 2^-48 is far below the FP32 form's rounding, and
-// the plain recurrence on tau itself is cheaper.
+// The recurrences of T_j(tau), j < q.  Doubles step the differences
+// d_{j+1} = T_{j+1} - T_j = d_j + 2 (|tau| - 1) T_j (with T_j(-x) = (-1)^j T_j(x)),
+// whose rounding grows with j where the three-term recurrence's grows with j^2
+// near the ends of the interval: three operations per degree.  Up to rank
+// kLapPlain the three-term recurrence, of two, stays within the 3 q units that
+// the barycentric weights' products had (16^2 / 2 units at the very ends, a few
+// elsewhere); in float pairs j^2 2^-48 is far below the FP32 form's rounding.
+constexpr int kLapPlain = 16;
 __device__ __forceinline__ float ff_round(ff a) { return a.hi + a.lo; }
 
 // acc[j] += c T_j(tau), j < q <= P.
 template <int P>
 __device__ __forceinline__ void cheb_moments(double tau, double c, int q, double* acc) {
+    if constexpr (P <= kLapPlain) {
+        const double x2 = tau + tau;
+        double t0 = 1.0, t1 = tau;
+        acc[0] += c;
+#pragma unroll
+        for (int j = 1; j < P; ++j) {
+            if (j < q) {
+                if (j > 1) {
+                    const double t2 = fma(x2, t1, -t0);
+                    t0 = t1;
+                    t1 = t2;
+                }
+                acc[j] = fma(c, t1, acc[j]);
+            }
+        }
+        return;
+    }
     const double e = fabs(tau) - 1.0, e2 = 2.0 * e, co = tau < 0.0 ? -c : c;
     double t = 1.0, d = e;
     acc[0] += c;
@@ -338,6 +364,17 @@ __device__ __forceinline__ void cheb_moments(ff tau, float c, int q, float* acc)
 
 // sum_i T_i(tau) a_i, i < q.
 __device__ __forceinline__ double cheb_sum(double tau, const double* __restrict__ a, int q) {
+    if (q <= kLapPlain) {
+        const double x2 = tau + tau;
+        double t0 = 1.0, t1 = tau, s = a[0];
+        for (int i = 1; i < q; ++i) {
+            s = fma(a[i], t1, s);
+            const double t2 = fma(x2, t1, -t0);
+            t0 = t1;
+            t1 = t2;
+        }
+        return s;
+    }
     const double e = fabs(tau) - 1.0, e2 = 2.0 * e;
     double t = 1.0, d = e, even = a[0], odd = 0.0;
     for (int i = 1; i < q; i += 2) {
@@ -376,36 +413,34 @@ struct LapItem {
 __device__ __forceinline__ float lap_shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ double lap_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 
-// Sums v[0 .. 2 H) over the lanes of a warp by halving: in step OFF a lane keeps
-// one half of its values and takes the partner's sums for it, so all P values
-// cost about P exchanges instead of 5 P; at the end lane l holds in v[0 .. P/32)
-// (P >= 32) or v[0] the sums of the entries it kept.
-template <int H, int OFF, typename T> __device__ __forceinline__ void halve_sum(T* v, int lane) {
-    if constexpr (OFF > 0) {
-        if constexpr (H > 0) {
-            const bool up = lane & OFF;
+// Sums v[0 .. 7] over the lanes of a warp: halving steps (a lane keeps one half of
+// its values and takes its partner's sums of that half), then two full ones; lane
+// l ends with the sum of entry 4 [l & 16] + 2 [l & 8] + [l & 4] in v[0].  Nine
+// exchanges for eight values instead of 40.
+template <typename T> __device__ __forceinline__ void sum8(T* v, int lane) {
 #pragma unroll
-            for (int i = 0; i < H; ++i) {
-                const T give = up ? v[i] : v[i + H];
-                const T keep = up ? v[i + H] : v[i];
-                v[i] = keep + lap_shfl(give, OFF);
-            }
-        } else {
-            v[0] += lap_shfl(v[0], OFF);
+    for (int h = 4, off = 16; h > 0; h >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const T give = up ? v[i] : v[i + h];
+            const T keep = up ? v[i + h] : v[i];
+            v[i] = keep + lap_shfl(give, off);
         }
-        halve_sum<H / 2, OFF / 2>(v, lane);
     }
+    v[0] += lap_shfl(v[0], 2);
+    v[0] += lap_shfl(v[0], 1);
 }
 
 // Moments u_j of one item, j < q <= P: each thread sums its elements over the
-// degrees in registers, a halving exchange sums the warp, shared memory the
-// warps, all in a fixed order.  Bound by the FP64 pipe (3 q operations per
-// element, 0.53e12 per second) in the FP64 form; N = 2^16, q = 11: 38.7 us for
-// the barycentric weights and the scan per degree, see k_lap_eval_cheb for what
-// it takes now.  In the FP32 form the recurrence runs in float pairs (N = 10^6:
-// 354 us before).
+// degrees in registers, exchanges sum the warp, shared memory the warps, all in a
+// fixed order.  P is q rounded up to 8 (64 accumulators at q = 34 left one CTA
+// per SM: 42 us at N = 2^16).  Bound by the FP64 pipe in the FP64 form (2 or 3
+// operations per element and degree, 0.53e12 per second); the barycentric
+// weights and a scan per degree took 38.7 us at N = 2^16, q = 11, and 354 us at
+// N = 10^6 in the FP32 form, whose recurrence runs in float pairs.
 template <typename T, int P>
-__global__ void __launch_bounds__(kLapThreads)
+__global__ void __launch_bounds__(kLapThreads, P <= 40 ? 2 : 1)
     k_lap_moments_cheb(const LapItem* __restrict__ items, const LapTau<T>* __restrict__ tau,
                        const int32_t* __restrict__ tperm, const T* __restrict__ c, int levels, int q,
                        T* __restrict__ partial) {
@@ -420,17 +455,11 @@ __global__ void __launch_bounds__(kLapThreads)
         const int64_t k = it.k0 + e;
         cheb_moments<P>(tau[k], c[tperm[k]], qb, acc);
     }
-    halve_sum<P / 2, 16>(acc, lane);
-    // the entry lane l holds in v[i]: bit 16 chose the upper P/2, bit 8 the upper P/4, ...
-    constexpr int R = P >= 32 ? P / 32 : 1;
-    int e0 = 0;
 #pragma unroll
-    for (int h = P / 2, off = 16; off > 0 && h > 0; h >>= 1, off >>= 1)
-        if (lane & off) e0 += h;
-    const bool own = P >= 32 || (lane & (32 / P - 1)) == 0;
-#pragma unroll
-    for (int i = 0; i < R; ++i)
-        if (own) red[w][e0 + i] = acc[i];
+    for (int j = 0; j < P; j += 8) {
+        sum8(acc + j, lane);
+        if ((lane & 3) == 0) red[w][j + (lane >> 2)] = acc[j];   // entry 4 [l & 16] + 2 [l & 8] + [l & 4] = l / 4
+    }
     __syncthreads();
     if (threadIdx.x < P && threadIdx.x < q) {
         T s = (T)0;
@@ -458,8 +487,8 @@ __global__ void k_lap_reduce_items(int levels, int q, const int* __restrict__ fi
 // a^{Y_m}_i = sum_{l = lo(m)}^{hi(m)} sum_j K''(m, l)_{ij} u^{Omega_l}_j, m = blockIdx.x
 // + 1, one warp per i (blockIdx.y: groups of 8), lanes striding over (l, j), a
 // fixed shuffle tree; written as LapTau<T> values.  Algorithm 1 (ell != nullptr):
-// l = l_m .. M - m; the generalised algorithm: l = 1 .. M - 1.  Block (0, 0)
-// also forms g_l = sum_{l' >= l} S_{l'} (S = u_0), g_{levels+1} = 0.
+// l = l_m .. M - m; the generalised algorithm: l = 1 .. M - 1.  The last block
+// (the least of the others' work) also forms g_l = sum_{l' >= l} S_{l'} (S = u_0), g_{levels+1} = 0.
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_lap_couple_cheb(int levels, int q, const int* __restrict__ ell, const int64_t* __restrict__ koff,
@@ -467,24 +496,22 @@ __global__ void __launch_bounds__(256)
                       LapTau<T>* __restrict__ ha, LapTau<T>* __restrict__ g) {
     const int m = blockIdx.x + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    if (blockIdx.x == gridDim.x - 1 && blockIdx.y == 0 && threadIdx.x <= levels) {   // a thread per l
+        const int l = threadIdx.x + 1;
         double s = 0.0;
-        g[levels + 1] = LapTau<T>(0.0);
-        for (int l = levels; l >= 1; --l) {
-            s += u[l * q];
-            g[l] = LapTau<T>(s);
-        }
+#pragma unroll 4
+        for (int k = levels; k >= l; --k) s += u[k * q];
+        g[l] = LapTau<T>(s);
     }
     const int i = blockIdx.y * 8 + warp;
     if (m >= levels || i >= q) return;
     const int l0 = ell ? ell[m] : 1, l1 = ell ? levels - m : levels - 1;
     const int tot = max(l1 - l0 + 1, 0) * q;
-    const double* K = Kt + (ell ? koff[m] : (int64_t)(m - 1) * (levels - 1) * q * q) + i * q;
+    const double* K = Kt + (ell ? koff[m] : (int64_t)(m - 1) * tot * q) + (int64_t)i * tot;
+    const double* ul = u + (int64_t)l0 * q;
     double acc = 0.0;
-    for (int x = lane; x < tot; x += 32) {
-        const int li = x / q, j = x - li * q;
-        acc += K[(int64_t)li * q * q + j] * u[(l0 + li) * q + j];
-    }
+#pragma unroll 8
+    for (int x = lane; x < tot; x += 32) acc += K[x] * ul[x];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (lane == 0) ha[m * q + i] = LapTau<T>(acc);
@@ -563,18 +590,17 @@ __device__ __forceinline__ double gen_kappa(int kind, double y, double xi) {
     return kind == 2 ? sqrt(1.5707963267948966192313216916398 / x) * exp(-x) : exp(-x);
 }
 
-// Kt[((m - 1)(M - 1) + l - 1) q^2 + s q + r] = kappa(y_s^{Y_m}, xi_r^{Omega_l}), block m.
+// Kt[((m - 1)(M - 1) + l - 1) q^2 + s q + r] = kappa(y_s^{Y_m}, xi_r^{Omega_l}), block (m, l).
 __global__ void k_gen_ktable(int kind, int levels, int q, double y1, double xi1,
                              const double* __restrict__ cheb, double* __restrict__ Kt) {
-    const int m = blockIdx.x + 1;
-    const int nb = levels - 1;
-    const double ay = ldexp(y1, -m);
-    for (int i = threadIdx.x; i < nb * q * q; i += blockDim.x) {
-        const int r = i % q, s = (i / q) % q, l = 1 + i / (q * q);
+    const int m = blockIdx.x + 1, l = blockIdx.y + 1;
+    const double ay = ldexp(y1, -m), ax = ldexp(xi1, -l);
+    double* out = Kt + ((int64_t)(m - 1) * (levels - 1) + l - 1) * q * q;
+    for (int i = threadIdx.x; i < q * q; i += blockDim.x) {
+        const int r = i % q, s = i / q;
         const double ys = 1.5 * ay + 0.5 * ay * cheb[s];
-        const double ax = ldexp(xi1, -l);
         const double xr = 1.5 * ax + 0.5 * ax * cheb[r];
-        Kt[(int64_t)(m - 1) * nb * q * q + i] = gen_kappa(kind, ys, xr);
+        out[i] = gen_kappa(kind, ys, xr);
     }
 }
 
@@ -744,10 +770,13 @@ static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
     int slot = -1;
     if (p.n_lap_items > 0) {
         timer_begin(p, "lap_moments", (double)p.N * (8 + 4 + sizeof(T)), st, &slot);
-        if (p.q <= 8) lap_moments_launch<T, 8>(p, c, partial, st);
-        else if (p.q <= 16) lap_moments_launch<T, 16>(p, c, partial, st);
-        else if (p.q <= 32) lap_moments_launch<T, 32>(p, c, partial, st);
-        else lap_moments_launch<T, 64>(p, c, partial, st);
+        switch ((p.q + 7) / 8) {
+#define FL_LAP_P(X) \
+    case X: lap_moments_launch<T, 8 * X>(p, c, partial, st); break;
+            FL_LAP_P(1) FL_LAP_P(2) FL_LAP_P(3) FL_LAP_P(4) FL_LAP_P(5) FL_LAP_P(6) FL_LAP_P(7) FL_LAP_P(8)
+#undef FL_LAP_P
+        default: return cudaErrorInvalidValue;
+        }
         timer_end(p, slot, st);
         ++p.launches;
     }
@@ -894,10 +923,10 @@ static cudaError_t lap_tables(Plan& p, bool last, std::vector<LapItem>* items, s
     return cudaSuccess;
 }
 
-// The plan's scratch with the item starts, the items, and (nk blocks of the
-// coupling table) the table's Chebyshev form.
+// The plan's scratch with the item starts, the items, and (nk blocks Kt of the
+// coupling table) the table's Chebyshev form p.d_lapK.
 static cudaError_t lap_upload(Plan& p, const std::vector<LapItem>& items, const std::vector<int>& first,
-                              const std::vector<int>& ell, int64_t nk, size_t* scratch, cudaStream_t st) {
+                              const std::vector<int>& ell, int64_t nk, double* Kt, size_t* scratch, cudaStream_t st) {
     p.n_lap_items = (int64_t)items.size();
     const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items, p.prec == FL_FP64 ? 8 : 4);
     *scratch = L.total + items.size() * sizeof(LapItem);
@@ -917,7 +946,11 @@ static cudaError_t lap_upload(Plan& p, const std::vector<LapItem>& items, const 
         const size_t smem = 3 * (size_t)p.q * p.q * sizeof(double);   // <= 96 KiB (q <= 64)
         e = cudaFuncSetAttribute(k_lap_kcheb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_lap_kcheb<<<(unsigned)nk, 256, smem, st>>>(p.q, p.d_lapK);
+        e = cudaMalloc((void**)&p.d_lapK, nk * p.q * p.q * sizeof(double));
+        if (e != cudaSuccess) return e;
+        const bool gen = ell.empty();
+        k_lap_kcheb<<<dim3((unsigned)(p.levels - 1), (unsigned)(p.levels - 1)), 256, smem, st>>>(
+            p.levels, p.q, gen ? nullptr : (const int*)(base + L.ell), p.d_lapKoff, Kt, p.d_lapK);
         e = cudaGetLastError();
     }
     return e;
@@ -996,21 +1029,22 @@ static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, in
         ktot += (int64_t)std::max(0, P.levels - m - P.ell[m] + 1) * P.q * P.q;
     }
     int* d_ell = nullptr;   // l_m for the table kernel
+    double* Kt = nullptr;   // the blocks at the Chebyshev points
     LAP_CUDA(cudaMalloc((void**)&p.d_lapKoff, koff.size() * sizeof(int64_t)), "cudaMalloc coupling offsets");
     LAP_CUDA(cudaMemcpyAsync(p.d_lapKoff, koff.data(), koff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st),
              "copy coupling offsets");
     if (ktot > 0) {
-        LAP_CUDA(cudaMalloc((void**)&p.d_lapK, ktot * sizeof(double)), "cudaMalloc coupling table");
+        LAP_CUDA(cudaMallocAsync((void**)&Kt, ktot * sizeof(double), st), "cudaMalloc coupling table");
         LAP_CUDA(cudaMalloc((void**)&d_ell, ell.size() * sizeof(int)), "cudaMalloc l_m");
         e = cudaMemcpyAsync(d_ell, ell.data(), ell.size() * sizeof(int), cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) {
-            k_lap_ktable<<<P.levels - 1, 256, 0, st>>>(P.levels, P.q, y1, xi1, d_ell, p.d_lapKoff, p.d_cheb,
-                                                       p.d_lapK);
+            k_lap_ktable<<<P.levels - 1, 256, 0, st>>>(P.levels, P.q, y1, xi1, d_ell, p.d_lapKoff, p.d_cheb, Kt);
             e = cudaGetLastError();
         }
     }
     size_t scratch = 0;
-    if (e == cudaSuccess) e = lap_upload(p, items, first, ell, ktot / (P.q * P.q), &scratch, st);
+    if (e == cudaSuccess) e = lap_upload(p, items, first, ell, ktot / (P.q * P.q), Kt, &scratch, st);
+    if (Kt) cudaFreeAsync(Kt, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the host arrays are released on return
     cudaFree(d_ell);
     LAP_CUDA(e, "fl_plan_laplace: tables");
@@ -1099,6 +1133,7 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
                                : lap_tables<float>(p, false, &items, &first, st),
              "fl_plan_kernel: moment items");
     int64_t nk = 0;   // blocks of the coupling table
+    double* Kt = nullptr;
     // the Omega_M near field: indices of the t_k in the last frequency band
     if (N && levels > 1) {
         std::vector<uint8_t> tb(N);
@@ -1115,12 +1150,15 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
                      "copy near field");
         }
         nk = (int64_t)(levels - 1) * (levels - 1);
-        LAP_CUDA(cudaMalloc((void**)&p.d_lapK, nk * qq * qq * sizeof(double)), "cudaMalloc coupling table");
-        k_gen_ktable<<<levels - 1, 256, 0, st>>>(kind, levels, qq, y1, xi1, p.d_cheb, p.d_lapK);
+        LAP_CUDA(cudaMallocAsync((void**)&Kt, nk * qq * qq * sizeof(double), st), "cudaMalloc coupling table");
+        k_gen_ktable<<<dim3((unsigned)(levels - 1), (unsigned)(levels - 1)), 256, 0, st>>>(kind, levels, qq, y1, xi1,
+                                                                                          p.d_cheb, Kt);
     }
     LAP_CUDA(cudaGetLastError(), "fl_plan_kernel: launch");
     size_t scratch = 0;
-    LAP_CUDA(lap_upload(p, items, first, std::vector<int>(), nk, &scratch, st), "fl_plan_kernel: tables");
+    e = lap_upload(p, items, first, std::vector<int>(), nk, Kt, &scratch, st);
+    if (Kt) cudaFreeAsync(Kt, st);
+    LAP_CUDA(e, "fl_plan_kernel: tables");
     LAP_CUDA(cudaStreamSynchronize(st), "fl_plan_kernel: synchronise");
     p.scratch_bytes = (double)scratch + (N + M) * (9.0 + 8.0) + (double)nk * qq * qq * 8.0;
     p.model_bytes = (double)N * (8 + 1 + tsz) + (double)M * (8 + 1 + tsz);
