@@ -416,8 +416,9 @@ __global__ void k_spread_starts(int total, const int4* __restrict__ groups, int 
 }
 
 template <typename E> static cudaError_t adj_upload(const std::vector<E>& v, E** dev, cudaStream_t st) {
-    cudaError_t e = cudaMalloc((void**)dev, std::max<size_t>(1, v.size()) * sizeof(E));
-    if (e == cudaSuccess && !v.empty())
+    if (v.empty()) return cudaSuccess;
+    cudaError_t e = cudaMalloc((void**)dev, v.size() * sizeof(E));
+    if (e == cudaSuccess)
         e = cudaMemcpyAsync(*dev, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice, st);
     return e;
 }
@@ -476,7 +477,7 @@ cudaError_t build_spread(Plan& p, cudaStream_t st) {
                 (int)nstart, p.d_dn_groups, (int)groups.size(), p.d_bands, p.d_cell, p.d_dn_start);
     }
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the host lists are released on return
+    if (e == cudaSuccess && !comb.empty()) e = cudaStreamSynchronize(st);   // the host lists are released on return
     return e;
 }
 

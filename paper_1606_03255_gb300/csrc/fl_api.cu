@@ -300,7 +300,7 @@ static void add_direct_band(Plan& p, const BandHost& bh) {
 // chunk's Horner blocks with `r` blocks per lane, r the largest power of two (up
 // to kDirMaxBlocks) that still leaves every SM about 1024 busy lanes (pinned
 // transforms: r = 1, or G = 1 for DirectSeg::pin = 2); an item
-// holds the nodes of one pass of its 256 threads, or of two when there are
+// holds the nodes of one pass of its threads, or of two when there are
 // plenty of items (the staged chunk then serves twice as many).  Adjoint: node
 // groups of `steps` nodes (pairs in FP32) per lane, doubled from 8 while the
 // launch keeps 24 warps per SM, since every group adds its sums to cdir with
@@ -329,12 +329,17 @@ static void build_direct_items(Plan& p) {
         const int64_t nblk = (std::min<int64_t>(s.K, kDirChunk) + kDirBlock - 1) / kDirBlock;
         return std::min(5, ilog2_ceil(s.pin ? nblk : (nblk + r - 1) / r));
     };
+    // few items (a small transform) in FP64 or pairs: CTAs of 64 threads, so that
+    // all SMs take part (46 CTAs of 256 threads at N = M = 1024 in FP64).  FP32 keeps
+    // 256: staging the coefficients is its larger part (3001 x 2500: 24.0 us, 28.7
+    // with 64)
+    p.direct_threads = 256;
     auto items = [&](int passes, bool make) {
         int64_t count = 0;
         for (size_t g = 0; g < p.direct_segs.size(); ++g) {
             const DirectSeg& s = p.direct_segs[g];
             const int lg = lanes(s);
-            const int64_t per = (int64_t)passes * np * (256 >> lg);
+            const int64_t per = (int64_t)passes * np * (p.direct_threads >> lg);
             for (int64_t n0 = 0; n0 < s.nodes; n0 += per) {
                 count += s.nchunk;
                 for (int ch = 0; make && ch < s.nchunk; ++ch)
@@ -343,7 +348,9 @@ static void build_direct_items(Plan& p) {
         }
         return count;
     };
-    items(items(1, false) >= 16 * kSMs ? 2 : 1, true);
+    const int64_t full = items(1, false);
+    if (np == 1 && full < 2 * kSMs) p.direct_threads = 64;
+    items(full >= 16 * kSMs ? 2 : 1, true);
     if (p.batched) return;   // forward only
     auto adj_items = [&](int64_t steps, bool make) {
         int64_t count = 0;
@@ -743,21 +750,22 @@ static fl_status plan_splits(Plan& p, const std::vector<int>& nfft, cudaStream_t
 // kernel's bound 1, at 0 .. kMaxQ points: the Chebyshev coefficients of
 // exp(-(c + h t) x) are 2 (-1)^j I_j(h x) e^{-c x}, and interpolation at q Chebyshev
 // points errs by at most twice the sum of the coefficients from q on; the
-// largest over x in (0, xmax] (sampled on a logarithmic grid; the bounds are
-// smooth and unimodal in x).
+// largest over x in (0, xmax], sampled four to the octave over the top three
+// octaves (the bounds are unimodal in x, and the bands reach at most about that
+// far beyond the peak).
 static void interp_error(double a, double b, double xmax, double* err) {
-    constexpr int kTerms = 128, kSamples = 24;
+    constexpr int kTerms = 96, kSamples = 13;
     const double h = 0.5 * (b - a);
     for (int q = 0; q <= kMaxQ; ++q) err[q] = 0.0;
     for (int i = 0; i < kSamples; ++i) {
-        const double x = xmax * pow(2.0, -0.25 * i), z = h * x;
+        const double x = xmax * pow(2.0, -0.25 * i), z = h * x, iz = 2.0 / z;
         // e^-z I_j(z) by backward recurrence, normalised by I_0 + 2 sum I_j = e^z
         double v[kTerms + 2];
         v[kTerms + 1] = 0.0;
         v[kTerms] = 1e-280;
         double sum = 2.0 * v[kTerms];
         for (int j = kTerms; j > 0; --j) {
-            v[j - 1] = v[j + 1] + 2.0 * j / z * v[j];
+            v[j - 1] = v[j + 1] + (j * iz) * v[j];
             if (v[j - 1] > 1e250) {   // rescale
                 for (int t = j - 1; t <= kTerms; ++t) v[t] *= 1e-250;
                 sum *= 1e-250;
@@ -780,10 +788,15 @@ static int merged_rank(Plan& p, double a, int octaves, double xmax, double tol) 
     const int key = (int)ceil(16.0 * log2(a * xmax));
     const auto hit = p.rank_memo.find({octaves, key});
     if (hit != p.rank_memo.end()) return hit->second;
-    double err[kMaxQ + 1];
-    interp_error(1.0, ldexp(1.0, octaves), pow(2.0, key / 16.0), err);
-    int r = 2;
-    while (r <= kMaxQ && err[r] > tol) ++r;
+    // beyond z = h x = 60 the coefficients fall below 1e-6 after kMaxQ only
+    const double b = ldexp(1.0, std::min(octaves, 60)), xm = pow(2.0, key / 16.0);
+    int r = kMaxQ + 1;
+    if (0.5 * (b - 1.0) * xm <= 60.0) {
+        double err[kMaxQ + 1];
+        interp_error(1.0, b, xm, err);
+        r = 2;
+        while (r <= kMaxQ && err[r] > tol) ++r;
+    }
     p.rank_memo[{octaves, key}] = r;
     return r;
 }

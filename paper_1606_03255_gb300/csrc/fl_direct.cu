@@ -199,7 +199,7 @@ __device__ __forceinline__ void dir_write(const DirectSeg& S, int64_t i, int chu
     f[j] = rmul ? cmulc(rmul[j], o) : o;
 }
 
-// One CTA per work item: consecutive sorted nodes of one segment against one
+// One CTA (64 or 256 threads) per work item: consecutive sorted nodes of one segment against one
 // chunk of up to kDirChunk coefficients staged in shared memory.  G = 2^lg
 // consecutive lanes share a node (two nodes in the FP32 form) and take its
 // Horner blocks l, l + G, ... of the chunk, so that a segment of few frequencies
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256)
     const int64_t k0 = (int64_t)it.chunk * kDirChunk;
     const int kn = (int)min(S.K - k0, (int64_t)kDirChunk);
     const int nblk = (kn + kDirBlock - 1) / kDirBlock;   // zeros past kn
-    for (int i = threadIdx.x; i < nblk * kDirBlock; i += 256) {
+    for (int i = threadIdx.x; i < nblk * kDirBlock; i += blockDim.x) {
         C v = dir_zero<C>();
         if (i < kn) {
             const int64_t k = k0 + i;
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(256)
     const int lg = it.lg, G = 1 << lg;
     const int sub = threadIdx.x & (G - 1);
     // every lane of a warp runs the same trips (the shuffles below)
-    for (int n0 = 0; n0 < it.nnodes; n0 += NP * (256 >> lg)) {
+    for (int n0 = 0; n0 < it.nnodes; n0 += NP * ((int)blockDim.x >> lg)) {
         const int n = n0 + NP * (threadIdx.x >> lg);
         const bool on = n < it.nnodes;
         const int64_t i = it.node0 + (on ? n : 0);
@@ -489,7 +489,7 @@ static cudaError_t direct_forward_t(Plan& p, const void* c, void* f, const void*
     if (e != cudaSuccess) return e;
     int slot;
     timer_begin(p, "direct", (double)p.direct_terms * sizeof(C) / 32.0, st, &slot);
-    kern<<<(unsigned)p.direct_work.size(), 256, smem, st>>>(
+    kern<<<(unsigned)p.direct_work.size(), p.direct_threads, smem, st>>>(
         p.d_direct, p.d_dsegs, p.d_ws, p.d_ntab, (const C*)p.d_dz, (const C*)c, p.d_perm, (const O*)rmul, (O*)f,
         (C*)p.d_dpart);
     if (p.direct_nodes > 0) {

@@ -224,6 +224,7 @@ struct Plan {
     std::vector<DirectRange> direct_ranges;   // the segments of several chunks
     int64_t direct_nodes = 0;                 // their nodes
     int64_t direct_terms = 0, dpart_elems = 0, direct_kmax = 0;
+    int direct_threads = 256;                 // per CTA of the forward items
 
     // device memory
     double2* d_ws = nullptr;       // nodes in sorted order (Re w, Im w)
