@@ -313,9 +313,15 @@ def _torch():
 
 
 def _stream_handle(stream=None) -> int:
+    """The cudaStream_t of `stream`, or of the current stream of the current device
+    (asked for as a raw handle: building the Stream object took 2.8 us of an
+    8 us call)."""
+    if stream is not None:
+        return int(stream.cuda_stream)
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if not torch.cuda.is_initialized():
+        return int(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t) -> int:
