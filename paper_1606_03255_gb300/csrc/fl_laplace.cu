@@ -445,6 +445,7 @@ __global__ void __launch_bounds__(kLapThreads, P <= 40 ? 2 : 1)
                        const int32_t* __restrict__ tperm, const T* __restrict__ c, int levels, int q,
                        T* __restrict__ partial) {
     __shared__ T red[kLapThreads / 32][P];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const LapItem it = items[blockIdx.x];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int qb = it.band < levels ? q : 1;         // the last band: its sum only
@@ -468,11 +469,35 @@ __global__ void __launch_bounds__(kLapThreads, P <= 40 ? 2 : 1)
     }
 }
 
+// The kernels of a planned transform depend on each other in turn and are short
+// (4 to 20 us): each lets the next one's launch begin while it runs, and a
+// kernel waits for the one before it to finish before it reads (programmatic
+// dependent launch; the first kernel of a call is launched normally).
+__device__ __forceinline__ void lap_wait_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+static cudaError_t lap_launch_after(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // u[l q + j] = sum over the items of band l of partial[item][j]: one warp per
 // entry, the lanes striding over the items, a fixed shuffle tree.
 template <typename T>
 __global__ void k_lap_reduce_items(int levels, int q, const int* __restrict__ first,
                                    const T* __restrict__ partial, double* __restrict__ u) {
+    lap_wait_previous();
     const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= (levels + 1) * q) return;               // uniform across the warp
@@ -494,6 +519,7 @@ __global__ void __launch_bounds__(256)
     k_lap_couple_cheb(int levels, int q, const int* __restrict__ ell, const int64_t* __restrict__ koff,
                       const double* __restrict__ Kt, const double* __restrict__ u,
                       LapTau<T>* __restrict__ ha, LapTau<T>* __restrict__ g) {
+    lap_wait_previous();
     const int m = blockIdx.x + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (blockIdx.x == gridDim.x - 1 && blockIdx.y == 0 && threadIdx.x <= levels) {   // a thread per l
@@ -524,6 +550,7 @@ __global__ void __launch_bounds__(256)
     k_lap_eval_cheb(int64_t M, const LapTau<T>* __restrict__ sigma, const uint8_t* __restrict__ sband,
                     int levels, int q, const LapTau<T>* __restrict__ ha, const LapTau<T>* __restrict__ g,
                     T* __restrict__ f) {
+    lap_wait_previous();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= M) return;
     const int m = sband[j];
@@ -612,6 +639,7 @@ __global__ void k_gen_eval(int64_t M, const double* __restrict__ sv, const LapTa
                            const LapTau<T>* __restrict__ ha, int64_t N, const double* __restrict__ t,
                            const T* __restrict__ c, const int32_t* __restrict__ nearT, int64_t nnear,
                            T* __restrict__ f) {
+    lap_wait_previous();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= M) return;
     const int m = sband[j];
@@ -783,24 +811,26 @@ static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
     // (bands without items sum to zero: no elements, no moments)
     if (!gen || (p.N > 0 && p.levels > 1)) {
         const int entries = (p.levels + 1) * p.q;
-        k_lap_reduce_items<T><<<(entries * 32 + 255) / 256, 256, 0, st>>>(p.levels, p.q, first, partial, u);
+        cudaError_t e = lap_launch_after(k_lap_reduce_items<T>, dim3((unsigned)((entries * 32 + 255) / 256)), dim3(256), st,
+                                         p.levels, p.q, first, partial, u);
         const dim3 grid((unsigned)std::max(1, p.levels - 1), (unsigned)((p.q + 7) / 8));
-        k_lap_couple_cheb<T><<<grid, 256, 0, st>>>(p.levels, p.q, gen ? nullptr : (const int*)(scratch + L.ell),
-                                                   p.d_lapKoff, p.d_lapK, u, ha, g);
+        if (e == cudaSuccess)
+            e = lap_launch_after(k_lap_couple_cheb<T>, grid, dim3(256), st, p.levels, p.q,
+                                 gen ? (const int*)nullptr : (const int*)(scratch + L.ell), p.d_lapKoff, p.d_lapK, u,
+                                 ha, g);
+        if (e != cudaSuccess) return e;
         p.launches += 2;
     }
     if (p.M > 0) {
         timer_begin(p, "lap_eval", (double)p.M * (8 + 1 + sizeof(T)), st, &slot);
-        const unsigned grid = (unsigned)((p.M + 255) / 256);
+        const dim3 grid((unsigned)((p.M + 255) / 256)), block(256);
         const LapTau<T>* sg = (const LapTau<T>*)p.d_stau;
-        if (p.lap_kernel == 2)
-            k_gen_eval<T, 2><<<grid, 256, 0, st>>>(p.M, p.d_s, sg, p.d_sband, p.levels, p.q, ha, p.N, p.d_t, c,
-                                                   p.d_nearT, p.n_nearT, f);
-        else if (p.lap_kernel == 1)
-            k_gen_eval<T, 1><<<grid, 256, 0, st>>>(p.M, p.d_s, sg, p.d_sband, p.levels, p.q, ha, p.N, p.d_t, c,
-                                                   p.d_nearT, p.n_nearT, f);
-        else
-            k_lap_eval_cheb<T><<<grid, 256, 0, st>>>(p.M, sg, p.d_sband, p.levels, p.q, ha, g, f);
+        const cudaError_t e =
+            p.lap_kernel == 0
+                ? lap_launch_after(k_lap_eval_cheb<T>, grid, block, st, p.M, sg, p.d_sband, p.levels, p.q, ha, g, f)
+                : lap_launch_after(p.lap_kernel == 2 ? k_gen_eval<T, 2> : k_gen_eval<T, 1>, grid, block, st, p.M,
+                                   p.d_s, sg, p.d_sband, p.levels, p.q, ha, p.N, p.d_t, c, p.d_nearT, p.n_nearT, f);
+        if (e != cudaSuccess) return e;
         timer_end(p, slot, st);
         p.launches += 1;
     }
