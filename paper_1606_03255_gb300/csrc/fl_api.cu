@@ -449,13 +449,6 @@ static double free_gather_cost(int64_t nodes, int nrhs, int64_t n, int log2n, in
 // in (tile rows TR of the length-n1 pass, rows l2 = g mod n2, column l1 = g /
 // n2); the window values are those of the gather kernel, phi_t = kb(frac(n x)
 // + m_w - 1 - t), in FP64 rounded once.
-static double kb_window_host(double t, double m, double b) {
-    const double s2 = m * m - t * t;
-    if (!(s2 > 0.0)) return b;
-    const double r = sqrt(s2);
-    return sinh(b * r) / r;
-}
-
 static fl_status build_fused(Plan& p, cudaStream_t st) {
     p.fused_bands = p.fused_entries = 0;
     if (p.prec != FL_FP32 || p.xi_mode || p.fuse_mode == 1 || p.M == 0) return FL_OK;
@@ -481,93 +474,91 @@ static fl_status build_fused(Plan& p, cudaStream_t st) {
         if (p.fuse_mode == 2 || fuse) cands.push_back({b, l1, l2, TR, P});
     }
     if (cands.empty()) return FL_OK;
-    std::vector<double2> hw(p.M);
-    FL_CUDA(cudaMemcpyAsync(hw.data(), p.d_ws, p.M * sizeof(double2), cudaMemcpyDeviceToHost, st),
-            "fl_plan: copy nodes");
-    FL_CUDA(cudaStreamSynchronize(st), "fl_plan: synchronise");
+    std::vector<FusedBand> list(cands.size());
+    int64_t chunks = 0, hist_len = 0;
+    int nrb_max = 0;
+    for (size_t c = 0; c < cands.size(); ++c) {
+        const Cand& cd = cands[c];
+        const BandDev& d = p.bands[cd.b].dev;
+        FusedBand& f = list[c];
+        f.node_off = p.bands[cd.b].node_off;
+        f.nodes = p.bands[cd.b].nodes;
+        f.n = d.n;
+        f.kb = d.kb;
+        f.l2 = cd.l2;
+        f.tr = cd.TR;
+        f.parts = cd.P;
+        f.nq = (cd.TR + 3) / 4;
+        f.nrb = (1 << cd.l2) / cd.TR;
+        f.chunk0 = (int)chunks;
+        f.hist0 = hist_len;
+        const int64_t nc = (f.nodes + kFusedChunk - 1) / kFusedChunk;
+        chunks += nc;
+        hist_len += nc * f.nrb;
+        nrb_max = std::max(nrb_max, f.nrb);
+    }
+    FusedBand* d_list = nullptr;
+    int32_t* d_hist = nullptr;
+    cudaError_t e = upload(list, &d_list, st);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_hist, hist_len * sizeof(int32_t));
+    std::vector<int32_t> hist(hist_len);
+    if (e == cudaSuccess) e = launch_fused_entries(p, d_list, (int)list.size(), chunks, nrb_max, false, d_hist, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(hist.data(), d_hist, hist_len * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    // first entry of every (row block, chunk of nodes), row blocks first
     std::vector<int32_t> rbs;
-    std::vector<int2> ent;
-    std::vector<float4> phi;
-    int64_t pp = 0;
-    for (const Cand& cd : cands) {
+    int64_t ents = 0, phis = 0, pp = 0;
+    for (size_t c = 0; c < cands.size() && e == cudaSuccess; ++c) {
+        const Cand& cd = cands[c];
         BandHost& bh = p.bands[cd.b];
         BandDev& d = bh.dev;
-        const int64_t n = d.n, n2 = (int64_t)1 << cd.l2, nrb = n2 / cd.TR;
-        const int NQ = (cd.TR + 3) / 4;
-        struct E {
-            int64_t rb;
-            int slot, l1;
-            float w[8];
-        };
-        std::vector<E> es;
-        es.reserve((size_t)(bh.nodes * ((cd.TR + taps - 1) / cd.TR + 1)));
-        for (int64_t jl = 0; jl < bh.nodes; ++jl) {
-            const double x = hw[bh.node_off + jl].x;
-            const double xr = x - floor(x);
-            const double t0 = (double)n * xr;
-            const double u = floor(t0);
-            const double fr = t0 - u;
-            const int64_t lo = (int64_t)u - (p.mw - 1);
-            int part = 0;
-            int64_t cur = -1;
-            for (int t = 0; t < taps; ++t) {
-                const int64_t g = ((lo + t) % n + n) % n;
-                const int64_t rho = g & (n2 - 1);
-                const int64_t rb = rho / cd.TR;
-                if (rb != cur) {
-                    if (part == cd.P)   // a window spans at most P row blocks (n2 >= 8 TR)
-                        return fail(FL_ECUDA, "fl_plan: fused gather entry count out of range");
-                    E e{};
-                    e.rb = rb;
-                    e.slot = (int)(jl * cd.P + part++);
-                    e.l1 = (int)(g >> cd.l2);
-                    es.push_back(e);
-                    cur = rb;
-                }
-                es.back().w[rho % cd.TR] = (float)kb_window_host(fr + (double)(p.mw - 1 - t), (double)p.mw, d.kb);
-            }
-        }
-        // bucket by row block (stable: node order within a block)
-        std::vector<int32_t> cnt(nrb + 1, 0);
-        for (const E& e : es) ++cnt[e.rb + 1];
-        for (int64_t r = 0; r < nrb; ++r) cnt[r + 1] += cnt[r];
+        FusedBand& f = list[c];
         d.fused = 1;
         d.pparts = cd.P;
-        d.ent_off = (int64_t)ent.size();
+        d.ent_off = f.ent_off = ents;
         d.rbs_off = (int64_t)rbs.size();
-        d.ph_off = (int64_t)phi.size();
+        d.ph_off = f.ph_off = phis;
         d.pp_off = pp;
-        bh.fentries = (int64_t)es.size();
-        rbs.insert(rbs.end(), cnt.begin(), cnt.end());
-        std::vector<int32_t> pos(cnt.begin(), cnt.end() - 1);
-        const size_t e0 = ent.size(), q0 = phi.size();
-        ent.resize(e0 + es.size());
-        phi.resize(q0 + es.size() * NQ);
-        for (const E& e : es) {
-            const int64_t k = pos[e.rb]++;
-            ent[e0 + k] = make_int2(e.slot, e.l1);
-            for (int qd = 0; qd < NQ; ++qd)
-                phi[q0 + k * NQ + qd] = make_float4(e.w[4 * qd], e.w[4 * qd + 1], e.w[4 * qd + 2], e.w[4 * qd + 3]);
+        const int64_t nc = (f.nodes + kFusedChunk - 1) / kFusedChunk;
+        int32_t run = 0;
+        for (int rb = 0; rb < f.nrb; ++rb) {
+            rbs.push_back(run);
+            for (int64_t k = 0; k < nc; ++k) {
+                int32_t& h = hist[f.hist0 + k * f.nrb + rb];
+                const int32_t cnt = h;
+                h = run;
+                run += cnt;
+            }
         }
-        pp += (int64_t)d.nrhs * bh.nodes * cd.P;   // per right-hand side: one slot per (node, row block)
+        rbs.push_back(run);
+        bh.fentries = run;
+        ents += run;
+        phis += (int64_t)run * f.nq;
+        pp += (int64_t)d.nrhs * f.nodes * cd.P;   // per right-hand side: one slot per (node, row block)
         ++p.fused_bands;
     }
-    p.fused_entries = (int64_t)ent.size();
-
-    FL_CUDA(cudaMalloc((void**)&p.d_frbs, rbs.size() * sizeof(int32_t)), "cudaMalloc fused starts");
-    FL_CUDA(cudaMalloc((void**)&p.d_fent, ent.size() * sizeof(int2)), "cudaMalloc fused entries");
-    FL_CUDA(cudaMalloc((void**)&p.d_fphi, phi.size() * sizeof(float4)), "cudaMalloc fused windows");
-    FL_CUDA(cudaMalloc((void**)&p.d_fpp, pp * sizeof(float2)), "cudaMalloc fused partials");
-    FL_CUDA(cudaMemcpyAsync(p.d_frbs, rbs.data(), rbs.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st),
-            "copy fused starts");
-    FL_CUDA(cudaMemcpyAsync(p.d_fent, ent.data(), ent.size() * sizeof(int2), cudaMemcpyHostToDevice, st),
-            "copy fused entries");
-    FL_CUDA(cudaMemcpyAsync(p.d_fphi, phi.data(), phi.size() * sizeof(float4), cudaMemcpyHostToDevice, st),
-            "copy fused windows");
+    p.fused_entries = ents;
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_frbs, rbs.size() * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_fent, ents * sizeof(int2));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_fphi, phis * sizeof(float4));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_fpp, pp * sizeof(float2));
+    if (e == cudaSuccess) e = cudaMemsetAsync(p.d_fphi, 0, phis * sizeof(float4), st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(p.d_frbs, rbs.data(), rbs.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(d_hist, hist.data(), hist_len * sizeof(int32_t), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(d_list, list.data(), list.size() * sizeof(FusedBand), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_fused_entries(p, d_list, (int)list.size(), chunks, nrb_max, true, d_hist, st);
+    // the host vectors and the lists are released on return
+    const cudaError_t es = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = es;
+    cudaFree(d_hist);
+    cudaFree(d_list);
+    FL_CUDA(e, "fl_plan: fused gather entries");
     // slots beyond a node's parts are never written and must read as zero
     FL_CUDA(cudaMemsetAsync(p.d_fpp, 0, pp * sizeof(float2), st), "clear fused partials");
-    // the host vectors are released on return: finish the copies first
-    FL_CUDA(cudaStreamSynchronize(st), "fl_plan: synchronise");
     return FL_OK;
 }
 

@@ -327,6 +327,16 @@ cudaError_t launch_copy_sorted(Plan& p, const Instance& in, const Instance& twin
 // cell[off .. off + n) >>= shift (node cells of a band moved to a grid 2^shift times smaller)
 // nodes [off, off + n), all of bands with one grid size, put in cell order (stable)
 // as the nodes of `band`
+// A band whose gather is fused into pass 2, and where its entries go: chunks of
+// kFusedChunk nodes from chunk0 on, hist[hist0 + chunk nrb + rb].
+constexpr int kFusedChunk = 1024;
+struct FusedBand {
+    int64_t node_off, nodes, n, hist0, ent_off, ph_off;
+    double kb;
+    int l2, tr, parts, nq, nrb, chunk0;
+};
+cudaError_t launch_fused_entries(const Plan& p, const FusedBand* list, int count, int64_t chunks, int nrb_max,
+                                 bool fill, int32_t* hist, cudaStream_t st);
 cudaError_t launch_cell_sort(Plan& p, int64_t off, int64_t n, int band, cudaStream_t st);
 cudaError_t launch_cell_shift(int32_t* cell, int64_t off, int64_t n, int shift, cudaStream_t st);
 
