@@ -363,7 +363,7 @@ __device__ __forceinline__ void cheb_moments(ff tau, float c, int q, float* acc)
 }
 
 // sum_i T_i(tau) a_i, i < q.
-__device__ __forceinline__ double cheb_sum(double tau, const double* __restrict__ a, int q) {
+__device__ __forceinline__ double cheb_sum(double tau, const double* a, int q) {
     if (q <= kLapPlain) {
         const double x2 = tau + tau;
         double t0 = 1.0, t1 = tau, s = a[0];
@@ -389,7 +389,7 @@ __device__ __forceinline__ double cheb_sum(double tau, const double* __restrict_
     }
     return tau < 0.0 ? even - odd : even + odd;
 }
-__device__ __forceinline__ ff cheb_sum(ff tau, const ff* __restrict__ a, int q) {
+__device__ __forceinline__ ff cheb_sum(ff tau, const ff* a, int q) {
     const ff x2 = ff(2.f * tau.hi, 2.f * tau.lo);
     ff t0 = ff(1.f), t1 = tau, s = a[0];
     for (int i = 1; i < q; ++i) {
@@ -472,14 +472,20 @@ __global__ void __launch_bounds__(kLapThreads, P <= 40 ? 2 : 1)
 // The kernels of a planned transform depend on each other in turn and are short
 // (4 to 20 us): each lets the next one's launch begin while it runs, and a
 // kernel waits for the one before it to finish before it reads (programmatic
-// dependent launch; the first kernel of a call is launched normally).
+// dependent launch; the first kernel of a call is launched normally, whichever
+// it is, so nothing of a call overlaps what precedes it on the stream).  A
+// dependent is resident while partial, u, ha and g are still being written:
+// they are passed as plain pointers (const __restrict__ would declare them
+// unchanged for the kernel's lifetime and allow their loads to be moved before
+// the wait), only the plan's tables and the caller's c and t as restricted ones.
 __device__ __forceinline__ void lap_wait_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <typename... P, typename... A>
-static cudaError_t lap_launch_after(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+static cudaError_t lap_launch_after(bool* dependent, void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st,
+                                    A... args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
@@ -488,7 +494,8 @@ static cudaError_t lap_launch_after(void (*kern)(P...), dim3 grid, dim3 block, c
     cfg.blockDim = block;
     cfg.stream = st;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = *dependent ? 1 : 0;
+    *dependent = true;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
@@ -496,7 +503,7 @@ static cudaError_t lap_launch_after(void (*kern)(P...), dim3 grid, dim3 block, c
 // entry, the lanes striding over the items, a fixed shuffle tree.
 template <typename T>
 __global__ void k_lap_reduce_items(int levels, int q, const int* __restrict__ first,
-                                   const T* __restrict__ partial, double* __restrict__ u) {
+                                   const T* partial, double* u) {
     lap_wait_previous();
     const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -517,8 +524,7 @@ __global__ void k_lap_reduce_items(int levels, int q, const int* __restrict__ fi
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_lap_couple_cheb(int levels, int q, const int* __restrict__ ell, const int64_t* __restrict__ koff,
-                      const double* __restrict__ Kt, const double* __restrict__ u,
-                      LapTau<T>* __restrict__ ha, LapTau<T>* __restrict__ g) {
+                      const double* __restrict__ Kt, const double* u, LapTau<T>* ha, LapTau<T>* g) {
     lap_wait_previous();
     const int m = blockIdx.x + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -548,8 +554,7 @@ __global__ void __launch_bounds__(256)
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_lap_eval_cheb(int64_t M, const LapTau<T>* __restrict__ sigma, const uint8_t* __restrict__ sband,
-                    int levels, int q, const LapTau<T>* __restrict__ ha, const LapTau<T>* __restrict__ g,
-                    T* __restrict__ f) {
+                    int levels, int q, const LapTau<T>* ha, const LapTau<T>* g, T* f) {
     lap_wait_previous();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= M) return;
@@ -636,9 +641,8 @@ __global__ void k_gen_ktable(int kind, int levels, int q, double y1, double xi1,
 template <typename T, int KIND>
 __global__ void k_gen_eval(int64_t M, const double* __restrict__ sv, const LapTau<T>* __restrict__ stau,
                            const uint8_t* __restrict__ sband, int levels, int q,
-                           const LapTau<T>* __restrict__ ha, int64_t N, const double* __restrict__ t,
-                           const T* __restrict__ c, const int32_t* __restrict__ nearT, int64_t nnear,
-                           T* __restrict__ f) {
+                           const LapTau<T>* ha, int64_t N, const double* __restrict__ t,
+                           const T* __restrict__ c, const int32_t* __restrict__ nearT, int64_t nnear, T* f) {
     lap_wait_previous();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= M) return;
@@ -796,6 +800,7 @@ static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
     const int* first = (const int*)(scratch + L.first);
     const bool gen = p.lap_kernel != 0;
     int slot = -1;
+    bool dependent = false;   // whether a kernel of this call precedes
     if (p.n_lap_items > 0) {
         timer_begin(p, "lap_moments", (double)p.N * (8 + 4 + sizeof(T)), st, &slot);
         switch ((p.q + 7) / 8) {
@@ -807,15 +812,16 @@ static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
         }
         timer_end(p, slot, st);
         ++p.launches;
+        dependent = true;
     }
     // (bands without items sum to zero: no elements, no moments)
     if (!gen || (p.N > 0 && p.levels > 1)) {
         const int entries = (p.levels + 1) * p.q;
-        cudaError_t e = lap_launch_after(k_lap_reduce_items<T>, dim3((unsigned)((entries * 32 + 255) / 256)), dim3(256), st,
-                                         p.levels, p.q, first, partial, u);
+        cudaError_t e = lap_launch_after(&dependent, k_lap_reduce_items<T>, dim3((unsigned)((entries * 32 + 255) / 256)),
+                                         dim3(256), st, p.levels, p.q, first, partial, u);
         const dim3 grid((unsigned)std::max(1, p.levels - 1), (unsigned)((p.q + 7) / 8));
         if (e == cudaSuccess)
-            e = lap_launch_after(k_lap_couple_cheb<T>, grid, dim3(256), st, p.levels, p.q,
+            e = lap_launch_after(&dependent, k_lap_couple_cheb<T>, grid, dim3(256), st, p.levels, p.q,
                                  gen ? (const int*)nullptr : (const int*)(scratch + L.ell), p.d_lapKoff, p.d_lapK, u,
                                  ha, g);
         if (e != cudaSuccess) return e;
@@ -827,8 +833,9 @@ static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
         const LapTau<T>* sg = (const LapTau<T>*)p.d_stau;
         const cudaError_t e =
             p.lap_kernel == 0
-                ? lap_launch_after(k_lap_eval_cheb<T>, grid, block, st, p.M, sg, p.d_sband, p.levels, p.q, ha, g, f)
-                : lap_launch_after(p.lap_kernel == 2 ? k_gen_eval<T, 2> : k_gen_eval<T, 1>, grid, block, st, p.M,
+                ? lap_launch_after(&dependent, k_lap_eval_cheb<T>, grid, block, st, p.M, sg, p.d_sband, p.levels, p.q,
+                                   ha, g, f)
+                : lap_launch_after(&dependent, p.lap_kernel == 2 ? k_gen_eval<T, 2> : k_gen_eval<T, 1>, grid, block, st, p.M,
                                    p.d_s, sg, p.d_sband, p.levels, p.q, ha, p.N, p.d_t, c, p.d_nearT, p.n_nearT, f);
         if (e != cudaSuccess) return e;
         timer_end(p, slot, st);
