@@ -48,8 +48,10 @@ class FourierLaplace(torch.nn.Module):
     """f = sum_k c_k exp(2 pi i k w_j) with autograd in c and in the nodes w.
 
     The plan (banding and sorting of the nodes, tables) is rebuilt when the
-    node tensor changes (new storage or an in-place update) and reused
-    otherwise.
+    node tensor changes (new storage, another layout or an in-place update) and
+    reused otherwise.  The module holds the tensor that its plan was made from,
+    so that no other can take its place in memory; an update that hides from
+    autograd's version counter (through ``.data``) is not seen.
     """
 
     def __init__(self, N: int, eps: float = 1e-6, precision: str = "fp32", q: int = 0):
@@ -60,15 +62,17 @@ class FourierLaplace(torch.nn.Module):
         self.q = int(q)
         self._plan = None
         self._key = None
+        self._nodes = None   # what the plan was made from (shares storage and version)
 
     def plan_for(self, nodes: torch.Tensor) -> fl.Plan:
-        key = (nodes.data_ptr(), nodes._version, tuple(nodes.shape), nodes.device)
+        key = (nodes.data_ptr(), nodes._version, tuple(nodes.shape), nodes.stride(), nodes.device)
         if self._plan is None or key != self._key:
             if self._plan is not None:
                 self._plan.close()
             self._plan = fl.Plan(self.N, nodes.detach(), self.eps, precision=self.precision,
                                  q=self.q)
             self._key = key
+            self._nodes = nodes.detach()
         return self._plan
 
     def forward(self, c: torch.Tensor, nodes: torch.Tensor) -> torch.Tensor:
