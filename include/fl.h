@@ -265,7 +265,8 @@ fl_status fl_execute_batched_ptrs(fl_plan_t p, const void *const *c_host, void *
 /*
  * fl_execute -- f~ ~= C c with C = (z_j^k), Algorithm 2.
  *   c_dev : device, N complex (plan precision).
- *   f_dev : device, M complex (plan precision), fully overwritten.
+ *   f_dev : device, M complex (plan precision), fully overwritten; it may
+ *           overlap c_dev (then the call may copy c first).
  * Asynchronous on `stream`.
  */
 fl_status fl_execute(fl_plan_t p, const void *c_dev, void *f_dev, void *stream);

@@ -1379,10 +1379,35 @@ static fl_status build_plan_tuned(const PlanSpec& sp, double bias, bool autotune
     return FL_OK;
 }
 
+// The forward transform where f may overlap c.  The direct bands write their
+// results while other blocks still read c, and the Z^0 nodes read c_0 in the last
+// kernel; the FFT passes are through with c before anything is written, and the
+// float-pair form reads a converted copy.  Where it matters, c is copied first
+// (stream-ordered scratch: the call stays asynchronous and can be captured).
+static bool reads_c_late(const Plan& p, const void* c, const void* f) {
+    if (p.z0_nodes == 0 && (p.direct_work.empty() || p.prec == FL_FP64_FF)) return false;
+    const size_t cs = p.prec != FL_FP32 ? 16 : 8;
+    const uintptr_t a = (uintptr_t)c, b = (uintptr_t)f;
+    return a < b + (size_t)p.M * cs && b < a + (size_t)p.N * cs;
+}
+
+static cudaError_t forward_call(Plan& p, const void* c, void* f, bool deriv, const void* rmul, cudaStream_t st) {
+    if (!reads_c_late(p, c, f)) return run_forward(p, c, f, deriv, st, rmul);
+    const size_t bytes = (size_t)p.N * (p.prec != FL_FP32 ? 16 : 8);
+    void* copy = nullptr;
+    cudaError_t e = cudaMallocAsync(&copy, bytes, st);
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(copy, c, bytes, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = run_forward(p, copy, f, deriv, st, rmul);
+    const cudaError_t e2 = cudaFreeAsync(copy, st);
+    return e != cudaSuccess ? e : e2;
+}
+
 // fl_execute through a CUDA graph of its launches, captured on the first call
 // (and again when the buffers or the stream change), then replayed.
 static cudaError_t forward_graphed(Plan& p, const void* c, void* f, cudaStream_t st) {
-    if (!p.use_graph || p.timing || st == nullptr) return run_forward(p, c, f, false, st);
+    if (!p.use_graph || p.timing || st == nullptr || reads_c_late(p, c, f))
+        return forward_call(p, c, f, false, nullptr, st);
     if (!p.gexec || p.g_c != c || p.g_f != f || p.g_st != st) {
         if (p.gexec) {
             cudaGraphExecDestroy(p.gexec);
@@ -1537,7 +1562,7 @@ fl_status fl_execute_deriv(fl_plan_t h, const void* c_dev, void* f_dev, void* st
     if (h->p.M > 0 && (!c_dev || !f_dev)) return fail(FL_EINVAL, "fl_execute_deriv: NULL buffer");
     if (h->p.batched) return fail(FL_EUNSUPPORTED, "fl_execute_deriv: batched plans are forward only");
     if (h->p.xi_mode) return fail(FL_EUNSUPPORTED, "fl_execute_deriv: real-exponent plans are forward only");
-    cudaError_t e = run_forward(h->p, c_dev, f_dev, true, (cudaStream_t)stream);
+    cudaError_t e = forward_call(h->p, c_dev, f_dev, true, nullptr, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "fl_execute_deriv");
     return FL_OK;
 }
@@ -1547,7 +1572,7 @@ fl_status fl_grad_w(fl_plan_t h, const void* c_dev, const void* r_dev, void* gw_
     if (h->p.M > 0 && (!c_dev || !r_dev || !gw_dev)) return fail(FL_EINVAL, "fl_grad_w: NULL buffer");
     if (h->p.batched) return fail(FL_EUNSUPPORTED, "fl_grad_w: batched plans are forward only");
     if (h->p.xi_mode) return fail(FL_EUNSUPPORTED, "fl_grad_w: real-exponent plans are forward only");
-    cudaError_t e = run_forward(h->p, c_dev, gw_dev, true, (cudaStream_t)stream, r_dev);
+    cudaError_t e = forward_call(h->p, c_dev, gw_dev, true, r_dev, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "fl_grad_w");
     return FL_OK;
 }
