@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(256)
     const double kb = XI ? kb_b : B.kb;
 #pragma unroll
     for (int t = 0; t < 2 * MW; ++t)
-        sp_phi[i * (2 * MW) + t] = T(kb_window<double>(fr + (double)(MW - 1 - t), (double)MW, kb));
+        sp_phi[i * (2 * MW) + t] = sizeof(T) == 8 ? T(kb_window_exact(fr, (double)(MW - 1 - t), (double)MW, kb))
+                                                  : T(kb_window<double>(fr + (double)(MW - 1 - t), (double)MW, kb));
     if (B.nrhs == 1) return;
     const double tau = (kTwoPiAdj * wv.y - B.yc) * B.yh_inv;
     const int q = B.nrhs;

@@ -95,8 +95,12 @@ __global__ void k_weights(BandDev B, int ellm, int Lm, int q, double xi1, int le
     double inv_phi = 1.0;
     if (!xis) {   // the window of this grid: shape B.kb (kb_b for sigma = 2)
         const double nu = (double)(k - B.Nm / 2) / (double)B.n;
-        const double arg = B.kb * B.kb - (kTwoPiD * nu) * (kTwoPiD * nu);
-        inv_phi = 1.0 / (kPi * cyl_bessel_i0((double)mw * sqrt(fmax(arg, 0.0))));
+        if constexpr (sizeof(T) == 8) {
+            inv_phi = 1.0 / (kPi * kb_transform_exact(nu, (double)mw, B.kb));
+        } else {
+            const double arg = B.kb * B.kb - (kTwoPiD * nu) * (kTwoPiD * nu);
+            inv_phi = 1.0 / (kPi * cyl_bessel_i0((double)mw * sqrt(fmax(arg, 0.0))));
+        }
     }
     // entry s of frequency k at Dk[s * ds]
     T* Dk = D + B.D_off + (B.dld ? k * B.dld : k);
@@ -549,7 +553,10 @@ __global__ void __launch_bounds__(256) k_gather(int64_t M, const double2* __rest
     }
     if (!tab) {
 #pragma unroll
-        for (int t = 0; t < 2 * MW; ++t) phi[t] = kb_window<T>(fr + (T)(MW - 1 - t), (T)MW, kb);
+        for (int t = 0; t < 2 * MW; ++t) {
+            if constexpr (sizeof(T) == 8) phi[t] = kb_window_exact(fr, (T)(MW - 1 - t), (T)MW, kb);
+            else phi[t] = kb_window<T>(fr + (T)(MW - 1 - t), (T)MW, kb);
+        }
     }
     const int64_t nmask = B.n - 1;
     const C* g = grid + B.grid_off;
