@@ -105,6 +105,22 @@ static int onesided_rank(double eps_K) {
     return kMaxQ + 1;
 }
 
+// FP64 plans that merge a directly summed band (merge_bands) take windows one
+// point wider on each side: nodes without a window error come under one, 1.2 times
+// the error against 64 bits of the bands before (5.5e-14 against 4.5e-14 at N = M =
+// 3000, eps = 1e-10).  A point more divides the window's error by
+// e^(2 pi sqrt(1 - 1/sigma)) (85 at sigma = 2: 8.7e-16 there) and costs two taps per
+// node and right-hand side.
+static void widen_windows(Plan& p) {
+    p.mw_extra = 1;
+    p.mw = std::min(12, p.mw + 1);
+}
+
+// The half-width of a sub-band NFFT of oversampling sigma.
+static int split_width(const Plan& p, double sigma) {
+    return std::min(12, window_width(p.eps_A, sigma) + p.mw_extra);
+}
+
 static fl_status select_common(Plan& p, int q_in) {
     p.eps_K = p.eps / 3.0;
     p.eps_A = p.eps / 3.0;
@@ -121,6 +137,7 @@ static fl_status select_common(Plan& p, int q_in) {
     // the latter's error amplified by up to Phi(0)/Phi(1/4) < 8 in the division
     // by Phi(x/2): each gets eps_A / 8
     p.mw = window_width(p.xi_mode ? p.eps_A / 8.0 : p.eps_A, 2.0);
+    p.mw_extra = 0;
     p.kb_b = M_PI * (2.0 - 1.0 / 2.0);
     return FL_OK;
 }
@@ -641,7 +658,7 @@ static SplitChoice best_split(const Plan& p, const BandHost& bh, double smin, in
             const int64_t n = (int64_t)1 << lg;
             if ((double)n >= 2.0 * (double)Nc) continue;   // no gain over sigma = 2
             // the half-width this sigma needs, and the FP32 limit at it
-            const int mc = std::max(mw, window_width(p.eps_A, (double)n / (double)Nc));
+            const int mc = std::max(mw, split_width(p, (double)n / (double)Nc));
             if (deconv_gain((double)n / (double)Nc, mc) > gain_max) continue;
             const double gather = free32    ? free_gather_cost(bh.nodes, d.nrhs, n, lg, mc, fusable, &fz)
                                   : fusable ? d.nrhs * fused_cost(bh.nodes, lg, mc)
@@ -691,7 +708,7 @@ static fl_status plan_splits(Plan& p, const std::vector<int>& nfft, cudaStream_t
             smin_used = std::min(smin_used, ldexp(1.0, c.log2n) / (double)c.Nc);
         }
     if (!any) return FL_OK;
-    p.mw = std::max(p.mw, window_width(p.eps_A, smin_used));
+    p.mw = std::max(p.mw, split_width(p, smin_used));
     p.sigma_min = smin_used;
     for (size_t i = 0; i < nfft.size(); ++i) {
         const SplitChoice c = best_ch[i];
@@ -735,7 +752,11 @@ static fl_status plan_splits(Plan& p, const std::vector<int>& nfft, cudaStream_t
 // Chebyshev points y_s of the union), at the rank that leaves no larger an
 // error than rank q leaves on a single dyadic band: at N = M = 2^20, eps = 1e-6 the
 // six bands of the clustered nodes take 35 right-hand sides instead of 72, at
-// 2^18 and 1e-12 nine bands 82 instead of 198.
+// 2^18 and 1e-12 nine bands 82 instead of 198.  In FP64 a directly summed band
+// only where another band goes through an NFFT anyway, and then with wider windows
+// (widen_windows): where all were direct, merging raised the error at 300 x 5000 and
+// eps = 1e-10 from 6.6e-15 to 3.8e-14 (adjoint 6.7e-16 to 8.9e-15), and the call took
+// 148 us instead of 45.
 
 // Bounds of the interpolation error of exp(-y x) on y in [a, b], relative to the
 // kernel's bound 1, at 0 .. kMaxQ points: the Chebyshev coefficients of
@@ -818,6 +839,10 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
         if (p.bands[in.band_base + lb].nodes > 0 && p.bands[in.band_base + lb].ell == 1) list.push_back(lb);
     const int n = (int)list.size();
     if (n == 0) return FL_OK;
+    // FP64: where every band is summed directly the transform has no error but
+    // rounding, and keeps it
+    bool merge_direct = p.prec != FL_FP64;
+    for (int lb = 1; lb <= in.levels; ++lb) merge_direct |= p.bands[in.band_base + lb].dev.route == 1;
     double tol;
     {
         double err[kMaxQ + 1];   // the dyadic band at rank q, over every x
@@ -850,6 +875,7 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
                                                    : nfft_cost(p, alone);
         best[j + 1] = Part{best[j].cost + single, j, 0};
         for (int i = j; i >= 0; --i) {
+            if (!merge_direct && p.bands[in.band_base + list[i]].dev.route == 2) break;
             const int r = merged_rank(p, ldexp(p.y1, -list[j]), list[j] - list[i] + 1, in.xi1, tol);
             if (r > kMaxQ) break;
             if (i == j && r >= p.q) continue;
@@ -860,6 +886,8 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
     for (int j = n; j > 0; j = best[j].from) {
         const int i = best[j].from, r = best[j].rank;
         if (r == 0) continue;
+        for (int t = i; t < j; ++t)
+            if (p.prec == FL_FP64 && p.mw_extra == 0 && p.bands[in.band_base + list[t]].dev.route == 2) widen_windows(p);
         const int lead = in.band_base + list[i];
         const BandHost g = merged(i, j - 1, r);
         for (int t = i; t < j; ++t) {
