@@ -27,8 +27,18 @@ __device__ __forceinline__ ff adj_shfl(ff v, int o) { return ff(adj_shfl(v.hi, o
 // the forward epilogue).  None depends on the values transformed, so an adjoint
 // call only forms r_j e_j; the FP64 and float-pair gathers read the taps and
 // weights too (they formed about 10^3 FP64 operations of them per node and
-// call).  In double, rounded once (FP32 with integer exponents: in float from
-// the node records, as the gather forms them).
+// call).  In double, rounded once.  FP32 with integer exponents: in float from
+// the node records (X = x 2^64, tau as a pair: in double this would be 1 ms of the
+// FP64 pipe at M = 2^18), each fraction the float nearest to 32 bits of X and each
+// difference tau - t_s rounded once.  (Fractions cut to 24 bits, as the gather
+// has them, turn every node the same way, by 2^-25 turns on average: 1.9e-7 of the
+// result.)
+__device__ __forceinline__ float adj_turns(uint64_t ph) { return (float)(int32_t)(ph >> 32) * 0x1p-32f; }
+__device__ __forceinline__ float adj_difference(float th, float tl, float ch, float cl) {
+    const float s = th - ch, z = s - th, e = (th - (s - z)) - (ch + z);   // th - ch = s + e
+    return s + (e + (tl - cl));
+}
+
 template <int MW>
 __global__ void __launch_bounds__(256)
     k_node_tables_f32(int64_t M, const uint4* __restrict__ ntab, const int32_t* __restrict__ bandid,
@@ -42,11 +52,10 @@ __global__ void __launch_bounds__(256)
     const uint64_t X = ((uint64_t)nd.y << 32) | nd.x;
     float2 e = {1.f, 0.f};
     if (B.nsub == 0) {
-        const float ph = (float)((int64_t)((uint64_t)(B.Nm >> 1) * X) >> 40) * 0x1p-24f;
-        e = expipi<float>(-2.f * ph);
+        e = expipi<float>(-2.f * adj_turns((uint64_t)(B.Nm >> 1) * X));
     }
     sp_e[i] = e;
-    const float fr = (float)((X << B.log2n) >> 40) * 0x1p-24f, kb = (float)B.kb;
+    const float fr = (float)(uint32_t)((X << B.log2n) >> 32) * 0x1p-32f, kb = (float)B.kb;
 #pragma unroll
     for (int t = 0; t < 2 * MW; ++t) sp_phi[i * (2 * MW) + t] = kb_window<float>(fr + (float)(MW - 1 - t), (float)MW, kb);
     if (B.nrhs == 1) return;
@@ -57,7 +66,7 @@ __global__ void __launch_bounds__(256)
     float den = 0.f;
     int hit = -1;
     for (int s = 0; s < q; ++s) {
-        const float d = (th - ch[s]) + (tl - ch[q + s]);
+        const float d = adj_difference(th, tl, ch[s], ch[q + s]);
         if (d == 0.f) hit = s;
         L[s] = ch[2 * q + s] / d;
         den += L[s];
@@ -133,8 +142,7 @@ __device__ __forceinline__ float2 adj_phase(int64_t kc, const uint4* __restrict_
                                             float) {
     const uint4 nd = ntab[j];
     const uint64_t X = ((uint64_t)nd.y << 32) | nd.x;
-    const float ph = (float)((int64_t)((uint64_t)kc * X) >> 40) * 0x1p-24f;
-    return expipi<float>(-2.f * ph);
+    return expipi<float>(-2.f * adj_turns((uint64_t)kc * X));
 }
 __device__ __forceinline__ double2 adj_phase(int64_t kc, const uint4*, const double2* __restrict__ ws, int64_t j,
                                              double) {
