@@ -518,9 +518,19 @@ __global__ void k_lap_reduce_items(int levels, int q, const int* __restrict__ fi
 
 // a^{Y_m}_i = sum_{l = lo(m)}^{hi(m)} sum_j K''(m, l)_{ij} u^{Omega_l}_j, m = blockIdx.x
 // + 1, one warp per i (blockIdx.y: groups of 8), lanes striding over (l, j), a
-// fixed shuffle tree; written as LapTau<T> values.  Algorithm 1 (ell != nullptr):
+// fixed shuffle tree; written as LapTau<T> values (an overflow or NaN in the high
+// part, with no low part).  Algorithm 1 (ell != nullptr):
 // l = l_m .. M - m; the generalised algorithm: l = 1 .. M - 1.  The last block
 // (the least of the others' work) also forms g_l = sum_{l' >= l} S_{l'} (S = u_0), g_{levels+1} = 0.
+template <typename T> __device__ __forceinline__ LapTau<T> lap_value(double x) {
+    if constexpr (sizeof(T) == 4) {
+        const float hi = (float)x;
+        return ff(hi, isfinite(hi) ? (float)(x - (double)hi) : 0.f);
+    } else {
+        return x;
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_lap_couple_cheb(int levels, int q, const int* __restrict__ ell, const int64_t* __restrict__ koff,
@@ -533,7 +543,7 @@ __global__ void __launch_bounds__(256)
         double s = 0.0;
 #pragma unroll 4
         for (int k = levels; k >= l; --k) s += u[k * q];
-        g[l] = LapTau<T>(s);
+        g[l] = lap_value<T>(s);
     }
     const int i = blockIdx.y * 8 + warp;
     if (m >= levels || i >= q) return;
@@ -546,7 +556,7 @@ __global__ void __launch_bounds__(256)
     for (int x = lane; x < tot; x += 32) acc += K[x] * ul[x];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) ha[m * q + i] = LapTau<T>(acc);
+    if (lane == 0) ha[m * q + i] = lap_value<T>(acc);
 }
 
 // f~_j = sum_i T_i(sigma_j) a_i + g_{L_m+1} (s_j in Y_m), g_1 (s_j in Y_M); the
@@ -560,9 +570,14 @@ __global__ void __launch_bounds__(256)
     if (j >= M) return;
     const int m = sband[j];
     LapTau<T> v = g[m >= levels ? 1 : levels - m + 1];
-    if (m < levels) v = cheb_sum(sigma[j], ha + m * q, q) + v;
-    if constexpr (sizeof(T) == 4) f[j] = ff_round(v);
-    else f[j] = v;
+    if constexpr (sizeof(T) == 4) {
+        const float far = v.hi;
+        if (m < levels) v = cheb_sum(sigma[j], ha + m * q, q) + v;
+        f[j] = isinf(far) && m < levels ? cheb_sum(sigma[j], ha + m * q, q).hi + far : ff_round(v);
+    } else {
+        if (m < levels) v = cheb_sum(sigma[j], ha + m * q, q) + v;
+        f[j] = v;
+    }
 }
 
 // f~_j: barycentric weights of s_j on Y_m (double), then sum_s L_s h_s + g_{L_m + 1}.
