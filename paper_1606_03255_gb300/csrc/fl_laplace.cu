@@ -312,6 +312,30 @@ __global__ void k_lap_starts(int64_t n, const uint8_t* __restrict__ band, int le
 constexpr int kLapPlain = 16;
 __device__ __forceinline__ float ff_round(ff a) { return a.hi + a.lo; }
 
+// What the moments are summed in: double, or (FP32 form) a float with the
+// rounding of all its sums beside it, so that a moment reaches the coupling sums
+// in more than FP32 accuracy -- the band functions' Chebyshev coefficients are as
+// large as the function at its larger end, and moments rounded to float were
+// off by up to 1.8 times what the float sums over Lagrange weights are (K_1/2 at 4431 x
+// 35414: 7.9e-8 against 4.5e-8; 2^-24 = 6e-8).  An overflow stays in hi.
+struct LapSum32 {
+    float hi, lo;
+    __device__ __forceinline__ LapSum32() : hi(0.f), lo(0.f) {}
+    __device__ __forceinline__ LapSum32(float h, float l) : hi(h), lo(l) {}
+    // exact sum of the high parts and their rounding
+    __device__ __forceinline__ LapSum32 operator+(LapSum32 b) const {
+        const float s = hi + b.hi, z = s - hi;
+        return LapSum32(s, lo + b.lo + ((hi - (s - z)) + (b.hi - z)));
+    }
+};
+template <typename T> struct lap_sum { using type = double; };
+template <> struct lap_sum<float> { using type = LapSum32; };
+template <typename T> using LapSum = typename lap_sum<T>::type;
+__device__ __forceinline__ double lap_total(double v) { return v; }
+__device__ __forceinline__ double lap_total(LapSum32 v) {
+    return isfinite(v.hi) ? (double)v.hi + (double)v.lo : (double)v.hi;
+}
+
 // acc[j] += c T_j(tau), j < q <= P.
 template <int P>
 __device__ __forceinline__ void cheb_moments(double tau, double c, int q, double* acc) {
@@ -345,10 +369,10 @@ __device__ __forceinline__ void cheb_moments(double tau, double c, int q, double
     }
 }
 template <int P>
-__device__ __forceinline__ void cheb_moments(ff tau, float c, int q, float* acc) {
+__device__ __forceinline__ void cheb_moments(ff tau, float c, int q, LapSum32* acc) {
     const ff x2 = ff(2.f * tau.hi, 2.f * tau.lo);
     ff t0 = ff(1.f), t1 = tau;
-    acc[0] += c;
+    acc[0] = acc[0] + LapSum32(c, 0.f);
 #pragma unroll
     for (int j = 1; j < P; ++j) {
         if (j < q) {
@@ -357,7 +381,8 @@ __device__ __forceinline__ void cheb_moments(ff tau, float c, int q, float* acc)
                 t0 = t1;
                 t1 = t2;
             }
-            acc[j] = fmaf(c, ff_round(t1), acc[j]);
+            const float p = c * t1.hi;
+            acc[j] = acc[j] + LapSum32(p, fmaf(c, t1.lo, fmaf(c, t1.hi, -p)));
         }
     }
 }
@@ -412,6 +437,7 @@ struct LapItem {
 
 __device__ __forceinline__ float lap_shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ double lap_shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ LapSum32 lap_shfl(LapSum32 v, int o) { return LapSum32(lap_shfl(v.hi, o), lap_shfl(v.lo, o)); }
 
 // Sums v[0 .. 7] over the lanes of a warp: halving steps (a lane keeps one half of
 // its values and takes its partner's sums of that half), then two full ones; lane
@@ -428,8 +454,8 @@ template <typename T> __device__ __forceinline__ void sum8(T* v, int lane) {
             v[i] = keep + lap_shfl(give, off);
         }
     }
-    v[0] += lap_shfl(v[0], 2);
-    v[0] += lap_shfl(v[0], 1);
+    v[0] = v[0] + lap_shfl(v[0], 2);
+    v[0] = v[0] + lap_shfl(v[0], 1);
 }
 
 // Moments u_j of one item, j < q <= P: each thread sums its elements over the
@@ -443,15 +469,16 @@ template <typename T, int P>
 __global__ void __launch_bounds__(kLapThreads, P <= 40 ? 2 : 1)
     k_lap_moments_cheb(const LapItem* __restrict__ items, const LapTau<T>* __restrict__ tau,
                        const int32_t* __restrict__ tperm, const T* __restrict__ c, int levels, int q,
-                       T* __restrict__ partial) {
-    __shared__ T red[kLapThreads / 32][P];
+                       double* __restrict__ partial) {
+    using S = LapSum<T>;
+    __shared__ double red[kLapThreads / 32][P];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const LapItem it = items[blockIdx.x];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int qb = it.band < levels ? q : 1;         // the last band: its sum only
-    T acc[P];
+    S acc[P];
 #pragma unroll
-    for (int j = 0; j < P; ++j) acc[j] = (T)0;
+    for (int j = 0; j < P; ++j) acc[j] = S();
     for (int e = threadIdx.x; e < it.count; e += kLapThreads) {
         const int64_t k = it.k0 + e;
         cheb_moments<P>(tau[k], c[tperm[k]], qb, acc);
@@ -459,11 +486,11 @@ __global__ void __launch_bounds__(kLapThreads, P <= 40 ? 2 : 1)
 #pragma unroll
     for (int j = 0; j < P; j += 8) {
         sum8(acc + j, lane);
-        if ((lane & 3) == 0) red[w][j + (lane >> 2)] = acc[j];   // entry 4 [l & 16] + 2 [l & 8] + [l & 4] = l / 4
+        if ((lane & 3) == 0) red[w][j + (lane >> 2)] = lap_total(acc[j]);   // entry 4 [l & 16] + 2 [l & 8] + [l & 4] = l / 4
     }
     __syncthreads();
     if (threadIdx.x < P && threadIdx.x < q) {
-        T s = (T)0;
+        double s = 0.0;
         for (int ww = 0; ww < kLapThreads / 32; ++ww) s += red[ww][threadIdx.x];
         partial[(int64_t)blockIdx.x * q + threadIdx.x] = s;
     }
@@ -501,16 +528,15 @@ static cudaError_t lap_launch_after(bool* dependent, void (*kern)(P...), dim3 gr
 
 // u[l q + j] = sum over the items of band l of partial[item][j]: one warp per
 // entry, the lanes striding over the items, a fixed shuffle tree.
-template <typename T>
 __global__ void k_lap_reduce_items(int levels, int q, const int* __restrict__ first,
-                                   const T* partial, double* u) {
+                                   const double* partial, double* u) {
     lap_wait_previous();
     const int i = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= (levels + 1) * q) return;               // uniform across the warp
     const int l = i / q, j = i - l * q;
     double s = 0.0;
-    for (int b = first[l] + lane; b < first[l + 1]; b += 32) s += (double)partial[(int64_t)b * q + j];
+    for (int b = first[l] + lane; b < first[l + 1]; b += 32) s += partial[(int64_t)b * q + j];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if (lane == 0) u[i] = s;
@@ -784,10 +810,10 @@ struct LapPlanLayout {
     size_t partial, u, ha, g, ell, first, total;
 };
 
-static LapPlanLayout lap_plan_layout(int levels, int q, int64_t items, size_t tsize) {
+static LapPlanLayout lap_plan_layout(int levels, int q, int64_t items) {
     LapPlanLayout L;
     size_t off = 0;
-    L.partial = off; off = align256(off + (size_t)items * q * tsize);
+    L.partial = off; off = align256(off + (size_t)items * q * sizeof(double));
     L.u = off;       off = align256(off + (size_t)(levels + 1) * q * sizeof(double));
     L.ha = off;      off = align256(off + (size_t)(levels + 1) * q * sizeof(double));
     L.g = off;       off = align256(off + (size_t)(levels + 2) * sizeof(double));
@@ -798,7 +824,7 @@ static LapPlanLayout lap_plan_layout(int levels, int q, int64_t items, size_t ts
 }
 
 template <typename T, int P>
-static void lap_moments_launch(Plan& p, const T* c, T* partial, cudaStream_t st) {
+static void lap_moments_launch(Plan& p, const T* c, double* partial, cudaStream_t st) {
     k_lap_moments_cheb<T, P><<<(unsigned)p.n_lap_items, kLapThreads, 0, st>>>(
         (const LapItem*)p.d_lapitems, (const LapTau<T>*)p.d_ttau, p.d_tperm, c, p.levels, p.q, partial);
 }
@@ -806,9 +832,9 @@ static void lap_moments_launch(Plan& p, const T* c, T* partial, cudaStream_t st)
 // moments -> reduce -> couple -> eval, both forms of the algorithm.
 template <typename T>
 static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
-    const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items, sizeof(T));
+    const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items);
     unsigned char* scratch = (unsigned char*)p.d_lap;
-    T* partial = (T*)(scratch + L.partial);
+    double* partial = (double*)(scratch + L.partial);
     double* u = (double*)(scratch + L.u);
     LapTau<T>* ha = (LapTau<T>*)(scratch + L.ha);
     LapTau<T>* g = (LapTau<T>*)(scratch + L.g);
@@ -832,7 +858,7 @@ static cudaError_t lap_plan_run(Plan& p, const T* c, T* f, cudaStream_t st) {
     // (bands without items sum to zero: no elements, no moments)
     if (!gen || (p.N > 0 && p.levels > 1)) {
         const int entries = (p.levels + 1) * p.q;
-        cudaError_t e = lap_launch_after(&dependent, k_lap_reduce_items<T>, dim3((unsigned)((entries * 32 + 255) / 256)),
+        cudaError_t e = lap_launch_after(&dependent, k_lap_reduce_items, dim3((unsigned)((entries * 32 + 255) / 256)),
                                          dim3(256), st, p.levels, p.q, first, partial, u);
         const dim3 grid((unsigned)std::max(1, p.levels - 1), (unsigned)((p.q + 7) / 8));
         if (e == cudaSuccess)
@@ -980,7 +1006,7 @@ static cudaError_t lap_tables(Plan& p, bool last, std::vector<LapItem>* items, s
 static cudaError_t lap_upload(Plan& p, const std::vector<LapItem>& items, const std::vector<int>& first,
                               const std::vector<int>& ell, int64_t nk, double* Kt, size_t* scratch, cudaStream_t st) {
     p.n_lap_items = (int64_t)items.size();
-    const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items, p.prec == FL_FP64 ? 8 : 4);
+    const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items);
     *scratch = L.total + items.size() * sizeof(LapItem);
     cudaError_t e = cudaMalloc(&p.d_lap, L.total);
     unsigned char* base = (unsigned char*)p.d_lap;

@@ -1,5 +1,8 @@
-"""Planned Laplace transforms: infinite coefficients leave the results that do not
-depend on them finite and the others as the allocation-free call has them."""
+"""The FP32 form of planned Laplace transforms: no less accurate than its single
+rounding of the result and the barycentric form of the allocation-free call allow
+(relative 2-norms against the oracle at an eps where interpolation errs far
+less than float rounding), and infinite coefficients leave the results that do
+not depend on them finite and the others as the allocation-free call has them."""
 import numpy as np
 import pytest
 
@@ -34,6 +37,16 @@ def _both(fl, c, t, s, eps, prec="fp32"):
                                     fl._precision(prec), torch.cuda.current_stream().cuda_stream)
     fl.check(st, "noalloc")
     return a, f.cpu().numpy().astype(np.float64)
+
+
+@pytest.mark.parametrize("N,M", [(300, 5000), (1810, 8274), (2208, 4045), (20000, 5000), (200000, 3000)])
+def test_fp32_rounding(fl, N, M):
+    c, t, s = W.laplace_inputs(N, M, seed=N)
+    c = c.astype(np.float32).astype(np.float64)
+    ref = oracle.laplace_direct(c, t, s)
+    a, b = _both(fl, c, t, s, 1e-9)
+    ea, eb = (np.linalg.norm(x - ref) / np.linalg.norm(ref) for x in (a, b))
+    assert ea <= max(eb, 2.0 ** -25), (ea, eb)
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
