@@ -47,7 +47,9 @@ __global__ void k_classify(int64_t M, const double* __restrict__ w,
             if (band > 0 && n > 0) {
                 const double xs = xhalf ? 0.5 * x : x;   // exact
                 const double xr = xs - floor(xs);        // exact
-                cell = (uint32_t)floor(xr * (double)n);  // exact: n is a power of two
+                // exact: n is a power of two.  xr rounds to 1 for x just below an integer
+                // (-2^-54 < x - k < 0): cell 0, as its taps take it
+                cell = (uint32_t)floor(xr * (double)n) & (uint32_t)(n - 1);
             }
         }
         keys[j] = ((uint32_t)band << 25) | cell;

@@ -253,7 +253,7 @@ __global__ void k_node_tab(int64_t M, const double2* __restrict__ ws, const int3
     if (i >= M) return;
     const double2 wv = ws[i];
     const double x = wv.x - floor(wv.x);
-    const uint64_t X = (uint64_t)ldexp(x, 64);
+    const uint64_t X = x < 1.0 ? (uint64_t)ldexp(x, 64) : 0;   // (x rounds to 1 just below an integer)
     const BandDev B = bands[bandid[i]];
     float th = 0.f, tl = 0.f;
     if (B.route == 2) {
