@@ -77,23 +77,28 @@ __global__ void __launch_bounds__(256)
 
 template <typename T, int MW, bool XI>
 __global__ void __launch_bounds__(256)
-    k_node_tables(int64_t M, const double2* __restrict__ ws, const int32_t* __restrict__ bandid,
-                  const BandDev* __restrict__ bands, const double* __restrict__ cheb, int ldl, double kb_b,
-                  T* __restrict__ sp_phi, T* __restrict__ sp_L, C_t<T>* __restrict__ sp_e) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    k_node_taps(int64_t M, const double2* __restrict__ ws, const int32_t* __restrict__ bandid,
+                const BandDev* __restrict__ bands, double kb_b, T* __restrict__ sp_phi, C_t<T>* __restrict__ sp_e) {
+    const int64_t x0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // a thread per node and tap
+    const int64_t i = x0 / (2 * MW);
+    const int t = (int)(x0 - i * (2 * MW));
     if (i >= M) return;
-    const BandDev B = bands[bandid[i]];
+    const BandDev& B = bands[bandid[i]];
     if (B.route != 1) return;
-    const double2 wv = ws[i];
-    const double xs = XI ? 0.5 * wv.x : wv.x;
+    const double wx = ws[i].x;
+    const double xs = XI ? 0.5 * wx : wx;
     const double x = xs - floor(xs);
     const double t0 = (double)B.n * x;
     const double fr = t0 - floor(t0);
+    const double kb = XI ? kb_b : B.kb;
+    sp_phi[x0] = sizeof(T) == 8 ? T(kb_window_exact(fr, (double)(MW - 1 - t), (double)MW, kb))
+                                : T(kb_window<double>(fr + (double)(MW - 1 - t), (double)MW, kb));
+    if (t > 0) return;
     double2 e = {1.0, 0.0};
     if constexpr (XI) {
-        const double v = kTwoPiAdj * 0.5 * wv.x, arg = kb_b * kb_b - v * v;
+        const double v = kTwoPiAdj * 0.5 * wx, arg = kb_b * kb_b - v * v;
         const double i0 = cyl_bessel_i0((double)MW * sqrt(arg > 0.0 ? arg : 0.0));
-        e = cscale(expipi<double>(-2.0 * frac_turns(B.xc, wv.x)), 1.0 / (kPiAdj * i0));
+        e = cscale(expipi<double>(-2.0 * frac_turns(B.xc, wx)), 1.0 / (kPiAdj * i0));
     } else if (B.nsub == 0) {
         double ph = (double)(B.Nm >> 1) * x;   // N_m a power of two: exact
         ph -= floor(ph);
@@ -101,25 +106,43 @@ __global__ void __launch_bounds__(256)
         e = expipi<double>(-2.0 * ph);
     }
     sp_e[i] = C_t<T>{T(e.x), T(e.y)};
-    const double kb = XI ? kb_b : B.kb;
-#pragma unroll
-    for (int t = 0; t < 2 * MW; ++t)
-        sp_phi[i * (2 * MW) + t] = sizeof(T) == 8 ? T(kb_window_exact(fr, (double)(MW - 1 - t), (double)MW, kb))
-                                                  : T(kb_window<double>(fr + (double)(MW - 1 - t), (double)MW, kb));
-    if (B.nrhs == 1) return;
-    const double tau = (kTwoPiAdj * wv.y - B.yc) * B.yh_inv;
-    const int q = B.nrhs;
-    const double* ch = cheb + 2 * B.choff;
-    double den = 0.0;
+}
+
+// The weights, 2^lg lanes per node (at most 32): one division each, the sum of
+// the quotients by exchanges.  A thread per node took 78 us for 1024 nodes (q = 18),
+// nearly all of it the latency of its divisions and windows in turn.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_node_weights(int64_t M, int lg, const double2* __restrict__ ws, const int32_t* __restrict__ bandid,
+                   const BandDev* __restrict__ bands, const double* __restrict__ cheb, int ldl, T* __restrict__ sp_L) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> lg;
+    const int G = 1 << lg, lane = threadIdx.x & (G - 1);
+    const BandDev* B = i < M ? &bands[bandid[i]] : nullptr;
+    const int q = B && B->route == 1 && B->nrhs > 1 ? B->nrhs : 0;
+    const double* ch = q ? cheb + 2 * B->choff : cheb;
+    const double tau = q ? (kTwoPiAdj * ws[i].y - B->yc) * B->yh_inv : 0.0;
+    static_assert(kMaxQ <= 64, "two weights per lane");
+    double w[2] = {0.0, 0.0}, den = 0.0;
     int hit = -1;
-    for (int s = 0; s < q; ++s) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int s = lane + k * G;
+        if (s >= q) continue;
         const double d = tau - ch[s];
         if (d == 0.0) hit = s;
-        den += ch[q + s] / d;
+        w[k] = ch[q + s] / d;
+        den += w[k];
+    }
+    for (int off = G >> 1; off > 0; off >>= 1) {
+        den += __shfl_xor_sync(0xffffffffu, den, off);
+        hit = max(hit, __shfl_xor_sync(0xffffffffu, hit, off));
     }
     const double inv = 1.0 / den;
-    for (int s = 0; s < q; ++s)
-        sp_L[i * ldl + s] = T(hit >= 0 ? (s == hit ? 1.0 : 0.0) : ch[q + s] / (tau - ch[s]) * inv);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int s = lane + k * G;
+        if (s < q) sp_L[i * ldl + s] = T(hit >= 0 ? (s == hit ? 1.0 : 0.0) : w[k] * inv);
+    }
 }
 
 // rv_j = r_j e_j in sorted order.
@@ -424,9 +447,9 @@ __global__ void k_spread_starts(int total, const int4* __restrict__ groups, int 
     start[i] = adj_lower(cell, (int)B.node_off, (int)(B.node_off + B.nodes), i - groups[lo].z);
 }
 
-template <typename E> static cudaError_t adj_upload(const std::vector<E>& v, E** dev, cudaStream_t st) {
+template <typename E> static cudaError_t adj_upload(Plan& p, const std::vector<E>& v, E** dev, cudaStream_t st) {
     if (v.empty()) return cudaSuccess;
-    cudaError_t e = cudaMalloc((void**)dev, v.size() * sizeof(E));
+    cudaError_t e = p.pool.get(dev, (int64_t)v.size());
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(*dev, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice, st);
     return e;
@@ -470,38 +493,40 @@ cudaError_t build_spread(Plan& p, cudaStream_t st) {
         g.z = (int)nstart;
         nstart += p.bands[g.y].dev.n + 1;
     }
-    cudaError_t e = adj_upload(blocks, &p.d_sp_blocks, st);
-    if (e == cudaSuccess) e = adj_upload(groups, &p.d_dn_groups, st);
-    if (e == cudaSuccess) e = adj_upload(comb, &p.d_comb, st);
+    cudaError_t e = adj_upload(p, blocks, &p.d_sp_blocks, st);
+    if (e == cudaSuccess) e = adj_upload(p, groups, &p.d_dn_groups, st);
+    if (e == cudaSuccess) e = adj_upload(p, comb, &p.d_comb, st);
     if (e == cudaSuccess && nblocks > 0) {
-        e = cudaMalloc((void**)&p.d_sp_ranges, nblocks * sizeof(int4));
+        e = p.pool.bytes((void**)&p.d_sp_ranges, nblocks * sizeof(int4));
         if (e == cudaSuccess)
             k_spread_ranges<<<(unsigned)((nblocks + 255) / 256), 256, 0, st>>>(
                 (int)nblocks, p.d_sp_blocks, p.n_sp_bands, p.d_bands, p.d_cell, p.mw, p.d_sp_ranges);
     }
     if (e == cudaSuccess && nstart > 0) {
-        e = cudaMalloc((void**)&p.d_dn_start, nstart * sizeof(int32_t));
+        e = p.pool.bytes((void**)&p.d_dn_start, nstart * sizeof(int32_t));
         if (e == cudaSuccess)
             k_spread_starts<<<(unsigned)((nstart + 255) / 256), 256, 0, st>>>(
                 (int)nstart, p.d_dn_groups, (int)groups.size(), p.d_bands, p.d_cell, p.d_dn_start);
     }
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess && !comb.empty()) e = cudaStreamSynchronize(st);   // the host lists are released on return
-    return e;
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <typename T, int MW> static cudaError_t node_tables_t(Plan& p, cudaStream_t st) {
-    const unsigned grid = (unsigned)((p.M + 255) / 256);
     if constexpr (sizeof(T) == 4) {
         if (!p.xi_mode) {
-            k_node_tables_f32<MW><<<grid, 256, 0, st>>>(p.M, p.d_ntab, p.d_bandid, p.d_bands, p.d_cheb32, p.qmax,
-                                                        (T*)p.d_sp_phi, (T*)p.d_sp_L, (C_t<T>*)p.d_sp_e);
+            k_node_tables_f32<MW><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(
+                p.M, p.d_ntab, p.d_bandid, p.d_bands, p.d_cheb32, p.qmax, (T*)p.d_sp_phi, (T*)p.d_sp_L,
+                (C_t<T>*)p.d_sp_e);
             return cudaGetLastError();
         }
     }
-    auto kern = p.xi_mode ? k_node_tables<T, MW, true> : k_node_tables<T, MW, false>;
-    kern<<<grid, 256, 0, st>>>(p.M, p.d_ws, p.d_bandid, p.d_bands, p.d_cheb, p.qmax, p.kb_b, (T*)p.d_sp_phi,
-                               (T*)p.d_sp_L, (C_t<T>*)p.d_sp_e);
+    auto kern = p.xi_mode ? k_node_taps<T, MW, true> : k_node_taps<T, MW, false>;
+    kern<<<(unsigned)((p.M * 2 * MW + 255) / 256), 256, 0, st>>>(p.M, p.d_ws, p.d_bandid, p.d_bands, p.kb_b,
+                                                                  (T*)p.d_sp_phi, (C_t<T>*)p.d_sp_e);
+    int lg = 0;
+    while (lg < 5 && (1 << lg) < p.qmax) ++lg;
+    k_node_weights<T><<<(unsigned)(((p.M << lg) + 255) / 256), 256, 0, st>>>(p.M, lg, p.d_ws, p.d_bandid, p.d_bands,
+                                                                             p.d_cheb, p.qmax, (T*)p.d_sp_L);
     return cudaGetLastError();
 }
 

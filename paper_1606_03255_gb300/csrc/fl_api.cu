@@ -38,12 +38,7 @@ static fl_status cuda_fail(cudaError_t e, const char* where) {
 
 Plan::~Plan() {
     if (gexec) cudaGraphExecDestroy(gexec);
-    void* ptrs[] = {d_ws, d_perm, d_bandid, d_bands, d_small, d_pass, d_cheb, d_D, d_grid, d_Y,
-                    d_stage_c, d_stage_f, d_stage_r, d_z0, d_t, d_s, d_tband, d_sband, d_lap, d_direct,
-                    d_dranges, d_dpart, d_cdir, d_dsegs, d_dadj, d_dz, d_cell, d_sp_phi,
-                    d_sp_L, d_sp_rv, d_sp_e, d_sp_blocks, d_dn_groups, d_sp_ranges, d_dn_start, d_comb, d_lapK, d_lapKoff, d_tw, d_nearT, d_cheb32, d_cff, d_tperm, d_ts, d_tbs, d_ttau, d_stau, d_lapitems,
-                    d_xis, d_xperm, d_xbk, d_xstart, d_xwin, d_xiphi, d_xcs, d_xsb,
-                    d_frbs, d_fent, d_fphi, d_fpp, d_ntab, d_boff, d_bptr};
+    void* ptrs[] = {d_stage_c, d_stage_f, d_stage_r, d_boff, d_bptr};   // made by calls
     for (void* q : ptrs)
         if (q) cudaFree(q);
     for (Timer& t : timers) {
@@ -310,7 +305,7 @@ static void add_direct_band(Plan& p, const BandHost& bh) {
             return;
         }
     }
-    p.direct_segs.push_back({bh.node_off, bh.nodes, d.K, d.c_off, 0, (int)((d.K + kDirChunk - 1) / kDirChunk), pin});
+    p.direct_segs.push_back({bh.node_off, bh.nodes, d.K, d.c_off, 0, 0, (int)((d.K + kDirChunk - 1) / kDirChunk), pin});
 }
 
 // Work items of the direct segments.  Forward: the lanes per node G cover the
@@ -328,11 +323,13 @@ static void build_direct_items(Plan& p) {
     p.direct_work.clear();
     p.dadj_work.clear();
     p.direct_ranges.clear();
-    p.direct_nodes = p.dpart_elems = p.direct_kmax = 0;
+    p.direct_nodes = p.dpart_elems = p.direct_kmax = p.base_nodes = 0;
     int64_t lane_blocks = 0;
     for (DirectSeg& s : p.direct_segs) {
         lane_blocks += (s.nodes + np - 1) / np * ((s.K + kDirBlock - 1) / kDirBlock);
         p.direct_kmax = std::max(p.direct_kmax, s.K);
+        s.z_off = p.base_nodes - s.node_off;
+        if (s.pin == 0 || !p.batched) p.base_nodes += s.nodes;   // (single plans: the adjoint reads them)
         if (s.nchunk == 1) continue;
         s.dslot = p.dpart_elems;
         p.dpart_elems += s.nodes * s.nchunk;
@@ -390,10 +387,11 @@ static void build_direct_items(Plan& p) {
     adj_items(steps, true);
 }
 
+// (pageable host memory: copied to staging memory before the call returns)
 template <typename E>
-static cudaError_t upload(const std::vector<E>& v, E** dev, cudaStream_t st) {
+static cudaError_t upload(DevPool& pool, const std::vector<E>& v, E** dev, cudaStream_t st) {
     if (v.empty()) return cudaSuccess;
-    cudaError_t e = cudaMalloc((void**)dev, v.size() * sizeof(E));
+    cudaError_t e = pool.get(dev, (int64_t)v.size());
     if (e == cudaSuccess) e = cudaMemcpyAsync(*dev, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice, st);
     return e;
 }
@@ -516,8 +514,8 @@ static fl_status build_fused(Plan& p, cudaStream_t st) {
     }
     FusedBand* d_list = nullptr;
     int32_t* d_hist = nullptr;
-    cudaError_t e = upload(list, &d_list, st);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_hist, hist_len * sizeof(int32_t));
+    cudaError_t e = upload(p.scratch(), list, &d_list, st);
+    if (e == cudaSuccess) e = p.scratch().get(&d_hist, hist_len);
     std::vector<int32_t> hist(hist_len);
     if (e == cudaSuccess) e = launch_fused_entries(p, d_list, (int)list.size(), chunks, nrb_max, false, d_hist, st);
     if (e == cudaSuccess)
@@ -556,10 +554,10 @@ static fl_status build_fused(Plan& p, cudaStream_t st) {
         ++p.fused_bands;
     }
     p.fused_entries = ents;
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_frbs, rbs.size() * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_fent, ents * sizeof(int2));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_fphi, phis * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_fpp, pp * sizeof(float2));
+    if (e == cudaSuccess) e = p.pool.bytes((void**)&p.d_frbs, rbs.size() * sizeof(int32_t));
+    if (e == cudaSuccess) e = p.pool.bytes((void**)&p.d_fent, ents * sizeof(int2));
+    if (e == cudaSuccess) e = p.pool.bytes((void**)&p.d_fphi, phis * sizeof(float4));
+    if (e == cudaSuccess) e = p.pool.bytes((void**)&p.d_fpp, pp * sizeof(float2));
     if (e == cudaSuccess) e = cudaMemsetAsync(p.d_fphi, 0, phis * sizeof(float4), st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(p.d_frbs, rbs.data(), rbs.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st);
@@ -568,11 +566,6 @@ static fl_status build_fused(Plan& p, cudaStream_t st) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_list, list.data(), list.size() * sizeof(FusedBand), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = launch_fused_entries(p, d_list, (int)list.size(), chunks, nrb_max, true, d_hist, st);
-    // the host vectors and the lists are released on return
-    const cudaError_t es = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) e = es;
-    cudaFree(d_hist);
-    cudaFree(d_list);
     FL_CUDA(e, "fl_plan: fused gather entries");
     // slots beyond a node's parts are never written and must read as zero
     FL_CUDA(cudaMemsetAsync(p.d_fpp, 0, pp * sizeof(float2), st), "clear fused partials");
@@ -627,6 +620,31 @@ struct SplitChoice {
     int64_t Kp = 0, Nc = 0;
 };
 
+// The splits of a band of K frequencies that sigma >= smin and the gain limit
+// admit at window half-width mw: the same for every band of these, so they are
+// listed once per plan (merge_bands asks for hundreds of estimates).
+static const std::vector<SplitOption>& split_options(const Plan& p, int64_t K, double smin, int mw) {
+    const auto key = std::make_tuple(K, smin, mw);
+    const auto hit = p.split_memo.find(key);
+    if (hit != p.split_memo.end()) return hit->second;
+    std::vector<SplitOption>& v = p.split_memo[key];
+    const double gain_max = p.prec == FL_FP32 ? kMaxDeconvGain : deconv_gain_limit64(p.eps_A);
+    // (the window shape and gain are those of the candidate's own sigma)
+    for (int P = 2; P <= 9; ++P) {
+        const int64_t Kp = (K + P - 1) / P;
+        const int64_t Nc = Kp + (Kp & 1);
+        const int lg = ilog2_ceil((int64_t)ceil(smin * (double)Nc));
+        if (lg <= kSmallMaxLog2 || lg > kMaxLog2n) continue;
+        const int64_t n = (int64_t)1 << lg;
+        if ((double)n >= 2.0 * (double)Nc) continue;   // no gain over sigma = 2
+        // the half-width this sigma needs, and the FP32 limit at it
+        const int mc = std::max(mw, split_width(p, (double)n / (double)Nc));
+        if (deconv_gain((double)n / (double)Nc, mc) > gain_max) continue;
+        v.push_back({P, lg, mc, Kp, Nc});
+    }
+    return v;
+}
+
 // Best split of band bh at sigma_min >= smin with window half-width mw
 // (P = 1: unsplit); force: fewest grid points regardless of the gather.
 static SplitChoice best_split(const Plan& p, const BandHost& bh, double smin, int mw, bool force,
@@ -647,29 +665,19 @@ static SplitChoice best_split(const Plan& p, const BandHost& bh, double smin, in
     double bc = force ? (double)d.n : c1;
     const bool eligible = smin < 2.0 && four_step && !p.xi_mode && bh.nodes > 0 &&
                           (fusable || p.prec == FL_FP64);
-    const double gain_max = p.prec == FL_FP32 ? kMaxDeconvGain : deconv_gain_limit64(p.eps_A);
-    // (the window shape and gain are those of the candidate's own sigma)
     if (eligible) {
-        for (int P = 2; P <= 9; ++P) {
-            const int64_t Kp = (d.K + P - 1) / P;
-            const int64_t Nc = Kp + (Kp & 1);
-            const int lg = ilog2_ceil((int64_t)ceil(smin * (double)Nc));
-            if (lg <= kSmallMaxLog2 || lg > kMaxLog2n) continue;
-            const int64_t n = (int64_t)1 << lg;
-            if ((double)n >= 2.0 * (double)Nc) continue;   // no gain over sigma = 2
-            // the half-width this sigma needs, and the FP32 limit at it
-            const int mc = std::max(mw, split_width(p, (double)n / (double)Nc));
-            if (deconv_gain((double)n / (double)Nc, mc) > gain_max) continue;
-            const double gather = free32    ? free_gather_cost(bh.nodes, d.nrhs, n, lg, mc, fusable, &fz)
-                                  : fusable ? d.nrhs * fused_cost(bh.nodes, lg, mc)
-                                            : unfused_cost(bh.nodes, d.nrhs, mc);
-            const double c = force ? (double)P * n : P * (fft_cost(d.nrhs, n, lg) + gather);
+        for (const SplitOption& o : split_options(p, d.K, smin, mw)) {
+            const int64_t n = (int64_t)1 << o.log2n;
+            const double gather = free32    ? free_gather_cost(bh.nodes, d.nrhs, n, o.log2n, o.mc, fusable, &fz)
+                                  : fusable ? d.nrhs * fused_cost(bh.nodes, o.log2n, o.mc)
+                                            : unfused_cost(bh.nodes, d.nrhs, o.mc);
+            const double c = force ? (double)o.P * n : o.P * (fft_cost(d.nrhs, n, o.log2n) + gather);
             if (c < bc) {
                 bc = c;
-                best.P = P;
-                best.log2n = lg;
-                best.Kp = Kp;
-                best.Nc = Nc;
+                best.P = o.P;
+                best.log2n = o.log2n;
+                best.Kp = o.Kp;
+                best.Nc = o.Nc;
             }
         }
     }
@@ -765,31 +773,43 @@ static fl_status plan_splits(Plan& p, const std::vector<int>& nfft, cudaStream_t
 // largest over x in (0, xmax], sampled four to the octave over the top three
 // octaves (the bounds are unimodal in x, and the bands reach at most about that
 // far beyond the peak).
-static void interp_error(double a, double b, double xmax, double* err) {
-    constexpr int kTerms = 96, kSamples = 13;
+static void interp_error(double a, double b, double xmax, double tol, double* err) {
+    constexpr int kTerms = 96, kSamples = 13, kPad = 16;   // (padded: the loops over the samples are vectors)
+    constexpr double kQuarter[4] = {1.0, 0.84089641525371454, 0.70710678118654752, 0.59460355750136053};
     const double h = 0.5 * (b - a);
-    for (int q = 0; q <= kMaxQ; ++q) err[q] = 0.0;
-    for (int i = 0; i < kSamples; ++i) {
-        const double x = xmax * pow(2.0, -0.25 * i), z = h * x, iz = 2.0 / z;
-        // e^-z I_j(z) by backward recurrence, normalised by I_0 + 2 sum I_j = e^z
-        double v[kTerms + 2];
-        v[kTerms + 1] = 0.0;
-        v[kTerms] = 1e-280;
-        double sum = 2.0 * v[kTerms];
-        for (int j = kTerms; j > 0; --j) {
-            v[j - 1] = v[j + 1] + (j * iz) * v[j];
-            if (v[j - 1] > 1e250) {   // rescale
-                for (int t = j - 1; t <= kTerms; ++t) v[t] *= 1e-250;
-                sum *= 1e-250;
-            }
-            sum += (j > 1 ? 2.0 : 1.0) * v[j - 1];
+    // e^-z I_j(z) <= (z/2)^j / j!: the terms from J on are below tol 10^-8 together
+    int J = 1;
+    for (double t = 0.5 * h * xmax; J < kTerms && t > 1e-9 * tol; t *= 0.5 * h * xmax / ++J)
+        ;
+    double iz[kPad], scale[kPad], sum[kPad], p[kTerms + 2][kPad];
+    for (int i = 0; i < kPad; ++i) {
+        const int k = std::min(i, kSamples - 1);
+        const double x = ldexp(xmax * kQuarter[k & 3], -(k >> 2));
+        iz[i] = 2.0 / (h * x);
+        scale[i] = 4.0 * exp(-a * x);
+        sum[i] = p[0][i] = 1.0;
+        p[J + 1][i] = 0.0;
+    }
+    for (int j = J + 1; j <= kMaxQ; ++j) err[j] = 0.0;
+    // I_j(z) / I_{j-1}(z) backwards, then I_j / I_0 = their products, normalised by I_0 + 2 sum I_j = e^z
+    for (int j = J; j > 0; --j)
+        for (int i = 0; i < kPad; ++i) p[j][i] = 1.0 / (j * iz[i] + p[j + 1][i]);
+    for (int j = 1; j <= J; ++j)
+        for (int i = 0; i < kPad; ++i) {
+            p[j][i] *= p[j - 1][i];
+            sum[i] += 2.0 * p[j][i];
         }
-        const double scale = 4.0 * exp(-a * x) / sum;
-        double tail = 0.0;
-        for (int j = kTerms; j >= 0; --j) {
-            tail += v[j] * scale;
-            if (j <= kMaxQ) err[j] = std::max(err[j], tail);
+    for (int i = 0; i < kPad; ++i) {
+        scale[i] /= sum[i];
+        sum[i] = 0.0;                            // from here the tails
+    }
+    for (int j = J; j >= 0; --j) {
+        double most = 0.0;
+        for (int i = 0; i < kPad; ++i) {
+            sum[i] += p[j][i] * scale[i];
+            most = std::max(most, sum[i]);
         }
+        if (j <= kMaxQ) err[j] = most;
     }
 }
 
@@ -805,7 +825,7 @@ static int merged_rank(Plan& p, double a, int octaves, double xmax, double tol) 
     int r = kMaxQ + 1;
     if (0.5 * (b - 1.0) * xm <= 60.0) {
         double err[kMaxQ + 1];
-        interp_error(1.0, b, xm, err);
+        interp_error(1.0, b, xm, tol, err);
         r = 2;
         while (r <= kMaxQ && err[r] > tol) ++r;
     }
@@ -816,7 +836,7 @@ static int merged_rank(Plan& p, double a, int octaves, double xmax, double tol) 
 // Estimated cost of an NFFT band (the units of route_of), at its best split.
 static double nfft_cost(const Plan& p, const BandHost& bh) {
     double best = 0.0;
-    const bool split = p.sigma_mode != 1 && !p.xi_mode && p.prec != FL_FP64_FF;
+    const bool split = p.sigma_mode != 1 && !p.xi_mode && p.prec != FL_FP64_FF && bh.dev.log2n > kSmallMaxLog2;
     for (double smin : {2.0, 1.75, 1.5, 1.25}) {
         double c = 0.0;
         best_split(p, bh, smin, p.mw, false, &c);
@@ -846,7 +866,7 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
     double tol;
     {
         double err[kMaxQ + 1];   // the dyadic band at rank q, over every x
-        interp_error(1.0, 2.0, 64.0, err);
+        interp_error(1.0, 2.0, 64.0, 0.0, err);
         tol = err[p.q];
         // in double an error below half a unit of rounding is none (rank 22 at
         // eps = 1e-12 leaves 6e-18)
@@ -857,10 +877,11 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
         int from, rank;
     };
     std::vector<Part> best(n + 1, Part{0.0, 0, 0});
+    std::vector<int64_t> before(n + 1, 0);          // nodes of the candidates before
+    for (int t = 0; t < n; ++t) before[t + 1] = before[t] + p.bands[in.band_base + list[t]].nodes;
     auto merged = [&](int i, int j, int rank) {   // candidates list[i .. j] as one band
         BandHost g = p.bands[in.band_base + list[i]];
-        g.nodes = 0;
-        for (int t = i; t <= j; ++t) g.nodes += p.bands[in.band_base + list[t]].nodes;
+        g.nodes = before[j + 1] - before[i];
         const double a = ldexp(p.y1, -list[j]), b = ldexp(p.y1, 1 - list[i]);
         g.dev.nodes = g.nodes;
         g.dev.yc = 0.5 * (a + b);
@@ -869,15 +890,20 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
         g.dev.nrhs = rank;
         return g;
     };
+    std::vector<int> floor_rank(n, 2);               // known of the interval from candidate i on
     for (int j = 0; j < n; ++j) {
         const BandHost& alone = p.bands[in.band_base + list[j]];
         const double single = alone.dev.route == 2 ? (double)alone.nodes * alone.dev.K * 6.0 * p.direct_bias
                                                    : nfft_cost(p, alone);
         best[j + 1] = Part{best[j].cost + single, j, 0};
+        int least = 2;   // the rank grows with the interval: no less than those of parts of it
         for (int i = j; i >= 0; --i) {
             if (!merge_direct && p.bands[in.band_base + list[i]].dev.route == 2) break;
+            least = floor_rank[i] = std::max(floor_rank[i], least);
+            if (best[i].cost + nfft_cost(p, merged(i, j, least)) >= best[j + 1].cost) continue;   // not even at that rank
             const int r = merged_rank(p, ldexp(p.y1, -list[j]), list[j] - list[i] + 1, in.xi1, tol);
             if (r > kMaxQ) break;
+            least = floor_rank[i] = r;
             if (i == j && r >= p.q) continue;
             const double c = best[i].cost + nfft_cost(p, merged(i, j, r));
             if (c < best[j + 1].cost) best[j + 1] = Part{c, i, r};
@@ -907,7 +933,7 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
         p.bands[lead].dev.choff = off;
         p.qmax = std::max(p.qmax, r);
         if (i == j - 1) continue;   // one band at a lower rank: its nodes are in order
-        const cudaError_t e = launch_cell_sort(p, g.node_off, g.nodes, lead, st);
+        const cudaError_t e = launch_cell_sort(p, g.node_off, g.nodes, lead, g.dev.log2n, st);
         if (e != cudaSuccess) return cuda_fail(e, "fl_plan: merged bands");
     }
     return FL_OK;
@@ -945,38 +971,39 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     p.levels = p.inst[0].levels;
     p.xi1 = p.inst[0].xi1;
     int nb = (int)p.bands.size();
-    FL_CUDA(cudaMalloc((void**)&p.d_bands, nb * sizeof(BandDev)), "cudaMalloc bands");
+    const auto al = DevPool::rounded;
+    const int64_t nodes_all = moff;
+    const int64_t sort_hist = 256 * ((maxM + 2047) / 2048);   // radix-sort tiles of 2048
+    const size_t sort_bytes = 5 * al(maxM * 4) + al(maxM * sizeof(double2)) + al(sort_hist * 4) +
+                              al(nb * sizeof(int64_t)) + al(sizeof(int));
+    p.small = nodes_all <= kSmallPlan;
+    FL_CUDA(p.pool.reserve(al(nb * sizeof(BandDev)) + al(16) + al(nodes_all * sizeof(double2)) + 3 * al(nodes_all * 4) +
+                           (p.small ? sort_bytes + ((size_t)1 << 17) : 0)),
+            "cudaMalloc nodes");
+    FL_CUDA(p.pool.bytes((void**)&p.d_bands, nb * sizeof(BandDev)), "cudaMalloc bands");
     std::vector<BandDev> hb(nb);
     for (int b = 0; b < nb; ++b) hb[b] = p.bands[b].dev;
     FL_CUDA(cudaMemcpyAsync(p.d_bands, hb.data(), nb * sizeof(BandDev), cudaMemcpyHostToDevice, st),
             "copy bands");
-    FL_CUDA(cudaMalloc(&p.d_z0, 2 * sizeof(double)), "cudaMalloc z0");
+    FL_CUDA(p.pool.bytes(&p.d_z0, 2 * sizeof(double)), "cudaMalloc z0");
 
     // classify and sort the nodes of every transform into its slice
     const int64_t M = p.M;
     std::vector<int64_t> counts(nb, 0);
     if (M > 0) {
-        FL_CUDA(cudaMalloc((void**)&p.d_ws, M * sizeof(double2)), "cudaMalloc nodes");
-        FL_CUDA(cudaMalloc((void**)&p.d_perm, M * sizeof(int32_t)), "cudaMalloc perm");
-        FL_CUDA(cudaMalloc((void**)&p.d_bandid, M * sizeof(int32_t)), "cudaMalloc band ids");
-        FL_CUDA(cudaMalloc((void**)&p.d_cell, M * sizeof(int32_t)), "cudaMalloc cells");
-        uint32_t *keys = nullptr, *keys2 = nullptr, *hist = nullptr;
-        int32_t *vals = nullptr, *vals2 = nullptr;
+        FL_CUDA(p.pool.bytes((void**)&p.d_ws, M * sizeof(double2)), "cudaMalloc nodes");
+        FL_CUDA(p.pool.bytes((void**)&p.d_perm, M * sizeof(int32_t)), "cudaMalloc perm");
+        FL_CUDA(p.pool.bytes((void**)&p.d_bandid, M * sizeof(int32_t)), "cudaMalloc band ids");
+        FL_CUDA(p.pool.bytes((void**)&p.d_cell, M * sizeof(int32_t)), "cudaMalloc cells");
+        SortScratch& ss = p.sort;
         int64_t* dcount = nullptr;
         int* dflag = nullptr;
-        const int64_t nblk = (maxM + 2047) / 2048;
-        cudaError_t e = cudaSuccess;
-        auto cleanup = [&]() {
-            cudaFree(keys); cudaFree(keys2); cudaFree(hist); cudaFree(vals); cudaFree(vals2);
-            cudaFree(dcount); cudaFree(dflag);
-        };
-        if ((e = cudaMalloc((void**)&keys, maxM * 4)) == cudaSuccess &&
-            (e = cudaMalloc((void**)&keys2, maxM * 4)) == cudaSuccess &&
-            (e = cudaMalloc((void**)&vals, maxM * 4)) == cudaSuccess &&
-            (e = cudaMalloc((void**)&vals2, maxM * 4)) == cudaSuccess &&
-            (e = cudaMalloc((void**)&hist, 256 * nblk * 4)) == cudaSuccess &&
-            (e = cudaMalloc((void**)&dcount, nb * sizeof(int64_t))) == cudaSuccess &&
-            (e = cudaMalloc((void**)&dflag, sizeof(int))) == cudaSuccess &&
+        cudaError_t e = p.scratch().reserve(sort_bytes);
+        if (e == cudaSuccess && (e = p.scratch().get(&ss.keys, maxM)) == cudaSuccess &&
+            (e = p.scratch().get(&ss.keys2, maxM)) == cudaSuccess && (e = p.scratch().get(&ss.vals, maxM)) == cudaSuccess &&
+            (e = p.scratch().get(&ss.vals2, maxM)) == cudaSuccess && (e = p.scratch().get(&ss.perm, maxM)) == cudaSuccess &&
+            (e = p.scratch().get(&ss.ws, maxM)) == cudaSuccess && (e = p.scratch().get(&ss.hist, sort_hist)) == cudaSuccess &&
+            (e = p.scratch().get(&dcount, nb)) == cudaSuccess && (e = p.scratch().get(&dflag, 1)) == cudaSuccess &&
             (e = cudaMemsetAsync(dcount, 0, nb * sizeof(int64_t), st)) == cudaSuccess &&
             (e = cudaMemsetAsync(dflag, 0, sizeof(int), st)) == cudaSuccess) {
             for (int i = 0; i < B && e == cudaSuccess; ++i) {
@@ -985,22 +1012,19 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
                     e = launch_copy_sorted(p, in, p.inst[in.twin], st);
                     continue;
                 }
-                if ((e = launch_classify(p, in, nodes, keys, vals, dcount, dflag, st)) == cudaSuccess &&
-                    (e = radix_sort_pairs(keys, vals, keys2, vals2, hist, in.M, 32, st)) == cudaSuccess)
-                    e = launch_permute(p, in, nodes, keys, vals, st);
+                if ((e = launch_classify(p, in, nodes, ss.keys, ss.vals, dcount, dflag, st)) == cudaSuccess &&
+                    (e = radix_sort_pairs(ss.keys, ss.vals, ss.keys2, ss.vals2, ss.hist, in.M, 32, st)) == cudaSuccess)
+                    e = launch_permute(p, in, nodes, ss.keys, ss.vals, st);
             }
             int flag = 0;
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(counts.data(), dcount, nb * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, dflag, sizeof(int), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e == cudaSuccess && flag) {
-                cleanup();
+            if (e == cudaSuccess && flag)
                 return fail(FL_EINVAL, p.xi_mode ? "fl_plan_xi: a node has Im w < 0, a non-finite part or |Re w| > 1/2"
                                                  : "fl_plan: a node has Im w < 0 or a non-finite part");
-            }
         }
-        cleanup();
         if (e != cudaSuccess) return cuda_fail(e, "fl_plan: node classification");
         for (const Instance& in : p.inst)
             if (in.twin >= 0)
@@ -1053,6 +1077,10 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
             if (d.route == 1) nfft_bands.push_back(b);
         }
     }
+    if (M > kTmpKeep) {   // large: planning's scratch given back before the grids are allocated
+        FL_CUDA(cudaStreamSynchronize(st), "fl_plan: synchronise");
+        p.tmp.release();
+    }
     // oversampling from the tolerance: split sparse bands into sub-bands
     if ((s = plan_splits(p, nfft_bands, st)) != FL_OK) return s;
     // a transform that copies its twin's nodes shares its twin's weight tables
@@ -1097,78 +1125,99 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     build_pass_groups(p);
     if ((s = build_fused(p, st)) != FL_OK) return s;
     if ((int)p.bands.size() != nb) {   // sub-bands were appended: a larger table
-        FL_CUDA(cudaStreamSynchronize(st), "fl_plan: synchronise");
-        FL_CUDA(cudaFree(p.d_bands), "cudaFree bands");
-        p.d_bands = nullptr;
         nb = (int)p.bands.size();
         hb.resize(nb);
-        FL_CUDA(cudaMalloc((void**)&p.d_bands, nb * sizeof(BandDev)), "cudaMalloc bands");
+        FL_CUDA(p.pool.bytes((void**)&p.d_bands, nb * sizeof(BandDev)), "cudaMalloc bands");
     }
     for (int b = 0; b < nb; ++b) hb[b] = p.bands[b].dev;
     FL_CUDA(cudaMemcpyAsync(p.d_bands, hb.data(), nb * sizeof(BandDev), cudaMemcpyHostToDevice, st),
             "copy bands");
+    const size_t cs = p.prec != FL_FP32 ? 16 : 8, rs = cs / 2;   // complex128 I/O for FP64 and float pairs
+    {   // one block for what follows (128 KiB of it for lists that are not known yet)
+        size_t n = (size_t)1 << 17;
+        auto add = [&](bool on, int64_t count, size_t size) { n += on ? al((size_t)count * size) : 0; };
+        const bool node_tables = !p.batched && !(p.small_work.empty() && p.large_bands.empty());
+        add(true, (int64_t)p.small_work.size(), sizeof(SmallWork));
+        add(true, (int64_t)p.pass_items.size(), sizeof(PassItem));
+        add(true, (int64_t)(p.direct_work.size() + p.dadj_work.size()), sizeof(DirectItem));
+        add(p.prec == FL_FP32 && !p.xi_mode, M, sizeof(uint4));
+        add(true, p.dpart_elems, cs);
+        add(!p.dadj_work.empty(), p.N, cs);
+        add(true, 2 * p.base_nodes, cs);
+        add(node_tables, M * 2 * p.mw, rs);
+        add(node_tables, M * p.qmax, rs);
+        add(node_tables, M, cs);
+        add(node_tables, M, cs);
+        add(true, p.grid_elems, cs);
+        add(true, p.D_elems, rs);
+        add(true, p.Y_elems, cs);
+        add(!p.small_work.empty() || p.Y_elems > 0, kTwEntries + 8192, cs);
+        add(p.prec == FL_FP64_FF, p.N, sizeof(ffc));
+        if (n > ((size_t)1 << 18) && n < kOneBlock) FL_CUDA(p.pool.reserve(n), "cudaMalloc tables and grids");
+    }
     if (p.prec == FL_FP32 && !p.xi_mode && p.M > 0) {
-        FL_CUDA(cudaMalloc((void**)&p.d_ntab, p.M * sizeof(uint4)), "cudaMalloc node records");
+        FL_CUDA(p.pool.bytes((void**)&p.d_ntab, p.M * sizeof(uint4)), "cudaMalloc node records");
         FL_CUDA(build_node_table(p, st), "fl_plan: node records");
     }
-    // complex128 I/O for FP64 and float pairs; real tables double or float pairs
-    const size_t cs = p.prec != FL_FP32 ? 16 : 8, rs = cs / 2;
     if (!p.small_work.empty()) {
-        FL_CUDA(cudaMalloc((void**)&p.d_small, p.small_work.size() * sizeof(SmallWork)), "cudaMalloc work");
+        FL_CUDA(p.pool.bytes((void**)&p.d_small, p.small_work.size() * sizeof(SmallWork)), "cudaMalloc work");
         FL_CUDA(cudaMemcpyAsync(p.d_small, p.small_work.data(), p.small_work.size() * sizeof(SmallWork),
                                 cudaMemcpyHostToDevice, st),
                 "copy work");
     }
     if (!p.pass_items.empty()) {
-        FL_CUDA(cudaMalloc((void**)&p.d_pass, p.pass_items.size() * sizeof(PassItem)), "cudaMalloc pass items");
+        FL_CUDA(p.pool.bytes((void**)&p.d_pass, p.pass_items.size() * sizeof(PassItem)), "cudaMalloc pass items");
         FL_CUDA(cudaMemcpyAsync(p.d_pass, p.pass_items.data(), p.pass_items.size() * sizeof(PassItem),
                                 cudaMemcpyHostToDevice, st),
                 "copy pass items");
     }
     if (!p.direct_work.empty()) {
-        FL_CUDA(upload(p.direct_segs, &p.d_dsegs, st), "fl_plan: direct segments");
-        FL_CUDA(upload(p.direct_work, &p.d_direct, st), "fl_plan: direct work");
-        FL_CUDA(upload(p.direct_ranges, &p.d_dranges, st), "fl_plan: direct ranges");
-        FL_CUDA(upload(p.dadj_work, &p.d_dadj, st), "fl_plan: adjoint work");
-        if (p.dpart_elems > 0) FL_CUDA(cudaMalloc(&p.d_dpart, p.dpart_elems * cs), "cudaMalloc direct partials");
-        if (!p.dadj_work.empty()) FL_CUDA(cudaMalloc(&p.d_cdir, p.N * cs), "cudaMalloc direct adjoint");
-        FL_CUDA(cudaMalloc(&p.d_dz, 2 * M * cs), "cudaMalloc direct bases");
-        FL_CUDA(build_direct_base(p, st), "fl_plan: direct bases");
+        FL_CUDA(upload(p.pool, p.direct_segs, &p.d_dsegs, st), "fl_plan: direct segments");
+        FL_CUDA(upload(p.pool, p.direct_work, &p.d_direct, st), "fl_plan: direct work");
+        FL_CUDA(upload(p.pool, p.direct_ranges, &p.d_dranges, st), "fl_plan: direct ranges");
+        FL_CUDA(upload(p.pool, p.dadj_work, &p.d_dadj, st), "fl_plan: adjoint work");
+        if (p.dpart_elems > 0) FL_CUDA(p.pool.bytes(&p.d_dpart, p.dpart_elems * cs), "cudaMalloc direct partials");
+        if (!p.dadj_work.empty()) FL_CUDA(p.pool.bytes(&p.d_cdir, p.N * cs), "cudaMalloc direct adjoint");
+        if (p.base_nodes > 0) {
+            FL_CUDA(p.pool.bytes(&p.d_dz, 2 * p.base_nodes * cs), "cudaMalloc direct bases");
+            FL_CUDA(build_direct_base(p, st), "fl_plan: direct bases");
+        }
     }
     // adjoint of the NFFT bands (single plans): per-node taps and weights, cell lists
     if (!p.batched && M > 0) {
         FL_CUDA(build_spread(p, st), "fl_plan: adjoint lists");
         if (p.n_sp_blocks + p.n_dn_groups[0] + p.n_dn_groups[1] > 0) {
-            FL_CUDA(cudaMalloc(&p.d_sp_phi, (size_t)M * 2 * p.mw * rs), "cudaMalloc adjoint taps");
-            FL_CUDA(cudaMalloc(&p.d_sp_L, (size_t)M * p.qmax * rs), "cudaMalloc adjoint weights");
-            FL_CUDA(cudaMalloc(&p.d_sp_e, (size_t)M * cs), "cudaMalloc adjoint shifts");
-            FL_CUDA(cudaMalloc(&p.d_sp_rv, (size_t)M * cs), "cudaMalloc adjoint residuals");
+            FL_CUDA(p.pool.bytes(&p.d_sp_phi, (size_t)M * 2 * p.mw * rs), "cudaMalloc adjoint taps");
+            FL_CUDA(p.pool.bytes(&p.d_sp_L, (size_t)M * p.qmax * rs), "cudaMalloc adjoint weights");
+            FL_CUDA(p.pool.bytes(&p.d_sp_e, (size_t)M * cs), "cudaMalloc adjoint shifts");
+            FL_CUDA(p.pool.bytes(&p.d_sp_rv, (size_t)M * cs), "cudaMalloc adjoint residuals");
         }
     }
-    if (p.grid_elems) FL_CUDA(cudaMalloc(&p.d_grid, p.grid_elems * cs), "cudaMalloc grids");
-    if (p.D_elems) FL_CUDA(cudaMalloc(&p.d_D, p.D_elems * rs), "cudaMalloc weights");
+    if (p.grid_elems) FL_CUDA(p.pool.bytes(&p.d_grid, p.grid_elems * cs), "cudaMalloc grids");
+    if (p.D_elems) FL_CUDA(p.pool.bytes(&p.d_D, p.D_elems * rs), "cudaMalloc weights");
     if (p.D_elems && p.xi_mode)   // the padding of the exponent-major rows
         FL_CUDA(cudaMemsetAsync(p.d_D, 0, p.D_elems * rs, st), "clear weights");
-    if (p.Y_elems) FL_CUDA(cudaMalloc(&p.d_Y, p.Y_elems * cs), "cudaMalloc intermediate");
+    if (p.Y_elems) FL_CUDA(p.pool.bytes(&p.d_Y, p.Y_elems * cs), "cudaMalloc intermediate");
     if (p.Y_elems || !p.small_work.empty()) {   // stage twiddles of the passes and the small FFTs
-        FL_CUDA(cudaMalloc(&p.d_tw, (size_t)(kTwEntries + (p.prec != FL_FP32 ? 8192 : 0)) * cs),
+        FL_CUDA(p.pool.bytes(&p.d_tw, (size_t)(kTwEntries + (p.prec != FL_FP32 ? 8192 : 0)) * cs),
                 "cudaMalloc twiddles");
         FL_CUDA(build_twiddles(p, st), "fl_plan: twiddles");
     }
     if (p.prec == FL_FP64_FF)
-        FL_CUDA(cudaMalloc(&p.d_cff, (size_t)p.N * sizeof(ffc)), "cudaMalloc float-pair coefficients");
+        FL_CUDA(p.pool.bytes(&p.d_cff, (size_t)p.N * sizeof(ffc)), "cudaMalloc float-pair coefficients");
     int cheb_len = 0;
     for (int r : p.ranks) cheb_len += r;
-    FL_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * cheb_len * sizeof(double)), "cudaMalloc cheb");
-    FL_CUDA(cudaMalloc((void**)&p.d_cheb32, 4 * cheb_len * sizeof(float)), "cudaMalloc cheb32");
+    FL_CUDA(p.pool.bytes((void**)&p.d_cheb, 2 * cheb_len * sizeof(double)), "cudaMalloc cheb");
+    FL_CUDA(p.pool.bytes((void**)&p.d_cheb32, 4 * cheb_len * sizeof(float)), "cudaMalloc cheb32");
     FL_CUDA(build_cheb(p, st), "fl_plan: tables");
     if (p.d_sp_phi) FL_CUDA(build_node_weights(p, st), "fl_plan: node weights");
     for (int i = 0; i < B; ++i)
         if (!shares_D[i]) FL_CUDA(build_tables(p, p.inst[i], st), "fl_plan: tables");
     FL_CUDA(cudaStreamSynchronize(st), "fl_plan: synchronise");
+    p.tmp.release();
     p.scratch_bytes = (double)p.grid_elems * cs + (double)p.D_elems * rs + (double)p.Y_elems * cs +
                       (double)M * (sizeof(double2) + 8) + (double)p.dpart_elems * cs +
-                      (p.direct_work.empty() ? 0.0 : 2.0 * M * cs + (double)(p.dadj_work.empty() ? 0 : p.N) * cs);
+                      (p.direct_work.empty() ? 0.0 : 2.0 * p.base_nodes * cs + (double)(p.dadj_work.empty() ? 0 : p.N) * cs);
     // algorithmic bytes of one execute: c once, D once, each grid written and read
     // once per FFT pass, the nodes, and f
     double mb = (double)p.N * cs + (double)p.D_elems * rs + (double)M * (sizeof(double2) + 8 + cs);
@@ -1685,8 +1734,8 @@ fl_status fl_plan_xi(fl_plan_t* out, int64_t N, const double* xi_dev, int64_t M,
         delete h;
         return s;
     };
-    cudaError_t e = cudaMalloc((void**)&p.d_xis, N * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_xperm, N * sizeof(int32_t));
+    cudaError_t e = p.pool.bytes((void**)&p.d_xis, N * sizeof(double));
+    if (e == cudaSuccess) e = p.pool.bytes((void**)&p.d_xperm, N * sizeof(int32_t));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(p.d_xis, p.h_xis.data(), N * sizeof(double), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)

@@ -119,21 +119,25 @@ __device__ __forceinline__ float2 dir_f32_base(const DirF32Node& d) {
     return cscale(expipi<float>(2.f * xr), expf(-d.yh));
 }
 
-// Plan time: z_j and z_j^8 of the nodes of every segment (entries 2 i and 2 i + 1
-// of node i), formed in double and rounded once.
+// Plan time: z_j and z_j^8 (entries 2 t and 2 t + 1 of the t-th node with a base),
+// formed in double and rounded once.
 template <typename A> __device__ __forceinline__ C_t<A> dir_round(double2 v) { return {A(v.x), A(v.y)}; }
 template <typename A>
-__global__ void k_dir_base(const DirectSeg* __restrict__ segs, const double2* __restrict__ ws,
-                           C_t<A>* __restrict__ z) {
-    const DirectSeg S = segs[blockIdx.y];
+__global__ void k_dir_base(int64_t total, const DirectSeg* __restrict__ segs, int nsegs,
+                           const double2* __restrict__ ws, C_t<A>* __restrict__ z) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= S.nodes) return;
-    const int64_t i = S.node_off + t;
-    const DirNode<double> n = dir_node<double>(ws, nullptr, i);
+    if (t >= total) return;
+    int lo = 0, hi = nsegs;                      // last segment whose first base is <= t
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (segs[mid].node_off + segs[mid].z_off <= t) lo = mid;
+        else hi = mid;
+    }
+    const DirNode<double> n = dir_node<double>(ws, nullptr, t - segs[lo].z_off);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
         const double k = e ? 8.0 : 1.0;
-        z[2 * i + e] = dir_round<A>(cscale(expipi<double>(2.0 * frac_turns(k, n.x)), exp(-n.y * k)));
+        z[2 * t + e] = dir_round<A>(cscale(expipi<double>(2.0 * frac_turns(k, n.x)), exp(-n.y * k)));
     }
 }
 
@@ -258,8 +262,9 @@ __global__ void __launch_bounds__(256)
             if (S.pin) {
                 z = dir_pair(dir_f32_base(na.d), dir_f32_base(nb.d));
             } else {
-                z = dir_pair(zb[2 * i], zb[2 * i1]);
-                z8 = dir_pair(zb[2 * i + 1], zb[2 * i1 + 1]);
+                const C *za = zb + 2 * (i + S.z_off), *zc = zb + 2 * (i1 + S.z_off);
+                z = dir_pair(za[0], zc[0]);
+                z8 = dir_pair(za[1], zc[1]);
             }
             const f2 nz = f2_make(-f2_lo(z.y), -f2_hi(z.y)), nz8 = f2_make(-f2_lo(z8.y), -f2_hi(z8.y));
             f2c acc = {f2_dup(0.f), f2_dup(0.f)};
@@ -308,7 +313,7 @@ __global__ void __launch_bounds__(256)
         } else {
             const DirNode<A> nd = dir_node<A>(ws, ntab, i);
             C acc = dir_zero<C>();
-            const C z = zb[2 * i], z8 = zb[2 * i + 1];
+            const C z = zb[2 * (i + S.z_off)], z8 = zb[2 * (i + S.z_off) + 1];
             for (int b = sub; on && b < nblk; b += G) {
                 C zk;
                 if (!dir_power<1>(nd, k0 + b * kDirBlock, &zk)) break;
@@ -386,6 +391,7 @@ __global__ void __launch_bounds__(32)
     const DirectItem it = items[blockIdx.x];
     const DirectSeg S = segs[it.seg];
     const int lane = threadIdx.x, lkb = it.lg, g = lane >> lkb, G = 32 >> lkb;
+    zb += 2 * S.z_off;
     const int64_t k0 = (int64_t)it.chunk * (32 * kAdjKL) + (int64_t)(lane & ((1 << lkb) - 1)) * kAdjKL;
     const bool active = k0 < S.K;
     C acc[kAdjKL];
@@ -463,12 +469,8 @@ __global__ void __launch_bounds__(32)
 
 template <typename A>
 static cudaError_t dir_base_t(Plan& p, cudaStream_t st) {
-    int64_t most = 0;
-    for (const DirectSeg& s : p.direct_segs) most = std::max(most, s.nodes);
-    const int64_t ns = (int64_t)p.direct_segs.size();
-    for (int64_t s0 = 0; s0 < ns; s0 += 65535)   // gridDim.y
-        k_dir_base<A><<<dim3((unsigned)((most + 255) / 256), (unsigned)std::min<int64_t>(65535, ns - s0)), 256, 0,
-                        st>>>(p.d_dsegs + s0, p.d_ws, (C_t<A>*)p.d_dz);
+    k_dir_base<A><<<(unsigned)((p.base_nodes + 255) / 256), 256, 0, st>>>(
+        p.base_nodes, p.d_dsegs, (int)p.direct_segs.size(), p.d_ws, (C_t<A>*)p.d_dz);
     return cudaGetLastError();
 }
 

@@ -277,13 +277,16 @@ template <typename T> using LapTau = typename lap_tau<T>::type;
 template <typename T>
 __global__ void k_lap_tau(int64_t n, const double* __restrict__ v, const uint8_t* __restrict__ band,
                           double v1, int levels, LapTau<T>* __restrict__ tau) {
+    __shared__ double inv[FL_MAX_LEVELS + 1];            // 2 / a of every band
+    for (int l = threadIdx.x; l < levels; l += blockDim.x) inv[l] = 1.0 / (0.5 * ldexp(v1, -l));
+    __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int l = band[i];
     double x = 0.0;
-    if (l < levels) {
-        const double a = ldexp(v1, -l);
-        x = (v[i] - 1.5 * a) / (0.5 * a);
+    if (l < levels) {   // the quotient by its reciprocal, corrected once
+        const double a = ldexp(v1, -l), h = 0.5 * a, d = v[i] - 1.5 * a, r = inv[l], q = d * r;
+        x = r > 1e-280 && r < 1e280 ? fma(fma(-q, h, d), r, q) : d / h;
     }
     tau[i] = LapTau<T>(x);
 }
@@ -926,30 +929,23 @@ static cudaError_t sort_t_by_band(Plan& p, cudaStream_t st) {
     const int64_t n = p.N;
     uint32_t *keys = nullptr, *ktmp = nullptr, *hist = nullptr;
     int32_t *vals = nullptr, *vtmp = nullptr;
-    double* ts = nullptr;
-    uint8_t* bs = nullptr;
     const int64_t nblocks = (n + 2047) / 2048;        // radix-sort tiles of 256 x 8
-    cudaError_t e = cudaMalloc((void**)&keys, n * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&ktmp, n * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&vals, n * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&vtmp, n * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&hist, 256 * nblocks * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_ts, n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_tbs, n);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p.d_tperm, n * sizeof(int32_t));
-    ts = p.d_ts;
-    bs = p.d_tbs;
-    if (e == cudaSuccess) {
-        k_lap_sortprep<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, p.d_tband, keys, vals);
-        e = radix_sort_pairs(keys, vals, ktmp, vtmp, hist, n, 8, st);
-    }
-    if (e == cudaSuccess) {
-        k_lap_sorted<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, p.d_t, keys, vals, ts, bs, p.d_tperm);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    for (void* ptr : {(void*)keys, (void*)ktmp, (void*)vals, (void*)vtmp, (void*)hist}) cudaFree(ptr);
-    return e;   // on failure the plan's destructor frees what was allocated
+    const auto al = DevPool::rounded;
+    cudaError_t e = p.scratch().reserve(4 * al(4 * n) + al(1024 * nblocks) + al(8 * n) + al(n));
+    if (e == cudaSuccess) e = p.scratch().get(&keys, n);
+    if (e == cudaSuccess) e = p.scratch().get(&ktmp, n);
+    if (e == cudaSuccess) e = p.scratch().get(&vals, n);
+    if (e == cudaSuccess) e = p.scratch().get(&vtmp, n);
+    if (e == cudaSuccess) e = p.scratch().get(&hist, 256 * nblocks);
+    if (e == cudaSuccess) e = p.scratch().get(&p.d_ts, n);
+    if (e == cudaSuccess) e = p.scratch().get(&p.d_tbs, n);
+    if (e == cudaSuccess) e = p.pool.get(&p.d_tperm, n);
+    if (e != cudaSuccess) return e;
+    k_lap_sortprep<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, p.d_tband, keys, vals);
+    e = radix_sort_pairs(keys, vals, ktmp, vtmp, hist, n, 8, st);
+    if (e != cudaSuccess) return e;
+    k_lap_sorted<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, p.d_t, keys, vals, p.d_ts, p.d_tbs, p.d_tperm);
+    return cudaGetLastError();
 }
 
 // Plan time, after sort_t_by_band: tau of the t_k in band order and of the s_j,
@@ -957,7 +953,7 @@ static cudaError_t sort_t_by_band(Plan& p, cudaStream_t st) {
 // the launch has about four items per SM up to E = kLapMaxPer (N = 2^16: 256
 // items of 256 elements, which the FP64 pipes of all SMs share; longer runs
 // only pay once that many items are there).  last: whether the last band is
-// summed too.  The sorted copies of the t_k are released.
+// summed too.
 template <typename T>
 static cudaError_t lap_tables(Plan& p, bool last, std::vector<LapItem>* items, std::vector<int>* first,
                               cudaStream_t st) {
@@ -965,16 +961,16 @@ static cudaError_t lap_tables(Plan& p, bool last, std::vector<LapItem>* items, s
     first->assign(p.levels + 2, 0);
     cudaError_t e = cudaSuccess;
     if (p.M > 0) {
-        e = cudaMalloc(&p.d_stau, p.M * sizeof(LapTau<T>));
+        e = p.pool.bytes(&p.d_stau, p.M * sizeof(LapTau<T>));
         if (e != cudaSuccess) return e;
         k_lap_tau<T><<<(unsigned)((p.M + 255) / 256), 256, 0, st>>>(p.M, p.d_s, p.d_sband, p.y1, p.levels,
                                                                     (LapTau<T>*)p.d_stau);
     }
     if (p.N == 0) return cudaGetLastError();
-    e = cudaMalloc(&p.d_ttau, p.N * sizeof(LapTau<T>));
+    e = p.pool.bytes(&p.d_ttau, p.N * sizeof(LapTau<T>));
     int64_t* d_first = nullptr;
     std::vector<int64_t> start(p.levels + 2);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_first, start.size() * sizeof(int64_t));
+    if (e == cudaSuccess) e = p.scratch().get(&d_first, (int64_t)start.size());
     if (e == cudaSuccess) {
         k_lap_tau<T><<<(unsigned)((p.N + 255) / 256), 256, 0, st>>>(p.N, p.d_ts, p.d_tbs, p.xi1, p.levels,
                                                                     (LapTau<T>*)p.d_ttau);
@@ -984,12 +980,8 @@ static cudaError_t lap_tables(Plan& p, bool last, std::vector<LapItem>* items, s
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(start.data(), d_first, start.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(d_first);
     if (e != cudaSuccess) return e;
-    cudaFree(p.d_ts);
-    cudaFree(p.d_tbs);
-    p.d_ts = nullptr;
-    p.d_tbs = nullptr;
+    if (p.N > kTmpKeep) p.tmp.release();   // (all of it has been used)
     const int64_t per = std::min<int64_t>(kLapMaxPer, std::max<int64_t>(1, p.N / (kLapThreads * 4 * 152)));
     for (int l = 1; l <= p.levels; ++l) {
         (*first)[l] = (int)items->size();
@@ -1008,14 +1000,14 @@ static cudaError_t lap_upload(Plan& p, const std::vector<LapItem>& items, const 
     p.n_lap_items = (int64_t)items.size();
     const LapPlanLayout L = lap_plan_layout(p.levels, p.q, p.n_lap_items);
     *scratch = L.total + items.size() * sizeof(LapItem);
-    cudaError_t e = cudaMalloc(&p.d_lap, L.total);
+    cudaError_t e = p.pool.bytes(&p.d_lap, L.total);
     unsigned char* base = (unsigned char*)p.d_lap;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(base + L.first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !ell.empty())
         e = cudaMemcpyAsync(base + L.ell, ell.data(), ell.size() * sizeof(int), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !items.empty()) {
-        e = cudaMalloc(&p.d_lapitems, items.size() * sizeof(LapItem));
+        e = p.pool.bytes(&p.d_lapitems, items.size() * sizeof(LapItem));
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(p.d_lapitems, items.data(), items.size() * sizeof(LapItem),
                                 cudaMemcpyHostToDevice, st);
@@ -1024,7 +1016,7 @@ static cudaError_t lap_upload(Plan& p, const std::vector<LapItem>& items, const 
         const size_t smem = 3 * (size_t)p.q * p.q * sizeof(double);   // <= 96 KiB (q <= 64)
         e = cudaFuncSetAttribute(k_lap_kcheb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        e = cudaMalloc((void**)&p.d_lapK, nk * p.q * p.q * sizeof(double));
+        e = p.pool.bytes((void**)&p.d_lapK, nk * p.q * p.q * sizeof(double));
         if (e != cudaSuccess) return e;
         const bool gen = ell.empty();
         k_lap_kcheb<<<dim3((unsigned)(p.levels - 1), (unsigned)(p.levels - 1)), 256, smem, st>>>(
@@ -1034,13 +1026,24 @@ static cudaError_t lap_upload(Plan& p, const std::vector<LapItem>& items, const 
     return e;
 }
 
+// The arrays of a plan whose sizes follow from N and M (one block for them).
+static size_t lap_known_bytes(const Plan& p) {
+    const auto al = DevPool::rounded;
+    const size_t N = (size_t)p.N, M = (size_t)p.M;
+    size_t n = al(8 * N) + al(N) + al(4 * N) + al(8 * N) + al(8 * M) + al(M) + al(8 * M) + al(128 * sizeof(double));
+    if (p.small) n += 5 * al(4 * N) + al(8 * N) + al(N) + ((size_t)1 << 17);   // the sort's too
+    return n;
+}
+
 static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, int q,
                                    cudaStream_t st) {
     // interval ends and validity
     unsigned long long* dmx = nullptr;
     int* dflag = nullptr;
-    LAP_CUDA(cudaMalloc((void**)&dmx, 2 * sizeof(unsigned long long)), "cudaMalloc");
-    cudaError_t e = cudaMalloc((void**)&dflag, sizeof(int));
+    p.small = p.N <= kSmallPlan && p.M <= kSmallPlan;
+    cudaError_t e = p.pool.reserve(lap_known_bytes(p));
+    if (e == cudaSuccess) e = p.scratch().get(&dmx, 2);
+    if (e == cudaSuccess) e = p.scratch().get(&dflag, 1);
     unsigned long long mx[2] = {0, 0};
     int flag = 0;
     if (e == cudaSuccess) e = cudaMemsetAsync(dmx, 0, 2 * sizeof(unsigned long long), st);
@@ -1052,8 +1055,6 @@ static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, in
     if (e == cudaSuccess) e = cudaMemcpyAsync(mx, dmx, sizeof(mx), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, dflag, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(dmx);
-    cudaFree(dflag);
     LAP_CUDA(e, "fl_plan_laplace: node scan");
     if (flag) return lap_fail(FL_EINVAL, "fl_plan_laplace: a t_k or s_j is negative or not finite");
     double xi1, y1;
@@ -1075,19 +1076,19 @@ static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, in
     // copies of the nodes and their band ids
     const size_t N = (size_t)p.N, M = (size_t)p.M;
     if (N) {
-        LAP_CUDA(cudaMalloc((void**)&p.d_t, N * sizeof(double)), "cudaMalloc t");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_t, N * sizeof(double)), "cudaMalloc t");
         LAP_CUDA(cudaMemcpyAsync(p.d_t, t, N * sizeof(double), cudaMemcpyDeviceToDevice, st), "copy t");
-        LAP_CUDA(cudaMalloc((void**)&p.d_tband, N), "cudaMalloc t bands");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_tband, N), "cudaMalloc t bands");
         k_lap_band<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(p.N, p.d_t, xi1, P.levels, p.d_tband);
         LAP_CUDA(sort_t_by_band(p, st), "fl_plan_laplace: band order");
     }
     if (M) {
-        LAP_CUDA(cudaMalloc((void**)&p.d_s, M * sizeof(double)), "cudaMalloc s");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_s, M * sizeof(double)), "cudaMalloc s");
         LAP_CUDA(cudaMemcpyAsync(p.d_s, s, M * sizeof(double), cudaMemcpyDeviceToDevice, st), "copy s");
-        LAP_CUDA(cudaMalloc((void**)&p.d_sband, M), "cudaMalloc s bands");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_sband, M), "cudaMalloc s bands");
         k_lap_band<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(p.M, p.d_s, y1, P.levels, p.d_sband);
     }
-    LAP_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * kMaxQ * sizeof(double)), "cudaMalloc cheb");
+    LAP_CUDA(p.pool.bytes((void**)&p.d_cheb, 2 * kMaxQ * sizeof(double)), "cudaMalloc cheb");
     k_lap_cheb<<<1, 64, 0, st>>>(P.q, p.d_cheb);
     const size_t tsz = p.prec == FL_FP64 ? 8 : 4;
     if ((size_t)kLapWarps * (P.levels + 1) * (P.q + 1) * tsz > 200 * 1024)
@@ -1108,12 +1109,12 @@ static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, in
     }
     int* d_ell = nullptr;   // l_m for the table kernel
     double* Kt = nullptr;   // the blocks at the Chebyshev points
-    LAP_CUDA(cudaMalloc((void**)&p.d_lapKoff, koff.size() * sizeof(int64_t)), "cudaMalloc coupling offsets");
+    LAP_CUDA(p.pool.bytes((void**)&p.d_lapKoff, koff.size() * sizeof(int64_t)), "cudaMalloc coupling offsets");
     LAP_CUDA(cudaMemcpyAsync(p.d_lapKoff, koff.data(), koff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st),
              "copy coupling offsets");
     if (ktot > 0) {
-        LAP_CUDA(cudaMallocAsync((void**)&Kt, ktot * sizeof(double), st), "cudaMalloc coupling table");
-        LAP_CUDA(cudaMalloc((void**)&d_ell, ell.size() * sizeof(int)), "cudaMalloc l_m");
+        LAP_CUDA(p.scratch().get(&Kt, ktot), "cudaMalloc coupling table");
+        LAP_CUDA(p.scratch().get(&d_ell, (int64_t)ell.size()), "cudaMalloc l_m");
         e = cudaMemcpyAsync(d_ell, ell.data(), ell.size() * sizeof(int), cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) {
             k_lap_ktable<<<P.levels - 1, 256, 0, st>>>(P.levels, P.q, y1, xi1, d_ell, p.d_lapKoff, p.d_cheb, Kt);
@@ -1122,10 +1123,9 @@ static fl_status plan_laplace_impl(Plan& p, const double* t, const double* s, in
     }
     size_t scratch = 0;
     if (e == cudaSuccess) e = lap_upload(p, items, first, ell, ktot / (P.q * P.q), Kt, &scratch, st);
-    if (Kt) cudaFreeAsync(Kt, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the host arrays are released on return
-    cudaFree(d_ell);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     LAP_CUDA(e, "fl_plan_laplace: tables");
+    p.tmp.release();
     const size_t ts = p.prec == FL_FP64 ? 8 : 4;
     p.scratch_bytes = (double)scratch + (N + M) * (9.0 + 8.0);
     p.model_bytes = (double)N * (8 + 1 + ts) + (double)M * (8 + 1 + ts);
@@ -1150,8 +1150,10 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
                                    cudaStream_t st) {
     unsigned long long* dmx = nullptr;
     int* dflag = nullptr;
-    LAP_CUDA(cudaMalloc((void**)&dmx, 2 * sizeof(unsigned long long)), "cudaMalloc");
-    cudaError_t e = cudaMalloc((void**)&dflag, 2 * sizeof(int));
+    p.small = p.N <= kSmallPlan && p.M <= kSmallPlan;
+    cudaError_t e = p.pool.reserve(lap_known_bytes(p));
+    if (e == cudaSuccess) e = p.scratch().get(&dmx, 2);
+    if (e == cudaSuccess) e = p.scratch().get(&dflag, 2);
     unsigned long long mx[2] = {0, 0};
     int flag[2] = {0, 0};
     if (e == cudaSuccess) e = cudaMemsetAsync(dmx, 0, 2 * sizeof(unsigned long long), st);
@@ -1164,8 +1166,6 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
     if (e == cudaSuccess) e = cudaMemcpyAsync(mx, dmx, sizeof(mx), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(flag, dflag, sizeof(flag), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(dmx);
-    cudaFree(dflag);
     LAP_CUDA(e, "fl_plan_kernel: node scan");
     if (flag[0]) return lap_fail(FL_EINVAL, "fl_plan_kernel: a t_k or s_j is negative or not finite");
     if (flag[1]) return lap_fail(FL_EINVAL, "fl_plan_kernel: the K_1/2 kernel needs every t_k, s_j > 0");
@@ -1188,19 +1188,19 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
     p.bands.assign(levels + 1, BandHost());
     const size_t N = (size_t)p.N, M = (size_t)p.M;
     if (N) {
-        LAP_CUDA(cudaMalloc((void**)&p.d_t, N * sizeof(double)), "cudaMalloc t");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_t, N * sizeof(double)), "cudaMalloc t");
         LAP_CUDA(cudaMemcpyAsync(p.d_t, t, N * sizeof(double), cudaMemcpyDeviceToDevice, st), "copy t");
-        LAP_CUDA(cudaMalloc((void**)&p.d_tband, N), "cudaMalloc t bands");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_tband, N), "cudaMalloc t bands");
         k_lap_band<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(p.N, p.d_t, xi1, levels, p.d_tband);
         LAP_CUDA(sort_t_by_band(p, st), "fl_plan_kernel: band order");
     }
     if (M) {
-        LAP_CUDA(cudaMalloc((void**)&p.d_s, M * sizeof(double)), "cudaMalloc s");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_s, M * sizeof(double)), "cudaMalloc s");
         LAP_CUDA(cudaMemcpyAsync(p.d_s, s, M * sizeof(double), cudaMemcpyDeviceToDevice, st), "copy s");
-        LAP_CUDA(cudaMalloc((void**)&p.d_sband, M), "cudaMalloc s bands");
+        LAP_CUDA(p.pool.bytes((void**)&p.d_sband, M), "cudaMalloc s bands");
         k_lap_band<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(p.M, p.d_s, y1, levels, p.d_sband);
     }
-    LAP_CUDA(cudaMalloc((void**)&p.d_cheb, 2 * kGenMaxQ * sizeof(double)), "cudaMalloc cheb");
+    LAP_CUDA(p.pool.bytes((void**)&p.d_cheb, 2 * kGenMaxQ * sizeof(double)), "cudaMalloc cheb");
     k_lap_cheb<<<1, kGenMaxQ, 0, st>>>(qq, p.d_cheb);
     const size_t tsz = p.prec == FL_FP64 ? 8 : 4;
     if ((size_t)(levels + 1) * (qq + 1) * tsz > 200 * 1024)
@@ -1222,22 +1222,22 @@ static fl_status plan_general_impl(Plan& p, int kind, const double* t, const dou
             if (tb[k] == levels) near.push_back((int32_t)k);
         p.n_nearT = (int64_t)near.size();
         if (!near.empty()) {
-            LAP_CUDA(cudaMalloc((void**)&p.d_nearT, near.size() * sizeof(int32_t)), "cudaMalloc near field");
+            LAP_CUDA(p.pool.bytes((void**)&p.d_nearT, near.size() * sizeof(int32_t)), "cudaMalloc near field");
             LAP_CUDA(cudaMemcpyAsync(p.d_nearT, near.data(), near.size() * sizeof(int32_t),
                                      cudaMemcpyHostToDevice, st),
                      "copy near field");
         }
         nk = (int64_t)(levels - 1) * (levels - 1);
-        LAP_CUDA(cudaMallocAsync((void**)&Kt, nk * qq * qq * sizeof(double), st), "cudaMalloc coupling table");
+        LAP_CUDA(p.scratch().get(&Kt, nk * qq * qq), "cudaMalloc coupling table");
         k_gen_ktable<<<dim3((unsigned)(levels - 1), (unsigned)(levels - 1)), 256, 0, st>>>(kind, levels, qq, y1, xi1,
                                                                                           p.d_cheb, Kt);
     }
     LAP_CUDA(cudaGetLastError(), "fl_plan_kernel: launch");
     size_t scratch = 0;
     e = lap_upload(p, items, first, std::vector<int>(), nk, Kt, &scratch, st);
-    if (Kt) cudaFreeAsync(Kt, st);
     LAP_CUDA(e, "fl_plan_kernel: tables");
     LAP_CUDA(cudaStreamSynchronize(st), "fl_plan_kernel: synchronise");
+    p.tmp.release();
     p.scratch_bytes = (double)scratch + (N + M) * (9.0 + 8.0) + (double)nk * qq * qq * 8.0;
     p.model_bytes = (double)N * (8 + 1 + tsz) + (double)M * (8 + 1 + tsz);
     return FL_OK;

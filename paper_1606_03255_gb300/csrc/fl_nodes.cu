@@ -268,32 +268,25 @@ __global__ void k_cell_permute(int64_t n, const uint32_t* __restrict__ keys, con
     cell[i] = (int32_t)keys[i];
 }
 
-cudaError_t launch_cell_sort(Plan& p, int64_t off, int64_t n, int band, cudaStream_t st) {
+cudaError_t launch_cell_sort(Plan& p, int64_t off, int64_t n, int band, int bits, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const int64_t blocks = (n + 2047) / 2048;          // radix-sort tiles
-    const size_t kb = (n * 4 + 255) / 256 * 256;
-    unsigned char* tmp = nullptr;                       // keys, vals (twice), perm, nodes, histogram
-    cudaError_t e = cudaMallocAsync((void**)&tmp, 5 * kb + n * sizeof(double2) + 256 * blocks * 4, st);
-    if (e != cudaSuccess) return e;
-    uint32_t *keys = (uint32_t*)tmp, *keys2 = (uint32_t*)(tmp + kb);
-    int32_t *vals = (int32_t*)(tmp + 2 * kb), *vals2 = (int32_t*)(tmp + 3 * kb), *perm = (int32_t*)(tmp + 4 * kb);
-    double2* ws = (double2*)(tmp + 5 * kb);
-    uint32_t* hist = (uint32_t*)(tmp + 5 * kb + n * sizeof(double2));
+    uint32_t *keys = p.sort.keys, *keys2 = p.sort.keys2, *hist = p.sort.hist;
+    int32_t *vals = p.sort.vals, *vals2 = p.sort.vals2, *perm = p.sort.perm;
+    double2* ws = p.sort.ws;
     const unsigned grid = (unsigned)((n + 255) / 256);
-    e = cudaMemcpyAsync(perm, p.d_perm + off, n * 4, cudaMemcpyDeviceToDevice, st);
+    cudaError_t e = cudaMemcpyAsync(perm, p.d_perm + off, n * 4, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(ws, p.d_ws + off, n * sizeof(double2), cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) {
         k_cell_keys<<<grid, 256, 0, st>>>(n, p.d_cell + off, keys, vals);
-        e = radix_sort_pairs(keys, vals, keys2, vals2, hist, n, 32, st);
+        e = radix_sort_pairs(keys, vals, keys2, vals2, hist, n, bits, st);
     }
     if (e == cudaSuccess) {
         k_cell_permute<<<grid, 256, 0, st>>>(n, keys, vals, ws, perm, band, p.d_ws + off, p.d_perm + off,
                                              p.d_bandid + off, p.d_cell + off);
         e = cudaGetLastError();
     }
-    const cudaError_t e2 = cudaFreeAsync(tmp, st);
-    return e != cudaSuccess ? e : e2;
+    return e;
 }
 
 // Plan time: the entries of the fused gather.  A node's window of 2 m_w grid points

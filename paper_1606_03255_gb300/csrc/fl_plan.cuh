@@ -7,6 +7,7 @@
 
 #include <map>
 #include <string>
+#include <tuple>
 #include <utility>
 #include <vector>
 
@@ -96,6 +97,7 @@ struct DirectSeg {
     int64_t K;                 // frequencies 0 .. K - 1
     int64_t c_off;             // first coefficient of the transform
     int64_t dslot;             // offset of its partial sums (nodes x nchunk; nchunk > 1)
+    int64_t z_off;             // bases of its nodes: entries 2 (i + z_off) and the next of Plan::d_dz, i sorted
     int nchunk;                // chunks of kDirChunk coefficients
     int pin;                   // pinned transforms (kPinnedN): 1, or 2 with the blocks of a node summed in order
 };
@@ -175,7 +177,87 @@ constexpr int64_t kPinnedN = (int64_t)1 << 18;
 // sum the blocks of a node in order
 constexpr int64_t kDirSeqK = 256, kDirSeqNodes = 128;
 
+// Device memory of a plan, or of planning, given back together: small arrays share
+// blocks of 256 KiB, larger ones have their own, and reserve() makes one block for
+// the arrays that follow.  A cudaMalloc that the driver has to map memory for takes
+// 32 us and its cudaFree 28 (any size up to 64 MiB); ones that fit the 2 MiB it has
+// just mapped 1.6 us each.  Arrays of 2 MiB and more begin on a 2 MiB page, as
+// those of their own did (packed, they cost 0.5 % of a call at 300007 x 250001).
+class DevPool {
+public:
+    DevPool() = default;
+    DevPool(const DevPool&) = delete;
+    DevPool& operator=(const DevPool&) = delete;
+    ~DevPool() { release(); }
+    static size_t rounded(size_t n) {   // what an array of n bytes takes, at most
+        return n < kPage ? (n ? (n + 255) & ~(size_t)255 : 256) : ((n + kPage - 1) & ~(kPage - 1)) + kPage;
+    }
+    cudaError_t reserve(size_t n) {   // n: a sum of rounded sizes
+        if (n <= left_) return cudaSuccess;
+        void* b = nullptr;
+        const cudaError_t e = cudaMalloc(&b, n);
+        if (e != cudaSuccess) return e;
+        blocks_.push_back(b);
+        cur_ = (unsigned char*)b;
+        left_ = n;
+        return cudaSuccess;
+    }
+    cudaError_t bytes(void** p, size_t n) {
+        const size_t skip = n < kPage ? 0 : (size_t)(-(uintptr_t)cur_) & (kPage - 1);   // to the next page
+        n = n < kPage ? rounded(n) : (n + 255) & ~(size_t)255;
+        if (skip + n <= left_) {
+            cur_ += skip;
+            left_ -= skip;
+        } else if (n > kBlock / 4) {
+            const cudaError_t e = cudaMalloc(p, n);
+            if (e == cudaSuccess) blocks_.push_back(*p);
+            return e;
+        }
+        const cudaError_t e = n > left_ ? reserve(kBlock) : cudaSuccess;
+        if (e != cudaSuccess) return e;
+        *p = cur_;
+        cur_ += n;
+        left_ -= n;
+        return cudaSuccess;
+    }
+    template <typename T> cudaError_t get(T** p, int64_t count) { return bytes((void**)p, (size_t)count * sizeof(T)); }
+    void release() {
+        for (void* b : blocks_) cudaFree(b);
+        blocks_.clear();
+        cur_ = nullptr;
+        left_ = 0;
+    }
+
+private:
+    static constexpr size_t kBlock = (size_t)1 << 18, kPage = (size_t)1 << 21;
+    std::vector<void*> blocks_;
+    unsigned char* cur_ = nullptr;
+    size_t left_ = 0;
+};
+
+constexpr int64_t kSmallPlan = 4096;             // nodes (elements) up to which Plan::small
+constexpr size_t kOneBlock = (size_t)1 << 30;    // bytes up to which a plan's tables and grids are one allocation
+constexpr int64_t kTmpKeep = (int64_t)1 << 22;   // elements up to which planning keeps its scratch to the end
+
+// One way to split a band into P sub-band NFFTs (fl_api.cu).
+struct SplitOption {
+    int P, log2n, mc;
+    int64_t Kp, Nc;
+};
+
+// Planning's arrays for the radix sorts, used by one after the other on the stream.
+struct SortScratch {
+    uint32_t *keys = nullptr, *keys2 = nullptr, *hist = nullptr;
+    int32_t *vals = nullptr, *vals2 = nullptr, *perm = nullptr;
+    double2* ws = nullptr;
+};
+
 struct Plan {
+    DevPool pool;           // what the plan keeps (everything below that planning makes)
+    DevPool tmp;            // what planning needs, given back at its end
+    SortScratch sort;       // in scratch()
+    bool small = false;     // few nodes: planning's scratch shares the plan's block
+    DevPool& scratch() { return small ? pool : tmp; }
     int kind = 0;           // 0 Fourier-Laplace, 1 Laplace
     fl_precision prec = FL_FP32;
     int64_t N = 0, M = 0;
@@ -199,6 +281,7 @@ struct Plan {
     bool q_given = false;          // q is the caller's, not from eps
     bool own_gather = false;       // bands may have ranks of their own (see merge_bands)
     std::map<std::pair<int, int>, int> rank_memo;   // see merged_rank
+    mutable std::map<std::tuple<int64_t, double, int>, std::vector<SplitOption>> split_memo;   // see split_options
     std::vector<int> ranks;        // ranks of the tables d_cheb, d_cheb32, in order
     int route_mode = 0;            // 0 by cost, 1 all NFFT, 2 all direct
     int variant = 0;               // 0 Algorithm 2 weights, 1 one-sided interpolation
@@ -224,6 +307,7 @@ struct Plan {
     std::vector<DirectItem> direct_work, dadj_work;
     std::vector<DirectRange> direct_ranges;   // the segments of several chunks
     int64_t direct_nodes = 0;                 // their nodes
+    int64_t base_nodes = 0;                   // nodes with bases (d_dz)
     int64_t direct_terms = 0, dpart_elems = 0, direct_kmax = 0;
     int direct_threads = 256;                 // per CTA of the forward items
 
@@ -267,7 +351,8 @@ struct Plan {
     DirectRange* d_dranges = nullptr;
     DirectSeg* d_dsegs = nullptr;
     DirectItem* d_dadj = nullptr;
-    void* d_dz = nullptr;          // direct route: z_j, z_j^8 per sorted node (complex, the plan's arithmetic)
+    void* d_dz = nullptr;          // direct route: z_j, z_j^8 per node of a segment (complex, the plan's
+                                   // arithmetic; not where pinned forward steps form z themselves)
     void* d_dpart = nullptr;       // direct route: partial sums (complex T)
     void* d_cdir = nullptr;        // direct route adjoint: N complex
     // fused gather (FuseArgs): row-block starts, entries, window values, partial sums
@@ -338,7 +423,7 @@ struct FusedBand {
 };
 cudaError_t launch_fused_entries(const Plan& p, const FusedBand* list, int count, int64_t chunks, int nrb_max,
                                  bool fill, int32_t* hist, cudaStream_t st);
-cudaError_t launch_cell_sort(Plan& p, int64_t off, int64_t n, int band, cudaStream_t st);
+cudaError_t launch_cell_sort(Plan& p, int64_t off, int64_t n, int band, int bits, cudaStream_t st);
 cudaError_t launch_cell_shift(int32_t* cell, int64_t off, int64_t n, int shift, cudaStream_t st);
 
 // Launchers (fl_transform.cu)

@@ -109,8 +109,9 @@ __global__ void k_weights(BandDev B, int ellm, int Lm, int q, double xi1, int le
         Dk[0] = (T)inv_phi;
         return;
     }
-    if (one_sided) {
-        for (int s = 0; s < q; ++s) {
+    if (one_sided) {   // (blockIdx.y: a part of the points each)
+        const int per = (q + gridDim.y - 1) / gridDim.y, end = min(q, ((int)blockIdx.y + 1) * per);
+        for (int s = blockIdx.y * per; s < end; ++s) {
             const double ys = B.yc + B.yh * cheb[s];
             Dk[s * ds] = (T)(exp(-ys * xk) * inv_phi);
         }
@@ -157,7 +158,7 @@ static cudaError_t build_tables_t(Plan& p, const Instance& in, cudaStream_t st) 
         kt_max = std::max<int64_t>(kt_max, (int64_t)(bh.Lm - bh.ell + 1) * p.q * p.q);
     }
     if (kt_max > 0) {
-        e = cudaMallocAsync((void**)&Kt, kt_max * sizeof(double), st);
+        e = p.scratch().get(&Kt, kt_max);
         if (e != cudaSuccess) return e;
     }
     for (int lb = 1; lb <= in.levels; ++lb) {
@@ -173,17 +174,16 @@ static cudaError_t build_tables_t(Plan& p, const Instance& in, cudaStream_t st) 
             const BandDev& d = bh.dev.nsub > 0 ? p.bands[bh.dev.sub0 + c].dev : bh.dev;
             if (d.K == 0) continue;   // real exponents: none below the band's cut
             const bool merged = bh.leader >= 0;   // interpolation in y alone, at the merged band's points
-            k_weights<T><<<(unsigned)((d.K + 255) / 256), 256, 0, st>>>(
+            // few frequencies: the points over several blocks (17 us a band of 1024 frequencies
+            // and 12 points, nearly all of it exponentials in turn)
+            const bool one_sided = (merged || p.variant == 1) && d.nrhs > 1;
+            const dim3 grid((unsigned)((d.K + 255) / 256), one_sided && d.K < 65536 ? (unsigned)((d.nrhs + 3) / 4) : 1);
+            k_weights<T><<<grid, 256, 0, st>>>(
                 d, bh.ell, bh.Lm, merged ? d.nrhs : p.q, in.xi1, in.levels, p.d_cheb + 2 * d.choff, Kt, p.mw,
                 p.kb_b, merged ? 1 : p.variant, p.xi_mode ? p.d_xis : nullptr, (T*)p.d_D);
         }
     }
-    e = cudaGetLastError();
-    if (Kt) {
-        cudaError_t e2 = cudaFreeAsync(Kt, st);
-        if (e == cudaSuccess) e = e2;
-    }
-    return e;
+    return cudaGetLastError();
 }
 
 // Stage twiddles of the four-step passes (layout in fl_common.cuh): entry

@@ -228,8 +228,8 @@ template <typename T>
 static cudaError_t xi_tables_t(Plan& p, cudaStream_t st) {
     const int64_t N = p.N;
     const int m = p.mw;
-    cudaError_t e = cudaMalloc((void**)&p.d_xbk, std::max<int64_t>(N, 1) * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&p.d_xwin, std::max<int64_t>(N, 1) * 2 * m * sizeof(T));
+    cudaError_t e = p.pool.bytes((void**)&p.d_xbk, std::max<int64_t>(N, 1) * sizeof(int32_t));
+    if (e == cudaSuccess) e = p.pool.bytes(&p.d_xwin, std::max<int64_t>(N, 1) * 2 * m * sizeof(T));
     if (e != cudaSuccess) return e;
     if (N > 0)
         k_xi_win<T><<<(unsigned)((N + 255) / 256), 256, 0, st>>>(N, p.d_xis, m, p.kb_b, p.d_xbk,
@@ -242,7 +242,7 @@ static cudaError_t xi_tables_t(Plan& p, cudaStream_t st) {
         while (k < N && (int64_t)floor(2.0 * p.h_xis[k]) < B) ++k;
         start[B] = (int32_t)k;
     }
-    e = cudaMalloc((void**)&p.d_xstart, start.size() * sizeof(int32_t));
+    e = p.pool.bytes((void**)&p.d_xstart, start.size() * sizeof(int32_t));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(p.d_xstart, start.data(), start.size() * sizeof(int32_t),
                             cudaMemcpyHostToDevice, st);
@@ -267,7 +267,7 @@ static cudaError_t xi_tables_t(Plan& p, cudaStream_t st) {
     }
     p.xiphi_elems = tot;
     if (tot > 0) {
-        e = cudaMalloc(&p.d_xiphi, tot * sizeof(T));
+        e = p.pool.bytes(&p.d_xiphi, tot * sizeof(T));
         if (e != cudaSuccess) return e;
         for (int lg = 0; lg <= kMaxLog2n; ++lg) {
             if (off[lg] < 0) continue;
@@ -289,12 +289,12 @@ static cudaError_t xi_tables_t(Plan& p, cudaStream_t st) {
     p.xsb_n = (int)sb.size();
     p.xsb_blocks = blocks;
     if (!sb.empty()) {
-        e = cudaMalloc((void**)&p.d_xsb, sb.size() * sizeof(int2));
+        e = p.pool.bytes((void**)&p.d_xsb, sb.size() * sizeof(int2));
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(p.d_xsb, sb.data(), sb.size() * sizeof(int2), cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return e;
     }
-    e = cudaMalloc(&p.d_xcs, std::max<int64_t>(N, 1) * sizeof(C_t<T>));
+    e = p.pool.bytes(&p.d_xcs, std::max<int64_t>(N, 1) * sizeof(C_t<T>));
     if (e != cudaSuccess) return e;
     // the band table with phi_off
     std::vector<BandDev> hb(p.bands.size());
