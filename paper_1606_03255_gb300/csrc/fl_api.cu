@@ -100,22 +100,6 @@ static int onesided_rank(double eps_K) {
     return kMaxQ + 1;
 }
 
-// FP64 plans that merge a directly summed band (merge_bands) take windows one
-// point wider on each side: nodes without a window error come under one, 1.2 times
-// the error against 64 bits of the bands before (5.5e-14 against 4.5e-14 at N = M =
-// 3000, eps = 1e-10).  A point more divides the window's error by
-// e^(2 pi sqrt(1 - 1/sigma)) (85 at sigma = 2: 8.7e-16 there) and costs two taps per
-// node and right-hand side.
-static void widen_windows(Plan& p) {
-    p.mw_extra = 1;
-    p.mw = std::min(12, p.mw + 1);
-}
-
-// The half-width of a sub-band NFFT of oversampling sigma.
-static int split_width(const Plan& p, double sigma) {
-    return std::min(12, window_width(p.eps_A, sigma) + p.mw_extra);
-}
-
 static fl_status select_common(Plan& p, int q_in) {
     p.eps_K = p.eps / 3.0;
     p.eps_A = p.eps / 3.0;
@@ -132,7 +116,6 @@ static fl_status select_common(Plan& p, int q_in) {
     // the latter's error amplified by up to Phi(0)/Phi(1/4) < 8 in the division
     // by Phi(x/2): each gets eps_A / 8
     p.mw = window_width(p.xi_mode ? p.eps_A / 8.0 : p.eps_A, 2.0);
-    p.mw_extra = 0;
     p.kb_b = M_PI * (2.0 - 1.0 / 2.0);
     return FL_OK;
 }
@@ -638,7 +621,7 @@ static const std::vector<SplitOption>& split_options(const Plan& p, int64_t K, d
         const int64_t n = (int64_t)1 << lg;
         if ((double)n >= 2.0 * (double)Nc) continue;   // no gain over sigma = 2
         // the half-width this sigma needs, and the FP32 limit at it
-        const int mc = std::max(mw, split_width(p, (double)n / (double)Nc));
+        const int mc = std::max(mw, window_width(p.eps_A, (double)n / (double)Nc));
         if (deconv_gain((double)n / (double)Nc, mc) > gain_max) continue;
         v.push_back({P, lg, mc, Kp, Nc});
     }
@@ -716,7 +699,7 @@ static fl_status plan_splits(Plan& p, const std::vector<int>& nfft, cudaStream_t
             smin_used = std::min(smin_used, ldexp(1.0, c.log2n) / (double)c.Nc);
         }
     if (!any) return FL_OK;
-    p.mw = std::max(p.mw, split_width(p, smin_used));
+    p.mw = std::max(p.mw, window_width(p.eps_A, smin_used));
     p.sigma_min = smin_used;
     for (size_t i = 0; i < nfft.size(); ++i) {
         const SplitChoice c = best_ch[i];
@@ -833,6 +816,19 @@ static int merged_rank(Plan& p, double a, int octaves, double xmax, double tol) 
     return r;
 }
 
+// FP64 plans that merge a directly summed band take windows one point wider on
+// each side: nodes without a window error come under one, 1.2 times the error
+// against 64 bits of the bands before (5.5e-14 against 4.5e-14 at N = M = 3000, eps =
+// 1e-10).  A point more divides the window's error by e^(2 pi sqrt(1 - 1/sigma)) (85
+// at sigma = 2: 8.7e-16 there) and costs two taps per node and right-hand side.  Not
+// below kWindowEps, where the NFFT errs by rounding (at 1e-12 1.0e-15 either way), and
+// not where the gain would pass its limit.
+constexpr double kWindowEps = 0x1p-36;
+static void widen_windows(Plan& p) {
+    if (p.prec != FL_FP64 || !p.merged_direct || p.eps < kWindowEps || p.mw >= 12) return;
+    if (deconv_gain(p.sigma_min, p.mw + 1) <= deconv_gain_limit64(p.eps_A)) ++p.mw;
+}
+
 // Estimated cost of an NFFT band (the units of route_of), at its best split.
 static double nfft_cost(const Plan& p, const BandHost& bh) {
     double best = 0.0;
@@ -913,7 +909,7 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
         const int i = best[j].from, r = best[j].rank;
         if (r == 0) continue;
         for (int t = i; t < j; ++t)
-            if (p.prec == FL_FP64 && p.mw_extra == 0 && p.bands[in.band_base + list[t]].dev.route == 2) widen_windows(p);
+            p.merged_direct |= p.bands[in.band_base + list[t]].dev.route == 2;
         const int lead = in.band_base + list[i];
         const BandHost g = merged(i, j - 1, r);
         for (int t = i; t < j; ++t) {
@@ -1042,7 +1038,7 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     p.z0_nodes = 0;
     p.ranks.assign(1, p.q);
     p.qmax = p.q;
-    p.own_gather = false;
+    p.own_gather = p.merged_direct = false;
     for (const Instance& in : p.inst) p.own_gather = p.own_gather || !pinned(p, in);
     std::vector<int> nfft_bands;   // bands evaluated by an NFFT, in order
     for (int i = 0; i < B; ++i) {
@@ -1083,6 +1079,7 @@ static fl_status plan_multi(Plan& p, int B, const int64_t* Ns, const int64_t* Ms
     }
     // oversampling from the tolerance: split sparse bands into sub-bands
     if ((s = plan_splits(p, nfft_bands, st)) != FL_OK) return s;
+    widen_windows(p);
     // a transform that copies its twin's nodes shares its twin's weight tables
     // (same N, bands and splits); shares_D[i] records that every band did
     std::vector<char> shares_D(B, 0);

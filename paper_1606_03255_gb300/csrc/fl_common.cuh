@@ -139,16 +139,18 @@ template <typename T> __device__ __forceinline__ T kb_window(T t, T m, T b) {
     return sinh(b * r) / r;
 }
 
-// u - v (u >= v >= 0, each as high + low part): its square root as r + *rlo.
-__device__ __forceinline__ double root_of_difference(double uh, double ul, double vh, double vl, double* rlo) {
+// u - v (u >= v >= 0, each as high + low part): its square root as r + *rlo, and 1 / r.
+__device__ __forceinline__ double root_of_difference(double uh, double ul, double vh, double vl, double* rlo,
+                                                     double* inv) {
     const double d = uh - vh, e = ((uh - d) - vh) + (ul - vl);
     const double s = d + e;
     if (!(s > 0.0)) {
-        *rlo = 0.0;
+        *rlo = *inv = 0.0;
         return 0.0;
     }
     const double r = sqrt(s);
-    *rlo = (fma(-r, r, s) + (e - (s - d))) / (2.0 * r);
+    *inv = 1.0 / r;
+    *rlo = (fma(-r, r, s) + (e - (s - d))) * (0.5 * *inv);
     return r;
 }
 
@@ -159,12 +161,12 @@ __device__ __forceinline__ double root_of_difference(double uh, double ul, doubl
 __device__ __forceinline__ double kb_window_exact(double fr, double c, double m, double b) {
     const double th = fr + c, tl = fr - (th - c);       // c an integer, |c| >= 1 or c = 0
     const double h = th * th;
-    double rl;
-    const double r = root_of_difference(m * m, 0.0, h, fma(th, th, -h) + 2.0 * th * tl, &rl);
+    double rl, inv;
+    const double r = root_of_difference(m * m, 0.0, h, fma(th, th, -h) + 2.0 * th * tl, &rl, &inv);
     if (r == 0.0) return b;
     const double a = b * r, al = fma(b, r, -a) + b * rl;
     const double v = sinh(a);
-    return fma(al, fmax(v, 1.0), v) / r;                // sinh(a + al), cosh a ~ max(sinh a, 1)
+    return fma(al, fmax(v, 1.0), v) * inv;              // sinh(a + al), cosh a ~ max(sinh a, 1)
 }
 
 // I_0(m sqrt(b^2 - (2 pi nu)^2)), likewise (nu exact; the argument is well above 1
@@ -173,8 +175,8 @@ __device__ __forceinline__ double kb_transform_exact(double nu, double m, double
     constexpr double kH = 6.283185307179586, kL = 2.4492935982947064e-16;   // 2 pi
     const double v = kH * nu, vl = fma(kH, nu, -v) + kL * nu;
     const double bb = b * b, vv = v * v;
-    double rl;
-    const double r = root_of_difference(bb, fma(b, b, -bb), vv, fma(v, v, -vv) + 2.0 * v * vl, &rl);
+    double rl, inv;
+    const double r = root_of_difference(bb, fma(b, b, -bb), vv, fma(v, v, -vv) + 2.0 * v * vl, &rl, &inv);
     const double a = m * r, al = fma(m, r, -a) + m * rl;
     const double i0 = cyl_bessel_i0(a);
     return a > 1.0 ? fma(i0 * (1.0 - 0.5 / a), al, i0) : i0;                 // I_1 ~ I_0 (1 - 1 / (2 a))

@@ -276,7 +276,7 @@ struct Plan {
     int fuse_mode = 0;             // window gather in pass 2: 0 by cost, 1 never, 2 wherever possible
     int sigma_mode = 0;            // oversampling: 0 by cost, 1 sigma = 2, 2 sub-bands wherever allowed
     double sigma_min = 2.0;        // smallest oversampling of the plan's grids
-    int mw_extra = 0;              // points added to every window half-width (see widen_windows)
+    bool merged_direct = false;    // a band that would be summed directly was merged (see widen_windows)
     int qmax = 0;                  // largest rank of a band (q unless bands were merged)
     bool q_given = false;          // q is the caller's, not from eps
     bool own_gather = false;       // bands may have ranks of their own (see merge_bands)
