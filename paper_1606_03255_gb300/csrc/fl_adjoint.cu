@@ -612,8 +612,11 @@ __global__ void k_z0_sum(int64_t z0, const int32_t* __restrict__ perm,
 // b_s[(k - k0 - N_m/2) mod n], one thread per k over a plan-time list of the grids
 // (three fields decide whether a grid holds k; the walk over the band table
 // read 200 bytes per band and thread).  Bound by reading D and the grids once;
-// the sums in the plan's arithmetic (float pairs: in pairs, where double took
-// 185 us of FP64 conversions and products at N = 2^18).
+// the sums in the plan's arithmetic.  Float pairs: in pairs, where double took
+// 185 us of FP64 conversions and products at N = 2^18; a term adds a rounding of
+// 2^-46 of the sum of the terms' magnitudes, so the up to 130 terms of a frequency
+// add 130^(1/2) 2^-46 = 1.6e-13 of it, below the 2^-46 of each of the 40 layers of
+// FFTs times the gain of 8.6 before it (measured: 4.6e-14 at N = M = 2^18, eps = 1e-12).
 template <typename A, typename O>
 __global__ void __launch_bounds__(128)
     k_combine(int64_t N, int n_items, const CombineItem* __restrict__ items, const A* __restrict__ D,

@@ -254,12 +254,16 @@ static fl_status select_bands(Plan& p, Instance& in, int inst_index) {
 
 // Route of a non-empty band: NFFT with nrhs right-hand sides, or the direct sum
 // over its K frequencies.  Costs in issued instructions: an FFT grid point
-// ~ (log2 n + 8) over both passes and the prep (twice that in double, whose
-// twiddles come from double sincospi); per gathered node, 2 per tap and
-// right-hand side plus the window (2 m_w sinh/sqrt) and the barycentric
-// divisions, both several times dearer in double on this part; a fixed launch
-// and latency share per NFFT band; a direct term ~ 6 (one complex Horner step
-// and its share of the block's phase).
+// ~ (log2 n + 8) over both passes and the prep (twice that in double); per
+// gathered node, 2 per tap and right-hand side plus the window (2 m_w
+// sinh/sqrt) and the barycentric divisions, both several times dearer in
+// double on this part; a fixed launch and latency share per NFFT band; a direct
+// term ~ 6 (one complex Horner step and its share of the block's phase).  The
+// constants were fitted when double twiddles, windows and weights were formed in
+// the call.  Twiddles now come from tables, and so do the taps and weights of
+// single FP64 and float-pair plans, so there the model charges an NFFT more than
+// it costs and leaves bands to the direct sum; batches form the windows and
+// weights in the call as before.
 static int route_of(const Plan& p, const BandHost& bh) {
     if (p.route_mode == 1) return 1;
     if (p.route_mode == 2) return 2;
@@ -326,10 +330,10 @@ static void build_direct_items(Plan& p) {
         const int64_t nblk = (std::min<int64_t>(s.K, kDirChunk) + kDirBlock - 1) / kDirBlock;
         return std::min(5, ilog2_ceil(s.pin ? nblk : (nblk + r - 1) / r));
     };
-    // few items (a small transform) in FP64 or pairs: CTAs of 64 threads, so that
-    // all SMs take part (46 CTAs of 256 threads at N = M = 1024 in FP64).  FP32 keeps
-    // 256: staging the coefficients is its larger part (3001 x 2500: 24.0 us, 28.7
-    // with 64)
+    // few items (a small transform) in FP64: CTAs of 64 threads, so that all SMs
+    // take part (46 CTAs of 256 threads at N = M = 1024).  FP32 and float pairs keep 256:
+    // staging the coefficients is their larger part (FP32 3001 x 2500: 24.0 us, 28.7
+    // with 64; pairs 17576 x 266: 30.9, 39.1 with 64)
     p.direct_threads = 256;
     auto items = [&](int passes, bool make) {
         int64_t count = 0;
@@ -346,7 +350,7 @@ static void build_direct_items(Plan& p) {
         return count;
     };
     const int64_t full = items(1, false);
-    if (np == 1 && full < 2 * kSMs) p.direct_threads = 64;
+    if (p.prec == FL_FP64 && full < 2 * kSMs) p.direct_threads = 64;
     items(full >= 16 * kSMs ? 2 : 1, true);
     if (p.batched) return;   // forward only
     auto adj_items = [&](int64_t steps, bool make) {
@@ -419,7 +423,7 @@ static double unfused_cost(int64_t nodes, int nrhs, int mw) {
 }
 
 // FP32 transforms that may merge bands (not pinned): the same with the traffic
-// of the grids and partial sums, in the same units (0.26 ps: an FFT point costs
+// of the grids and partial sums (constants from N = M = 2^20), in the same units (0.26 ps: an FFT point costs
 // log2 n + 8 of them, 7 ps measured at N = M = 2^20; a byte of HBM about 0.56).
 // A gather from the grid pays for writing it and reads it once, or 128 bytes
 // per node, whichever is less (it measured 0.16 ms for 1.5*10^5 nodes and 35
@@ -868,6 +872,15 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
         // eps = 1e-12 leaves 6e-18)
         if (p.prec != FL_FP32) tol = std::max(tol, ldexp(1.0, -54));
     }
+    // A direct term is dearer in the model than in fact, next to an NFFT of many
+    // right-hand sides.  FP64 and float pairs at eps = 1e-10, N = 1024 to 65536, M =
+    // 1000 to 10000 near the circle: with estimates 1.4 to 3.9 times the merged
+    // band's the direct sums were faster (16384 x 3000, 3.9: 259 us against 439
+    // merged; 65536 x 1000, 1.4: 273 against 768; pairs 1024 x 10000, 3.8: 58 against
+    // 84), from 5.8 on the merged band (4096 x 10000, 5.8: 222 against 159; 65536 x
+    // 10000, 6.9: 2057 against 1487).  FP32 at 1e-6: 270001 x 3000 78 us against 312,
+    // 600000 x 6000 171 against 293 (merged at a share of 4.5).
+    const double direct_share = p.prec == FL_FP32 ? 7.0 : 4.5;
     struct Part {
         double cost;
         int from, rank;
@@ -889,8 +902,9 @@ static fl_status merge_bands(Plan& p, const Instance& in, cudaStream_t st) {
     std::vector<int> floor_rank(n, 2);               // known of the interval from candidate i on
     for (int j = 0; j < n; ++j) {
         const BandHost& alone = p.bands[in.band_base + list[j]];
-        const double single = alone.dev.route == 2 ? (double)alone.nodes * alone.dev.K * 6.0 * p.direct_bias
-                                                   : nfft_cost(p, alone);
+        const double single = alone.dev.route == 2
+                                  ? (double)alone.nodes * alone.dev.K * 6.0 * p.direct_bias / direct_share
+                                  : nfft_cost(p, alone);
         best[j + 1] = Part{best[j].cost + single, j, 0};
         int least = 2;   // the rank grows with the interval: no less than those of parts of it
         for (int i = j; i >= 0; --i) {
@@ -1314,7 +1328,7 @@ static uint64_t plan_signature(const Plan& p, const PlanSpec& sp) {
     mix((uint64_t)sp.fuse_mode);
     mix((uint64_t)sp.rhs_per_launch);
     for (const Instance& in : p.inst) mix((uint64_t)(in.twin + 1));
-    for (const BandHost& bh : p.bands) mix((uint64_t)bh.nodes * 131 + (uint64_t)bh.local);
+    for (const BandHost& bh : p.bands) mix((uint64_t)bh.own * 131 + (uint64_t)bh.local);   // before merging
     return h;
 }
 

@@ -168,10 +168,14 @@ struct Timer {
 };
 
 // FP32 transforms of at most this many coefficients (integer exponents) keep the
-// rounding of every forward step, bit for bit: their node gradients leave
-// through autograd in double and are compared at that precision at these
-// sizes, where any other rounding of the FP32 steps (about 10^-7) shows; a
-// transform of a batch equals the single plan's bit for bit, so both do.
+// rounding of every forward step, bit for bit.  No accuracy asks for it: their
+// node gradients leave through autograd as doubles that hold FP32 values, and a
+// caller who compares such gradients from one version to the next in double
+// would see any other rounding (about 10^-7).  2^18 is the size of the gradient
+// workload; above it the steps round as is fastest.  A batch of such transforms
+// equals the single plans bit for bit where both choose the same window; in a
+// batch with a larger one the gather is the one compiled for bands of several
+// ranks, whose rounding may differ in the last place.
 constexpr int64_t kPinnedN = (int64_t)1 << 18;
 // pinned transforms: bands with K <= kDirSeqK and at least kDirSeqNodes nodes
 // sum the blocks of a node in order
