@@ -147,15 +147,17 @@ def method_bytes(info: dict, q: int, cs: int = 8, n_min: int = 0) -> float:
     """Bytes the method moves through the band grids per execute (its per-unit
     figure): one grid write and one read per right-hand side of every
     NFFT, 2 cs n each (cs = bytes per complex; a band evaluated as P sub-band
-    NFFTs has P grids of band_n points); only grids above n_min."""
+    NFFTs has P grids of band_n points); only grids above n_min.  The right-hand
+    sides are the plan's (band_rhs: bands evaluated together count once), or q
+    of every band but the last where the plan does not say."""
     total = 0.0
     L = info["levels"]
     parts = info.get("band_parts") or [1] * (L + 1)
+    rhs = info.get("band_rhs") or [q] * L + [1]
     for b in range(1, L + 1):
         if info["band_route"][b] != 1 or info["band_n"][b] <= n_min:
             continue
-        nrhs = 1 if b == L else q
-        total += nrhs * parts[b] * 2.0 * cs * info["band_n"][b]
+        total += rhs[b] * parts[b] * 2.0 * cs * info["band_n"][b]
     return total
 
 

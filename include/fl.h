@@ -425,6 +425,13 @@ fl_status fl_laplace_real_noalloc(int64_t N, int64_t M, const double *t_dev,
 /* Plan parameters and sizes (host call, no device work). */
 fl_status fl_get_info(fl_plan_t p, fl_info *info);
 
+/* Right-hand sides of band b's grids, b < count (host call; count at most
+ * FL_MAX_LEVELS; bands as in fl_info, index 0 and bands beyond the plan's get 0).
+ * 0 also for empty and directly summed bands and for bands that are evaluated
+ * together with an earlier one, whose entry has the right-hand sides of all of
+ * them (fl_info gives such bands the route, grid size and parts of that one). */
+fl_status fl_get_band_rhs(fl_plan_t p, int *rhs, int count);
+
 /* Enable (1) or disable (0) per-kernel CUDA-event timing; resets counters. */
 fl_status fl_set_timing(fl_plan_t p, int enable);
 

@@ -185,9 +185,10 @@ __device__ __forceinline__ ffc adj_phase(int64_t, const uint4*, const double2*, 
 // plan-time range: consecutive in cell order) are staged in shared memory with
 // their taps, weights and phased values, and a thread sums its few covering
 // nodes in registers.  A thread per cell that searched its nodes and kept all
-// sums in local memory took 430 us for 4.3*10^6 cells at 300007 x 250001; blocks
-// of 256 cells that went over the right-hand sides in turn, staging again,
-// 318 us for 1.6*10^6.
+// sums in local memory took 430 us for 4.3*10^6 cells at 300007 x 250001 (97 us
+// now); blocks of 256 cells that went over the right-hand sides in turn, staging
+// again, 318 us for 1.6*10^6.  On the 2^18 disk nodes 40 % of the issue slots and
+// 34 % of L1 are used, with the staging loads' latency beside them.
 constexpr int kSpThreads = 256, kSpTile = 128, kSpQ = 8;
 
 template <typename T> static size_t sp_smem(int mw, int q) {
@@ -304,8 +305,9 @@ template <int H, int OFF, typename T> __device__ __forceinline__ void adj_halve(
 // sides per warp (WPG = 1), or per CTA where the covering nodes are several
 // hundred (WPG = 8); the lanes stride over the nodes (plan-time cell starts), the
 // sums in registers -- a node's weights are read once for CG cells -- then a
-// halving exchange, and the warps in order.  A CTA per cell with the sums in
-// local memory took 82 us on the 2^18 disk nodes in FP32 and 222 us in pairs.
+// halving exchange, and the warps in order.  Bound by load latency at 20 % of
+// the warps (115 registers): 17 and 20 us on the 2^18 disk nodes in FP32, where a CTA
+// per cell with the sums in local memory took 82 us (222 us in pairs).
 template <typename T> struct SpreadDense {
     static constexpr int CG = sizeof(T) == 4 ? 4 : 2;
 };
@@ -611,8 +613,9 @@ __global__ void k_z0_sum(int64_t z0, const int32_t* __restrict__ perm,
 // c_out[k] = [k == 0] z0sum + cdir[k] + sum over the grids of sum_s D[s][k - k0]
 // b_s[(k - k0 - N_m/2) mod n], one thread per k over a plan-time list of the grids
 // (three fields decide whether a grid holds k; the walk over the band table
-// read 200 bytes per band and thread).  Bound by reading D and the grids once;
-// the sums in the plan's arithmetic.  Float pairs: in pairs, where double took
+// read 200 bytes per band and thread).  Bound by the latency of its loads of D and
+// the grids (N = M = 2^18 FP32: 23 warps waiting on them per issue, DRAM at 12 % of its
+// peak); the sums in the plan's arithmetic.  Float pairs: in pairs, where double took
 // 185 us of FP64 conversions and products at N = 2^18; a term adds a rounding of
 // 2^-46 of the sum of the terms' magnitudes, so the up to 130 terms of a frequency
 // add 130^(1/2) 2^-46 = 1.6e-13 of it, below the 2^-46 of each of the 40 layers of

@@ -1899,6 +1899,15 @@ fl_status fl_execute_batched_ptrs(fl_plan_t h, const void* const* c_host, void* 
     return FL_OK;
 }
 
+fl_status fl_get_band_rhs(fl_plan_t h, int* rhs, int count) {
+    if (!h || !rhs || count < 0 || count > FL_MAX_LEVELS) return fail(FL_EINVAL, "fl_get_band_rhs: invalid argument");
+    const Plan& p = h->p;
+    const int nb = p.kind == 0 && !p.inst.empty() ? p.inst[0].levels + 1 : 0;
+    for (int b = 0; b < count; ++b)
+        rhs[b] = b > 0 && b < nb && p.bands[b].dev.route == 1 ? p.bands[b].dev.nrhs : 0;
+    return FL_OK;
+}
+
 fl_status fl_get_info(fl_plan_t h, fl_info* info) {
     if (!h || !info) return fail(FL_EINVAL, "fl_get_info: NULL argument");
     const Plan& p = h->p;

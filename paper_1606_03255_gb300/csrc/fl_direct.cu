@@ -209,7 +209,9 @@ __device__ __forceinline__ void dir_write(const DirectSeg& S, int64_t i, int chu
 // Horner blocks l, l + G, ... of the chunk, so that a segment of few frequencies
 // keeps all lanes busy: a whole warp per node left 30 of 32 lanes idle at K =
 // 64.  Bound by the FMA pipe of its arithmetic (4 operations a term; FP64: 16
-// cycles of the SM per warp instruction, active lanes or not).  The FP32 form
+// cycles of the SM per warp instruction, active lanes or not, 93 % of the pipe at N
+// = M = 2^18), the FP32 form there by the staging loads too (FMA pipe 40 %).  The
+// FP32 form
 // steps two nodes at once in packed pairs (fl_f32x2.cuh), 5 issues per term and
 // node pair against 2 x 7.
 //
@@ -378,7 +380,8 @@ __global__ void k_direct_reduce(int nranges, const DirectRange* __restrict__ ran
 // groups).  The FP32 form steps two nodes at once in packed pairs.  The node
 // groups are cut so that the launch has several warps per SM: at 256 nodes each
 // the K = 512 band of N = M = 2^18 disk nodes had 160 warps (float pairs:
-// 570 us, and the bands with K <= 256 in double 990 us).
+// 570 us, and the bands with K <= 256 in double 990 us).  Still bound by its few
+// warps there (14 % active, 18 % of the issue slots).
 constexpr int kAdjKL = kDirAdjKL;
 static_assert(kAdjKL == 16, "two chains of eight steps");
 

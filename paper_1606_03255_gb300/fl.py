@@ -36,7 +36,7 @@ EXPORTED = ["fl_plan", "fl_plan_ex", "fl_plan_batched", "fl_execute_batched", "f
             "fl_execute_batched_ptrs", "fl_execute", "fl_execute_deriv", "fl_grad_w", "fl_execute_host",
             "fl_adjoint", "fl_transposed", "fl_plan_xi",
             "fl_plan_laplace", "fl_plan_kernel", "fl_laplace_real", "fl_laplace_real_noalloc", "fl_get_info",
-            "fl_set_timing", "fl_get_timing", "fl_destroy", "fl_last_error", "fl_version"]
+            "fl_get_band_rhs", "fl_set_timing", "fl_get_timing", "fl_destroy", "fl_last_error", "fl_version"]
 
 
 class fl_info(ctypes.Structure):
@@ -138,6 +138,7 @@ def load(path: str | None = None):
         "fl_laplace_real": [vp, vp, vp, vp],
         "fl_laplace_real_noalloc": [i64, i64, vp, vp, vp, vp, ci, cd, ci, vp],
         "fl_get_info": [vp, ctypes.POINTER(fl_info)],
+        "fl_get_band_rhs": [vp, ctypes.POINTER(ci), ci],
         "fl_set_timing": [vp, ci],
         "fl_get_timing": [vp, ctypes.POINTER(fl_timing)],
         "fl_destroy": [vp],
@@ -269,6 +270,12 @@ def fl_get_info(plan):
     info = fl_info()
     st = load().fl_get_info(plan, ctypes.byref(info))
     return st, info
+
+
+def fl_get_band_rhs(plan, count):
+    rhs = (ctypes.c_int * max(int(count), 1))()
+    st = load().fl_get_band_rhs(plan, rhs, int(count))
+    return st, list(rhs)[:max(int(count), 0)]
 
 
 def fl_set_timing(plan, enable):
@@ -456,7 +463,9 @@ class Plan:
     def info(self) -> dict:
         st, inf = fl_get_info(self._handle)
         check(st, "fl_get_info")
-        return info_dict(inf)
+        st, rhs = fl_get_band_rhs(self._handle, inf.levels + 1)
+        check(st, "fl_get_band_rhs")
+        return {**info_dict(inf), "band_rhs": rhs}
 
     def set_timing(self, enable: bool):
         check(fl_set_timing(self._handle, enable), "fl_set_timing")
